@@ -4,8 +4,9 @@
 
 namespace mpsvqe {
 
+// Aligned to its size, so that one entry moves as one 64- or 128-bit load or store.
 template <class R>
-struct Cx {
+struct alignas(2 * sizeof(R)) Cx {
   R x, y;
 };
 
@@ -50,6 +51,22 @@ __device__ __forceinline__ void cmac_conj(Cx<R>& acc, Cx<R> a, Cx<R> b) {
   acc.x = fma(a.x, b.x, acc.x);
   acc.x = fma(a.y, b.y, acc.x);
   acc.y = fma(a.x, b.y, acc.y);
+  acc.y = fma(-a.y, b.x, acc.y);
+}
+// acc += a * conj(b)
+template <class R>
+__device__ __forceinline__ void cmac_bconj(Cx<R>& acc, Cx<R> a, Cx<R> b) {
+  acc.x = fma(a.x, b.x, acc.x);
+  acc.x = fma(a.y, b.y, acc.x);
+  acc.y = fma(-a.x, b.y, acc.y);
+  acc.y = fma(a.y, b.x, acc.y);
+}
+// acc -= a * b
+template <class R>
+__device__ __forceinline__ void cmsub(Cx<R>& acc, Cx<R> a, Cx<R> b) {
+  acc.x = fma(-a.x, b.x, acc.x);
+  acc.x = fma(a.y, b.y, acc.x);
+  acc.y = fma(-a.x, b.y, acc.y);
   acc.y = fma(-a.y, b.x, acc.y);
 }
 template <class R>

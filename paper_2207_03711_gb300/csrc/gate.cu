@@ -1,0 +1,1152 @@
+// The gate engine: persistent kernel that applies a list of two-site gates to each MPS
+// slot, one thread-block cluster per slot.
+//
+// Per gate: Eq. (7) contraction and 4x4 gate, Eq. (8) row scaling by lambda_{n-1}, Eq. (9)
+// truncated SVD (bidiagonal route; one-sided Jacobi for spectra that stay degenerate),
+// Eq. (10) updates. One evaluation's gate chain is serial, so what a gate costs is its own
+// latency; a cluster of C blocks spreads every stage of it over C SMs, and keeps M' in
+// distributed shared memory where one block's is too small. C depends on the precision and
+// the bond cap only, never on how many slots run together, so a slot's result does not
+// depend on its company.
+#include <cstring>
+#include <mutex>
+
+#include "../../include/mpsvqe.h"
+#include "gate.cuh"
+
+namespace mpsvqe {
+
+template <class R>
+struct Eps;
+template <>
+struct Eps<double> {
+  static constexpr double v = 2.220446049250313e-16;
+};
+template <>
+struct Eps<float> {
+  static constexpr float v = 1.1920929e-7f;
+};
+
+// Algorithmic real flops of one gate step, counted as the textbook dense algorithms:
+// contraction theta = B_n B_{n+1} (2 rl x rm x 2 rr complex MACs), the 4x4 gate on
+// (i, j), Golub-Reinsch SVD of the (m x n) complex M' computing singular values and
+// right vectors (4 (4 m n^2 + 8 n^3) real flops for m >= n, roles swapped otherwise),
+// and the site update B_n = M V^H (2 rl x 2 rr x k complex MACs). A complex MAC is 8.
+__device__ __forceinline__ double flops_per_gate(int rl, int rm, int rr, int k) {
+  const float m = 2.0f * rl, n = 2.0f * rr;   // products stay below 2^31: exact enough for a count
+  const float big = m >= n ? m : n, small = m >= n ? n : m;
+  const double contract = 8.0f * m * rm * n + 8.0f * 4.0f * m * n;
+  const double svd = 4.0f * (4.0f * big * small * small + 8.0f * small * small * small);
+  const double update = 8.0f * m * n * k;
+  return contract + svd + update;
+}
+
+// Capacity of bond b (b = -1 and b = n-1 are the trivial outer bonds): the largest rank
+// an n-site MPS with bond cap chi can have there, min(chi, 2^min(b+1, n-1-b)).
+__device__ __forceinline__ int bond_cap(int b, int n, int chi) {
+  if (b < 0 || b >= n - 1) return 1;
+  const int e = min(min(b + 1, n - 1 - b), 30);
+  return min(chi, 1 << e);
+}
+
+namespace gate {
+
+// Shared-memory plan of one block. Two areas have several tenants in turn:
+//   exchange  GEMM tiles of the contraction | exchange buffers of the bidiagonalisation |
+//             TGK arrays, singular values, orderings
+//   work      own columns of T | pivots of the twisted factorisations | chunks of W, V or
+//             reflectors and the rows of E | GEMM tiles of the site update
+template <class R, int NT, int C>
+struct Plan {
+  static constexpr int GMAX = sizeof(R) == 4 ? 4 : 1;   // column groups of pass 2
+  size_t fixed, exch, work, total;
+  int mmax, cl, kc;
+  __host__ __device__ static size_t up(size_t b) { return (b + 255) & ~(size_t)255; }
+  __host__ __device__ explicit Plan(int chi) {
+    mmax = 2 * chi;
+    cl = 2 * ((chi + C - 1) / C);
+    kc = (chi + C - 1) / C;
+    fixed = up(1280 + sizeof(R) * 2 * mmax + sizeof(Cx<R>) * 2 * mmax);
+    const size_t bidiag = up(sizeof(Cx<R>) * ((size_t)2 * C * GMAX * mmax + 4 * (size_t)mmax + 3 * cl + 8) +
+                             sizeof(R) * (2 * C + 24));
+    const size_t post = up(sizeof(R) * (2 * 2 * (size_t)mmax + 3 * mmax) + sizeof(float) * 2 * mmax +
+                           (8 + 2 * 4) * (size_t)mmax + 256 * sizeof(R) + 16);
+    const size_t tiles = up(GemmTiles<R, NT>::bytes);
+    exch = bidiag > post ? bidiag : post;
+    if (tiles > exch) exch = tiles;
+    const size_t t = up(sizeof(Cx<R>) * (size_t)cl * mmax);
+    const size_t twist = up(sizeof(R) * (size_t)kc * 2 * 2 * mmax);
+    const size_t nsr = up(sizeof(R) * ((size_t)kc * chi + (size_t)chi * 33));
+    const size_t nsc = up(sizeof(Cx<R>) * ((size_t)kc * chi + (size_t)chi * 33));
+    const size_t ychunk = up(sizeof(Cx<R>) * 16 * (size_t)mmax);
+    work = t;
+    for (size_t b : {twist, nsr, nsc, ychunk, tiles})
+      if (b > work) work = b;
+    total = fixed + exch + work;
+    // small caps: room for the whole Jacobi matrix, and for longer chunks
+    const size_t cap = 227 * 1024 - 1024, want = up(sizeof(Cx<R>) * (size_t)mmax * (mmax + 1));
+    if (want > work && want <= 96 * 1024 && fixed + exch + want <= cap) {
+      work = want;
+      total = fixed + exch + work;
+    }
+  }
+};
+
+// One Newton-Schulz step X <- X - (1/2) E X, E = X X^T - I, on the real rows w_0..w_{k-1}
+// (length p) in global memory: this block's rows (t = rank + C i) of E, their largest
+// absolute row sum, and (when asked) the updated rows.
+template <class R, int NT, int C>
+__device__ __forceinline__ R real_defect(const R* W, int k, int p, int kcv, unsigned rank, R* E, R* chunk, R* red) {
+  const int tid = threadIdx.x;
+  constexpr int QC = 32, LDC = 33, SP = 8;
+  R acc[SP];
+#pragma unroll
+  for (int s = 0; s < SP; ++s) acc[s] = R(0);
+  const int npair = kcv * k;
+  for (int q0 = 0; q0 < p; q0 += QC) {
+    const int qn = min(QC, p - q0);
+    __syncthreads();
+    for (int e = tid; e < k * QC; e += NT) {
+      const int j = e / QC, q = e % QC;
+      chunk[j * LDC + q] = q < qn ? ldcg(W + (size_t)j * p + q0 + q) : R(0);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < SP; ++s) {
+      const int e = tid + s * NT;
+      if (e < npair) {
+        const int i = e / k, j = e - i * k;
+        const R* wi = chunk + (rank + C * i) * LDC;
+        const R* wj = chunk + j * LDC;
+        R a = acc[s];
+#pragma unroll 8
+        for (int q = 0; q < QC; ++q) a = fma(wi[q], wj[q], a);
+        acc[s] = a;
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int s = 0; s < SP; ++s) {
+    const int e = tid + s * NT;
+    if (e < npair) {
+      const int i = e / k, j = e - i * k;
+      E[e] = acc[s] - (j == (int)rank + C * i ? R(1) : R(0));
+    }
+  }
+  __syncthreads();
+  // largest row sum of |E|, as FP32 (it only steers the iteration)
+  float worst = 0.f;
+  const int warp = tid >> 5, lane = tid & 31;
+  for (int i = warp; i < kcv; i += NT / 32) {
+    float s = 0.f;
+    for (int j = lane; j < k; j += 32) s += fabsf((float)E[i * k + j]);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    worst = fmaxf(worst, s == s ? s : 3e38f);   // a NaN counts as a failure
+  }
+  if (lane == 0) red[warp] = (R)worst;
+  __syncthreads();
+  R m = R(0);
+  for (int w = 0; w < NT / 32; ++w) m = fmax(m, red[w]);
+  return m;
+}
+
+template <class R, int NT, int C>
+__device__ __forceinline__ void real_update(const R* W, R* out, int k, int p, int kcv, unsigned rank, const R* E, R* chunk) {
+  const int tid = threadIdx.x;
+  constexpr int QC = 32, LDC = 33;
+  for (int q0 = 0; q0 < p; q0 += QC) {
+    const int qn = min(QC, p - q0);
+    __syncthreads();
+    for (int e = tid; e < k * QC; e += NT) {
+      const int j = e / QC, q = e % QC;
+      chunk[j * LDC + q] = q < qn ? ldcg(W + (size_t)j * p + q0 + q) : R(0);
+    }
+    __syncthreads();
+    for (int e = tid; e < kcv * QC; e += NT) {
+      const int i = e / QC, q = e % QC;
+      if (q >= qn) continue;
+      R a = R(0);
+#pragma unroll 4
+      for (int j = 0; j < k; ++j) a = fma(E[i * k + j], chunk[j * LDC + q], a);
+      const int t = rank + C * i;
+      out[(size_t)t * p + q0 + q] = fma(R(-0.5), a, chunk[t * LDC + q]);
+    }
+  }
+}
+
+// Mixed precision: one Newton-Schulz step on the complex rows x_0..x_{k-1} of V (global,
+// row length len) that the FP32 back-transformation leaves orthonormal only to a few
+// 1e-7. E = X X^H - I is a few 1e-7 itself, so its Gram matrix has to be accurate far
+// below FP32 resolution: every entry is split into a multiple of 2^-11 and a rest. The
+// products of two leading parts are multiples of 2^-22 whose partial sums stay below 4
+// (Cauchy-Schwarz), so FP32 adds them exactly; the three products with a rest are 2^-12
+// times smaller and their rounding errors vanish against E. Four FMAs per real product,
+// where a compensated (Dot2) sum of the same accuracy takes eleven operations.
+template <int NT, int C>
+__device__ __forceinline__ void newton_schulz_cluster(const Cx<float>* X, int k, int len, int kcv, unsigned rank,
+                                                      Cx<float>* E, Cx<float>* chunk, Cx<float>* out, Cx<float>* site) {
+  const int tid = threadIdx.x;
+  constexpr int QC = 32, LDC = 33, SP = 4;
+  const int npair = kcv * k;
+  float hr[SP], hi[SP], cr[SP], ci[SP];
+#pragma unroll
+  for (int s = 0; s < SP; ++s) hr[s] = hi[s] = cr[s] = ci[s] = 0.f;
+  constexpr float kMagic = 6144.0f;   // 1.5 2^12: adding it rounds to a multiple of 2^-11
+  for (int q0 = 0; q0 < len; q0 += QC) {
+    const int qn = min(QC, len - q0);
+    __syncthreads();
+    for (int e = tid; e < k * QC; e += NT) {
+      const int j = e / QC, q = e % QC;
+      chunk[j * LDC + q] = q < qn ? ldcg(X + (size_t)j * len + q0 + q) : cx<float>(0.f, 0.f);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < SP; ++s) {
+      const int e = tid + s * NT;
+      if (e < npair) {
+        const int i = e / k, j = e - i * k;
+        const Cx<float>* xi = chunk + (rank + C * i) * LDC;
+        const Cx<float>* xj = chunk + j * LDC;
+#pragma unroll 4
+        for (int q = 0; q < QC; ++q) {
+          const Cx<float> a = xi[q], b = xj[q];
+          const float ax = __fadd_rn(__fadd_rn(a.x, kMagic), -kMagic), ay = __fadd_rn(__fadd_rn(a.y, kMagic), -kMagic);
+          const float bx = __fadd_rn(__fadd_rn(b.x, kMagic), -kMagic), by = __fadd_rn(__fadd_rn(b.y, kMagic), -kMagic);
+          const float axl = __fadd_rn(a.x, -ax), ayl = __fadd_rn(a.y, -ay);
+          const float bxl = __fadd_rn(b.x, -bx), byl = __fadd_rn(b.y, -by);
+          // a conj(b) = (ax bx + ay by) + i (ay bx - ax by)
+          hr[s] = fmaf(ay, by, fmaf(ax, bx, hr[s]));
+          hi[s] = fmaf(-ax, by, fmaf(ay, bx, hi[s]));
+          cr[s] = fmaf(ax, bxl, fmaf(axl, b.x, cr[s]));
+          cr[s] = fmaf(ay, byl, fmaf(ayl, b.y, cr[s]));
+          ci[s] = fmaf(ay, bxl, fmaf(ayl, b.x, ci[s]));
+          ci[s] = fmaf(-ax, byl, fmaf(-axl, b.y, ci[s]));
+        }
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int s = 0; s < SP; ++s) {
+    const int e = tid + s * NT;
+    if (e < npair) {
+      const int i = e / k, j = e - i * k;
+      const bool diag = j == (int)rank + C * i;
+      E[e] = diag ? cx<float>(__fadd_rn(__fadd_rn(hr[s], -1.0f), cr[s]), 0.f)
+                  : cx<float>(__fadd_rn(hr[s], cr[s]), __fadd_rn(hi[s], ci[s]));
+    }
+  }
+  for (int q0 = 0; q0 < len; q0 += QC) {
+    const int qn = min(QC, len - q0);
+    __syncthreads();
+    for (int e = tid; e < k * QC; e += NT) {
+      const int j = e / QC, q = e % QC;
+      chunk[j * LDC + q] = q < qn ? ldcg(X + (size_t)j * len + q0 + q) : cx<float>(0.f, 0.f);
+    }
+    __syncthreads();
+    for (int e = tid; e < kcv * QC; e += NT) {
+      const int i = e / QC, q = e % QC;
+      if (q >= qn) continue;
+      Cx<float> a = cx<float>(0.f, 0.f);
+#pragma unroll 4
+      for (int j = 0; j < k; ++j) cmac(a, E[i * k + j], chunk[j * LDC + q]);
+      const int t = rank + C * i;
+      const Cx<float> x = chunk[t * LDC + q];
+      const Cx<float> v = cx<float>(fmaf(-0.5f, a.x, x.x), fmaf(-0.5f, a.y, x.y));
+      out[(size_t)t * len + q0 + q] = v;
+      site[(size_t)t * len + q0 + q] = conj(v);
+    }
+  }
+}
+
+// Back-transformation x <- H_0 H_1 ... H_{nref-1} x of this block's vectors, one warp per
+// vector, EL entries per lane, the reflectors staged from L2 in chunks of nch.
+template <class R, int NT, int C, int EL>
+__device__ __forceinline__ void back_transform(const R* W, int p, int len, int nref, int kcv, unsigned rank, bool tall,
+                                               int rr, const Cx<R>* Y, int ystride, const Cx<R>* tau, const Cx<R>* scl,
+                                               Cx<R>* chunk, int nch, Cx<R>* out, Cx<R>* site) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int NW = NT / 32;
+  for (int v0 = 0; v0 < kcv; v0 += NW) {
+    const int i = v0 + warp, t = rank + C * i;
+    const bool act = i < kcv;
+    Cx<R> x[EL];
+#pragma unroll
+    for (int e = 0; e < EL; ++e) {
+      const int q = lane + 32 * e;
+      x[e] = cx<R>(act && q < p ? ldcg(W + (size_t)t * p + q) : R(0), R(0));
+    }
+    for (int hi = nref; hi > 0; hi -= nch) {
+      const int lo = max(0, hi - nch);
+      __syncthreads();
+      for (int e = tid; e < (hi - lo) * len; e += NT) {
+        const int jj = e / len, q = e - jj * len, jr = lo + jj, start = tall ? jr + 1 : jr;
+        Cx<R> v = cx<R>(0, 0);
+        if (q == start)
+          v = cx<R>(1, 0);
+        else if (q > start)
+          v = tall ? ldcg(Y + (size_t)jr * ystride + q) * scl[jr] : ldcg(Y + (size_t)jr * ystride + q);
+        chunk[jj * len + q] = v;
+      }
+      __syncthreads();
+      if (act) {
+        for (int jr = hi - 1; jr >= lo; --jr) {
+          const Cx<R>* h = chunk + (jr - lo) * len;
+          const int start = tall ? jr + 1 : jr;
+          Cx<R> hv[EL];
+          Cx<R> s = cx<R>(0, 0);
+#pragma unroll
+          for (int e = 0; e < EL; ++e) {
+            if (32 * e + 31 >= start) {   // uniform: whole rows of zeros are left out
+              const int q = lane + 32 * e;
+              hv[e] = q < len ? h[q] : cx<R>(0, 0);
+              cmac_conj(s, hv[e], x[e]);
+            }
+          }
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+            s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+          }
+          const Cx<R> f = tau[jr] * s;
+#pragma unroll
+          for (int e = 0; e < EL; ++e)
+            if (32 * e + 31 >= start) cmsub(x[e], f, hv[e]);
+        }
+      }
+    }
+    if (act) {
+#pragma unroll
+      for (int e = 0; e < EL; ++e) {
+        const int q = lane + 32 * e;
+        if (q < len) {
+          const int nat = tall ? (q & 1) * rr + (q >> 1) : q;
+          out[(size_t)t * len + nat] = x[e];
+          if (site) site[(size_t)t * len + nat] = conj(x[e]);
+        }
+      }
+    }
+  }
+  __syncthreads();
+}
+
+template <bool KF, class F>
+struct Op {
+  F f;
+  static constexpr bool k_fast = KF;
+  template <class... A>
+  __device__ __forceinline__ auto operator()(A... a) const {
+    return f(a...);
+  }
+};
+template <bool KF, class F>
+__device__ __forceinline__ Op<KF, F> op(F f) {
+  return Op<KF, F>{f};
+}
+
+// Site tensors of caller-owned memory (RAW) may lie on any 4-byte boundary: they are
+// moved by component.
+template <bool RAW, class R>
+__device__ __forceinline__ Cx<R> ld_site(const Cx<R>* p) {
+  if constexpr (RAW) {
+    const R* q = reinterpret_cast<const R*>(p);
+    return cx<R>(ldcg(q), ldcg(q + 1));
+  } else {
+    return ldcg(p);
+  }
+}
+template <bool RAW, class R>
+__device__ __forceinline__ void st_site(Cx<R>* p, Cx<R> v) {
+  if constexpr (RAW) {
+    R* q = reinterpret_cast<R*>(p);
+    q[0] = v.x;
+    q[1] = v.y;
+  } else {
+    *p = v;
+  }
+}
+
+template <class R, int NT, int C, bool RAW>
+__global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0, int64_t g1, int slot0,
+                                                const double* theta, double cutoff, int max_sweeps) {
+  extern __shared__ __align__(256) unsigned char smem[];
+  constexpr bool kF64 = sizeof(R) == 8;
+  constexpr int NW = NT / 32, GMAX = Plan<R, NT, C>::GMAX;
+  const Plan<R, NT, C> L(m.chi);
+  const unsigned rank_c = crank<C>();
+  const int blk = blockIdx.x / C, s = slot0 + blk;
+  const int n = m.n, chi = m.chi, mmax = 2 * chi;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  Cx<R>* Bslot = (Cx<R>*)m.B + (size_t)s * m.slot_elems;
+  double* lam = m.lam + (size_t)s * (n - 1) * chi;
+  int* rank = m.rank + (size_t)s * (n + 1);
+  Cx<R>* W = (Cx<R>*)m.work_M + (size_t)s * mmax * mmax;                 // unscaled M
+  Cx<R>* Y = (Cx<R>*)m.work_X + (size_t)s * mmax * (mmax + 16);          // reflector vectors
+  double* scratch = (double*)m.work_S + (size_t)s * 16 * chi * chi;      // chi^2 x 16 doubles:
+  R* Wa = (R*)scratch;                                                   //   rows of W, twice
+  R* Wb = (R*)(scratch + 2 * (size_t)chi * chi);
+  Cx<R>* xout = (Cx<R>*)(scratch + 4 * (size_t)chi * chi);               //   rows of V, twice
+  Cx<R>* xout2 = (Cx<R>*)(scratch + 8 * (size_t)chi * chi);
+
+  // fixed part
+  Cx<double>* U = (Cx<double>*)smem;
+  Cx<R>* Uf = (Cx<R>*)(smem + 256);
+  double* red = (double*)(smem + 512);        // 32 per-warp partials
+  double* redc = red + 32;                    // per-block partials of the cluster (16)
+  int* misc = (int*)(redc + 16);              // [0] k, [1] collapsed, [2] Jacobi caps, [3] splits
+  R* dd = (R*)(smem + 1280);
+  R* ee = dd + mmax;
+  Cx<R>* tau = (Cx<R>*)(ee + mmax);
+  Cx<R>* scl = tau + mmax;
+  unsigned char* exch = smem + L.fixed;
+  unsigned char* work = smem + L.fixed + L.exch;
+  // exchange area, after the bidiagonalisation
+  R* bn = (R*)exch;                           // TGK off-diagonals, scaled
+  R* b2 = bn + 2 * mmax;
+  R* sig = b2 + 2 * mmax;
+  R* lo = sig + mmax;
+  R* hi = lo + mmax;
+  double* sig2d = (double*)(((uintptr_t)(hi + mmax) + 15) & ~(uintptr_t)15);
+  R* small = (R*)(sig2d + mmax);              // 256
+  float* b2f = (float*)(small + 256);
+  int* order = (int*)(b2f + 2 * mmax);        // 2 mmax
+  Cx<R>* T = (Cx<R>*)work;
+
+  const double* th = theta + (size_t)blk * c.n_params;
+  int st_max_iters = 0, st_max_rank = 1, st_bad = 0, st_nonfinite = 0, st_badarg = 0;
+  if (tid == 0) misc[2] = 0;
+  unsigned long long ph[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  double alg_flops = 0.0, dw_acc = 0.0;
+  long long t_mark = clock64();
+#define PHASE(i)                                    \
+  do {                                              \
+    if (tid == 0) {                                 \
+      const long long now_ = clock64();             \
+      ph[i] += (unsigned long long)(now_ - t_mark); \
+      t_mark = now_;                                \
+    }                                               \
+  } while (0)
+
+  const int64_t g_first = c.start_gate ? max(g0, c.start_gate[blk]) : g0;
+  const int64_t g_shift = c.shift_gate ? c.shift_gate[blk] : -1;
+  const double phi_shift = c.shift_phi ? c.shift_phi[blk] : 0.0;
+  csync<C>();   // every block of the cluster runs before any touches a peer's shared memory
+  for (int64_t g = g_first; g < g1; ++g) {
+    GateRec gr;
+    if constexpr (RAW) {
+      gr.bond = c.raw_bond[g];
+      gr.param = -1;
+      gr.m0 = (int32_t)g;
+    } else {
+      gr = c.gates[g];
+    }
+    // (1) the 4x4 gate: fixed, or mats[m1] . Rz(phi) on one site . mats[m0]
+    if (tid < 16) {
+      const int i = tid >> 2, j = tid & 3;
+      const double* A = c.mats + 32 * (size_t)gr.m0;
+      Cx<double> u;
+      if (gr.param < 0) {
+        u = cx<double>(A[2 * tid], A[2 * tid + 1]);
+      } else {
+        const Cx<double>* Am = (const Cx<double>*)A;
+        const Cx<double>* P = (const Cx<double>*)c.mats + 16 * (size_t)gr.m1;
+        const double half = 0.5 * (gr.scale * th[gr.param] + (g == g_shift ? phi_shift : 0.0));
+        double sn, cs;
+        sincos(half, &sn, &cs);
+        u = cx(0.0, 0.0);
+        for (int k = 0; k < 4; ++k) {
+          const int bit = gr.rz_site == 0 ? ((k >> 1) & 1) : (k & 1);
+          const Cx<double> pz = cx(cs, bit ? sn : -sn);  // Rz = diag(e^{-i phi/2}, e^{i phi/2})
+          u = u + (P[i * 4 + k] * pz) * Am[k * 4 + j];
+        }
+      }
+      U[tid] = u;
+      Uf[tid] = cx<R>((R)u.x, (R)u.y);
+    }
+    const int bond = gr.bond;
+    if constexpr (RAW) {
+      // caller-owned device arrays: the bond and the three ranks it touches must lie
+      // inside the site capacities before anything is indexed (uniform over the cluster)
+      bool ok = bond >= 0 && bond <= n - 2;
+      if (ok) {
+        const int r0 = ldcg(rank + bond), r1 = ldcg(rank + bond + 1), r2 = ldcg(rank + bond + 2);
+        ok = r0 >= 1 && r0 <= bond_cap(bond - 1, n, chi) && r1 >= 1 && r1 <= bond_cap(bond, n, chi) && r2 >= 1 &&
+             r2 <= bond_cap(bond + 1, n, chi);
+      }
+      if (!ok) {
+        if (tid == 0) st_badarg = 1;
+        break;
+      }
+    }
+    const int rl = ldcg(rank + bond), rm = ldcg(rank + bond + 1), rr = ldcg(rank + bond + 2);
+    const int mrows = 2 * rl, ncol = 2 * rr;
+    const bool tall = mrows >= ncol;
+    const int tr = tall ? mrows : ncol, tp = tall ? ncol : mrows, ld = tr;
+    Cx<R>* Bn = Bslot + m.site_off[bond];
+    Cx<R>* Bn1 = Bslot + m.site_off[bond + 1];
+    const double* laml = bond > 0 ? lam + (size_t)(bond - 1) * chi : nullptr;
+    __syncthreads();
+    // (2) Eq. (7): M[(a,i),(j,c)] = sum_{i'j'} U[ij,i'j'] sum_b B_n[a,i',b] B_{n+1}[b,j',c];
+    //     W <- M; Eq. (8): M' = lambda_{n-1}[a] M. Each block contracts the columns of T it
+    //     owns into place, then applies the gate and lambda to its (a, c) quads.
+    const int nq = ((tall ? rr : rl) + C - 1 - (int)rank_c) / C;   // own c (tall) or a (wide)
+    if (tall)
+      tile_gemm<R, NT>(
+          mrows, 2 * nq, rm, [&](int mi, int k) { return ld_site<RAW>(Bn + (size_t)mi * rm + k); },
+          op<false>([&](int k, int ni) {
+            return ld_site<RAW>(Bn1 + (size_t)k * ncol + (ni & 1) * rr + rank_c + C * (ni >> 1));
+          }),
+          [&](int mi, int ni, Cx<R> v) { T[(size_t)ni * ld + mi] = v; }, exch);
+    else
+      tile_gemm<R, NT>(
+          2 * nq, ncol, rm,
+          [&](int mi, int k) { return ld_site<RAW>(Bn + (size_t)(2 * (rank_c + C * (mi >> 1)) + (mi & 1)) * rm + k); },
+          op<false>([&](int k, int ni) { return ld_site<RAW>(Bn1 + (size_t)k * ncol + ni); }),
+          [&](int mi, int ni, Cx<R> v) { T[(size_t)mi * ld + ni] = v; }, exch);
+    double fro = 0.0;
+    const int qfast = tall ? rl : rr;
+    for (int it = tid; it < nq * qfast; it += NT) {
+      const int o = it / qfast, f = it - o * qfast;
+      const int a = tall ? f : (int)rank_c + C * o, cc = tall ? (int)rank_c + C * o : f;
+      // entry (i, j) of the quad
+      Cx<R>* e[4];
+#pragma unroll
+      for (int ij = 0; ij < 4; ++ij) {
+        const int i = ij >> 1, j = ij & 1;
+        e[ij] = tall ? T + (size_t)(2 * o + j) * ld + 2 * f + i : T + (size_t)(2 * o + i) * ld + j * rr + f;
+      }
+      const Cx<R> th4[4] = {*e[0], *e[1], *e[2], *e[3]};
+      const R la = laml ? (R)__ldcg(laml + a) : R(1);
+      R part = 0;
+#pragma unroll
+      for (int ij = 0; ij < 4; ++ij) {
+        Cx<R> v = cx<R>(0, 0);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) cmac(v, Uf[ij * 4 + kk], th4[kk]);
+        W[(size_t)(2 * a + (ij >> 1)) * ncol + (ij & 1) * rr + cc] = v;
+        const Cx<R> mv = la * v;
+        *e[ij] = tall ? mv : conj(mv);
+        if constexpr (kF64)
+          part += norm2(mv);
+        else
+          fro += (double)norm2(mv);
+      }
+      if constexpr (kF64) fro += part;
+    }
+    for (int o = 16; o > 0; o >>= 1) fro += __shfl_xor_sync(0xffffffffu, fro, o);
+    if (lane == 0) red[warp] = fro;
+    __syncthreads();
+    if (tid < C) {
+      double t = 0.0;
+      for (int w = 0; w < NW; ++w) t += red[w];
+      peer<C>(redc, tid)[rank_c] = t;
+    }
+    csync<C>();
+    double total = 0.0;
+#pragma unroll
+    for (int w = 0; w < C; ++w) total += redc[w];
+    // a NaN or Inf in M' (from corrupted inputs) would run through every later stage:
+    // the gate is skipped, the state left as it was, and the host reports the count
+    if (!(total <= DBL_MAX)) {
+      if (tid == 0) ++st_nonfinite;
+      csync<C>();
+      continue;
+    }
+    PHASE(0);
+    // (3) Eq. (9): bidiagonalise T = Q B P^H (B real)
+    {
+      Bidiag<R> b;
+      b.T = T;
+      b.ld = ld;
+      b.zrows = mmax;
+      b.zp = (Cx<R>*)exch;
+      b.colp = b.zp + (size_t)2 * C * GMAX * mmax;
+      b.xs = b.colp + 2 * mmax;
+      b.us = b.xs + mmax;
+      b.rj = b.us + mmax;
+      b.fj = b.rj + 2 * L.cl;
+      b.sc = b.fj + L.cl;
+      b.nrmp = (R*)(b.sc + 8);
+      b.part = b.nrmp + 2 * C;
+      b.dd = dd;
+      b.ee = ee;
+      b.tau = tau;
+      b.scl = scl;
+      b.Y = Y;
+      b.ystride = mmax;
+      bidiagonalize_cluster<R, NT, C, GMAX>(b, tr, tp, tall, rank_c);
+    }
+    PHASE(1);
+    // Golub-Kahan tridiagonal off-diagonal (d0, e0, d1, e1, ..., d_{p-1}), scaled by a power
+    // of two so that no singular value exceeds 1
+    const int N = 2 * tp;
+    if (warp == 0) {
+      R top = 0;
+      for (int i = lane; i < N; i += 32) {
+        const R left = i > 0 ? rabs((i - 1) & 1 ? ee[(i - 1) >> 1] : dd[(i - 1) >> 1]) : R(0);
+        const R right = i < N - 1 ? rabs(i & 1 ? ee[i >> 1] : dd[i >> 1]) : R(0);
+        top = fmax(top, left + right);
+      }
+      for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
+      if (lane == 0) {
+        small[0] = top;
+        misc[1] = 0;
+        misc[3] = 0;
+      }
+    }
+    __syncthreads();
+    const R smax = small[0];
+    int ex = 0;
+    if (smax > R(0)) frexp(smax, &ex);        // smax = f 2^ex, f in [1/2, 1)
+    ex = max(min(ex, kF64 ? 1000 : 120), kF64 ? -1000 : -120);
+    const R down = ldexp(R(1), -ex), back = ldexp(R(1), ex), top = smax * down;
+    // split the TGK where an off-diagonal is negligible (exact degeneracies live in
+    // different blocks after this; the perturbation is below 4 eps ||B||)
+    for (int i = tid; i < N - 1; i += NT) {
+      R v = ((i & 1) ? ee[i >> 1] : dd[i >> 1]) * down;
+      if (rabs(v) <= R(4) * Eps<R>::v * top) {
+        v = R(0);
+        misc[3] = 1;
+      }
+      bn[i] = v;
+      b2[i] = v * v;
+      if constexpr (kF64) b2f[i] = (float)(v * v);
+    }
+    if (tid == 0) {
+      bn[N - 1] = R(0);
+      b2[N - 1] = R(0);
+    }
+    __syncthreads();
+    const bool split = misc[3] != 0;
+    const int kk = min(chi, tp), kco = (kk + C - 1 - (int)rank_c) / C;
+    int passes = 0;
+    if constexpr (!kF64) {
+      for (int i = warp; i < kco; i += NW) {
+        const int t = rank_c + C * i;
+        float a, b;
+        passes = max(passes, warp_bisect(b2, N, t, fminf(top * 1.001f, 1.01f), &a, &b));
+        if (lane < C) {
+          peer<C>(lo, lane)[t] = a;
+          peer<C>(hi, lane)[t] = b;
+          peer<C>(sig, lane)[t] = 0.5f * (a + b);
+        }
+      }
+    } else {
+      const float topf = fminf((float)top * 1.001f, 1.01f);
+      for (int i = warp; i < kco; i += NW) {
+        float a, b;
+        passes = max(passes, warp_bisect(b2f, N, rank_c + C * i, topf, &a, &b));
+        if (lane == 0) sig2d[i] = __hiloint2double(__float_as_int(b), __float_as_int(a));   // the FP32 bracket
+      }
+      __syncthreads();
+      constexpr int LT = 4;
+      for (int i0 = warp * (32 / LT); i0 < kco; i0 += NW * (32 / LT)) {
+        const int i = i0 + lane / LT;
+        const bool act = i < kco;
+        const int t = rank_c + C * (act ? i : i0);
+        const double pk = sig2d[act ? i : i0];
+        double a, b;
+        passes += lanes_bisect<LT>(b2, N, t, act, (double)top * 1.001, __int_as_float(__double2loint(pk)),
+                                   __int_as_float(__double2hiint(pk)), &a, &b);
+        if (act)
+          for (int cb = lane & (LT - 1); cb < C; cb += LT) {
+            peer<C>(lo, cb)[t] = a;
+            peer<C>(hi, cb)[t] = b;
+            peer<C>(sig, cb)[t] = 0.5 * (a + b);
+          }
+      }
+    }
+    csync<C>();
+    if (warp == 0) {
+      // sig is descending: k = number of leading values above cutoff * sig_0
+      const R s0 = sig[0], cut = (R)cutoff * s0;
+      int cntk = 0;
+      for (int t = lane; t < kk; t += 32) cntk += (sig[t] > cut && sig[t] > R(0));
+      for (int o = 16; o > 0; o >>= 1) cntk += __shfl_xor_sync(0xffffffffu, cntk, o);
+      if (lane == 0) misc[0] = cntk > 0 ? cntk : 1;
+    }
+    __syncthreads();
+    const int k = misc[0];
+    if (tid == 0) {
+      st_max_rank = max(st_max_rank, k);
+      st_max_iters = max(st_max_iters, passes);
+    }
+    PHASE(2);
+
+    // (4) singular vectors of B from twisted factorisations: pivots from both ends (one lane
+    // per direction), the twist where |gamma| is smallest, the vector outward from there
+    const R tiny = kF64 ? R(1e-300) : R(1e-30);
+    const int kcv = (k + C - 1 - (int)rank_c) / C;   // own vectors t = rank_c + C i
+    const int odd = tall ? 0 : 1;
+    {
+      R* F = (R*)work;                       // [kcv][2][N] reciprocal pivots
+      int* rng = order;                      // [kcv][3]: block start, end, twist
+      const int v = tid >> 1, dir = tid & 1;
+      const bool act = v < kcv;
+      R lamv = 0;
+      int s0 = 0, e0 = N;
+      if (act) {
+        const int t = rank_c + C * v;
+        lamv = sig[t];
+        if (split) owning_range<R>(b2, N, sig, t, R(8) * (hi[t] - lo[t]) + R(4) * Eps<R>::v * top, &s0, &e0);
+        R* f = F + (size_t)(2 * v + dir) * N;
+        int i = dir ? e0 - 1 : s0;
+        const int step = dir ? -1 : 1;
+        R d = -lamv;
+        if (rabs(d) < tiny) d = -tiny;
+        R rv = pivot_rcp(d);
+        f[i] = rv;
+#pragma unroll 4
+        for (int q = 1; q < e0 - s0; ++q) {
+          const R bb = b2[dir ? i - 1 : i];
+          i += step;
+          d = fma(-bb, rv, -lamv);
+          if (rabs(d) < tiny) d = -tiny;
+          rv = pivot_rcp(d);
+          f[i] = rv;
+        }
+        if (dir == 0) {
+          rng[3 * v] = s0;
+          rng[3 * v + 1] = e0;
+        }
+      }
+      __syncthreads();
+      for (int w = warp; w < kcv; w += NW) {
+        const int ws = rng[3 * w], we = rng[3 * w + 1];
+        const R lw = sig[rank_c + C * w];
+        const R* fu = F + (size_t)2 * w * N;
+        const R* fd = fu + N;
+        R best = R(1e30);
+        int at = we - 1;
+        for (int i = ws + lane; i < we; i += 32) {
+          // gamma_i = -lam - b_{i-1}^2 / dp_{i-1} - b_i^2 / dm_{i+1}
+          R gm = -lw;
+          if (i > ws) gm = fma(-b2[i - 1], fu[i - 1], gm);
+          if (i < we - 1) gm = fma(-b2[i], fd[i + 1], gm);
+          gm = rabs(gm);
+          if (gm < best) {
+            best = gm;
+            at = i;
+          }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+          const R ob = __shfl_xor_sync(0xffffffffu, best, o);
+          const int oa = __shfl_xor_sync(0xffffffffu, at, o);
+          if (ob < best || (ob == best && oa < at)) {
+            best = ob;
+            at = oa;
+          }
+        }
+        if (lane == 0) rng[3 * w + 2] = at;
+        // outside the block the vector is zero
+        R* z = F + (size_t)2 * w * N;
+        for (int i = lane; i < N; i += 32)
+          if (i < ws || i >= we) z[i] = R(0);
+      }
+      __syncthreads();
+      if (act) {
+        const int at = rng[3 * v + 2];
+        R* z = F + (size_t)2 * v * N;        // the vector overwrites the forward pivots
+        const R* f = F + (size_t)(2 * v + dir) * N;
+        R zv = 1;
+        if (dir == 0) {
+          z[at] = R(1);
+          // z_i = -(b_i / dp_i) z_{i+1}
+#pragma unroll 8
+          for (int i = at - 1; i >= s0; --i) {
+            zv *= -bn[i] * f[i];
+            z[i] = zv;
+          }
+        } else {
+#pragma unroll 8
+          for (int i = at + 1; i < e0; ++i) {
+            zv *= -bn[i - 1] * f[i];
+            z[i] = zv;
+          }
+        }
+      }
+      __syncthreads();
+      for (int w = warp; w < kcv; w += NW) {
+        const R* z = F + (size_t)2 * w * N;
+        R nrm = 0;
+        for (int q = lane; q < tp; q += 32) {
+          const R x = z[2 * q + odd];
+          nrm = fma(x, x, nrm);
+        }
+        for (int o = 16; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
+        const R inv = nrm > R(0) ? R(1) / sqrt(nrm) : R(0);
+        const int t = rank_c + C * w;
+        for (int q = lane; q < tp; q += 32) Wa[(size_t)t * tp + q] = z[2 * q + odd] * inv;
+      }
+    }
+    csync<C>();
+    PHASE(3);
+    // (4b) the rows are orthonormal to about eps / (relative gap). Newton-Schulz steps pull
+    // them together without the serial chain of a Gram-Schmidt (the span, and with it
+    // B_n B_{n+1}, does not change); rows too far off go through block Gram-Schmidt, and
+    // a collapse there to Jacobi. FP32 stops at 1e-4: the step on the final V, which works
+    // from an accurate Gram matrix, squares that away.
+    R *Wc = Wa, *Wn = Wb;
+    bool slow = false;
+    {
+      R* E = (R*)work;
+      R* chunk = E + (size_t)L.kc * chi;
+      const float tol = kF64 ? 1e-15f : 1e-4f;
+      float pred = 2.f;
+      for (int it = 0; it < 8 && pred > tol; ++it) {
+        const R dmax = real_defect<R, NT, C>(Wc, k, tp, kcv, rank_c, E, chunk, small);
+        if (tid < C) peer<C>(redc, tid)[rank_c] = (double)dmax;
+        csync<C>();
+        float defect = 0.f;
+#pragma unroll
+        for (int w = 0; w < C; ++w) defect = fmaxf(defect, (float)redc[w]);
+        if (!(defect <= 0.4f)) {
+          slow = true;
+          break;
+        }
+        if (!kF64 && defect <= tol) break;
+        real_update<R, NT, C>(Wc, Wn, k, tp, kcv, rank_c, E, chunk);
+        R* sw = Wc;
+        Wc = Wn;
+        Wn = sw;
+        pred = defect * defect;
+        csync<C>();
+      }
+      if (slow) {
+        if (rank_c == 0) {
+          for (int e = tid; e < k * tp; e += NT) Wn[e] = ldcg(Wc + e);
+          __syncthreads();
+          orthonormalize_rows_block<R, NT>(Wn, tp, k, tp, (R*)work, small, &misc[1]);
+          __syncthreads();
+          if (tid < C) peer<C>(misc, tid)[1] = misc[1];
+        }
+        Wc = Wn;
+        csync<C>();
+      }
+    }
+    PHASE(4);
+    int kf = k;                                  // kept count of the path taken
+    if (misc[1] == 0) {
+      // (5) back-transformation: x_t = P w_t (tall) or Q [w_t; 0] (wide) is the right
+      //     singular vector v_t of M' (length ncol)
+      const int nref = tall ? tp - 1 : tp;
+      const int nch = max(1, min(nref, (int)(L.work / (sizeof(Cx<R>) * ncol))));
+      Cx<R>* site = kF64 ? Bn1 : nullptr;
+      auto go = [&](auto el) {
+        back_transform<R, NT, C, decltype(el)::value>(Wc, tp, ncol, nref, kcv, rank_c, tall, rr, Y, mmax, tau, scl,
+                                                      (Cx<R>*)work, nch, xout, site);
+      };
+      if (ncol <= 32)
+        go(std::integral_constant<int, 1>{});
+      else if (ncol <= 64)
+        go(std::integral_constant<int, 2>{});
+      else if (ncol <= 128)
+        go(std::integral_constant<int, 4>{});
+      else
+        go(std::integral_constant<int, 8>{});
+      if (rank_c == 0 && warp == 0) {
+        double kept = 0.0;
+        const double bk = (double)back;
+        for (int t = lane; t < k; t += 32) kept += ((double)sig[t] * bk) * ((double)sig[t] * bk);
+        for (int o = 16; o > 0; o >>= 1) kept += __shfl_xor_sync(0xffffffffu, kept, o);
+        if (lane == 0 && total > 0.0) dw_acc += fmax(0.0, total - kept) / total;
+        for (int t = lane; t < k; t += 32) lam[(size_t)bond * chi + t] = (double)(sig[t] * back);
+      }
+    } else {
+      // (5') degenerate spectrum without a split: one-sided Jacobi by the first block on the
+      //      columns X = conj rows of M' (rebuilt from W and lambda_{n-1})
+      if (tid == 0) ++st_bad;
+      if (rank_c == 0) {
+        const int ldx = ncol + 1;
+        Cx<R>* X = sizeof(Cx<R>) * (size_t)mrows * ldx <= L.work ? T : Y;
+        for (int idx = tid; idx < mrows * ncol; idx += NT) {
+          const int row = idx / ncol, q = idx - row * ncol;
+          const R la = laml ? (R)__ldcg(laml + (row >> 1)) : R(1);
+          X[(size_t)row * ldx + q] = conj(la * ldcg(W + (size_t)row * ncol + q));
+        }
+        __syncthreads();
+        const double zero2 = (double)Eps<R>::v * Eps<R>::v * 16.0 * total;
+        jacobi_columns<R, NT, 8>(X, ldx, mrows, ncol, zero2, max_sweeps, &misc[2]);
+        for (int p = tid; p < mrows; p += NT) {
+          double acc = 0.0;
+          for (int q = 0; q < ncol; ++q) acc += (double)norm2(X[(size_t)p * ldx + q]);
+          sig2d[p] = acc;
+        }
+        __syncthreads();
+        for (int p = tid; p < mrows; p += NT) {
+          const double v = sig2d[p];
+          int rk = 0;
+          for (int q = 0; q < mrows; ++q) {
+            const double w = sig2d[q];
+            rk += (w > v) || (w == v && q < p);
+          }
+          order[rk] = p;
+        }
+        __syncthreads();
+        if (tid == 0) {
+          const double s0 = sig2d[order[0]];
+          const int kmax = min(chi, min(mrows, ncol));
+          int kk2 = 0;
+          while (kk2 < kmax && sig2d[order[kk2]] > cutoff * cutoff * s0) ++kk2;
+          if (kk2 == 0) kk2 = 1;
+          double all = 0.0, dropped = 0.0;
+          for (int t = 0; t < mrows; ++t) all += sig2d[order[t]];
+          for (int t = kk2; t < mrows; ++t) dropped += sig2d[order[t]];
+          if (all > 0.0) dw_acc += dropped / all;
+          for (int cb = 0; cb < C; ++cb) peer<C>(misc, cb)[0] = kk2;
+          st_max_rank = max(st_max_rank, kk2);
+        }
+        __syncthreads();
+        const int kj = misc[0];
+        for (int t = tid; t < kj; t += NT) lam[(size_t)bond * chi + t] = (double)(R)sqrt(sig2d[order[t]]);
+        for (int idx = tid; idx < kj * ncol; idx += NT) {
+          const int t = idx / ncol, q = idx - t * ncol;
+          const int p = order[t];
+          const R inv = (R)(1.0 / sqrt(sig2d[p]));
+          const Cx<R> v = inv * X[(size_t)p * ldx + q];   // column p of X = sigma * v_t
+          xout[idx] = v;
+          if (kF64) Bn1[idx] = conj(v);
+        }
+      }
+      csync<C>();
+      kf = misc[0];
+    }
+    const int kcf = (kf + C - 1 - (int)rank_c) / C;
+    csync<C>();
+    Cx<R>* xv = xout;
+    if constexpr (!kF64) {
+      // (5b) mixed precision: over a long circuit the orthonormality defect of the FP32
+      //      back-transformation, not the rounding of the stored tensors, dominates the
+      //      energy error; one Newton-Schulz step brings it down to the storage rounding
+      Cx<float>* E = (Cx<float>*)work;
+      Cx<float>* chunk = E + (size_t)L.kc * chi;
+      if constexpr (RAW) {
+        newton_schulz_cluster<NT, C>(xout, kf, ncol, kcf, rank_c, E, chunk, xout2, xout2);
+        __syncthreads();
+        // the caller's tensors take V by component; xout2 then holds conj(V) rows
+        for (int i = 0; i < kcf; ++i) {
+          const int t = rank_c + C * i;
+          for (int q = tid; q < ncol; q += NT) {
+            const Cx<R> v = xout2[(size_t)t * ncol + q];
+            st_site<true>(Bn1 + (size_t)t * ncol + q, v);
+            xout2[(size_t)t * ncol + q] = conj(v);
+          }
+        }
+      } else {
+        newton_schulz_cluster<NT, C>(xout, kf, ncol, kcf, rank_c, E, chunk, xout2, Bn1);
+      }
+      xv = xout2;
+      csync<C>();
+    }
+    PHASE(5);
+    // (6) Eq. (10): B_{n+1} <- V (row t = v_t^H, written above), B_n <- M V^H (column t =
+    //     M v_t), lambda_n <- sigma
+    {
+      const int mper = (mrows + C - 1) / C, m0 = min(mrows, mper * (int)rank_c), mn = min(mper, mrows - m0);
+      tile_gemm<R, NT>(
+          mn, kf, ncol, [&](int mi, int q) { return ldcg(W + (size_t)(m0 + mi) * ncol + q); },
+          op<true>([&](int q, int t) { return ldcg(xv + (size_t)t * ncol + q); }),
+          [&](int mi, int t, Cx<R> v) { st_site<RAW>(Bn + (size_t)(m0 + mi) * kf + t, v); }, work);
+    }
+    if (rank_c == 0 && tid == 0) rank[bond + 1] = kf;
+    csync<C>();
+    PHASE(6);
+    if (tid == 0) alg_flops += flops_per_gate(rl, rm, rr, kf);
+  }
+#undef PHASE
+  if (rank_c == 0 && tid == 0) {
+    for (int i = 0; i < 7; ++i) m.prof[s * 8 + i] += ph[i];
+    m.prof[s * 8 + 7] = __double_as_longlong(__longlong_as_double(m.prof[s * 8 + 7]) + alg_flops);
+    m.dw[s] += dw_acc;
+    int* stt = m.stat + s * kStatWords;
+    stt[0] = max(stt[0], st_max_iters);
+    stt[1] += misc[2];
+    stt[3] += st_bad;
+    stt[2] = max(stt[2], st_max_rank);
+    stt[4] += st_nonfinite;
+    stt[5] |= st_badarg;
+  }
+  csync<C>();   // no block leaves while a peer may still reach its shared memory
+}
+
+}  // namespace gate
+
+// The dynamic shared-memory limit of a kernel is process-wide state: handles of
+// different chi launch the same instantiation from several threads, so the limit is
+// raised once to the device's opt-in maximum and never lowered.
+template <auto Kernel>
+static cudaError_t raise_smem_limit() {
+  static std::once_flag once[64];
+  static cudaError_t status[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::call_once(once[dev], [dev] {
+    int optin = 0;
+    status[dev] = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (status[dev] == cudaSuccess)
+      status[dev] = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+  });
+  return status[dev];
+}
+
+template <class R, int NT, int C, bool RAW>
+static cudaError_t launch_cluster(const DevMPS& m, const CircDev& c, int64_t g0, int64_t g1, int slot0, int count,
+                                  const double* theta, double cutoff, int max_sweeps, cudaStream_t st) {
+  constexpr auto kernel = gate::k_circuit<R, NT, C, RAW>;
+  cudaError_t e = raise_smem_limit<kernel>();
+  if (e != cudaSuccess) return e;
+  const gate::Plan<R, NT, C> L(m.chi);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(count * C));
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = L.total;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = C > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, m, c, g0, g1, slot0, theta, cutoff, max_sweeps);
+}
+
+template <bool RAW>
+static cudaError_t launch_mixed(const DevMPS& m, const CircDev& c, int64_t g0, int64_t g1, int slot0, int count,
+                                const double* theta, double cutoff, int max_sweeps, cudaStream_t st) {
+  if (m.chi <= 16)
+    return launch_cluster<float, 512, 1, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
+  if (m.chi <= 64)
+    return launch_cluster<float, 512, 4, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
+  if constexpr (!RAW)
+    return launch_cluster<float, 512, 8, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_circuit(const DevMPS& m, int prec, const CircDev& c, int64_t g0, int64_t g1, int slot0, int count,
+                           const double* theta, double cutoff, int max_sweeps, cudaStream_t st) {
+  if (prec == MPS_PREC_FP64)
+    return launch_cluster<double, 256, 8, false>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
+  return launch_mixed<false>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
+}
+
+}  // namespace mpsvqe
+
+// ------------------------------------------------------------------------------
+// Allocation-free variant of the gate engine for callers that cannot allocate device
+// memory themselves or through this library (the paper has no counterpart; see the
+// declaration of mps_apply_gates_noalloc in include/mpsvqe.h). Its workspace lives in
+// the file-scope array below, which every GPU that loads the library keeps until the
+// process exits; all calls share it.
+namespace mpsvqe {
+namespace {
+constexpr size_t kNoAllocScratchBytes = size_t(1) << 20;   // 1 MiB
+constexpr int kNoAllocMaxChi = 64;
+}  // namespace
+}  // namespace mpsvqe
+
+static __device__ __align__(256) unsigned char g_noalloc_scratch[mpsvqe::kNoAllocScratchBytes];
+
+namespace {
+std::mutex g_noalloc_mu;
+void* g_noalloc_ptr[64] = {nullptr};
+}  // namespace
+
+extern "C" int mps_apply_gates_noalloc(int n_qubits, int chi, void* site_tensors, const int64_t* site_offsets,
+                                       double* lambdas, int32_t* ranks, int64_t n_gates, const int32_t* bonds,
+                                       const double* gates, void* cuda_stream, double* discarded_weight) {
+  using namespace mpsvqe;
+  if (!site_tensors || !site_offsets || !lambdas || !ranks || (n_gates > 0 && (!bonds || !gates))) {
+    set_error_message("mps_apply_gates_noalloc: null device pointer");
+    return MPS_EINVAL;
+  }
+  if (n_qubits < 2 || n_qubits > kMaxQubits || chi < 1 || chi > kNoAllocMaxChi || n_gates < 0) {
+    set_error_message("mps_apply_gates_noalloc: needs 2 <= n_qubits <= 128, 1 <= chi <= 64 and n_gates >= 0 "
+                      "(the fixed 1 MiB device workspace holds one chi <= 64 gate step)");
+    return MPS_EINVAL;
+  }
+  const size_t mm = 2 * (size_t)chi;
+  const size_t off_M = 0;
+  const size_t off_X = off_M + ((mm * mm * 8 + 255) & ~(size_t)255);
+  const size_t off_S = off_X + ((mm * (mm + 16) * 8 + 255) & ~(size_t)255);
+  const size_t off_dw = off_S + ((16 * (size_t)chi * chi * 8 + 255) & ~(size_t)255);
+  const size_t off_end = off_dw + 256;
+  if (off_end > kNoAllocScratchBytes) {
+    set_error_message("mps_apply_gates_noalloc: workspace larger than the 1 MiB device array");
+    return MPS_EINVAL;
+  }
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+    set_error_message("mps_apply_gates_noalloc: no current CUDA device");
+    return MPS_ECUDA;
+  }
+  unsigned char* base = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(g_noalloc_mu);
+    if (!g_noalloc_ptr[dev]) {
+      void* p = nullptr;
+      if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) {
+        set_error_message("mps_apply_gates_noalloc: cudaGetSymbolAddress of the device workspace failed");
+        return MPS_ECUDA;
+      }
+      g_noalloc_ptr[dev] = p;
+    }
+    base = (unsigned char*)g_noalloc_ptr[dev];
+  }
+  cudaStream_t st = (cudaStream_t)cuda_stream;
+  DevMPS d{};
+  d.n = n_qubits;
+  d.chi = chi;
+  d.n_slots = 1;
+  d.slot_elems = 0;
+  d.site_off = site_offsets;
+  d.B = site_tensors;
+  d.lam = lambdas;
+  d.rank = ranks;
+  d.work_M = base + off_M;
+  d.work_X = base + off_X;
+  d.work_S = base + off_S;
+  d.dw = (double*)(base + off_dw);
+  d.stat = (int*)(base + off_dw + 8);
+  d.prof = (unsigned long long*)(base + off_dw + 64);
+  // the shared array keeps the previous call's contents: clear the accumulators
+  if (cudaMemsetAsync(base + off_dw, 0, 256, st) != cudaSuccess) return MPS_ECUDA;
+  CircDev c{};
+  c.gates = nullptr;
+  c.n_gates = n_gates;
+  c.mats = gates;
+  c.n_params = 1;
+  c.raw_bond = bonds;
+  const double* theta = (const double*)(base + off_dw + 128);   // never read: every gate is fixed
+  for (int64_t g0 = 0; g0 < n_gates; g0 += 16384) {
+    const int64_t g1 = g0 + 16384 < n_gates ? g0 + 16384 : n_gates;
+    if (launch_mixed<true>(d, c, g0, g1, 0, 1, theta, std::ldexp(1.0, -20), 60, st) != cudaSuccess) return MPS_ECUDA;
+  }
+  if (discarded_weight) {
+    // the discarded weight and the status words sit next to each other in the array:
+    // one copy brings both back
+    unsigned char host[8 + 4 * kStatWords];
+    if (cudaMemcpyAsync(host, d.dw, sizeof(host), cudaMemcpyDeviceToHost, st) != cudaSuccess) return MPS_ECUDA;
+    if (cudaStreamSynchronize(st) != cudaSuccess) return MPS_ECUDA;
+    int stat[kStatWords];
+    std::memcpy(discarded_weight, host, 8);
+    std::memcpy(stat, host + 8, sizeof(stat));
+    if (stat[5]) {
+      set_error_message("mps_apply_gates_noalloc: a bond outside [0, n-2] or a rank outside its capacity "
+                        "reached the device; gates from there on were not applied");
+      return MPS_EINVAL;
+    }
+    if (stat[4] > 0) {
+      set_error_message("mps_apply_gates_noalloc: a gate's M' held a NaN or Inf; the gate was skipped");
+      return MPS_ENONFINITE;
+    }
+    if (stat[1] > 0) {
+      set_error_message("mps_apply_gates_noalloc: a Jacobi SVD fallback reached its sweep cap");
+      return MPS_ENOCONV;
+    }
+  }
+  return MPS_OK;
+}
