@@ -53,31 +53,36 @@ namespace gate {
 
 // Shared-memory plan of one block. Two areas have several tenants in turn:
 //   exchange  GEMM tiles of the contraction | exchange buffers of the bidiagonalisation |
-//             TGK arrays, singular values, orderings
+//             TGK arrays, its blocks, singular values, orderings
 //   work      own columns of T | pivots of the twisted factorisations | chunks of W, V or
 //             reflectors and the rows of E | GEMM tiles of the site update
 template <class R, int NT, int C>
 struct Plan {
-  static constexpr int GMAX = sizeof(R) == 4 ? 4 : 1;   // column groups of pass 2
+  static constexpr size_t kFixed = 3072;   // gate, record, reductions, ranks, site offsets
   size_t fixed, exch, work, total;
-  int mmax, cl, kc;
+  int mmax, cl, kc, gmax;
   __host__ __device__ static size_t up(size_t b) { return (b + 255) & ~(size_t)255; }
+  // leading dimension of T: 8 (mod 16) complex<float> entries, so that the two 8-lane
+  // column walks of a half warp fall into different banks
+  __host__ __device__ static int lead(int rows) { return sizeof(R) == 4 ? (rows + 15) / 16 * 16 + 8 : rows; }
   __host__ __device__ explicit Plan(int chi) {
     mmax = 2 * chi;
     cl = 2 * ((chi + C - 1) / C);
     kc = (chi + C - 1) / C;
-    fixed = up(1280 + sizeof(R) * 2 * mmax + sizeof(Cx<R>) * 2 * mmax);
-    const size_t bidiag = up(sizeof(Cx<R>) * ((size_t)2 * C * GMAX * mmax + 4 * (size_t)mmax + 3 * cl + 8) +
+    gmax = chi > 64 ? 1 : 2;   // column groups of pass 2: as many as there are threads for the rows
+    fixed = up(kFixed + sizeof(R) * 2 * mmax + sizeof(Cx<R>) * 2 * mmax);
+    const size_t bidiag = up(sizeof(Cx<R>) * ((size_t)2 * C * gmax * mmax + 4 * (size_t)mmax + 4 * cl + 8) +
                              sizeof(R) * (2 * C + 24));
-    const size_t post = up(sizeof(R) * (2 * 2 * (size_t)mmax + 3 * mmax) + sizeof(float) * 2 * mmax +
-                           (8 + 2 * 4) * (size_t)mmax + 256 * sizeof(R) + 16);
-    const size_t tiles = up(GemmTiles<R, NT>::bytes);
+    const size_t post = up(sizeof(R) * (2 * 2 * (size_t)mmax + 2 * mmax) + sizeof(float) * 2 * mmax +
+                           (8 + 2 * 4) * (size_t)mmax + 256 * sizeof(R) + 48 + sizeof(int) * (8 * (size_t)mmax + 4) +
+                           sizeof(R) * 2 * kc * (2 * (size_t)mmax / SturmGroup<R>::v + 1));
+    const size_t tiles = up(gemm_tile_bytes<NT>());
     exch = bidiag > post ? bidiag : post;
     if (tiles > exch) exch = tiles;
-    const size_t t = up(sizeof(Cx<R>) * (size_t)cl * mmax);
+    const size_t t = up(sizeof(Cx<R>) * (size_t)cl * lead(mmax));
     const size_t twist = up(sizeof(R) * (size_t)kc * 2 * 2 * mmax);
     const size_t nsr = up(sizeof(R) * ((size_t)kc * chi + (size_t)chi * 33));
-    const size_t nsc = up(sizeof(Cx<R>) * ((size_t)kc * chi + (size_t)chi * 33));
+    const size_t nsc = sizeof(R) == 4 ? up(8 * (size_t)kc * chi + 16 * (size_t)chi * 33 + 16) : 0;
     const size_t ychunk = up(sizeof(Cx<R>) * 16 * (size_t)mmax);
     work = t;
     for (size_t b : {twist, nsr, nsc, ychunk, tiles})
@@ -178,81 +183,75 @@ __device__ __forceinline__ void real_update(const R* W, R* out, int k, int p, in
 // Mixed precision: one Newton-Schulz step on the complex rows x_0..x_{k-1} of V (global,
 // row length len) that the FP32 back-transformation leaves orthonormal only to a few
 // 1e-7. E = X X^H - I is a few 1e-7 itself, so its Gram matrix has to be accurate far
-// below FP32 resolution: every entry is split into a multiple of 2^-11 and a rest. The
-// products of two leading parts are multiples of 2^-22 whose partial sums stay below 4
-// (Cauchy-Schwarz), so FP32 adds them exactly; the three products with a rest are 2^-12
-// times smaller and their rounding errors vanish against E. Four FMAs per real product,
-// where a compensated (Dot2) sum of the same accuracy takes eleven operations.
+// below FP32 resolution: the split products of the contractions give that (leading parts
+// summed exactly, the rest 2^-12 times smaller) at four FMAs per real product, where a
+// compensated (Dot2) sum takes eleven operations. One thread: column j of E and up to SP
+// of this block's rows, so that a split entry of x_j serves them all.
 template <int NT, int C>
 __device__ __forceinline__ void newton_schulz_cluster(const Cx<float>* X, int k, int len, int kcv, unsigned rank,
-                                                      Cx<float>* E, Cx<float>* chunk, Cx<float>* out, Cx<float>* site) {
+                                                      Cx<float>* E, SplitF* chunk, Cx<float>* out, Cx<float>* site) {
   const int tid = threadIdx.x;
-  constexpr int QC = 32, LDC = 33, SP = 4;
-  const int npair = kcv * k;
-  float hr[SP], hi[SP], cr[SP], ci[SP];
+  constexpr int QC = 32, LDC = 33, SP = 8;
+  const int jsh = row_shift(k), j = tid & ((1 << jsh) - 1), i0 = tid >> jsh, istep = NT >> jsh;
+  SplitAcc acc[SP];
 #pragma unroll
-  for (int s = 0; s < SP; ++s) hr[s] = hi[s] = cr[s] = ci[s] = 0.f;
-  constexpr float kMagic = 6144.0f;   // 1.5 2^12: adding it rounds to a multiple of 2^-11
-  for (int q0 = 0; q0 < len; q0 += QC) {
+  for (int s = 0; s < SP; ++s) zero(acc[s]);
+  const int ns = (kcv + istep - 1) / istep;   // rows per thread, uniform
+  auto load = [&](int q0) {
     const int qn = min(QC, len - q0);
     __syncthreads();
     for (int e = tid; e < k * QC; e += NT) {
-      const int j = e / QC, q = e % QC;
-      chunk[j * LDC + q] = q < qn ? ldcg(X + (size_t)j * len + q0 + q) : cx<float>(0.f, 0.f);
+      const int jj = e / QC, q = e % QC;
+      chunk[jj * LDC + q] = to_elem(q < qn ? ldcg(X + (size_t)jj * len + q0 + q) : cx<float>(0.f, 0.f));
     }
     __syncthreads();
+    return qn;
+  };
+  for (int q0 = 0; q0 < len; q0 += QC) {
+    load(q0);
+    if (j < k) {
+#pragma unroll 2
+      for (int q = 0; q < QC; ++q) {
+        SplitF b = chunk[j * LDC + q];
+        b.v.z = -b.v.z;   // conj
+        b.v.w = -b.v.w;
 #pragma unroll
-    for (int s = 0; s < SP; ++s) {
-      const int e = tid + s * NT;
-      if (e < npair) {
-        const int i = e / k, j = e - i * k;
-        const Cx<float>* xi = chunk + (rank + C * i) * LDC;
-        const Cx<float>* xj = chunk + j * LDC;
-#pragma unroll 4
-        for (int q = 0; q < QC; ++q) {
-          const Cx<float> a = xi[q], b = xj[q];
-          const float ax = __fadd_rn(__fadd_rn(a.x, kMagic), -kMagic), ay = __fadd_rn(__fadd_rn(a.y, kMagic), -kMagic);
-          const float bx = __fadd_rn(__fadd_rn(b.x, kMagic), -kMagic), by = __fadd_rn(__fadd_rn(b.y, kMagic), -kMagic);
-          const float axl = __fadd_rn(a.x, -ax), ayl = __fadd_rn(a.y, -ay);
-          const float bxl = __fadd_rn(b.x, -bx), byl = __fadd_rn(b.y, -by);
-          // a conj(b) = (ax bx + ay by) + i (ay bx - ax by)
-          hr[s] = fmaf(ay, by, fmaf(ax, bx, hr[s]));
-          hi[s] = fmaf(-ax, by, fmaf(ay, bx, hi[s]));
-          cr[s] = fmaf(ax, bxl, fmaf(axl, b.x, cr[s]));
-          cr[s] = fmaf(ay, byl, fmaf(ayl, b.y, cr[s]));
-          ci[s] = fmaf(ay, bxl, fmaf(ayl, b.x, ci[s]));
-          ci[s] = fmaf(-ax, byl, fmaf(-axl, b.y, ci[s]));
-        }
+        for (int s = 0; s < SP; ++s)
+          if (s < ns) mac(acc[s], chunk[(rank + C * min(i0 + s * istep, kcv - 1)) * LDC + q], b);
       }
     }
   }
   __syncthreads();
+  if (j < k) {
 #pragma unroll
-  for (int s = 0; s < SP; ++s) {
-    const int e = tid + s * NT;
-    if (e < npair) {
-      const int i = e / k, j = e - i * k;
-      const bool diag = j == (int)rank + C * i;
-      E[e] = diag ? cx<float>(__fadd_rn(__fadd_rn(hr[s], -1.0f), cr[s]), 0.f)
-                  : cx<float>(__fadd_rn(hr[s], cr[s]), __fadd_rn(hi[s], ci[s]));
+    for (int s = 0; s < SP; ++s) {
+      const int i = i0 + s * istep;
+      if (s < ns && i < kcv) {
+        const bool diag = j == (int)rank + C * i;
+        E[i * k + j] = diag ? cx<float>(__fadd_rn(__fadd_rn(acc[s].hx, -1.0f), acc[s].lx), 0.f) : value(acc[s]);
+      }
     }
   }
   for (int q0 = 0; q0 < len; q0 += QC) {
-    const int qn = min(QC, len - q0);
-    __syncthreads();
-    for (int e = tid; e < k * QC; e += NT) {
-      const int j = e / QC, q = e % QC;
-      chunk[j * LDC + q] = q < qn ? ldcg(X + (size_t)j * len + q0 + q) : cx<float>(0.f, 0.f);
-    }
-    __syncthreads();
+    const int qn = load(q0);
     for (int e = tid; e < kcv * QC; e += NT) {
       const int i = e / QC, q = e % QC;
       if (q >= qn) continue;
-      Cx<float> a = cx<float>(0.f, 0.f);
-#pragma unroll 4
-      for (int j = 0; j < k; ++j) cmac(a, E[i * k + j], chunk[j * LDC + q]);
+      Cx<float> a = cx<float>(0.f, 0.f), a2 = a;
+      int jj = 0;
+      for (; jj + 1 < k; jj += 2) {
+        const SplitF x0 = chunk[jj * LDC + q], x1 = chunk[(jj + 1) * LDC + q];
+        cmac(a, E[i * k + jj], cx<float>(x0.v.x + x0.v.y, x0.v.z + x0.v.w));
+        cmac(a2, E[i * k + jj + 1], cx<float>(x1.v.x + x1.v.y, x1.v.z + x1.v.w));
+      }
+      if (jj < k) {
+        const SplitF x0 = chunk[jj * LDC + q];
+        cmac(a, E[i * k + jj], cx<float>(x0.v.x + x0.v.y, x0.v.z + x0.v.w));
+      }
+      a = a + a2;
       const int t = rank + C * i;
-      const Cx<float> x = chunk[t * LDC + q];
+      const SplitF xs = chunk[t * LDC + q];
+      const Cx<float> x = cx<float>(xs.v.x + xs.v.y, xs.v.z + xs.v.w);   // exact: the split parts add up to x
       const Cx<float> v = cx<float>(fmaf(-0.5f, a.x, x.x), fmaf(-0.5f, a.y, x.y));
       out[(size_t)t * len + q0 + q] = v;
       site[(size_t)t * len + q0 + q] = conj(v);
@@ -260,89 +259,102 @@ __device__ __forceinline__ void newton_schulz_cluster(const Cx<float>* X, int k,
   }
 }
 
-// Back-transformation x <- H_0 H_1 ... H_{nref-1} x of this block's vectors, one warp per
-// vector, EL entries per lane, the reflectors staged from L2 in chunks of nch.
-template <class R, int NT, int C, int EL>
+// Back-transformation x <- H_0 H_1 ... H_{nref-1} x of this block's vectors: V vectors per
+// warp (independent chains that share a reflector's loads), EL entries per lane, the
+// reflectors staged from L2 in chunks of nch.
+template <class R, int NT, int C, int EL, int V>
 __device__ __forceinline__ void back_transform(const R* W, int p, int len, int nref, int kcv, unsigned rank, bool tall,
                                                int rr, const Cx<R>* Y, int ystride, const Cx<R>* tau, const Cx<R>* scl,
                                                Cx<R>* chunk, int nch, Cx<R>* out, Cx<R>* site) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int NW = NT / 32;
-  for (int v0 = 0; v0 < kcv; v0 += NW) {
-    const int i = v0 + warp, t = rank + C * i;
-    const bool act = i < kcv;
-    Cx<R> x[EL];
+  for (int v0 = 0; v0 < kcv; v0 += NW * V) {
+    Cx<R> x[V][EL];
+    bool act[V];
 #pragma unroll
-    for (int e = 0; e < EL; ++e) {
-      const int q = lane + 32 * e;
-      x[e] = cx<R>(act && q < p ? ldcg(W + (size_t)t * p + q) : R(0), R(0));
+    for (int v = 0; v < V; ++v) {
+      const int i = v0 + warp + v * NW, t = rank + C * i;
+      act[v] = i < kcv;
+#pragma unroll
+      for (int e = 0; e < EL; ++e) {
+        const int q = lane + 32 * e;
+        x[v][e] = cx<R>(act[v] && q < p ? ldcg(W + (size_t)t * p + q) : R(0), R(0));
+      }
     }
     for (int hi = nref; hi > 0; hi -= nch) {
       const int lo = max(0, hi - nch);
       __syncthreads();
-      for (int e = tid; e < (hi - lo) * len; e += NT) {
-        const int jj = e / len, q = e - jj * len, jr = lo + jj, start = tall ? jr + 1 : jr;
-        Cx<R> v = cx<R>(0, 0);
-        if (q == start)
-          v = cx<R>(1, 0);
-        else if (q > start)
-          v = tall ? ldcg(Y + (size_t)jr * ystride + q) * scl[jr] : ldcg(Y + (size_t)jr * ystride + q);
-        chunk[jj * len + q] = v;
+      for (int jj = warp; jj < hi - lo; jj += NW) {
+        const int jr = lo + jj, start = tall ? jr + 1 : jr;
+        const Cx<R> sc = scl[jr];
+        const Cx<R>* y = Y + (size_t)jr * ystride;
+        Cx<R> v[EL];
+#pragma unroll
+        for (int e = 0; e < EL; ++e) {
+          const int q = lane + 32 * e;
+          v[e] = q > start && q < len ? ldcg(y + q) : cx<R>(0, 0);
+        }
+#pragma unroll
+        for (int e = 0; e < EL; ++e) {
+          const int q = lane + 32 * e;
+          if (tall) v[e] = v[e] * sc;
+          if (q < len) chunk[jj * len + q] = q == start ? cx<R>(1, 0) : v[e];
+        }
       }
       __syncthreads();
-      if (act) {
+      if (act[0]) {
         for (int jr = hi - 1; jr >= lo; --jr) {
           const Cx<R>* h = chunk + (jr - lo) * len;
           const int start = tall ? jr + 1 : jr;
           Cx<R> hv[EL];
-          Cx<R> s = cx<R>(0, 0);
+          Cx<R> s[V];
+#pragma unroll
+          for (int v = 0; v < V; ++v) s[v] = cx<R>(0, 0);
 #pragma unroll
           for (int e = 0; e < EL; ++e) {
+            hv[e] = cx<R>(0, 0);
             if (32 * e + 31 >= start) {   // uniform: whole rows of zeros are left out
               const int q = lane + 32 * e;
-              hv[e] = q < len ? h[q] : cx<R>(0, 0);
-              cmac_conj(s, hv[e], x[e]);
+              if (q < len) hv[e] = h[q];
+#pragma unroll
+              for (int v = 0; v < V; ++v) cmac_conj(s[v], hv[e], x[v][e]);
             }
           }
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) {
-            s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
-            s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
-          }
-          const Cx<R> f = tau[jr] * s;
+          for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-          for (int e = 0; e < EL; ++e)
-            if (32 * e + 31 >= start) cmsub(x[e], f, hv[e]);
+            for (int v = 0; v < V; ++v) {
+              s[v].x += __shfl_xor_sync(0xffffffffu, s[v].x, o);
+              s[v].y += __shfl_xor_sync(0xffffffffu, s[v].y, o);
+            }
+          const Cx<R> tj = tau[jr];
+#pragma unroll
+          for (int v = 0; v < V; ++v) {
+            const Cx<R> f = tj * s[v];
+#pragma unroll
+            for (int e = 0; e < EL; ++e)
+              if (32 * e + 31 >= start) cmsub(x[v][e], f, hv[e]);
+          }
         }
       }
     }
-    if (act) {
 #pragma unroll
-      for (int e = 0; e < EL; ++e) {
-        const int q = lane + 32 * e;
-        if (q < len) {
-          const int nat = tall ? (q & 1) * rr + (q >> 1) : q;
-          out[(size_t)t * len + nat] = x[e];
-          if (site) site[(size_t)t * len + nat] = conj(x[e]);
+    for (int v = 0; v < V; ++v) {
+      const int t = rank + C * (v0 + warp + v * NW);
+      if (act[v]) {
+#pragma unroll
+        for (int e = 0; e < EL; ++e) {
+          const int q = lane + 32 * e;
+          if (q < len) {
+            const int nat = tall ? (q & 1) * rr + (q >> 1) : q;
+            out[(size_t)t * len + nat] = x[v][e];
+            if (site) site[(size_t)t * len + nat] = conj(x[v][e]);
+          }
         }
       }
     }
   }
   __syncthreads();
-}
-
-template <bool KF, class F>
-struct Op {
-  F f;
-  static constexpr bool k_fast = KF;
-  template <class... A>
-  __device__ __forceinline__ auto operator()(A... a) const {
-    return f(a...);
-  }
-};
-template <bool KF, class F>
-__device__ __forceinline__ Op<KF, F> op(F f) {
-  return Op<KF, F>{f};
 }
 
 // Site tensors of caller-owned memory (RAW) may lie on any 4-byte boundary: they are
@@ -372,7 +384,7 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
                                                 const double* theta, double cutoff, int max_sweeps) {
   extern __shared__ __align__(256) unsigned char smem[];
   constexpr bool kF64 = sizeof(R) == 8;
-  constexpr int NW = NT / 32, GMAX = Plan<R, NT, C>::GMAX;
+  constexpr int NW = NT / 32;
   const Plan<R, NT, C> L(m.chi);
   const unsigned rank_c = crank<C>();
   const int blk = blockIdx.x / C, s = slot0 + blk;
@@ -390,12 +402,15 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
   Cx<R>* xout2 = (Cx<R>*)(scratch + 8 * (size_t)chi * chi);
 
   // fixed part
-  Cx<double>* U = (Cx<double>*)smem;
-  Cx<R>* Uf = (Cx<R>*)(smem + 256);
+  Cx<R>* Uh = (Cx<R>*)smem;                   // the gate matrix; FP32: leading parts,
+  Cx<R>* Ul = (Cx<R>*)(smem + 256);           // and what they leave of the FP64 entries
+  GateRec* rec = (GateRec*)(smem + 384);
   double* red = (double*)(smem + 512);        // 32 per-warp partials
   double* redc = red + 32;                    // per-block partials of the cluster (16)
   int* misc = (int*)(redc + 16);              // [0] k, [1] collapsed, [2] Jacobi caps, [3] splits
-  R* dd = (R*)(smem + 1280);
+  int64_t* soff = (int64_t*)(smem + 1024);    // site offsets (128)
+  int* ranks = (int*)(smem + 2048);           // bond ranks (129): every block keeps its own copy
+  R* dd = (R*)(smem + Plan<R, NT, C>::kFixed);
   R* ee = dd + mmax;
   Cx<R>* tau = (Cx<R>*)(ee + mmax);
   Cx<R>* scl = tau + mmax;
@@ -405,12 +420,16 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
   R* bn = (R*)exch;                           // TGK off-diagonals, scaled
   R* b2 = bn + 2 * mmax;
   R* sig = b2 + 2 * mmax;
-  R* lo = sig + mmax;
-  R* hi = lo + mmax;
-  double* sig2d = (double*)(((uintptr_t)(hi + mmax) + 15) & ~(uintptr_t)15);
+  R* usig = sig + mmax;                       // the same before sorting
+  double* sig2d = (double*)(((uintptr_t)(usig + mmax) + 15) & ~(uintptr_t)15);
   R* small = (R*)(sig2d + mmax);              // 256
   float* b2f = (float*)(small + 256);
   int* order = (int*)(b2f + 2 * mmax);        // 2 mmax
+  int* bs = order + 2 * mmax;                 // block of each singular value: start, end
+  int* be = bs + mmax;
+  int* bstart = be + mmax;                    // unreduced blocks of the TGK: starts (2 mmax + 1),
+  int* bpre = bstart + 2 * mmax + 1;          // values asked of the blocks before (2 mmax + 1)
+  R* gscale = (R*)(((uintptr_t)(bpre + 2 * mmax + 1) + 15) & ~(uintptr_t)15);
   Cx<R>* T = (Cx<R>*)work;
 
   const double* th = theta + (size_t)blk * c.n_params;
@@ -431,8 +450,11 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
   const int64_t g_first = c.start_gate ? max(g0, c.start_gate[blk]) : g0;
   const int64_t g_shift = c.shift_gate ? c.shift_gate[blk] : -1;
   const double phi_shift = c.shift_phi ? c.shift_phi[blk] : 0.0;
-  csync<C>();   // every block of the cluster runs before any touches a peer's shared memory
-  for (int64_t g = g_first; g < g1; ++g) {
+  for (int i = tid; i <= n; i += NT) ranks[i] = ldcg(rank + i);
+  for (int i = tid; i < n; i += NT) soff[i] = m.site_off[i];
+  // gate g by 16 lanes: fixed, or mats[m1] . Rz(phi) on one site . mats[m0]. Done for gate
+  // g + 1 by a warp that idles while the twisted factorisations of gate g run.
+  auto fetch_gate = [&](int64_t g, int l) {
     GateRec gr;
     if constexpr (RAW) {
       gr.bond = c.raw_bond[g];
@@ -441,36 +463,39 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
     } else {
       gr = c.gates[g];
     }
-    // (1) the 4x4 gate: fixed, or mats[m1] . Rz(phi) on one site . mats[m0]
-    if (tid < 16) {
-      const int i = tid >> 2, j = tid & 3;
-      const double* A = c.mats + 32 * (size_t)gr.m0;
-      Cx<double> u;
-      if (gr.param < 0) {
-        u = cx<double>(A[2 * tid], A[2 * tid + 1]);
-      } else {
-        const Cx<double>* Am = (const Cx<double>*)A;
-        const Cx<double>* P = (const Cx<double>*)c.mats + 16 * (size_t)gr.m1;
-        const double half = 0.5 * (gr.scale * th[gr.param] + (g == g_shift ? phi_shift : 0.0));
-        double sn, cs;
-        sincos(half, &sn, &cs);
-        u = cx(0.0, 0.0);
-        for (int k = 0; k < 4; ++k) {
-          const int bit = gr.rz_site == 0 ? ((k >> 1) & 1) : (k & 1);
-          const Cx<double> pz = cx(cs, bit ? sn : -sn);  // Rz = diag(e^{-i phi/2}, e^{i phi/2})
-          u = u + (P[i * 4 + k] * pz) * Am[k * 4 + j];
-        }
+    const int i = l >> 2, j = l & 3;
+    const double* A = c.mats + 32 * (size_t)gr.m0;
+    Cx<double> u;
+    if (gr.param < 0) {
+      u = cx<double>(A[2 * l], A[2 * l + 1]);
+    } else {
+      const Cx<double>* Am = (const Cx<double>*)A;
+      const Cx<double>* P = (const Cx<double>*)c.mats + 16 * (size_t)gr.m1;
+      const double half = 0.5 * (gr.scale * th[gr.param] + (g == g_shift ? phi_shift : 0.0));
+      double sn, cs;
+      sincos(half, &sn, &cs);
+      u = cx(0.0, 0.0);
+      for (int k = 0; k < 4; ++k) {
+        const int bit = gr.rz_site == 0 ? ((k >> 1) & 1) : (k & 1);
+        const Cx<double> pz = cx(cs, bit ? sn : -sn);  // Rz = diag(e^{-i phi/2}, e^{i phi/2})
+        u = u + (P[i * 4 + k] * pz) * Am[k * 4 + j];
       }
-      U[tid] = u;
-      Uf[tid] = cx<R>((R)u.x, (R)u.y);
     }
-    const int bond = gr.bond;
+    const Cx<R> h = cx<R>((R)u.x, (R)u.y);
+    Uh[l] = h;
+    if constexpr (!kF64) Ul[l] = cx<R>((R)(u.x - (double)h.x), (R)(u.y - (double)h.y));
+    if (l == 0) rec->bond = gr.bond;
+  };
+  if (tid < 16 && g_first < g1) fetch_gate(g_first, tid);
+  csync<C>();   // every block of the cluster runs before any touches a peer's shared memory
+  for (int64_t g = g_first; g < g1; ++g) {
+    const int bond = rec->bond;
     if constexpr (RAW) {
       // caller-owned device arrays: the bond and the three ranks it touches must lie
       // inside the site capacities before anything is indexed (uniform over the cluster)
       bool ok = bond >= 0 && bond <= n - 2;
       if (ok) {
-        const int r0 = ldcg(rank + bond), r1 = ldcg(rank + bond + 1), r2 = ldcg(rank + bond + 2);
+        const int r0 = ranks[bond], r1 = ranks[bond + 1], r2 = ranks[bond + 2];
         ok = r0 >= 1 && r0 <= bond_cap(bond - 1, n, chi) && r1 >= 1 && r1 <= bond_cap(bond, n, chi) && r2 >= 1 &&
              r2 <= bond_cap(bond + 1, n, chi);
       }
@@ -479,31 +504,28 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
         break;
       }
     }
-    const int rl = ldcg(rank + bond), rm = ldcg(rank + bond + 1), rr = ldcg(rank + bond + 2);
+    const int rl = ranks[bond], rm = ranks[bond + 1], rr = ranks[bond + 2];
     const int mrows = 2 * rl, ncol = 2 * rr;
     const bool tall = mrows >= ncol;
-    const int tr = tall ? mrows : ncol, tp = tall ? ncol : mrows, ld = tr;
-    Cx<R>* Bn = Bslot + m.site_off[bond];
-    Cx<R>* Bn1 = Bslot + m.site_off[bond + 1];
+    const int tr = tall ? mrows : ncol, tp = tall ? ncol : mrows, ld = Plan<R, NT, C>::lead(tr);
+    Cx<R>* Bn = Bslot + soff[bond];
+    Cx<R>* Bn1 = Bslot + soff[bond + 1];
     const double* laml = bond > 0 ? lam + (size_t)(bond - 1) * chi : nullptr;
-    __syncthreads();
     // (2) Eq. (7): M[(a,i),(j,c)] = sum_{i'j'} U[ij,i'j'] sum_b B_n[a,i',b] B_{n+1}[b,j',c];
     //     W <- M; Eq. (8): M' = lambda_{n-1}[a] M. Each block contracts the columns of T it
     //     owns into place, then applies the gate and lambda to its (a, c) quads.
     const int nq = ((tall ? rr : rl) + C - 1 - (int)rank_c) / C;   // own c (tall) or a (wide)
     if (tall)
-      tile_gemm<R, NT>(
-          mrows, 2 * nq, rm, [&](int mi, int k) { return ld_site<RAW>(Bn + (size_t)mi * rm + k); },
-          op<false>([&](int k, int ni) {
-            return ld_site<RAW>(Bn1 + (size_t)k * ncol + (ni & 1) * rr + rank_c + C * (ni >> 1));
-          }),
-          [&](int mi, int ni, Cx<R> v) { T[(size_t)ni * ld + mi] = v; }, exch);
+      tile_gemm<R, NT, false>(
+          mrows, 2 * nq, rm, [&](int mi, int k) { return ld_site<RAW>(Bn + mi * rm + k); },
+          [&](int k, int ni) { return ld_site<RAW>(Bn1 + k * ncol + (ni & 1) * rr + rank_c + C * (ni >> 1)); },
+          [&](int mi, int ni, Cx<R> v) { T[ni * ld + mi] = v; }, exch);
     else
-      tile_gemm<R, NT>(
+      tile_gemm<R, NT, false>(
           2 * nq, ncol, rm,
-          [&](int mi, int k) { return ld_site<RAW>(Bn + (size_t)(2 * (rank_c + C * (mi >> 1)) + (mi & 1)) * rm + k); },
-          op<false>([&](int k, int ni) { return ld_site<RAW>(Bn1 + (size_t)k * ncol + ni); }),
-          [&](int mi, int ni, Cx<R> v) { T[(size_t)mi * ld + ni] = v; }, exch);
+          [&](int mi, int k) { return ld_site<RAW>(Bn + (2 * (rank_c + C * (mi >> 1)) + (mi & 1)) * rm + k); },
+          [&](int k, int ni) { return ld_site<RAW>(Bn1 + k * ncol + ni); },
+          [&](int mi, int ni, Cx<R> v) { T[mi * ld + ni] = v; }, exch);
     double fro = 0.0;
     const int qfast = tall ? rl : rr;
     for (int it = tid; it < nq * qfast; it += NT) {
@@ -523,16 +545,17 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
       for (int ij = 0; ij < 4; ++ij) {
         Cx<R> v = cx<R>(0, 0);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) cmac(v, Uf[ij * 4 + kk], th4[kk]);
+        for (int kk = 0; kk < 4; ++kk) {
+          if constexpr (!kF64) cmac(v, Ul[ij * 4 + kk], th4[kk]);
+        }
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) cmac(v, Uh[ij * 4 + kk], th4[kk]);
         W[(size_t)(2 * a + (ij >> 1)) * ncol + (ij & 1) * rr + cc] = v;
         const Cx<R> mv = la * v;
         *e[ij] = tall ? mv : conj(mv);
-        if constexpr (kF64)
-          part += norm2(mv);
-        else
-          fro += (double)norm2(mv);
+        part += norm2(mv);
       }
-      if constexpr (kF64) fro += part;
+      fro += (double)part;
     }
     for (int o = 16; o > 0; o >>= 1) fro += __shfl_xor_sync(0xffffffffu, fro, o);
     if (lane == 0) red[warp] = fro;
@@ -550,6 +573,7 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
     // the gate is skipped, the state left as it was, and the host reports the count
     if (!(total <= DBL_MAX)) {
       if (tid == 0) ++st_nonfinite;
+      if (tid < 16 && g + 1 < g1) fetch_gate(g + 1, tid);
       csync<C>();
       continue;
     }
@@ -561,12 +585,11 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
       b.ld = ld;
       b.zrows = mmax;
       b.zp = (Cx<R>*)exch;
-      b.colp = b.zp + (size_t)2 * C * GMAX * mmax;
+      b.colp = b.zp + (size_t)2 * C * L.gmax * mmax;
       b.xs = b.colp + 2 * mmax;
       b.us = b.xs + mmax;
-      b.rj = b.us + mmax;
-      b.fj = b.rj + 2 * L.cl;
-      b.sc = b.fj + L.cl;
+      b.cs = (ColState<R>*)(b.us + mmax);
+      b.sc = (Cx<R>*)(b.cs + L.cl);
       b.nrmp = (R*)(b.sc + 8);
       b.part = b.nrmp + 2 * C;
       b.dd = dd;
@@ -575,7 +598,7 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
       b.scl = scl;
       b.Y = Y;
       b.ystride = mmax;
-      bidiagonalize_cluster<R, NT, C, GMAX>(b, tr, tp, tall, rank_c);
+      bidiagonalize_cluster<R, NT, C>(b, L.gmax, tr, tp, tall, rank_c);
     }
     PHASE(1);
     // Golub-Kahan tridiagonal off-diagonal (d0, e0, d1, e1, ..., d_{p-1}), scaled by a power
@@ -592,7 +615,6 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
       if (lane == 0) {
         small[0] = top;
         misc[1] = 0;
-        misc[3] = 0;
       }
     }
     __syncthreads();
@@ -601,70 +623,175 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
     if (smax > R(0)) frexp(smax, &ex);        // smax = f 2^ex, f in [1/2, 1)
     ex = max(min(ex, kF64 ? 1000 : 120), kF64 ? -1000 : -120);
     const R down = ldexp(R(1), -ex), back = ldexp(R(1), ex), top = smax * down;
-    // split the TGK where an off-diagonal is negligible (exact degeneracies live in
-    // different blocks after this; the perturbation is below 4 eps ||B||)
+    // split the TGK where an off-diagonal is negligible (the perturbation is below 4 eps
+    // ||B||): exact degeneracies, as symmetry sectors make them, live in different blocks
     for (int i = tid; i < N - 1; i += NT) {
       R v = ((i & 1) ? ee[i >> 1] : dd[i >> 1]) * down;
-      if (rabs(v) <= R(4) * Eps<R>::v * top) {
-        v = R(0);
-        misc[3] = 1;
-      }
+      if (rabs(v) <= R(4) * Eps<R>::v * top) v = R(0);
       bn[i] = v;
       b2[i] = v * v;
-      if constexpr (kF64) b2f[i] = (float)(v * v);
+      if constexpr (kF64) b2f[i] = rabs(v) <= R(4) * (R)Eps<float>::v * top ? 0.f : (float)(v * v);   // FP32 range and resolution
     }
     if (tid == 0) {
       bn[N - 1] = R(0);
       b2[N - 1] = R(0);
+      if constexpr (kF64) b2f[N - 1] = 0.f;
     }
     __syncthreads();
-    const bool split = misc[3] != 0;
-    const int kk = min(chi, tp), kco = (kk + C - 1 - (int)rank_c) / C;
+    const float* bf = kF64 ? b2f : (const float*)b2;
+    const float topf = fminf((float)top * 1.001f, 1.01f);
+    const int kk = min(chi, tp);
     int passes = 0;
-    if constexpr (!kF64) {
-      for (int i = warp; i < kco; i += NW) {
-        const int t = rank_c + C * i;
-        float a, b;
-        passes = max(passes, warp_bisect(b2, N, t, fminf(top * 1.001f, 1.01f), &a, &b));
-        if (lane < C) {
-          peer<C>(lo, lane)[t] = a;
-          peer<C>(hi, lane)[t] = b;
-          peer<C>(sig, lane)[t] = 0.5f * (a + b);
+    // Blocks, and how many of its values each has to give. A block of m indices has
+    // floor(m / 2) positive values. If all blocks together have more than kk, those below
+    // a bound under the kk-th value of the whole (with a margin far above rounding) are
+    // left out. Every value is then asked of one block, so no two vectors can coincide.
+    if (warp == 0) {
+      int nb = 0;
+      for (int i0 = 0; i0 < N; i0 += 32) {
+        const int i = i0 + lane;
+        const bool end = i < N && b2[i] == R(0);
+        const unsigned mk = __ballot_sync(0xffffffffu, end);
+        if (end) bstart[nb + 1 + __popc(mk & ((1u << lane) - 1u))] = i + 1;
+        nb += __popc(mk);
+      }
+      float cut_at = 0.f;
+      if (nb > 1) {
+        int have = 0;
+        __syncwarp();
+        for (int i = lane; i < nb; i += 32) have += (bstart[i + 1] - (i ? bstart[i] : 0)) >> 1;
+        for (int o = 16; o > 0; o >>= 1) have += __shfl_xor_sync(0xffffffffu, have, o);
+        if (have > kk) {
+          const int t = kk - 1;
+          float a, b;
+          warp_bisect<1>(bf, 0, N, &t, topf, &a, &b);
+          // values near the FP32 resolution are all asked for
+          cut_at = a > 1e-5f * topf ? a * (1.0f - 1e-4f) : 0.f;
         }
       }
-    } else {
-      const float topf = fminf((float)top * 1.001f, 1.01f);
-      for (int i = warp; i < kco; i += NW) {
-        float a, b;
-        passes = max(passes, warp_bisect(b2f, N, rank_c + C * i, topf, &a, &b));
-        if (lane == 0) sig2d[i] = __hiloint2double(__float_as_int(b), __float_as_int(a));   // the FP32 bracket
+      if (lane == 0) {
+        bstart[0] = 0;
+        misc[3] = nb;
+        small[1] = (R)cut_at;
       }
+    }
+    __syncthreads();
+    const int nb = misc[3];
+    {
+      const float cut_at = (float)small[1];
+      for (int i = tid; i < nb; i += NT) {
+        const int s = bstart[i], e = bstart[i + 1];
+        int cnt = nb == 1 ? kk : (e - s) >> 1;
+        if (cut_at > 0.f && cnt > 0) cnt = min(cnt, sturm_ge1<float>(bf, s, e, cut_at));
+        bpre[i + 1] = cnt;
+      }
+    }
+    __syncthreads();
+    if (warp == 0) {
+      int base = 0;
+      for (int i0 = 0; i0 < nb; i0 += 32) {
+        const int i = i0 + lane;
+        int v = i < nb ? bpre[i + 1] : 0;
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, v, o);
+          if (lane >= o) v += y;
+        }
+        __syncwarp();
+        if (i < nb) bpre[i + 1] = base + v;
+        base += __shfl_sync(0xffffffffu, v, 31);
+      }
+      if (lane == 0) bpre[0] = 0;
+    }
+    __syncthreads();
+    // value u (in block order) is the (u - bpre[block])-th of its block; this block of the
+    // cluster finds u = rank + C i
+    const int nval = bpre[nb], kco = (nval + C - 1 - (int)rank_c) / C;
+    auto block_of = [&](int u) {
+      int a = 0, b = nb;
+      while (b - a > 1) {
+        const int mid = (a + b) >> 1;
+        if (bpre[mid] <= u) a = mid; else b = mid;
+      }
+      return a;
+    };
+    for (int i = warp; i < kco; i += NW) {
+      const int u = rank_c + C * i;
+      float a[2], b[2];
+      int nv = 1;
+      if (nb == 1) {
+        // two values per warp at a time where there are more values than warps
+        const int t[2] = {u, (int)rank_c + C * min(i + NW, kco - 1)};
+        if (i + NW < kco) {
+          passes = max(passes, warp_bisect<2>(bf, 0, N, t, topf, a, b));
+          nv = 2;
+        } else {
+          passes = max(passes, warp_bisect<1>(bf, 0, N, t, topf, a, b));
+        }
+      } else {
+        const int ib = block_of(u), t = u - bpre[ib];
+        passes = max(passes, warp_bisect<1>(bf, bstart[ib], bstart[ib + 1], &t, topf, a, b));
+      }
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        if (v >= nv) break;
+        if constexpr (kF64) {
+          // the bracket for the FP64 passes
+          if (lane == 0) sig2d[i + v * NW] = __hiloint2double(__float_as_int(b[v]), __float_as_int(a[v]));
+        } else if (lane < C) {
+          peer<C>(usig, lane)[u + C * v * NW] = 0.5f * (a[v] + b[v]);
+        }
+      }
+      if (nv == 2) i += NW;
+    }
+    if constexpr (kF64) {
       __syncthreads();
-      constexpr int LT = 4;
-      for (int i0 = warp * (32 / LT); i0 < kco; i0 += NW * (32 / LT)) {
-        const int i = i0 + lane / LT;
+      for (int i0 = warp * 8; i0 < kco; i0 += NW * 8) {
+        const int i = i0 + lane / 4;
         const bool act = i < kco;
-        const int t = rank_c + C * (act ? i : i0);
+        const int u = rank_c + C * (act ? i : i0), ib = block_of(u);
         const double pk = sig2d[act ? i : i0];
         double a, b;
-        passes += lanes_bisect<LT>(b2, N, t, act, (double)top * 1.001, __int_as_float(__double2loint(pk)),
-                                   __int_as_float(__double2hiint(pk)), &a, &b);
+        passes += lanes_bisect(b2, bstart[ib], bstart[ib + 1], u - bpre[ib], act, (double)top * 1.001,
+                               __int_as_float(__double2loint(pk)), __int_as_float(__double2hiint(pk)), &a, &b);
         if (act)
-          for (int cb = lane & (LT - 1); cb < C; cb += LT) {
-            peer<C>(lo, cb)[t] = a;
-            peer<C>(hi, cb)[t] = b;
-            peer<C>(sig, cb)[t] = 0.5 * (a + b);
-          }
+          for (int cb = lane & 3; cb < C; cb += 4) peer<C>(usig, cb)[u] = 0.5 * (a + b);
       }
     }
     csync<C>();
+    // descending order over all blocks
+    for (int u = tid; u < nval; u += NT) {
+      const R x = usig[u];
+      int r = u;
+      if (nb > 1) {
+        r = 0;
+        for (int w = 0; w < nval; ++w) {
+          const R y = usig[w];
+          r += (y > x) || (y == x && w < u);
+        }
+      }
+      if (r < kk) {
+        const int ib = block_of(u);
+        sig[r] = x;
+        bs[r] = bstart[ib];
+        be[r] = bstart[ib + 1];
+      }
+    }
+    __syncthreads();
+    const int nsig = min(kk, nval);
     if (warp == 0) {
       // sig is descending: k = number of leading values above cutoff * sig_0
-      const R s0 = sig[0], cut = (R)cutoff * s0;
+      const R s0 = nsig > 0 ? sig[0] : R(0), cut = (R)cutoff * s0;
       int cntk = 0;
-      for (int t = lane; t < kk; t += 32) cntk += (sig[t] > cut && sig[t] > R(0));
+      for (int t = lane; t < nsig; t += 32) cntk += (sig[t] > cut && sig[t] > R(0));
       for (int o = 16; o > 0; o >>= 1) cntk += __shfl_xor_sync(0xffffffffu, cntk, o);
-      if (lane == 0) misc[0] = cntk > 0 ? cntk : 1;
+      if (lane == 0) {
+        misc[0] = cntk > 0 ? cntk : 1;
+        if (nsig == 0) {   // M' = 0
+          sig[0] = R(0);
+          bs[0] = 0;
+          be[0] = N;
+        }
+      }
     }
     __syncthreads();
     const int k = misc[0];
@@ -674,50 +801,101 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
     }
     PHASE(2);
 
-    // (4) singular vectors of B from twisted factorisations: pivots from both ends (one lane
-    // per direction), the twist where |gamma| is smallest, the vector outward from there
-    const R tiny = kF64 ? R(1e-300) : R(1e-30);
+    // (4) singular vectors of B from twisted factorisations of TGK - sigma. Leading minors
+    // p_i from both ends by the division-free recurrence (one lane per vector and end: the
+    // only serial chain, one multiply-add a step); the pivots' reciprocals p_{i-1} / p_i,
+    // the twist where |gamma| is smallest and the ratios of neighbouring entries by whole
+    // warps; then the running products of the ratios outward from the twist.
     const int kcv = (k + C - 1 - (int)rank_c) / C;   // own vectors t = rank_c + C i
-    const int odd = tall ? 0 : 1;
     {
-      R* F = (R*)work;                       // [kcv][2][N] reciprocal pivots
+      constexpr int STEP = SturmGroup<R>::v;
+      const R big = kF64 ? R(1e300) : R(1e30);
+      const int odd = tall ? 0 : 1;
+      R* F = (R*)work;                       // [kcv][2][N]: minors, then reciprocal pivots, ratios, entries
+      const int ns = N / STEP + 1;
+      R* S = gscale;                         // [kcv][2][ns]: scale of each group of steps
       int* rng = order;                      // [kcv][3]: block start, end, twist
+      if (warp == NW - 1 && lane < 16 && g + 1 < g1) fetch_gate(g + 1, lane);
       const int v = tid >> 1, dir = tid & 1;
       const bool act = v < kcv;
-      R lamv = 0;
       int s0 = 0, e0 = N;
       if (act) {
         const int t = rank_c + C * v;
-        lamv = sig[t];
-        if (split) owning_range<R>(b2, N, sig, t, R(8) * (hi[t] - lo[t]) + R(4) * Eps<R>::v * top, &s0, &e0);
-        R* f = F + (size_t)(2 * v + dir) * N;
-        int i = dir ? e0 - 1 : s0;
-        const int step = dir ? -1 : 1;
-        R d = -lamv;
-        if (rabs(d) < tiny) d = -tiny;
-        R rv = pivot_rcp(d);
-        f[i] = rv;
-#pragma unroll 4
-        for (int q = 1; q < e0 - s0; ++q) {
-          const R bb = b2[dir ? i - 1 : i];
-          i += step;
-          d = fma(-bb, rv, -lamv);
-          if (rabs(d) < tiny) d = -tiny;
-          rv = pivot_rcp(d);
-          f[i] = rv;
-        }
+        const R x = sig[t];
+        s0 = bs[t];
+        e0 = be[t];
         if (dir == 0) {
           rng[3 * v] = s0;
           rng[3 * v + 1] = e0;
+        }
+        // entry q of the walk is index i0 + st q; its off-diagonal is b2[i0 + st q + bo]
+        const int st = dir ? -1 : 1, i0 = dir ? e0 - 1 : s0, bo = dir ? 0 : -1, len = e0 - s0;
+        R* f = F + (size_t)(2 * v + dir) * N;
+        R* sg = S + (size_t)(2 * v + dir) * ns;
+        R prev = R(1), cur = -x;
+        f[i0] = cur;
+        int q = 1, gi = 0;
+        for (; q + STEP <= len; q += STEP) {
+          R bb[STEP], o[STEP];
+#pragma unroll
+          for (int u = 0; u < STEP; ++u) bb[u] = b2[i0 + st * (q + u) + bo];
+#pragma unroll
+          for (int u = 0; u < STEP; ++u) {
+            const R nxt = fma(-x, cur, -(bb[u] * prev));
+            prev = cur;
+            cur = nxt;
+            o[u] = cur;
+          }
+          const R sc = rescale_factor(prev, cur);
+          prev *= sc;
+          cur *= sc;
+          o[STEP - 1] = cur;   // the last of a group is kept scaled; the group's scale beside it
+#pragma unroll
+          for (int u = 0; u < STEP; ++u) f[i0 + st * (q + u)] = o[u];
+          sg[gi++] = sc;
+        }
+        for (; q < len; ++q) {
+          const R nxt = fma(-x, cur, -(b2[i0 + st * q + bo] * prev));
+          prev = cur;
+          cur = nxt;
+          f[i0 + st * q] = cur;
         }
       }
       __syncthreads();
       for (int w = warp; w < kcv; w += NW) {
         const int ws = rng[3 * w], we = rng[3 * w + 1];
+        R* fu = F + (size_t)2 * w * N;
+        R* fd = fu + N;
+        // reciprocal pivots in place, walking against the recurrence so that the minor
+        // before is still there: entry q needs entries q and q - 1 of its walk
+        const int len = we - ws;
+        for (int hi_q = len; hi_q > 0; hi_q -= 32) {
+          const int q = hi_q - 1 - lane;
+          R r0 = 0, r1 = 0;
+          if (q >= 0) {
+#pragma unroll
+            for (int d = 0; d < 2; ++d) {
+              const R* f = d ? fd : fu;
+              const R* sg = S + (size_t)(2 * w + d) * ns;
+              const int at = d ? we - 1 - q : ws + q, pv = d ? at + 1 : at - 1;
+              R num = q > 0 ? f[pv] : R(1);
+              // q closes group (q - 1) / STEP when q = STEP, 2 STEP, ..., if that group was whole
+              if (q > 0 && q % STEP == 0) num *= sg[q / STEP - 1];
+              const R den = f[at];
+              R r = num * inverse(den);
+              if (!(rabs(r) <= big)) r = -big;   // a zero pivot counts as a tiny negative one
+              (d ? r1 : r0) = r;
+            }
+          }
+          __syncwarp();
+          if (q >= 0) {
+            fu[ws + q] = r0;
+            fd[we - 1 - q] = r1;
+          }
+          __syncwarp();
+        }
         const R lw = sig[rank_c + C * w];
-        const R* fu = F + (size_t)2 * w * N;
-        const R* fd = fu + N;
-        R best = R(1e30);
+        R best = big;
         int at = we - 1;
         for (int i = ws + lane; i < we; i += 32) {
           // gamma_i = -lam - b_{i-1}^2 / dp_{i-1} - b_i^2 / dm_{i+1}
@@ -739,31 +917,34 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
           }
         }
         if (lane == 0) rng[3 * w + 2] = at;
-        // outside the block the vector is zero
-        R* z = F + (size_t)2 * w * N;
-        for (int i = lane; i < N; i += 32)
-          if (i < ws || i >= we) z[i] = R(0);
+        // ratios z_i / z_{i+1} = -b_i / dp_i above the twist, z_i / z_{i-1} = -b_{i-1} / dm_i below
+        for (int i = lane; i < N; i += 32) {
+          R r = 0;
+          if (i >= ws && i < at) r = -bn[i] * fu[i];
+          if (i > at && i < we) r = -bn[i - 1] * fd[i];
+          if (i == at) r = R(1);
+          fu[i] = r;
+        }
       }
       __syncthreads();
       if (act) {
-        const int at = rng[3 * v + 2];
-        R* z = F + (size_t)2 * v * N;        // the vector overwrites the forward pivots
-        const R* f = F + (size_t)(2 * v + dir) * N;
+        const int at = rng[3 * v + 2], st = dir ? 1 : -1, len = dir ? e0 - 1 - at : at - s0;
+        R* z = F + (size_t)2 * v * N + at;
         R zv = 1;
-        if (dir == 0) {
-          z[at] = R(1);
-          // z_i = -(b_i / dp_i) z_{i+1}
-#pragma unroll 8
-          for (int i = at - 1; i >= s0; --i) {
-            zv *= -bn[i] * f[i];
-            z[i] = zv;
+        int q = 1;
+        for (; q + 7 <= len; q += 8) {
+          R r[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) r[u] = z[st * (q + u)];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            zv *= r[u];
+            z[st * (q + u)] = zv;
           }
-        } else {
-#pragma unroll 8
-          for (int i = at + 1; i < e0; ++i) {
-            zv *= -bn[i - 1] * f[i];
-            z[i] = zv;
-          }
+        }
+        for (; q <= len; ++q) {
+          zv *= z[st * q];
+          z[st * q] = zv;
         }
       }
       __syncthreads();
@@ -834,8 +1015,13 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
       const int nch = max(1, min(nref, (int)(L.work / (sizeof(Cx<R>) * ncol))));
       Cx<R>* site = kF64 ? Bn1 : nullptr;
       auto go = [&](auto el) {
-        back_transform<R, NT, C, decltype(el)::value>(Wc, tp, ncol, nref, kcv, rank_c, tall, rr, Y, mmax, tau, scl,
-                                                      (Cx<R>*)work, nch, xout, site);
+        constexpr int EL = decltype(el)::value;
+        if (kcv > NW)
+          back_transform<R, NT, C, EL, 2>(Wc, tp, ncol, nref, kcv, rank_c, tall, rr, Y, mmax, tau, scl, (Cx<R>*)work,
+                                          nch, xout, site);
+        else
+          back_transform<R, NT, C, EL, 1>(Wc, tp, ncol, nref, kcv, rank_c, tall, rr, Y, mmax, tau, scl, (Cx<R>*)work,
+                                          nch, xout, site);
       };
       if (ncol <= 32)
         go(std::integral_constant<int, 1>{});
@@ -920,7 +1106,7 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
       //      back-transformation, not the rounding of the stored tensors, dominates the
       //      energy error; one Newton-Schulz step brings it down to the storage rounding
       Cx<float>* E = (Cx<float>*)work;
-      Cx<float>* chunk = E + (size_t)L.kc * chi;
+      SplitF* chunk = (SplitF*)(E + ((size_t)L.kc * chi + 1) / 2 * 2);
       if constexpr (RAW) {
         newton_schulz_cluster<NT, C>(xout, kf, ncol, kcf, rank_c, E, chunk, xout2, xout2);
         __syncthreads();
@@ -944,12 +1130,15 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
     //     M v_t), lambda_n <- sigma
     {
       const int mper = (mrows + C - 1) / C, m0 = min(mrows, mper * (int)rank_c), mn = min(mper, mrows - m0);
-      tile_gemm<R, NT>(
-          mn, kf, ncol, [&](int mi, int q) { return ldcg(W + (size_t)(m0 + mi) * ncol + q); },
-          op<true>([&](int q, int t) { return ldcg(xv + (size_t)t * ncol + q); }),
-          [&](int mi, int t, Cx<R> v) { st_site<RAW>(Bn + (size_t)(m0 + mi) * kf + t, v); }, work);
+      tile_gemm<R, NT, true>(
+          mn, kf, ncol, [&](int mi, int q) { return ldcg(W + (m0 + mi) * ncol + q); },
+          [&](int q, int t) { return ldcg(xv + t * ncol + q); },
+          [&](int mi, int t, Cx<R> v) { st_site<RAW>(Bn + (m0 + mi) * kf + t, v); }, work);
     }
-    if (rank_c == 0 && tid == 0) rank[bond + 1] = kf;
+    if (tid == 0) {
+      ranks[bond + 1] = kf;
+      if (rank_c == 0) rank[bond + 1] = kf;
+    }
     csync<C>();
     PHASE(6);
     if (tid == 0) alg_flops += flops_per_gate(rl, rm, rr, kf);
@@ -1018,11 +1207,11 @@ template <bool RAW>
 static cudaError_t launch_mixed(const DevMPS& m, const CircDev& c, int64_t g0, int64_t g1, int slot0, int count,
                                 const double* theta, double cutoff, int max_sweeps, cudaStream_t st) {
   if (m.chi <= 16)
-    return launch_cluster<float, 512, 1, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
+    return launch_cluster<float, 256, 1, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
   if (m.chi <= 64)
-    return launch_cluster<float, 512, 4, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
+    return launch_cluster<float, 256, 4, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
   if constexpr (!RAW)
-    return launch_cluster<float, 512, 8, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
+    return launch_cluster<float, 256, 8, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
   return cudaErrorInvalidValue;
 }
 

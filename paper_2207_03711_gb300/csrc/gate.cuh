@@ -68,67 +68,172 @@ __device__ __forceinline__ double ldcg(const double* p) { return __ldcg(p); }
 __device__ __forceinline__ int ldcg(const int* p) { return __ldcg(p); }
 
 // ------------------------------------------------------------------------- tiled GEMM
-// out(m, n) = sum_k a(m, k) b(k, n) for m < M, n < N by one block: NT / 16 rows x 64
-// columns per tile, 32-deep K tiles in shared memory, four columns per thread. The
-// operands come from L2 through functors, so orientation, conjugation and the cyclic
-// column spread cost nothing extra. As: (NT / 16) x 33, Bs: 32 x 65.
-template <class R, int NT>
-struct GemmTiles {
-  static constexpr int TM = NT / 16, KT = 32;
-  static constexpr size_t bytes = sizeof(Cx<R>) * (TM * (KT + 1) + KT * 65);
+// Operand entries in shared memory and their accumulators. FP32: an entry is split into a
+// multiple of 2^-11 and a rest; products of two leading parts are multiples of 2^-22 and,
+// with rows and columns of norm <= 1 (isometries), their partial sums stay below 4, so FP32
+// adds them exactly, while the three products with a rest are 2^-12 times smaller and so
+// are their rounding errors. The sum comes out rounded once, at the price of four FMAs per
+// real product; larger entries only lose the exactness, not the value. These contractions
+// are a few per cent of a gate, and their plain FP32 rounding was the largest part of a
+// mixed-precision energy's error after the truncation itself.
+struct SplitF {
+  float4 v;   // x leading, x rest, y leading, y rest
+};
+struct SplitAcc {
+  float hx, hy, lx, ly;
+};
+__device__ __forceinline__ float lead11(float x) {
+  constexpr float kMagic = 6144.0f;   // 1.5 2^12: adding it rounds to a multiple of 2^-11
+  return __fadd_rn(__fadd_rn(x, kMagic), -kMagic);
+}
+__device__ __forceinline__ SplitF to_elem(Cx<float> a) {
+  const float hx = lead11(a.x), hy = lead11(a.y);
+  return SplitF{make_float4(hx, __fadd_rn(a.x, -hx), hy, __fadd_rn(a.y, -hy))};
+}
+__device__ __forceinline__ Cx<double> to_elem(Cx<double> a) { return a; }
+__device__ __forceinline__ void zero(SplitAcc& a) { a.hx = a.hy = a.lx = a.ly = 0.f; }
+__device__ __forceinline__ void zero(Cx<double>& a) { a = cx<double>(0, 0); }
+// acc += a b
+__device__ __forceinline__ void mac(SplitAcc& c, const SplitF& a, const SplitF& b) {
+  c.hx = fmaf(-a.v.z, b.v.z, fmaf(a.v.x, b.v.x, c.hx));
+  c.hy = fmaf(a.v.z, b.v.x, fmaf(a.v.x, b.v.z, c.hy));
+  c.lx = fmaf(a.v.y, b.v.x, fmaf(a.v.x, b.v.y, c.lx));
+  c.ly = fmaf(a.v.y, b.v.z, fmaf(a.v.x, b.v.w, c.ly));
+  c.lx = fmaf(-a.v.w, b.v.z, fmaf(-a.v.z, b.v.w, c.lx));
+  c.ly = fmaf(a.v.w, b.v.x, fmaf(a.v.z, b.v.y, c.ly));
+  c.lx = fmaf(-a.v.w, b.v.w, fmaf(a.v.y, b.v.y, c.lx));
+  c.ly = fmaf(a.v.w, b.v.y, fmaf(a.v.y, b.v.w, c.ly));
+}
+__device__ __forceinline__ void mac(Cx<double>& c, const Cx<double>& a, const Cx<double>& b) { cmac(c, a, b); }
+__device__ __forceinline__ Cx<float> value(const SplitAcc& a) {
+  return cx<float>(__fadd_rn(a.hx, a.lx), __fadd_rn(a.hy, a.ly));
+}
+__device__ __forceinline__ Cx<double> value(const Cx<double>& a) { return a; }
+template <class R>
+struct Gemm;
+template <>
+struct Gemm<float> {
+  using E = SplitF;
+  using A = SplitAcc;
+};
+template <>
+struct Gemm<double> {
+  using E = Cx<double>;
+  using A = Cx<double>;
 };
 
-template <class R, int NT, class FA, class FB, class FC>
-__device__ __forceinline__ void tile_gemm(int M, int N, int K, FA fa, FB fb, FC fc, unsigned char* smem) {
-  constexpr int TM = GemmTiles<R, NT>::TM, KT = GemmTiles<R, NT>::KT;
-  Cx<R>(*As)[KT + 1] = reinterpret_cast<Cx<R>(*)[KT + 1]>(smem);
-  Cx<R>(*Bs)[65] = reinterpret_cast<Cx<R>(*)[65]>(smem + sizeof(Cx<R>) * TM * (KT + 1));
+// out(m, n) = sum_k a(m, k) b(k, n) for m < M, n < N by one block. The operands come from
+// L2 through functors, so orientation, conjugation and the cyclic column spread cost
+// nothing extra. RM x JN outputs per thread: tiles of (NT / 16) RM rows by 16 JN columns,
+// KT deep, the next K tile loaded to registers while the present one is used. KF: b's k
+// index runs fastest in memory.
+constexpr int kKT = 16;
+template <int NT>
+__host__ __device__ constexpr size_t gemm_tile_bytes() {   // of the largest tile shape below; entries are 16 bytes
+  constexpr int TY = NT / 16;
+  return 16 * (size_t)((4 * TY) * (kKT + 1) + kKT * (64 + 1));
+}
+template <class R, int NT, int RM, int JN, bool KF, class FA, class FB, class FC>
+__device__ __forceinline__ void tile_gemm_shape(int M, int N, int K, FA fa, FB fb, FC fc, unsigned char* smem) {
+  using E = typename Gemm<R>::E;
+  constexpr int TY = NT / 16, TM = TY * RM, TN = 16 * JN, KT = kKT;
+  constexpr int NA = TM * KT / NT, NB = KT * TN / NT > 0 ? KT * TN / NT : 1;
+  E(*As)[KT + 1] = reinterpret_cast<E(*)[KT + 1]>(smem);
+  E(*Bs)[TN + 1] = reinterpret_cast<E(*)[TN + 1]>(smem + sizeof(E) * TM * (KT + 1));
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   for (int m0 = 0; m0 < M; m0 += TM)
-    for (int n0 = 0; n0 < N; n0 += 64) {
-      Cx<R> acc[4];
+    for (int n0 = 0; n0 < N; n0 += TN) {
+      typename Gemm<R>::A acc[RM][JN];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[j] = cx<R>(0, 0);
-      const int jn = (min(64, N - n0) + 15) >> 4;
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < JN; ++j) zero(acc[i][j]);
+      Cx<R> ra[NA], rb[NB];
+      auto fetch = [&](int k0) {
+#pragma unroll
+        for (int e = 0; e < NA; ++e) {
+          const int x = tid + e * NT, r = x / KT, kk = x % KT;
+          ra[e] = (m0 + r < M && k0 + kk < K) ? fa(m0 + r, k0 + kk) : cx<R>(0, 0);
+        }
+#pragma unroll
+        for (int e = 0; e < NB; ++e) {
+          const int x = tid + e * NT, kk = KF ? x % KT : x / TN, n = KF ? x / KT : x % TN;
+          rb[e] = (x < KT * TN && n0 + n < N && k0 + kk < K) ? fb(k0 + kk, n0 + n) : cx<R>(0, 0);
+        }
+      };
+      fetch(0);
       for (int k0 = 0; k0 < K; k0 += KT) {
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < NA; ++e) {
+          const int x = tid + e * NT;
+          As[x / KT][x % KT] = to_elem(ra[e]);
+        }
+#pragma unroll
+        for (int e = 0; e < NB; ++e) {
+          const int x = tid + e * NT, kk = KF ? x % KT : x / TN, n = KF ? x / KT : x % TN;
+          if (x < KT * TN) Bs[kk][n] = to_elem(rb[e]);
+        }
+        __syncthreads();
+        if (k0 + KT < K) fetch(k0 + KT);
         const int kt = min(KT, K - k0);
-        __syncthreads();
-        for (int e = tid; e < TM * KT; e += NT) {
-          const int r = e / KT, kk = e % KT;
-          As[r][kk] = (m0 + r < M && kk < kt) ? fa(m0 + r, k0 + kk) : cx<R>(0, 0);
-        }
-        for (int e = tid; e < KT * 64; e += NT) {
-          const int kk = fb.k_fast ? e % KT : e >> 6, n = fb.k_fast ? e / KT : e & 63;
-          Bs[kk][n] = (n0 + n < N && kk < kt) ? fb(k0 + kk, n0 + n) : cx<R>(0, 0);
-        }
-        __syncthreads();
-        if (m0 + ty < M) {
-          if (jn == 4) {
-#pragma unroll 8
-            for (int kk = 0; kk < kt; ++kk) {
-              const Cx<R> a = As[ty][kk];
+        if (kt == KT) {
+#pragma unroll 4
+          for (int kk = 0; kk < KT; ++kk) {
+            E a[RM], b[JN];
 #pragma unroll
-              for (int j = 0; j < 4; ++j) cmac(acc[j], a, Bs[kk][tx + 16 * j]);
-            }
-          } else {
-            for (int kk = 0; kk < kt; ++kk) {
-              const Cx<R> a = As[ty][kk];
+            for (int i = 0; i < RM; ++i) a[i] = As[ty + TY * i][kk];
 #pragma unroll
-              for (int j = 0; j < 4; ++j)
-                if (j < jn) cmac(acc[j], a, Bs[kk][tx + 16 * j]);
-            }
+            for (int j = 0; j < JN; ++j) b[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+            for (int i = 0; i < RM; ++i)
+#pragma unroll
+              for (int j = 0; j < JN; ++j) mac(acc[i][j], a[i], b[j]);
+          }
+        } else {
+          for (int kk = 0; kk < kt; ++kk) {
+            E a[RM], b[JN];
+#pragma unroll
+            for (int i = 0; i < RM; ++i) a[i] = As[ty + TY * i][kk];
+#pragma unroll
+            for (int j = 0; j < JN; ++j) b[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+            for (int i = 0; i < RM; ++i)
+#pragma unroll
+              for (int j = 0; j < JN; ++j) mac(acc[i][j], a[i], b[j]);
           }
         }
       }
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (m0 + ty < M && n0 + tx + 16 * j < N) fc(m0 + ty, n0 + tx + 16 * j, acc[j]);
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < JN; ++j) {
+          const int mi = m0 + ty + TY * i, ni = n0 + tx + 16 * j;
+          if (mi < M && ni < N) fc(mi, ni, value(acc[i][j]));
+        }
     }
   __syncthreads();
 }
 
+// Shape by the narrow side: what one thread computes is kept at four outputs where the
+// product has them, and small products spread over all threads.
+template <class R, int NT, bool KF, class FA, class FB, class FC>
+__device__ __forceinline__ void tile_gemm(int M, int N, int K, FA fa, FB fb, FC fc, unsigned char* smem) {
+  constexpr int TY = NT / 16;
+  if (N <= 16) {
+    if (M <= TY)
+      tile_gemm_shape<R, NT, 1, 1, KF>(M, N, K, fa, fb, fc, smem);
+    else
+      tile_gemm_shape<R, NT, 4, 1, KF>(M, N, K, fa, fb, fc, smem);
+  } else if (N <= 32 && M > TY) {
+    tile_gemm_shape<R, NT, 2, 2, KF>(M, N, K, fa, fb, fc, smem);
+  } else {
+    tile_gemm_shape<R, NT, 1, 4, KF>(M, N, K, fa, fb, fc, smem);
+  }
+}
+
 // -------------------------------------------------------------------- bidiagonalisation
-// T = Q B P^H (LAPACK reflector conventions, svd.cuh) with a single cluster barrier per
+// T = Q B P^H (LAPACK reflector conventions) with a single cluster barrier per
 // step: the updates by right reflector k-1 and left reflector k go over the trailing
 // columns together, the next row comes out of that pass, and the product z with the next
 // right reflector is formed from the unscaled row (its norm, hence its scale, is known one
@@ -137,17 +242,82 @@ __device__ __forceinline__ void tile_gemm(int M, int N, int K, FA fa, FB fb, FC 
 // z partials, the next column before its right update, the partial norms of the row.
 // The trailing matrix is read twice and written once per step, where two separate half
 // steps read and write it twice.
+// LAPACK-style reflector H = I - tau v v^H, v_0 = 1, for x = (alpha, tail) with ||tail||^2 =
+// xn2: H^H x = beta e_1 with beta real, v = scale tail. A vector whose squared norm is
+// within 16x of the smallest normal number counts as zero: the squares that make up that
+// norm have lost their bits to underflow (entries below ~5e-19 in FP32, ~6e-154 in FP64),
+// so the norm could come out as 0 while alpha is not, and 1 / (alpha - beta) would be a
+// division by zero. The identity is taken there and the entries (absolutely that small)
+// are dropped from the bidiagonal. The root and the reciprocals are the hardware estimates
+// with Newton-Raphson steps, whose dependent chain is a quarter of a library square root's
+// and four divisions': it runs twice per step of a serial recurrence.
+// FP64 takes one third-order step from the 22-bit estimates (e the residual: 1 + e/2 +
+// 3 e^2 / 8 for the inverse root, 1 + e + e^2 for the inverse), which is shorter in
+// dependent operations than two second-order steps; FP64 latency is what it costs.
+__device__ __forceinline__ void root_and_inverse(float x, float* root, float* inv) {
+  const float y = rsqrtf(x);
+  float r = x * y;
+  r = fmaf(0.5f * y, fmaf(-r, r, x), r);
+  *root = r;
+  *inv = fmaf(y, fmaf(-r, y, 1.0f), y);
+}
+__device__ __forceinline__ void root_and_inverse(double x, double* root, double* inv) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x * y, y, 1.0);
+  y = fma(y * e, fma(0.375, e, 0.5), y);
+  const double r = x * y;
+  *root = fma(0.5 * y, fma(-r, r, x), r);
+  *inv = y;
+}
+__device__ __forceinline__ float inverse(float d) {
+  const float r = __fdividef(1.0f, d);
+  return fmaf(r, fmaf(-d, r, 1.0f), r);
+}
+__device__ __forceinline__ double inverse(double d) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+  const double e = fma(-d, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+template <class R>
+__device__ __forceinline__ void reflector(Cx<R> alpha, R xn2, Cx<R>* tau, R* beta, Cx<R>* scale) {
+  constexpr R kTiny2 = R(16) * (sizeof(R) == 4 ? R(FLT_MIN) : R(DBL_MIN));
+  const R n2 = alpha.x * alpha.x + alpha.y * alpha.y + xn2;
+  if ((xn2 == R(0) && alpha.y == R(0)) || !(n2 > kTiny2)) {
+    *tau = cx<R>(0, 0);
+    *beta = alpha.x;
+    *scale = cx<R>(0, 0);
+    return;
+  }
+  R nrm, inv;
+  root_and_inverse(n2, &nrm, &inv);
+  const R b = alpha.x >= R(0) ? -nrm : nrm, rb = alpha.x >= R(0) ? -inv : inv;
+  *beta = b;
+  *tau = cx<R>((b - alpha.x) * rb, -alpha.y * rb);
+  const Cx<R> den = cx<R>(alpha.x - b, alpha.y);
+  const R rd = inverse(norm2(den));
+  *scale = cx<R>(den.x * rd, -den.y * rd);
+}
+
+// Per own column: left factor, pending and new row entry (the pending right update uses
+// the row entry of the step before).
+template <class R>
+struct alignas(16) ColState {
+  Cx<R> f, ro, rn, pad;
+};
+
 template <class R>
 struct Bidiag {
   Cx<R>* T;            // own columns, leading dimension ld (>= r)
   int ld;
   int zrows;
-  Cx<R>* zp;           // [2][C][GMAX][zrows] z partials
+  Cx<R>* zp;           // [2][C][gmax][zrows] z partials
   Cx<R>* colp;         // [2][zrows] next column before its right update
-  Cx<R>* sc;           // [2] row entry of the next column, [2]: X of the leading row, [3..6]: scalars
+  Cx<R>* sc;           // [0..1] row entry of the next column, [2]: X of the leading row, [3..7]: scalars
   R* nrmp;             // [2][C] partial |row|^2
   Cx<R>*xs, *us;       // [zrows] X conj(right scale), the column (unscaled left reflector)
-  Cx<R>*rj, *fj;       // [2][own] row entries, [own] factors of the left update
+  ColState<R>* cs;     // [own]
   R* part;             // [24] per-warp partial sums
   R *dd, *ee;
   Cx<R>*tau, *scl;     // factor and scale per reflector of the side the back-transformation needs
@@ -155,28 +325,29 @@ struct Bidiag {
   int ystride;
 };
 
-// Smallest power of two >= rows, at least a warp.
-__device__ __forceinline__ int pow2_rows(int rows) {
-  return rows <= 32 ? 32 : 1 << (32 - __clz(rows - 1));
-}
+// log2 of the smallest power of two >= rows, at least a warp's.
+__device__ __forceinline__ int row_shift(int rows) { return rows <= 32 ? 5 : 32 - __clz(rows - 1); }
 
-template <class R, int NT, int C, int GMAX>
-__device__ __noinline__ void bidiagonalize_cluster(const Bidiag<R>& b, int r, int p, bool right_side, unsigned rank) {
+template <class R, int NT, int C>
+__device__ __forceinline__ void bidiagonalize_cluster(const Bidiag<R> b, const int gmax, const int r, const int p,
+                                                      const bool right_side, const unsigned rank) {
   const int tid = threadIdx.x;
   // On this chip a SM does two FP64 operations a clock: scalar work in FP64 runs in one
   // warp and is passed on through shared memory. In FP32 every warp does it for itself,
   // which saves the barrier.
   constexpr bool kOneWarp = sizeof(R) == 8;
-  constexpr int GL = 16, NG = NT / GL;   // lanes per column, columns at a time
+  constexpr int GL = 8, NG = NT / GL;   // lanes per column, columns at a time
+  constexpr int kLogNT = NT == 512 ? 9 : NT == 256 ? 8 : 7;
+  static_assert(NT == 1 << kLogNT, "threads: a power of two");
   const int own = 2 * (((p >> 1) + C - 1 - (int)rank) / C);   // p is even: pairs are never split
   Cx<R> tauR = cx<R>(0, 0), scR = cx<R>(0, 0);
-  for (int i = tid; i < 2 * own; i += NT) b.rj[i] = cx<R>(0, 0);
+  for (int i = tid; i < own; i += NT) b.cs[i].rn = cx<R>(0, 0);
   for (int k = 0; k < p; ++k) {
     const int par = k & 1, rows = r - k;
     const bool have_old = k > 0;
     // ---- the next column and the right-update vector X, one thread per row
-    const int rp = pow2_rows(rows);
-    if (tid < rp) {
+    const int rsh = row_shift(rows);
+    if (tid < (1 << rsh)) {
       R pn = 0;
       Cx<R> pd = cx<R>(0, 0);
       if (tid < rows) {
@@ -184,16 +355,20 @@ __device__ __noinline__ void bidiagonalize_cluster(const Bidiag<R>& b, int r, in
         if (!have_old) {
           col = peer<C>(b.T, 0)[tid];
         } else {
-          const int groups = min(GMAX, NT / rp);
-          Cx<R> z = cx<R>(0, 0);
-          const Cx<R>* zq = b.zp + (size_t)par * C * GMAX * b.zrows + tid;
-#pragma unroll
-          for (int c = 0; c < C; ++c) {
-#pragma unroll
-            for (int g = 0; g < GMAX; ++g)
-              if (g < groups) z = z + zq[(c * GMAX + g) * b.zrows];
-          }
+          const Cx<R>* zq = b.zp + par * C * gmax * b.zrows + tid;
           const Cx<R> a = b.colp[par * b.zrows + tid];
+          Cx<R> zc[C];
+#pragma unroll
+          for (int c = 0; c < C; ++c) zc[c] = zq[c * gmax * b.zrows];
+          if (min(gmax, NT >> rsh) == 2) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) zc[c] = zc[c] + zq[(c * gmax + 1) * b.zrows];
+          }
+#pragma unroll
+          for (int h = C / 2; h > 0; h >>= 1)
+#pragma unroll
+            for (int c = 0; c < h; ++c) zc[c] = zc[c] + zc[c + h];
+          const Cx<R> z = zc[0];
           X = tauR * (a + scR * z);
           col = a - X;
           b.xs[tid] = X * conj(scR);
@@ -222,14 +397,16 @@ __device__ __noinline__ void bidiagonalize_cluster(const Bidiag<R>& b, int r, in
     // ---- left reflector u = (1, col scL) of that column; g = u^H (X conj(scR))
     Cx<R> scL, ct, g;
     if (!kOneWarp || tid < 32) {
-      R xn2 = 0, betaL;
-      Cx<R> dot = cx<R>(0, 0), tauL;
-      for (int w = 0; w < rp / 32; ++w) {
-        xn2 += b.part[w];
-        dot.x += b.part[8 + w];
-        dot.y += b.part[16 + w];
-      }
-      make_reflector(b.us[0], xn2, &tauL, &betaL, &scL);
+      R xn2 = b.part[0], betaL;
+      Cx<R> dot = cx<R>(b.part[8], b.part[16]), tauL;
+#pragma unroll
+      for (int w = 1; w < 8; ++w)
+        if (w < (1 << rsh) / 32) {
+          xn2 += b.part[w];
+          dot.x += b.part[8 + w];
+          dot.y += b.part[16 + w];
+        }
+      reflector(b.us[0], xn2, &tauL, &betaL, &scL);
       g = have_old ? (b.sc[2] + conj(scL) * dot) * conj(scR) : cx<R>(0, 0);
       ct = conj(tauL);
       if (tid == 0) {
@@ -259,21 +436,19 @@ __device__ __noinline__ void bidiagonalize_cluster(const Bidiag<R>& b, int r, in
     const int l0 = 2 * ((((k + 1) >> 1) + C - 1 - (int)rank) / C);   // own pairs from column k (or k + 1) on
     const int first = 2 * (C * (l0 >> 1) + (int)rank) > k ? l0 : l0 + 1;   // own columns after k
     const int lane = tid & (GL - 1), grp = tid / GL;
-    const Cx<R>* rold = b.rj + (par ^ 1) * own;
-    Cx<R>* rnew = b.rj + par * own;
     auto finish = [&](int lc, Cx<R> s) {
-      const Cx<R> a0 = b.T[(size_t)lc * b.ld + k];
+      const Cx<R> a0 = b.T[lc * b.ld + k], ro = b.cs[lc].rn;
       s = a0 + conj(scL) * s;
       Cx<R> rn = a0;
       if (have_old) {
-        const Cx<R> ro = rold[lc];
         cmsub(s, g, ro);
         cmsub(rn, b.xs[0], ro);
       }
       const Cx<R> f = ct * s;
       rn = rn - f;
-      b.fj[lc] = f;
-      rnew[lc] = rn;
+      b.cs[lc].f = f;
+      b.cs[lc].ro = ro;
+      b.cs[lc].rn = rn;
       if (right_side) b.Y[(size_t)k * b.ystride + 2 * (C * (lc >> 1) + (int)rank) + (lc & 1)] = conj(rn);
     };
     for (int base = first; base < own; base += NG) {
@@ -281,9 +456,26 @@ __device__ __noinline__ void bidiagonalize_cluster(const Bidiag<R>& b, int r, in
       const bool act = lc < own;
       Cx<R> s = cx<R>(0, 0);
       if (act) {
-        const Cx<R>* a = b.T + (size_t)lc * b.ld + k;
-#pragma unroll 4
-        for (int i = lane == 0 ? GL : lane; i < rows; i += GL) cmac_conj(s, b.us[i], a[i]);
+        // four partial sums: the dependent chain, not the arithmetic, is what this costs
+        const Cx<R>* a = b.T + lc * b.ld + k;
+        Cx<R> sp[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sp[e] = cx<R>(0, 0);
+        int i = lane == 0 ? GL : lane;
+        for (; i + 3 * GL < rows; i += 4 * GL) {
+          Cx<R> av[4], uv[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            av[e] = a[i + e * GL];
+            uv[e] = b.us[i + e * GL];
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e) cmac_conj(sp[e], uv[e], av[e]);
+        }
+#pragma unroll
+        for (int e = 0; e < 3; ++e)
+          if (i + e * GL < rows) cmac_conj(sp[e], b.us[i + e * GL], a[i + e * GL]);
+        s = (sp[0] + sp[1]) + (sp[2] + sp[3]);
       }
 #pragma unroll
       for (int o = 1; o < GL; o <<= 1) {
@@ -292,59 +484,73 @@ __device__ __noinline__ void bidiagonalize_cluster(const Bidiag<R>& b, int r, in
       }
       if (act && lane == 0) {
         if constexpr (kOneWarp)
-          b.fj[lc] = s;
+          b.cs[lc].f = s;
         else
           finish(lc, s);
       }
     }
     __syncthreads();
     if constexpr (kOneWarp) {
-      for (int lc = first + tid; lc < own; lc += NT) finish(lc, b.fj[lc]);
+      for (int lc = first + tid; lc < own; lc += NT) finish(lc, b.cs[lc].f);
       __syncthreads();
     }
     // ---- pass 2: both updates, one thread per row and column group; z = sum a_j conj(r_j)
     // over the columns after k + 1; column k + 1 goes out whole
-    const int nrow = rows - 1, rp2 = pow2_rows(nrow), groups = min(GMAX, NT / rp2);
-    const int row = tid & (rp2 - 1), cgp = tid / rp2, npar = par ^ 1;
+    const int nrow = rows - 1, rsh2 = row_shift(nrow), groups = min(gmax, NT >> rsh2);
+    const int row = tid & ((1 << rsh2) - 1), cgp = tid >> rsh2, npar = par ^ 1;
     const int lnext = ((k + 1) >> 1) % C == (int)rank ? 2 * (((k + 1) >> 1) / C) + ((k + 1) & 1) : -1;
     if (cgp < groups && row < nrow) {
-      Cx<R> z = cx<R>(0, 0);
+      Cx<R> z = cx<R>(0, 0), z2 = cx<R>(0, 0);
       const Cx<R> u = b.us[row + 1] * scL;
       const Cx<R> x = have_old ? b.xs[row + 1] : cx<R>(0, 0);
       int lc = first + cgp;
-      Cx<R>* a = b.T + (size_t)lc * b.ld + k + 1 + row;
+      Cx<R>* a = b.T + lc * b.ld + k + 1 + row;
       if (lc == lnext) {   // first own column: only group 0 can meet it
         Cx<R> v = *a;
-        cmsub(v, x, rold[lc]);
-        cmsub(v, b.fj[lc], u);
+        cmsub(v, x, b.cs[lc].ro);
+        cmsub(v, b.cs[lc].f, u);
 #pragma unroll
         for (int c = 0; c < C; ++c) peer<C>(b.colp, c)[npar * b.zrows + row] = v;
         lc += groups;
-        a += (size_t)groups * b.ld;
+        a += groups * b.ld;
       }
-#pragma unroll 2
-      for (; lc < own; lc += groups, a += (size_t)groups * b.ld) {
-        Cx<R> v = *a;
-        cmsub(v, x, rold[lc]);
-        cmsub(v, b.fj[lc], u);
-        *a = v;
-        cmac_bconj(z, v, rnew[lc]);
+      const int step = groups * b.ld;
+      for (; lc + groups < own; lc += 2 * groups, a += 2 * step) {
+        const ColState<R> q = b.cs[lc], q2 = b.cs[lc + groups];
+        Cx<R> v = a[0], v2 = a[step];
+        cmsub(v, x, q.ro);
+        cmsub(v2, x, q2.ro);
+        cmsub(v, q.f, u);
+        cmsub(v2, q2.f, u);
+        a[0] = v;
+        a[step] = v2;
+        cmac_bconj(z, v, q.rn);
+        cmac_bconj(z2, v2, q2.rn);
       }
+      if (lc < own) {
+        const ColState<R> q = b.cs[lc];
+        Cx<R> v = a[0];
+        cmsub(v, x, q.ro);
+        cmsub(v, q.f, u);
+        a[0] = v;
+        cmac_bconj(z, v, q.rn);
+      }
+      z = z + z2;
 #pragma unroll
       for (int c = 0; c < C; ++c)
-        peer<C>(b.zp, c)[(size_t)((npar * C + (int)rank) * GMAX + cgp) * b.zrows + row] = z;
+        peer<C>(b.zp, c)[((npar * C + (int)rank) * gmax + cgp) * b.zrows + row] = z;
     }
     // partial norm of the new row (columns after k + 1) and its leading entry
     if (tid >= NT - 32) {
       const int l = tid & 31;
       R nn = 0;
       for (int lc = first + l; lc < own; lc += 32)
-        if (lc != lnext) nn += norm2(rnew[lc]);
+        if (lc != lnext) nn += norm2(b.cs[lc].rn);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, o);
       if (l < C) {
         peer<C>(b.nrmp, l)[npar * C + (int)rank] = nn;
-        if (lnext >= 0) peer<C>(b.sc, l)[npar] = rnew[lnext];
+        if (lnext >= 0) peer<C>(b.sc, l)[npar] = b.cs[lnext].rn;
       }
     }
     csync<C>();
@@ -353,7 +559,7 @@ __device__ __noinline__ void bidiagonalize_cluster(const Bidiag<R>& b, int r, in
       R rn2 = 0, betaR;
 #pragma unroll
       for (int c = 0; c < C; ++c) rn2 += b.nrmp[npar * C + c];
-      make_reflector(conj(b.sc[npar]), rn2, &tauR, &betaR, &scR);
+      reflector(conj(b.sc[npar]), rn2, &tauR, &betaR, &scR);
       if (tid == 0) {
         b.ee[k] = betaR;
         if (right_side) {
@@ -383,129 +589,202 @@ __device__ __noinline__ void bidiagonalize_cluster(const Bidiag<R>& b, int r, in
 // range: entries are scaled to |b| <= 1 and split off below 4 eps, so two steps shrink
 // the larger of a pair by at most (4 eps)^2. An exact zero counts once either way, because
 // its neighbours have opposite signs. Returns the number of eigenvalues >= x.
+__device__ __forceinline__ float rescale_factor(float a, float b) {
+  const unsigned m = max((__float_as_uint(a) >> 23) & 255u, (__float_as_uint(b) >> 23) & 255u);
+  return __uint_as_float((254u - min(m, 253u)) << 23);
+}
+__device__ __forceinline__ double rescale_factor(double a, double b) {
+  const unsigned m = max(((unsigned)__double2hiint(a) >> 20) & 2047u, ((unsigned)__double2hiint(b) >> 20) & 2047u);
+  return __hiloint2double((int)((2046u - min(m, 2045u)) << 20), 0);
+}
+__device__ __forceinline__ unsigned sign_bits(float a, float b) { return (__float_as_uint(a) ^ __float_as_uint(b)) >> 31; }
+__device__ __forceinline__ unsigned sign_bits(double a, double b) {
+  return (unsigned)(__double2hiint(a) ^ __double2hiint(b)) >> 31;
+}
 template <class R>
-__device__ __forceinline__ int sturm_ge(const R* b2, int s, int e, R x);
-
+struct SturmGroup;   // steps between rescalings
 template <>
-__device__ __forceinline__ int sturm_ge<float>(const float* b2, int s, int e, float x) {
-  float prev = 1.f, cur = -x;
-  unsigned neg = __float_as_uint(cur) >> 31;
-  int i = s + 1;
-#pragma unroll 2
-  for (; i + 3 < e; i += 4) {
+struct SturmGroup<float> {
+  static constexpr int v = 4;
+};
+template <>
+struct SturmGroup<double> {
+  static constexpr int v = 8;
+};
+// V shifts at once, for as many independent chains. last (optional): p_e with its binary
+// exponent, for interpolation.
+template <class R, int V>
+__device__ __forceinline__ void sturm_ge(const R* b2, int s, int e, const R* x, int* ge, R* last = nullptr,
+                                         int* last_exp = nullptr) {
+  constexpr int GRP = SturmGroup<R>::v;
+  R prev[V], cur[V];
+  unsigned neg[V];
+  int ex[V];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const float nxt = fmaf(-x, cur, -(b2[i + u - 1] * prev));
-      neg += (__float_as_uint(nxt) ^ __float_as_uint(cur)) >> 31;
-      prev = cur;
-      cur = nxt;
+  for (int v = 0; v < V; ++v) {
+    prev[v] = R(1);
+    cur[v] = -x[v];
+    neg[v] = sign_bits(cur[v], prev[v]);
+    ex[v] = 0;
+  }
+  int i = s + 1;
+  for (; i + GRP <= e; i += GRP) {
+    R bb[GRP];
+#pragma unroll
+    for (int u = 0; u < GRP; ++u) bb[u] = b2[i + u - 1];
+#pragma unroll
+    for (int u = 0; u < GRP; ++u)
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const R nxt = fma(-x[v], cur[v], -(bb[u] * prev[v]));
+        neg[v] += sign_bits(nxt, cur[v]);
+        prev[v] = cur[v];
+        cur[v] = nxt;
+      }
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const R sc = rescale_factor(prev[v], cur[v]);
+      prev[v] *= sc;
+      cur[v] *= sc;
+      if (last) ex[v] += 1023 - (int)(((unsigned)__double2hiint((double)sc) >> 20) & 2047u);
     }
-    const unsigned m = max((__float_as_uint(prev) >> 23) & 255u, (__float_as_uint(cur) >> 23) & 255u);
-    const float sc = __uint_as_float((254u - min(m, 253u)) << 23);
-    prev *= sc;
-    cur *= sc;
   }
   for (; i < e; ++i) {
-    const float nxt = fmaf(-x, cur, -(b2[i - 1] * prev));
-    neg += (__float_as_uint(nxt) ^ __float_as_uint(cur)) >> 31;
-    prev = cur;
-    cur = nxt;
-  }
-  return (e - s) - (int)neg;
-}
-
-template <>
-__device__ __forceinline__ int sturm_ge<double>(const double* b2, int s, int e, double x) {
-  double prev = 1.0, cur = -x;
-  unsigned neg = (unsigned)__double2hiint(cur) >> 31;
-  int i = s + 1;
-  for (; i + 7 < e; i += 8) {
+    const R bi = b2[i - 1];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const double nxt = fma(-x, cur, -(b2[i + u - 1] * prev));
-      neg += (unsigned)(__double2hiint(nxt) ^ __double2hiint(cur)) >> 31;
-      prev = cur;
-      cur = nxt;
+    for (int v = 0; v < V; ++v) {
+      const R nxt = fma(-x[v], cur[v], -(bi * prev[v]));
+      neg[v] += sign_bits(nxt, cur[v]);
+      prev[v] = cur[v];
+      cur[v] = nxt;
     }
-    const unsigned m = max(((unsigned)__double2hiint(prev) >> 20) & 2047u, ((unsigned)__double2hiint(cur) >> 20) & 2047u);
-    const double sc = __hiloint2double((int)((2046u - min(m, 2045u)) << 20), 0);
-    prev *= sc;
-    cur *= sc;
   }
-  for (; i < e; ++i) {
-    const double nxt = fma(-x, cur, -(b2[i - 1] * prev));
-    neg += (unsigned)(__double2hiint(nxt) ^ __double2hiint(cur)) >> 31;
-    prev = cur;
-    cur = nxt;
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    ge[v] = (e - s) - (int)neg[v];
+    if (last) {
+      last[v] = cur[v];
+      last_exp[v] = ex[v];
+    }
   }
-  return (e - s) - (int)neg;
+}
+template <class R>
+__device__ __forceinline__ int sturm_ge1(const R* b2, int s, int e, R x) {
+  int ge;
+  sturm_ge<R, 1>(b2, s, e, &x, &ge);
+  return ge;
 }
 
-// Singular value t (0-based, descending) in FP32 by one warp: 32 shifts per pass, each
-// pass narrows the bracket 33-fold. First pass on a log grid over eight decades, then
-// linear to the working precision. lo/hi bracket the value (scaled to smax ~ 1).
-__device__ __forceinline__ int warp_bisect(const float* b2, int N, int t, float top, float* lo_out, float* hi_out) {
+// Singular values t[0..V) (0-based, descending) of the TGK block [s, e) in FP32 by one
+// warp: 32 shifts per value and pass, each pass narrows a bracket 33-fold. First pass on a
+// log grid over eight decades, then linear to the working precision. lo/hi bracket the
+// values.
+template <int V>
+__device__ __forceinline__ int warp_bisect(const float* b2, int s, int e, const int* t, float top, float* lo,
+                                           float* hi) {
   const int lane = threadIdx.x & 31;
-  float lo = 0.f, hi = top;
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    lo[v] = 0.f;
+    hi[v] = top;
+  }
   int passes = 0;
   for (int it = 0; it < 9; ++it) {
-    float x;
-    if (it == 0) {
-      x = top * exp10f(-8.0f * (float)(32 - lane) / 32.0f);
-    } else {
-      x = fmaf(hi - lo, (float)(lane + 1) / 33.0f, lo);
+    float x[V];
+    int ge[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+      x[v] = it == 0 ? top * exp10f(-8.0f * (float)(32 - lane) / 32.0f)
+                     : fmaf(hi[v] - lo[v], (float)(lane + 1) / 33.0f, lo[v]);
+    sturm_ge<float, V>(b2, s, e, x, ge);
+    bool open = false;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      // counts fall with x: the number of shifts below the value locates it
+      const int m = __popc(__ballot_sync(0xffffffffu, ge[v] >= t[v] + 1));
+      const float nlo = __shfl_sync(0xffffffffu, x[v], max(m - 1, 0));
+      const float nhi = __shfl_sync(0xffffffffu, x[v], min(m, 31));
+      if (m > 0) lo[v] = nlo;
+      if (m < 32) hi[v] = nhi;
+      open = open || hi[v] - lo[v] > 1.2e-7f * hi[v];   // not yet two neighbours of the working precision
     }
-    const unsigned ge = __ballot_sync(0xffffffffu, sturm_ge<float>(b2, 0, N, x) >= t + 1);
-    // counts fall with x: the number of shifts below the value locates it
-    const int m = __popc(ge);
-    const float nlo = __shfl_sync(0xffffffffu, x, max(m - 1, 0)), nhi = __shfl_sync(0xffffffffu, x, min(m, 31));
-    if (m > 0) lo = nlo;
-    if (m < 32) hi = nhi;
     ++passes;
-    if (hi - lo <= 1.2e-7f * hi) break;   // the bracket is two neighbours of the working precision
+    if (!open) break;
   }
-  *lo_out = lo;
-  *hi_out = hi;
   return passes;
 }
 
-// The same in FP64 from the FP32 bracket: LT lanes per value (LT = 4: on this chip FP64
-// runs at two lanes a clock per SM, and few shifts per pass cost the least per bit), the
-// bracket first checked with FP64 counts and opened up if it does not hold. Stops at the
+// Value t of block [s, e) in FP64 from the FP32 bracket, LT = 4 lanes per value (a warp's FP64 operation
+// takes 16 clocks whatever the lanes do, so few shifts per pass cost the least). The
+// bracket is checked with FP64 counts first and opened up if it does not hold. Then every
+// other way of placing the shifts: two on either side of the secant estimate of the root
+// of p_N inside the bracket (w 2^-16 and w 2^-6 away; a simple root gains 5 to 15 bits a
+// pass), or, when that gained less than a plain section would, evenly. The bracket itself
+// always moves by counts, so a wrong estimate costs a pass and nothing else. Stops at the
 // working precision relative to the value, or at 2^-60 of the largest one.
-template <int LT>
-__device__ __forceinline__ int lanes_bisect(const double* b2, int N, int t, bool act, double top, float lo_f,
+__device__ __forceinline__ int lanes_bisect(const double* b2, int s, int e, int t, bool act, double top, float lo_f,
                                             float hi_f, double* lo_out, double* hi_out) {
-  const int lane = threadIdx.x & (LT - 1);
+  constexpr int LT = 4;
+  const int wl = threadIdx.x & 31, lane = wl & (LT - 1), base = wl & ~(LT - 1);
   double lo = (double)lo_f * (1.0 - 4e-6), hi = fmin(top, (double)hi_f * (1.0 + 4e-6) + 1e-30);
-  bool done = !act;
+  double flo = 0.0, fhi = 0.0;   // p_N at the ends, in a common scale; 0: not known
+  bool done = !act, even = false;
   int passes = 0;
   for (int it = 0; it < 64; ++it) {
-    // pass 0 checks the bracket: lane 0 its lower end, the last lane its upper end
+    const double w = hi - lo;
     double x;
-    if (it == 0)
-      x = lane == 0 ? lo : hi;
-    else
-      x = fma(hi - lo, (double)(lane + 1) / (double)(LT + 1), lo);
-    const int ge = sturm_ge<double>(b2, 0, N, x) >= t + 1;
-    const unsigned mask = __ballot_sync(0xffffffffu, ge) >> ((threadIdx.x & 31) & ~(LT - 1)) & ((1u << LT) - 1u);
-    ++passes;
+    // secant estimate; both ends have to be known and of opposite sign
+    const bool secant = it > 0 && flo * fhi < 0.0 && !even;
     if (it == 0) {
-      if (!(mask & 1u)) {
-        hi = lo;    // value below the bracket
-        lo = 0.0;
-      } else if (mask >> (LT - 1)) {
-        lo = hi;    // value at or above it
-        hi = top;
-      }
+      x = lane == 0 ? lo : hi;
+    } else if (secant) {
+      const double off = lane == 0 ? -0x1p-6 : lane == 1 ? -0x1p-16 : lane == 2 ? 0x1p-16 : 0x1p-6;
+      x = fma(w, fmin(fmax(fma(flo, inverse(flo - fhi), off), 0x1p-30), 1.0 - 0x1p-30), lo);
+    } else {
+      x = fma(w, (double)(lane + 1) * 0.2, lo);
+    }
+    int ge1, ex;
+    double f;
+    sturm_ge<double, 1>(b2, s, e, &x, &ge1, &f, &ex);
+    const unsigned mask = (__ballot_sync(0xffffffffu, ge1 >= t + 1) >> base) & 15u;
+    ++passes;
+    int il, ih;   // lanes that become the new ends (-1: the old one stays)
+    bool reopen = false;
+    if (it == 0) {
+      il = 0;
+      ih = LT - 1;
+      if (!(mask & 1u) || (mask >> (LT - 1))) reopen = true;
     } else {
       const int m = __popc(mask);
-      const int base = (threadIdx.x & 31) & ~(LT - 1);
-      const double nlo = __shfl_sync(0xffffffffu, x, base + max(m - 1, 0));
-      const double nhi = __shfl_sync(0xffffffffu, x, base + min(m, LT - 1));
-      if (!done) {
-        if (m > 0) lo = nlo;
-        if (m < LT) hi = nhi;
+      il = m > 0 ? m - 1 : -1;
+      ih = m < LT ? m : -1;
+    }
+    const double xl = __shfl_sync(0xffffffffu, x, base + max(il, 0)), xh = __shfl_sync(0xffffffffu, x, base + max(ih, 0));
+    const double fl = __shfl_sync(0xffffffffu, f, base + max(il, 0)), fh = __shfl_sync(0xffffffffu, f, base + max(ih, 0));
+    const int el = __shfl_sync(0xffffffffu, ex, base + max(il, 0)), eh = __shfl_sync(0xffffffffu, ex, base + max(ih, 0));
+    if (!done) {
+      if (reopen) {
+        if (!(mask & 1u)) {
+          hi = lo;    // value below the bracket
+          lo = 0.0;
+        } else {
+          lo = hi;    // value at or above it
+          hi = top;
+        }
+        flo = fhi = 0.0;
+      } else {
+        // an end that stays keeps no usable scale next to a new one: the estimate then
+        // waits for the next pass
+        if (il >= 0) lo = xl;
+        if (ih >= 0) hi = xh;
+        if (il >= 0 && ih >= 0) {
+          const int d = max(-900, min(900, el - eh));
+          flo = ldexp(fl, d > 0 ? 0 : d);
+          fhi = ldexp(fh, d > 0 ? -d : 0);
+        } else {
+          flo = fhi = 0.0;
+        }
+        even = secant && !(hi - lo < 0.2 * w);
       }
     }
     done = done || hi - lo <= fmax(2.3e-16 * hi, 8.7e-19);
@@ -514,43 +793,6 @@ __device__ __forceinline__ int lanes_bisect(const double* b2, int N, int t, bool
   *lo_out = lo;
   *hi_out = hi;
   return passes;
-}
-
-// ------------------------------------------------------------------ twisted vectors
-// 1 / d for the pivots: FP32 the fast reciprocal; FP64 the hardware estimate and two
-// Newton-Raphson steps r <- r + r (1 - d r), which square the relative error each time.
-__device__ __forceinline__ float pivot_rcp(float d) { return __fdividef(1.f, d); }
-__device__ __forceinline__ double pivot_rcp(double d) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-  r = fma(r, fma(-d, r, 1.0), r);
-  r = fma(r, fma(-d, r, 1.0), r);
-  return r;
-}
-
-// Block [s, e) of the split TGK that owns target t (see svd.cuh owning_block), by counts
-// without divisions. lam, delta in the units of b2.
-template <class R>
-__device__ void owning_range(const R* b2, int N, const R* sig, int t, R delta, int* s_out, int* e_out) {
-  const R lam = sig[t];
-  int m = 0;
-  for (int u = 0; u < t; ++u) m += rabs(sig[u] - lam) <= delta;
-  int occ = 0, bs = 0;
-  *s_out = 0;
-  *e_out = N;
-  for (int i = 0; i < N; ++i) {
-    const bool end = (i == N - 1) || (b2[i] == R(0));
-    if (!end) continue;
-    const int e = i + 1;
-    const int inwin = sturm_ge<R>(b2, bs, e, lam - delta) - sturm_ge<R>(b2, bs, e, lam + delta);
-    if (inwin > 0 && occ + inwin > m) {
-      *s_out = bs;
-      *e_out = e;
-      return;
-    }
-    occ += inwin;
-    bs = e;
-  }
 }
 
 }  // namespace gate
