@@ -1,6 +1,7 @@
 // C ABI of the MPS-VQE engine: handles, device memory layout and the host-side
 // orchestration of the kernels in kernels.cu. See include/mpsvqe.h for the contract.
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -94,16 +95,10 @@ struct ham_s {
   // device copies (current device at upload)
   bool uploaded = false;
   double* d_coeff = nullptr;
-  std::vector<int32_t*> d_parent, d_cnode, d_cterm;
+  std::vector<int32_t*> d_parent, d_cnode, d_cterm, d_cbegin;
   std::vector<uint8_t*> d_edge, d_cletter;
-  ~ham_s() {
-    dfree(d_coeff);
-    for (auto p : d_parent) dfree(p);
-    for (auto p : d_cnode) dfree(p);
-    for (auto p : d_cterm) dfree(p);
-    for (auto p : d_edge) dfree(p);
-    for (auto p : d_cletter) dfree(p);
-  }
+  void* d_all = nullptr;   // one allocation holds d_coeff and the arrays of all levels
+  ~ham_s() { dfree(d_all); }
 };
 
 struct circ_s {
@@ -170,6 +165,8 @@ struct mps_s {
     dfree(tc.err, st);
     dfree(w.vals, st);
     dfree(w.out, st);
+    dfree(w.part, st);
+    dfree(w.done, st);
     dfree(d_theta, st);
     dfree(d_occ, st);
     dfree(d_start_gate, st);
@@ -199,34 +196,48 @@ static int make_ham(int n, std::vector<Term> terms, ham_t* out) {
   return MPS_OK;
 }
 
+// All device arrays of a Hamiltonian in one allocation and one copy: a small one (a list
+// of strings measured once) costs its transfer, not a call per array and level.
 static int upload_ham(ham_s* h) {
   if (h->uploaded) return MPS_OK;
   const int n = h->n;
-  std::vector<double> co(h->terms.size());
-  for (size_t t = 0; t < co.size(); ++t) co[t] = h->terms[t].coeff;
-  TRY(dalloc(&h->d_coeff, co.size()));
-  CU(cudaMemcpy(h->d_coeff, co.data(), co.size() * 8, cudaMemcpyHostToDevice));
-  h->d_parent.assign(n, nullptr);
-  h->d_edge.assign(n, nullptr);
-  h->d_cnode.assign(n, nullptr);
-  h->d_cletter.assign(n, nullptr);
-  h->d_cterm.assign(n, nullptr);
   const Trie& t = h->trie;
+  std::vector<char> host;
+  auto put = [&](const void* p, size_t bytes) {
+    const size_t at = (host.size() + 15) & ~(size_t)15;
+    host.resize(at + bytes);
+    if (bytes) std::memcpy(host.data() + at, p, bytes);
+    return at;
+  };
+  std::vector<double> co(h->terms.size());
+  for (size_t i = 0; i < co.size(); ++i) co[i] = h->terms[i].coeff;
+  const size_t at_co = put(co.data(), co.size() * 8);
+  std::vector<std::array<size_t, 6>> at(n);
   for (int k = 0; k < n; ++k) {
-    if (!t.parent[k].empty()) {
-      TRY(dalloc(&h->d_parent[k], t.parent[k].size()));
-      TRY(dalloc(&h->d_edge[k], t.edge[k].size()));
-      CU(cudaMemcpy(h->d_parent[k], t.parent[k].data(), t.parent[k].size() * 4, cudaMemcpyHostToDevice));
-      CU(cudaMemcpy(h->d_edge[k], t.edge[k].data(), t.edge[k].size(), cudaMemcpyHostToDevice));
-    }
-    if (!t.close_term[k].empty()) {
-      TRY(dalloc(&h->d_cnode[k], t.close_node[k].size()));
-      TRY(dalloc(&h->d_cletter[k], t.close_letter[k].size()));
-      TRY(dalloc(&h->d_cterm[k], t.close_term[k].size()));
-      CU(cudaMemcpy(h->d_cnode[k], t.close_node[k].data(), t.close_node[k].size() * 4, cudaMemcpyHostToDevice));
-      CU(cudaMemcpy(h->d_cletter[k], t.close_letter[k].data(), t.close_letter[k].size(), cudaMemcpyHostToDevice));
-      CU(cudaMemcpy(h->d_cterm[k], t.close_term[k].data(), t.close_term[k].size() * 4, cudaMemcpyHostToDevice));
-    }
+    auto put_vec = [&](const auto& v) { return put(v.data(), v.size() * sizeof(v[0])); };
+    at[k] = {put_vec(t.parent[k]),     put_vec(t.edge[k]),       put_vec(t.child_begin[k]),
+             put_vec(t.close_node[k]), put_vec(t.close_letter[k]), put_vec(t.close_term[k])};
+  }
+  dfree(h->d_all);   // of an upload that failed half way
+  h->d_all = nullptr;
+  char* d = nullptr;
+  TRY(dalloc(&d, host.size()));
+  h->d_all = d;
+  CU(cudaMemcpy(d, host.data(), host.size(), cudaMemcpyHostToDevice));
+  h->d_coeff = (double*)(d + at_co);
+  h->d_parent.resize(n);
+  h->d_edge.resize(n);
+  h->d_cbegin.resize(n);
+  h->d_cnode.resize(n);
+  h->d_cletter.resize(n);
+  h->d_cterm.resize(n);
+  for (int k = 0; k < n; ++k) {
+    h->d_parent[k] = (int32_t*)(d + at[k][0]);
+    h->d_edge[k] = (uint8_t*)(d + at[k][1]);
+    h->d_cbegin[k] = (int32_t*)(d + at[k][2]);
+    h->d_cnode[k] = (int32_t*)(d + at[k][3]);
+    h->d_cletter[k] = (uint8_t*)(d + at[k][4]);
+    h->d_cterm[k] = (int32_t*)(d + at[k][5]);
   }
   h->uploaded = true;
   return MPS_OK;
@@ -273,33 +284,25 @@ static int ensure_theta(mps_s* m, size_t count) {
 constexpr int kTcMinDim = 128;    // levels with both bonds >= 128 use the tensor cores
 struct MeasPlan {
   std::vector<int32_t> cap;
-  int tc_nodes = 0;
   size_t level_bytes = 0, tc_bytes = 0;
 };
+// Bytes of T per node: two D x D' blocks, or T^T with its padded node stride.
+static size_t t_bytes(int chi, size_t es) {
+  return chi <= kFusedMax ? 0 : 2 * (size_t)chi * env_tc_node_stride(chi) * es;
+}
 static MeasPlan meas_plan(const Trie& t, int chi, size_t es, bool mixed, size_t budget = 0) {
   MeasPlan p;
   const size_t chi2 = (size_t)chi * chi, node_bytes = 3 * chi2 * es;
-  const bool explicit_budget = budget != 0;
   if (budget == 0) budget = (chi <= 128 ? size_t(4) : size_t(48)) << 30;
   const size_t per_level = budget / (size_t)std::max(1, t.n_levels);
   const int32_t U = (int32_t)std::max<size_t>(16, per_level / node_bytes);
   p.cap.assign(t.n, 0);
-  int32_t cmax = 1;
   for (int k = 0; k < t.n_levels; ++k) {
     p.cap[k] = std::min(t.level_nodes[k], U);
-    cmax = std::max(cmax, p.cap[k]);
-    p.level_bytes += (size_t)p.cap[k] * node_bytes;
+    // bonds up to kFusedMax keep T in shared memory
+    p.level_bytes += (size_t)p.cap[k] * (chi2 * es + t_bytes(chi, es));
   }
-  if (mixed && chi >= kTcMinDim) {
-    const size_t per_node = 24 * chi2;    // bytes of the W rows and GEMM-C output per child
-    // a quarter of an explicit budget, else 1 GiB (chi <= 128) or 4 GiB
-    const size_t tc_budget = explicit_budget ? std::max<size_t>(size_t(64) << 20, budget / 4)
-                                             : (chi <= 128 ? size_t(1) : size_t(4)) << 30;
-    // at most 65 535 children per chunk: the W-row kernel puts one child per grid z index
-    p.tc_nodes = (int)std::min<size_t>(std::min<size_t>((size_t)cmax, 65535),
-                                       std::max<size_t>(32, tc_budget / per_node));
-    p.tc_bytes = env_tc_scratch_floats(chi, p.tc_nodes) * sizeof(float) + 256;
-  }
+  if (mixed && chi >= kTcMinDim) p.tc_bytes = env_tc_scratch_floats(chi) * sizeof(float);
   return p;
 }
 
@@ -327,27 +330,30 @@ static int ensure_meas(mps_s* m, ham_s* h) {
     m->lvl_L[k] = m->lvl_T[k] = nullptr;
     m->lvl_cap[k] = 0;
     TRY(dev_alloc(&m->lvl_L[k], (size_t)plan.cap[k] * chi2 * m->es, "environment buffer", m->st));
-    TRY(dev_alloc(&m->lvl_T[k], (size_t)plan.cap[k] * 2 * chi2 * m->es, "T buffer", m->st));
+    if (m->chi > kFusedMax)
+      TRY(dev_alloc(&m->lvl_T[k], (size_t)plan.cap[k] * t_bytes(m->chi, m->es), "T buffer", m->st));
     m->lvl_cap[k] = plan.cap[k];
   }
-  if (plan.tc_nodes > m->tc.max_nodes) {
-    dfree(m->tc.scratch, m->st);
-    m->tc.scratch = nullptr;
-    m->tc.max_nodes = 0;
+  if (plan.tc_bytes && !m->tc.scratch) {
     void* p;
     TRY(dev_alloc(&p, plan.tc_bytes, "tensor-core scratch", m->st));
     m->tc.scratch = (float*)p;
     if (!m->tc.err) TRY(dalloc(&m->tc.err, 1, m->st));
     m->tc.chi = m->chi;
-    m->tc.max_nodes = plan.tc_nodes;
   }
   if (terms > m->w_terms) {
     dfree(m->w.vals, m->st);
     dfree(m->w.out, m->st);
-    m->w.vals = m->w.out = nullptr;
+    dfree(m->w.part, m->st);
+    m->w.vals = m->w.out = m->w.part = nullptr;
     m->w_terms = 0;
     TRY(dalloc(&m->w.vals, (size_t)terms * 2, m->st));
     TRY(dalloc(&m->w.out, 4 + (size_t)terms * 2, m->st));
+    TRY(dalloc(&m->w.part, 2 * (size_t)energy_sum_blocks(terms), m->st));
+    if (!m->w.done) {
+      TRY(dalloc(&m->w.done, 1, m->st));
+      CU(cudaMemsetAsync(m->w.done, 0, sizeof(unsigned), m->st));
+    }
     m->w_terms = terms;
   }
   return MPS_OK;
@@ -481,19 +487,23 @@ static int meas_chunk(MeasWalk& c, int k, int u0, int u1) {
   // the tensor-core route reads L in place as rows of 2D floats, which TMA needs 16-byte
   // aligned: levels with an odd left bond stay on the CUDA-core kernels
   const bool tc = m->prec == MPS_MIXED && m->tc.scratch && D >= kTcMinDim && Dp >= kTcMinDim && (D & 1) == 0;
-  if (tc) {
+  const bool fused = !tc && D <= kFusedMax && Dp <= kFusedMax;
+  const bool leaf = k + 1 >= t.n_levels || k + 1 >= m->n;
+  if (tc && !leaf) {
     const Cx<float>* Bk = (const Cx<float>*)m->dm.B + (size_t)c.slot * m->dm.slot_elems + m->site_off[k];
     CU(env_tc_site(m->tc, Bk, D, Dp, m->st));
     ++c.launches;
     cudaEvent_t e0, e1;
     TRY(next_event_pair(m, &e0, &e1));
-    CU(env_tc_T(m->tc, (const Cx<float>*)L, (Cx<float>*)T, U, D, Dp, m->st, e0, e1));
+    CU(env_tc_T(m->tc, (const Cx<float>*)L, (float*)T, U, D, Dp, m->st, e0, e1));
     c.launches += 1;
     m->stats.tc_gemm_launches += 1;
     m->stats.tc_gemm_flops += 2.0 * ((double)U * D) * (4.0 * Dp) * (2.0 * D);
-  } else {
-    CU(launch_env_T(m->dm, m->prec, c.slot, k, L, T, U, m->st));
-    ++c.launches;
+  } else if (!tc) {
+    if (!fused && !leaf) {
+      CU(launch_env_T(m->dm, m->prec, c.slot, k, L, T, U, c.h->d_cbegin[k] + u0, m->st));
+      ++c.launches;
+    }
   }
   // strings closing at level k on this chunk's nodes
   const auto& cn = t.close_node[k];
@@ -508,13 +518,13 @@ static int meas_chunk(MeasWalk& c, int k, int u0, int u1) {
     if (e1) CU(cudaEventRecord(e1, m->st));
     ++c.launches;
   }
-  if (k + 1 >= t.n_levels || k + 1 >= m->n) return MPS_OK;
+  if (leaf) return MPS_OK;
   const auto& par = t.parent[k + 1];
   int64_t a = std::lower_bound(par.begin(), par.end(), u0) - par.begin();
   const int64_t c1 = std::lower_bound(par.begin(), par.end(), u1) - par.begin();
   while (a < c1) {
     int64_t b = a + 1;
-    while (b < c1 && b - a < m->lvl_cap[k + 1] && (!tc || b - a < m->tc.max_nodes)) ++b;
+    while (b < c1 && b - a < m->lvl_cap[k + 1]) ++b;
     if (tc) {
       // the shared operands of site k live in the scratch, which the deeper levels of
       // the previous sub-chunk have used for their own sites: rebuild them
@@ -524,11 +534,15 @@ static int meas_chunk(MeasWalk& c, int k, int u0, int u1) {
       cudaEvent_t e0, e1;
       TRY(next_event_pair(m, &e0, &e1));
       const int nch = (int)(b - a);
-      CU(env_tc_children(m->tc, (const Cx<float>*)T, c.h->d_parent[k + 1] + a, c.h->d_edge[k + 1] + a, nch, u0,
-                         D, Dp, (Cx<float>*)m->lvl_L[k + 1], m->st, e0, e1));
-      c.launches += 3;
+      CU(env_tc_children(m->tc, (const float*)T, c.h->d_parent[k + 1] + a, c.h->d_edge[k + 1] + a, nch, u0, U, D, Dp,
+                         (Cx<float>*)m->lvl_L[k + 1], m->st, e0, e1));
+      c.launches += 1;
       m->stats.tc_gemm_launches += 1;
       m->stats.tc_gemm_flops += 2.0 * (2.0 * Dp) * ((double)nch * Dp) * (4.0 * D);
+    } else if (fused) {
+      CU(launch_level_fused(m->dm, m->prec, c.slot, k, D, Dp, par[a], par[b - 1] + 1, u0, (int)a, (int)b,
+                            c.h->d_cbegin[k], c.h->d_parent[k + 1], c.h->d_edge[k + 1], L, m->lvl_L[k + 1], m->st));
+      ++c.launches;
     } else {
       CU(launch_env_child(m->dm, m->prec, c.slot, k, T, c.h->d_parent[k + 1] + a, c.h->d_edge[k + 1] + a,
                           (int)(b - a), u0, m->lvl_L[k + 1], m->st));
@@ -551,7 +565,7 @@ static int run_measure(mps_s* m, ham_s* h, int slot, double* out_host, bool term
   if (m->tc.err) CU(cudaMemsetAsync(m->tc.err, 0, sizeof(int), m->st));
   m->kev_used = 0;
   CU(cudaEventRecord(m->ev[2], m->st));
-  CU(launch_right_envs(m->dm, m->prec, slot, c.r.data(), m->site_off.data(), m->w, m->st, &c.launches));
+  CU(launch_right_envs(m->dm, m->prec, slot, c.r.data(), m->w, m->st, &c.launches));
   const Trie& t = h->trie;
   if (t.n_levels > 0) {
     // root environment L_0 = [1] (one node, D_0 = 1)
@@ -561,7 +575,7 @@ static int run_measure(mps_s* m, ham_s* h, int slot, double* out_host, bool term
                        cudaMemcpyHostToDevice, m->st));
     TRY(meas_chunk(c, 0, 0, t.level_nodes[0]));
   }
-  CU(launch_energy_sum(m->dm, m->prec, slot, m->w, T, h->d_coeff, h->id_term >= 0 ? h->id_coeff : 0.0,
+  CU(launch_energy_sum(m->prec, m->w, T, h->d_coeff, h->id_term >= 0 ? h->id_coeff : 0.0,
                        h->id_term, m->st));
   ++c.launches;
   CU(cudaEventRecord(m->ev[3], m->st));
@@ -762,7 +776,7 @@ int mps_estimate_bytes(int n_qubits, int chi, int precision, int n_slots, circ_t
     const size_t T = ham->terms.size();
     const MeasPlan plan = meas_plan(ham->trie, chi, es, precision == MPS_MIXED);
     b += plan.level_bytes + plan.tc_bytes + (4 + 4 * T) * 8;   // chunk buffers, tensor-core scratch, values
-    b += T * (8 + 4 + 1 + 4) + T * (size_t)n;                  // coefficients and the trie arrays
+    b += T * (8 + 4 + 1 + 4) + (size_t)ham->trie.total_nodes * 9;   // coefficients and the trie arrays
   }
   *bytes = b;
   return MPS_OK;
@@ -879,9 +893,6 @@ int mps_set_meas_budget(mps_t m, size_t bytes) {
     p = nullptr;
   }
   std::fill(m->lvl_cap.begin(), m->lvl_cap.end(), 0);
-  dfree(m->tc.scratch, m->st);
-  m->tc.scratch = nullptr;
-  m->tc.max_nodes = 0;
   m->meas_budget = bytes;
   return MPS_OK;
 }

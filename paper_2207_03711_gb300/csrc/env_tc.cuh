@@ -8,28 +8,30 @@
 
 namespace mpsvqe {
 
-// Scratch of one handle for chunks of up to max_nodes children at bond cap chi.
+// Scratch of one handle at bond cap chi: the shared operands of one site.
 struct EnvTc {
-  float* scratch = nullptr;   // env_tc_scratch_floats(chi, max_nodes) floats, 256-byte aligned
+  float* scratch = nullptr;   // env_tc_scratch_floats(chi) floats, 256-byte aligned
   int* err = nullptr;         // device int: set by a tensor-core pipeline wait that ran out
   int chi = 0;
-  int max_nodes = 0;
 };
 
-size_t env_tc_scratch_floats(int chi, int max_nodes);
+size_t env_tc_scratch_floats(int chi);
+
+// Floats from one node's T^T to the next: D rounded up to a multiple of 4.
+inline int env_tc_node_stride(int D) { return (D + 3) & ~3; }
 
 // Shared operands of site k (D = left bond, Dp = right bond), once per level chunk.
 cudaError_t env_tc_site(const EnvTc& s, const Cx<float>* Bk, int D, int Dp, cudaStream_t st);
-// T_j[u] = L[u] B^j for the U nodes of a dense level chunk (L[u] at u D^2; T written as
-// T_j[u][a][c] at ((u D + a) 2 + j) D' + c; both 16-byte aligned, D and D' even).
+// T_j[u] = L[u] B^j for the U nodes of a dense level chunk (L[u] at u D^2, D even), as T^T:
+// 4 Dp rows (j, re/im, c) over columns (u, a), env_tc_node_stride(D) floats per node.
 // e0 / e1 (optional) are recorded on st right before and after the tensor-core GEMM.
-cudaError_t env_tc_T(const EnvTc& s, const Cx<float>* L, Cx<float>* T, int U, int D, int Dp, cudaStream_t st,
+cudaError_t env_tc_T(const EnvTc& s, const Cx<float>* L, float* Tt, int U, int D, int Dp, cudaStream_t st,
                      cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr);
-// L[child] = sum_ij P_ij (B^i)^+ T_j[parent] for nc <= max_nodes children (parent: trie
-// node indices, node_base = the trie index of T's entry 0; edge: the letters P), written
-// densely (child c at c D'^2).
-cudaError_t env_tc_children(const EnvTc& s, const Cx<float>* T, const int32_t* parent, const uint8_t* edge, int nc,
-                            int node_base, int D, int Dp, Cx<float>* Lout, cudaStream_t st,
+// L[child] = sum_ij P_ij (B^i)^+ T_j[parent] for nc children (parent: trie node indices,
+// node_base = the trie index of T^T's entry 0; edge: the letters P), written densely
+// (child c at c D'^2).
+cudaError_t env_tc_children(const EnvTc& s, const float* Tt, const int32_t* parent, const uint8_t* edge, int nc,
+                            int node_base, int U, int D, int Dp, Cx<float>* Lout, cudaStream_t st,
                             cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr);
 
 }  // namespace mpsvqe

@@ -13,6 +13,7 @@
 
 #include "../../include/mpsvqe.h"
 #include "gate.cuh"
+#include "smem_limit.cuh"
 
 namespace mpsvqe {
 
@@ -1161,31 +1162,11 @@ __global__ void __launch_bounds__(NT) k_circuit(DevMPS m, CircDev c, int64_t g0,
 
 }  // namespace gate
 
-// The dynamic shared-memory limit of a kernel is process-wide state: handles of
-// different chi launch the same instantiation from several threads, so the limit is
-// raised once to the device's opt-in maximum and never lowered.
-template <auto Kernel>
-static cudaError_t raise_smem_limit() {
-  static std::once_flag once[64];
-  static cudaError_t status[64];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  std::call_once(once[dev], [dev] {
-    int optin = 0;
-    status[dev] = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (status[dev] == cudaSuccess)
-      status[dev] = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
-  });
-  return status[dev];
-}
-
 template <class R, int NT, int C, bool RAW>
 static cudaError_t launch_cluster(const DevMPS& m, const CircDev& c, int64_t g0, int64_t g1, int slot0, int count,
                                   const double* theta, double cutoff, int max_sweeps, cudaStream_t st) {
   constexpr auto kernel = gate::k_circuit<R, NT, C, RAW>;
-  cudaError_t e = raise_smem_limit<kernel>();
+  cudaError_t e = gate::raise_smem_limit<kernel>();
   if (e != cudaSuccess) return e;
   const gate::Plan<R, NT, C> L(m.chi);
   cudaLaunchConfig_t cfg = {};

@@ -654,6 +654,14 @@ void build_trie(int n, const std::vector<Term>& terms, Trie* t) {
     t->max_level_nodes = std::max(t->max_level_nodes, t->level_nodes[k]);
     t->max_level_closes = std::max(t->max_level_closes, (int32_t)t->close_term[k].size());
   }
+  // children of a node are consecutive: first child of each, and the end
+  t->child_begin.assign(n, {});
+  for (int k = 0; k + 1 < t->n_levels; ++k) {
+    auto& cb = t->child_begin[k];
+    cb.assign((size_t)t->level_nodes[k] + 1, 0);
+    for (int32_t p : t->parent[k + 1]) ++cb[(size_t)p + 1];
+    for (int32_t u = 0; u < t->level_nodes[k]; ++u) cb[(size_t)u + 1] += cb[u];
+  }
 }
 
 }  // namespace mpsvqe

@@ -46,6 +46,8 @@ struct Trie {
   // node -> parent (level k+1 refers into level k) and the Pauli letter on edge
   std::vector<std::vector<int32_t>> parent;
   std::vector<std::vector<uint8_t>> edge;
+  // first child (index in level k + 1) of each node of level k, and the end of the last
+  std::vector<std::vector<int32_t>> child_begin;
   // closes at level k: (node at level k, letter at site k, term index)
   std::vector<std::vector<int32_t>> close_node;
   std::vector<std::vector<uint8_t>> close_letter;

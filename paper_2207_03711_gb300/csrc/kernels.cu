@@ -8,8 +8,13 @@
 #include <cmath>
 #include <cstdint>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "cx.cuh"
+#include "gemm.cuh"
 #include "kernels.cuh"
+#include "smem_limit.cuh"
 
 namespace mpsvqe {
 
@@ -118,97 +123,196 @@ __device__ void block_gemm(int Mdim, int Ndim, int K, const GemmTerm<R>* terms, 
     for (int n0 = 0; n0 < Ndim; n0 += 64) gemm_tile<R, NTH>(m0, n0, Mdim, Ndim, K, terms, nterm, C, ldc, As, Bs);
 }
 
-// The same product spread over a grid: one 64 x 64 tile per thread block, blockIdx.z
-// selecting one of up to four independent products.
-template <class R>
-struct GridGemm {
-  GemmTerm<R> t[4][2];
-  int nterm;
-  Cx<R>* C[4];
-  int ldc, M, N, K;
-};
-
-template <class R>
-__global__ void __launch_bounds__(256) k_cgemm_grid(GridGemm<R> g) {
-  __shared__ Cx<R> As[64][17];
-  __shared__ Cx<R> Bs[16][65];
-  const int z = blockIdx.z;
-  gemm_tile<R, 256>(blockIdx.y * 64, blockIdx.x * 64, g.M, g.N, g.K, g.t[z], g.nterm, g.C[z], g.ldc, As, Bs);
+// --------------------------------------------------------- right environments
+// R_n = [1]; Bhat_k^i = B_k^i R_{k+1} (same layout as B_k); R_k = sum_i Bhat_k^i (B_k^i)^+.
+// A site is a chain of two products, both plain GEMMs on the stored layout: Bhat = (2 Dl x
+// Dr) R and R_k = Bhat B^+ over (i, c) as one inner index. The per-letter blocks
+//   Q_k^P = sum_ij conj(P_ij) Bhat_k^i (B_k^j)^+,  P = X, Y, Z
+// (a string closing at site k with letter P has <P> = sum_ab L[a][b] conj(Q_k^P[a][b]),
+// Eq. 11 with the right part contracted; no string closes with I) hang off the chain and
+// run for all sites in one launch afterwards, from three sums over the four pairs of
+// operand entries: G01 and G10 give X and Y, the difference of G00 and G11 gives Z.
+template <class R, int NT>
+__device__ __forceinline__ void renv_bhat(const Cx<R>* Bk, const Cx<R>* Rn, Cx<R>* Bh, int Dl, int Dr, int tile, int ntiles,
+                                          unsigned char* smem) {
+  // rows are dealt to blocks in slabs
+  const int M = 2 * Dl, per = (M + ntiles - 1) / ntiles, m0 = min(M, per * tile), mn = min(per, M - m0);
+  gate::tile_gemm<R, NT, false>(
+      mn, Dr, Dr, [&](int i, int k) { return Bk[(size_t)(m0 + i) * Dr + k]; },
+      [&](int k, int j) { return Rn ? gate::ldcg(Rn + (size_t)k * Dr + j) : cx<R>(R(1), R(0)); },   // R_n = [1]
+      [&](int i, int j, Cx<R> v) { Bh[(size_t)(m0 + i) * Dr + j] = v; }, smem);
+}
+template <class R, int NT>
+__device__ __forceinline__ void renv_close(const Cx<R>* Bk, const Cx<R>* Bh, Cx<R>* Rk, int Dl, int Dr, int tile, int ntiles,
+                                           unsigned char* smem) {
+  const int per = (Dl + ntiles - 1) / ntiles, m0 = min(Dl, per * tile), mn = min(per, Dl - m0);
+  gate::tile_gemm<R, NT, true>(
+      mn, Dl, 2 * Dr, [&](int i, int k) { return gate::ldcg(Bh + (size_t)(m0 + i) * 2 * Dr + k); },
+      [&](int k, int j) { return conj(Bk[(size_t)j * 2 * Dr + k]); },
+      [&](int i, int j, Cx<R> v) { Rk[(size_t)(m0 + i) * Dl + j] = v; }, smem);
 }
 
-// --------------------------------------------------------- right environments
-// R_n = [1]; R_k = sum_i Bhat_k^i (B_k^i)^+ with Bhat_k^i = B_k^i R_{k+1} (same layout as
-// B_k). Per site two grid launches (the two Bhat^i products side by side, then R_k), so
-// large bond dimensions use many SMs. ranks: the slot's bond ranks on the host
-// (ranks[k] = left dimension of site k).
-template <class R>
-static cudaError_t right_envs_t(const DevMPS& m, int slot, const int* ranks, const int64_t* site_off, Cx<R>* Renv,
-                                Cx<R>* Bhat, Cx<R>* Q, cudaStream_t st) {
-  const int n = m.n;
-  const size_t chi2 = (size_t)m.chi * m.chi;
+// The whole chain by one cluster of C blocks (small bonds: a launch per product would cost
+// more than the product).
+template <class R, int C>
+__global__ void __launch_bounds__(256) k_renv_chain(DevMPS m, int slot, Cx<R>* Renv, Cx<R>* Bhat) {
+  extern __shared__ __align__(256) unsigned char smem[];
+  const int* rank = m.rank + (size_t)slot * (m.n + 1);
   const Cx<R>* Bslot = (const Cx<R>*)m.B + (size_t)slot * m.slot_elems;
-  static const Cx<R> one = cx<R>(1, 0);
-  cudaError_t e = cudaMemcpyAsync(Renv + (size_t)n * chi2, &one, sizeof(Cx<R>), cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) return e;
-  for (int k = n - 1; k >= 0; --k) {
-    const int Dl = ranks[k], Dr = ranks[k + 1];
-    const Cx<R>* Bk = Bslot + site_off[k];
-    Cx<R>* Bh = Bhat + site_off[k];
-    const Cx<R>* Rn = Renv + (size_t)(k + 1) * chi2;
-    GridGemm<R> g{};
-    g.nterm = 1;
-    g.ldc = 2 * Dr;
-    g.M = Dl;
-    g.N = Dr;
-    g.K = Dr;
-    for (int i = 0; i < 2; ++i) {   // Bhat^i = B^i R_{k+1}: (Dl x Dr)(Dr x Dr)
-      g.t[i][0] = GemmTerm<R>{Bk + i * Dr, 2 * Dr, false, Rn, Dr, cx<R>(1, 0), false};
-      g.C[i] = Bh + i * Dr;
-    }
-    k_cgemm_grid<R><<<dim3((Dr + 63) / 64, (Dl + 63) / 64, 2), 256, 0, st>>>(g);
-    // R_k = sum_i Bhat^i (B^i)^+: B^i read as (Dl x Dr) transposed and conjugated
-    GridGemm<R> h{};
-    h.nterm = 2;
-    h.ldc = Dl;
-    h.M = Dl;
-    h.N = Dl;
-    h.K = Dr;
-    for (int i = 0; i < 2; ++i) h.t[0][i] = GemmTerm<R>{Bh + i * Dr, 2 * Dr, false, Bk + i * Dr, 2 * Dr, cx<R>(1, 0), true, true};
-    h.C[0] = Renv + (size_t)k * chi2;
-    k_cgemm_grid<R><<<dim3((Dl + 63) / 64, (Dl + 63) / 64, 1), 256, 0, st>>>(h);
-    // Q_k^P = sum over the letter's two entries (i, j, s) of conj(s) Bhat^i (B^j)^+, one
-    // product per letter I, X, Y, Z: a string closing at site k with letter P has
-    // <P> = sum_ab L[a][b] conj(Q_k^P[a][b]) (Eq. 11 with the right part contracted)
-    GridGemm<R> q{};
-    q.nterm = 2;
-    q.ldc = Dl;
-    q.M = Dl;
-    q.N = Dl;
-    q.K = Dr;
-    for (int l = 0; l < 4; ++l) {
-      const int ii[4][2] = {{0, 1}, {0, 1}, {0, 1}, {0, 1}};
-      const int jj[4][2] = {{0, 1}, {1, 0}, {1, 0}, {0, 1}};
-      // conj of the letter's entries: I (1, 1), X (1, 1), Y (-i, i) -> (i, -i), Z (1, -1)
-      const Cx<R> cs[4][2] = {{cx<R>(1, 0), cx<R>(1, 0)},
-                              {cx<R>(1, 0), cx<R>(1, 0)},
-                              {cx<R>(0, 1), cx<R>(0, -1)},
-                              {cx<R>(1, 0), cx<R>(-1, 0)}};
-      for (int e = 0; e < 2; ++e)
-        q.t[l][e] = GemmTerm<R>{Bh + ii[l][e] * Dr, 2 * Dr, false, Bk + jj[l][e] * Dr, 2 * Dr, cs[l][e], true, true};
-      q.C[l] = Q + ((size_t)k * 4 + l) * chi2;
-    }
-    k_cgemm_grid<R><<<dim3((Dl + 63) / 64, (Dl + 63) / 64, 4), 256, 0, st>>>(q);
+  const size_t chi2 = (size_t)m.chi * m.chi;
+  const int c = (int)gate::crank<C>();
+  for (int k = m.n - 1; k >= 0; --k) {
+    const int Dl = rank[k], Dr = rank[k + 1];
+    const Cx<R>* Bk = Bslot + m.site_off[k];
+    Cx<R>* Bh = Bhat + m.site_off[k];
+    renv_bhat<R, 256>(Bk, k == m.n - 1 ? nullptr : Renv + (size_t)(k + 1) * chi2, Bh, Dl, Dr, c, C, smem);
+    gate::csync<C>();
+    renv_close<R, 256>(Bk, Bh, Renv + (size_t)k * chi2, Dl, Dr, c, C, smem);
+    gate::csync<C>();
   }
+}
+// One product of one site over a grid (large bonds).
+template <class R>
+__global__ void __launch_bounds__(256) k_renv_step(DevMPS m, int slot, int k, int stage, Cx<R>* Renv, Cx<R>* Bhat) {
+  extern __shared__ __align__(256) unsigned char smem[];
+  const int* rank = m.rank + (size_t)slot * (m.n + 1);
+  const size_t chi2 = (size_t)m.chi * m.chi;
+  const int Dl = rank[k], Dr = rank[k + 1];
+  const Cx<R>* Bk = (const Cx<R>*)m.B + (size_t)slot * m.slot_elems + m.site_off[k];
+  Cx<R>* Bh = Bhat + m.site_off[k];
+  // blockIdx.y: column slabs of 64 (the tile shape's width)
+  const int N = stage == 0 ? Dr : Dl, n0 = blockIdx.y * 64, nn = min(64, N - n0);
+  if (nn <= 0) return;
+  const int M = stage == 0 ? 2 * Dl : Dl, per = (M + gridDim.x - 1) / gridDim.x, m0 = min(M, per * (int)blockIdx.x),
+            mn = min(per, M - m0);
+  const Cx<R>* Rn = k == m.n - 1 ? nullptr : Renv + (size_t)(k + 1) * chi2;
+  Cx<R>* Rk = Renv + (size_t)k * chi2;
+  if (stage == 0)
+    gate::tile_gemm<R, 256, false>(
+        mn, nn, Dr, [&](int i, int q) { return Bk[(size_t)(m0 + i) * Dr + q]; },
+        [&](int q, int j) { return Rn ? gate::ldcg(Rn + (size_t)q * Dr + n0 + j) : cx<R>(R(1), R(0)); },
+        [&](int i, int j, Cx<R> v) { Bh[(size_t)(m0 + i) * Dr + n0 + j] = v; }, smem);
+  else
+    gate::tile_gemm<R, 256, true>(
+        mn, nn, 2 * Dr, [&](int i, int q) { return gate::ldcg(Bh + (size_t)(m0 + i) * 2 * Dr + q); },
+        [&](int q, int j) { return conj(Bk[(size_t)(n0 + j) * 2 * Dr + q]); },
+        [&](int i, int j, Cx<R> v) { Rk[(size_t)(m0 + i) * Dl + n0 + j] = v; }, smem);
+}
+
+// Q_k^X, Q_k^Y, Q_k^Z of all sites: output tiles of 16 TI x 16 TI, TI^2 outputs per thread
+// and sum, 16-deep tiles of the four operands. Grid (tiles, sites). TI = 2 in FP32; 1 in
+// FP64, whose tiles are worth more blocks.
+template <class R, int TI>
+__global__ void __launch_bounds__(256) k_letter_blocks(DevMPS m, int slot, const Cx<R>* Bhat, Cx<R>* Q) {
+  __shared__ Cx<R> A[2][16 * TI][17];
+  __shared__ Cx<R> B[2][16 * TI][17];
+  const int k = blockIdx.y;
+  const int* rank = m.rank + (size_t)slot * (m.n + 1);
+  const int Dl = rank[k], Dr = rank[k + 1], TS = 16 * TI, nt = (Dl + TS - 1) / TS;
+  if ((int)blockIdx.x >= nt * nt) return;
+  const int m0 = blockIdx.x / nt * TS, n0 = blockIdx.x % nt * TS;
+  const Cx<R>* Bk = (const Cx<R>*)m.B + (size_t)slot * m.slot_elems + m.site_off[k];
+  const Cx<R>* Bh = Bhat + m.site_off[k];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  Cx<R> g01[TI][TI], g10[TI][TI], gz[TI][TI];
+#pragma unroll
+  for (int i = 0; i < TI; ++i)
+#pragma unroll
+    for (int j = 0; j < TI; ++j) g01[i][j] = g10[i][j] = gz[i][j] = cx<R>(0, 0);
+  for (int k0 = 0; k0 < Dr; k0 += 16) {
+    __syncthreads();
+    for (int e = tid; e < 2 * TS * 16; e += 256) {
+      const int q = e & 15, r = (e >> 4) % TS, s = (e >> 4) / TS, c = k0 + q;
+      A[s][r][q] = (m0 + r < Dl && c < Dr) ? Bh[((size_t)(m0 + r) * 2 + s) * Dr + c] : cx<R>(0, 0);
+      B[s][r][q] = (n0 + r < Dl && c < Dr) ? Bk[((size_t)(n0 + r) * 2 + s) * Dr + c] : cx<R>(0, 0);
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int q = 0; q < 16; ++q) {
+      Cx<R> a0[TI], a1[TI], b0[TI], b1[TI];
+#pragma unroll
+      for (int i = 0; i < TI; ++i) {
+        a0[i] = A[0][ty + 16 * i][q];
+        a1[i] = A[1][ty + 16 * i][q];
+        b0[i] = B[0][tx + 16 * i][q];
+        b1[i] = B[1][tx + 16 * i][q];
+      }
+#pragma unroll
+      for (int i = 0; i < TI; ++i)
+#pragma unroll
+        for (int j = 0; j < TI; ++j) {
+          cmac_bconj(g01[i][j], a0[i], b1[j]);
+          cmac_bconj(g10[i][j], a1[i], b0[j]);
+          cmac_bconj(gz[i][j], a0[i], b0[j]);
+          cmac_bconj(gz[i][j], cx<R>(-a1[i].x, -a1[i].y), b1[j]);
+        }
+    }
+  }
+  Cx<R>* q = Q + (size_t)k * 4 * m.chi * m.chi;
+  const size_t chi2 = (size_t)m.chi * m.chi;
+#pragma unroll
+  for (int i = 0; i < TI; ++i)
+#pragma unroll
+    for (int j = 0; j < TI; ++j) {
+      const int r = m0 + ty + 16 * i, c = n0 + tx + 16 * j;
+      if (r < Dl && c < Dl) {
+        const size_t o = (size_t)r * Dl + c;
+        const Cx<R> d = g01[i][j] - g10[i][j];
+        q[chi2 + o] = g01[i][j] + g10[i][j];
+        q[2 * chi2 + o] = cx<R>(-d.y, d.x);   // i G01 - i G10
+        q[3 * chi2 + o] = gz[i][j];
+      }
+    }
+}
+
+// Bonds up to this run the chain in one cluster launch. FP64 products of larger bonds are
+// worth more SMs than a cluster has.
+template <class R>
+constexpr int kChainMax = sizeof(R) == 4 ? 64 : 32;
+
+template <class R>
+static cudaError_t right_envs_t(const DevMPS& m, int slot, const int* ranks, Cx<R>* Renv, Cx<R>* Bhat, Cx<R>* Q,
+                                cudaStream_t st, int* launches) {
+  const size_t smem = gate::gemm_tile_bytes<256>();
+  int top = 1;
+  for (int k = 0; k <= m.n; ++k) top = std::max(top, ranks[k]);
+  if (top <= kChainMax<R>) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(8);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 8;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_renv_chain<R, 8>, m, slot, Renv, Bhat);
+    if (e != cudaSuccess) return e;
+    *launches += 1;
+  } else {
+    for (int k = m.n - 1; k >= 0; --k) {
+      const int Dl = ranks[k], Dr = ranks[k + 1];
+      // slabs of 16 rows: the shortest time for one product of a serial chain
+      k_renv_step<R><<<dim3((2 * Dl + 15) / 16, (Dr + 63) / 64), 256, smem, st>>>(m, slot, k, 0, Renv, Bhat);
+      k_renv_step<R><<<dim3((Dl + 15) / 16, (Dl + 63) / 64), 256, smem, st>>>(m, slot, k, 1, Renv, Bhat);
+    }
+    *launches += 2 * m.n;
+  }
+  constexpr int TI = sizeof(R) == 4 ? 2 : 1;
+  const int nt = (top + 16 * TI - 1) / (16 * TI);
+  k_letter_blocks<R, TI><<<dim3(nt * nt, m.n), 256, 0, st>>>(m, slot, Bhat, Q);
+  *launches += 1;
   return cudaGetLastError();
 }
 
-cudaError_t launch_right_envs(const DevMPS& m, int prec, int slot, const int* ranks, const int64_t* site_off,
-                              MeasDev& w, cudaStream_t st, int* launches) {
-  *launches += 3 * m.n;
+cudaError_t launch_right_envs(const DevMPS& m, int prec, int slot, const int* ranks, MeasDev& w, cudaStream_t st,
+                              int* launches) {
   if (prec == MPS_PREC_FP64)
-    return right_envs_t<double>(m, slot, ranks, site_off, (Cx<double>*)w.R, (Cx<double>*)w.Bhat, (Cx<double>*)w.Q,
-                                st);
-  return right_envs_t<float>(m, slot, ranks, site_off, (Cx<float>*)w.R, (Cx<float>*)w.Bhat, (Cx<float>*)w.Q, st);
+    return right_envs_t<double>(m, slot, ranks, (Cx<double>*)w.R, (Cx<double>*)w.Bhat, (Cx<double>*)w.Q, st, launches);
+  return right_envs_t<float>(m, slot, ranks, (Cx<float>*)w.R, (Cx<float>*)w.Bhat, (Cx<float>*)w.Q, st, launches);
 }
 
 // ------------------------------------------------------------------ trie level
@@ -227,10 +331,12 @@ __device__ __forceinline__ void letter_entries(uint8_t l, int* ii, int* jj, Cx<R
 // and, on the CUDA-core route, T_j at (2u + j) Dk Dk1 (leading dimension Dk1).
 // T_j[u] = L_k[u] B_k^j  (Dk x Dk)(Dk x Dk1), grid (nodes, 2)
 template <class R>
-__global__ void __launch_bounds__(256) k_level_T(DevMPS m, int slot, int k, const Cx<R>* Lin, Cx<R>* T) {
+__global__ void __launch_bounds__(256) k_level_T(DevMPS m, int slot, int k, const Cx<R>* Lin, Cx<R>* T,
+                                                 const int32_t* cb) {
   __shared__ Cx<R> As[64][17];
   __shared__ Cx<R> Bs[16][65];
   const int u = blockIdx.x, j = blockIdx.y;
+  if (cb[u] == cb[u + 1]) return;
   const int* rank = m.rank + (size_t)slot * (m.n + 1);
   const int Dk = rank[k], Dk1 = rank[k + 1];
   const Cx<R>* Bk = (const Cx<R>*)m.B + (size_t)slot * m.slot_elems + m.site_off[k];
@@ -257,6 +363,204 @@ __global__ void __launch_bounds__(256) k_level_child(DevMPS m, int slot, int k, 
   for (int e = 0; e < 2; ++e)
     t[e] = GemmTerm<R>{Bk + ii[e] * Dk1, 2 * Dk1, true, T + ((size_t)u * 2 + jj[e]) * Dk * Dk1, Dk1, sg[e], false};
   block_gemm<R, 256>(Dk1, Dk1, Dk, t, 2, Lout + (size_t)c * Dk1 * Dk1, Dk1, As, Bs);
+}
+
+// Fused level for bonds up to 64: both T_j of a group of parents stay in shared memory and
+// the group's children are formed from them at once, so T never travels through memory,
+// nodes without children cost nothing but their rows, and small bonds share a block (64
+// rows of L and 64 columns of children at a time, whatever D and D').
+// cb: first child of each node of the level (trie indices); children outside [c_lo, c_hi)
+// are left to another launch; child c is written to Lout[c - c_lo].
+struct LevelArgs {
+  int slot, k;
+  int u_lo, u_hi;           // parents (trie indices)
+  int node_base;            // trie index of Lin's entry 0
+  int c_lo, c_hi;
+  const int32_t* cb;
+  const int32_t* parent;
+  const uint8_t* edge;
+};
+
+// FP32: site tensor, L rows and T in shared memory; 4 x JT outputs per thread for T, RM x 4
+// for the children, DP: right bond rounded up to a power of two.
+template <int DP>
+__global__ void __launch_bounds__(256) k_level_fused(DevMPS m, LevelArgs g, const Cx<float>* Lin, Cx<float>* Lout) {
+  extern __shared__ __align__(256) unsigned char smem[];
+  constexpr int JT = DP >= 16 ? DP / 8 : 1, RM = DP >= 16 ? DP / 16 : 1;
+  const int* rank = m.rank + (size_t)g.slot * (m.n + 1);
+  const int D = rank[g.k], Dp = rank[g.k + 1], W = 2 * Dp;
+  const int P = max(1, 64 / D), u0 = g.u_lo + blockIdx.x * P, u1 = min(u0 + P, g.u_hi);
+  const int c0 = max(g.cb[u0], g.c_lo), c1 = min(g.cb[u1], g.c_hi);
+  if (c0 >= c1) return;
+  Cx<float>* Bs = (Cx<float>*)smem;             // [D][2 D'], as stored
+  Cx<float>* Ls = Bs + D * W;                   // [rows][D + 1]
+  Cx<float>* Ts = Ls + 64 * (D + 1);            // [rows][2 D']
+  const Cx<float>* Bk = (const Cx<float>*)m.B + (size_t)g.slot * m.slot_elems + m.site_off[g.k];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int rows = (u1 - u0) * D;
+  const Cx<float>* Lu = Lin + (size_t)(u0 - g.node_base) * D * D;
+  for (int e = tid; e < D * W; e += 256) Bs[e] = Bk[e];
+  for (int e = tid; e < rows * D; e += 256) {
+    const int r = e / D, c = e - r * D;
+    Ls[r * (D + 1) + c] = Lu[e];
+  }
+  __syncthreads();
+  {
+    Cx<float> acc[4][JT];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < JT; ++j) acc[i][j] = cx<float>(0.f, 0.f);
+    int ro[4], co[JT];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) ro[i] = min(ty + 16 * i, rows - 1) * (D + 1);
+#pragma unroll
+    for (int j = 0; j < JT; ++j) co[j] = min(tx + 16 * j, W - 1);
+#pragma unroll 2
+    for (int q = 0; q < D; ++q) {
+      Cx<float> a[4], b[JT];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = Ls[ro[i] + q];
+#pragma unroll
+      for (int j = 0; j < JT; ++j) b[j] = Bs[q * W + co[j]];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < JT; ++j) cmac(acc[i][j], a[i], b[j]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < JT; ++j)
+        if (ty + 16 * i < rows && tx + 16 * j < W) Ts[(ty + 16 * i) * W + tx + 16 * j] = acc[i][j];
+  }
+  __syncthreads();
+  // children: columns (child, c) in turn, 64 at a time; out = s0 (B^0)^+ T_{j0} + s1 (B^1)^+ T_{j1}
+  const int ncol = (c1 - c0) * Dp;
+  for (int n0 = 0; n0 < ncol; n0 += 64) {
+    Cx<float> acc[RM][4];
+    int off[4], j0[4], ch[4], cc[4];
+    uint8_t let[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int nn = min(n0 + tx + 16 * j, ncol - 1);
+      ch[j] = nn / Dp;
+      cc[j] = nn - ch[j] * Dp;
+      let[j] = g.edge[c0 + ch[j]];
+      off[j] = (g.parent[c0 + ch[j]] - u0) * D * W + cc[j];
+      j0[j] = (let[j] == 1 || let[j] == 2) ? Dp : 0;   // X, Y swap the T_j
+#pragma unroll
+      for (int i = 0; i < RM; ++i) acc[i][j] = cx<float>(0.f, 0.f);
+    }
+    int bo[RM];
+#pragma unroll
+    for (int i = 0; i < RM; ++i) bo[i] = min(ty + 16 * i, Dp - 1);
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+#pragma unroll 2
+      for (int q = 0; q < D; ++q) {
+        Cx<float> a[RM], b[4];
+#pragma unroll
+        for (int i = 0; i < RM; ++i) a[i] = Bs[q * W + half * Dp + bo[i]];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) b[j] = Ts[off[j] + (half ? Dp - j0[j] : j0[j]) + q * W];
+#pragma unroll
+        for (int i = 0; i < RM; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) cmac_conj(acc[i][j], a[i], b[j]);
+      }
+      if (half == 0) {
+        // s0 / s1 = 1 for I and X, -1 for Y (-i, i) and Z (1, -1)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (let[j] >= 2) {
+#pragma unroll
+            for (int i = 0; i < RM; ++i) acc[i][j] = cx<float>(-acc[i][j].x, -acc[i][j].y);
+          }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (n0 + tx + 16 * j >= ncol) continue;
+      Cx<float>* o = Lout + (size_t)(c0 + ch[j] - g.c_lo) * Dp * Dp + cc[j];
+#pragma unroll
+      for (int i = 0; i < RM; ++i) {
+        const int r = ty + 16 * i;
+        if (r >= Dp) continue;
+        Cx<float> v = acc[i][j];
+        if (let[j] == 2) v = cx<float>(-v.y, v.x);       // s1 = i
+        if (let[j] == 3) v = cx<float>(-v.x, -v.y);      // s1 = -1
+        o[(size_t)r * Dp] = v;
+      }
+    }
+  }
+}
+
+// FP64: what a block does is bound by the FP64 pipe (two lanes a clock), so the operands
+// come through the tiled GEMM's staging; only T stays in shared memory.
+__global__ void __launch_bounds__(256) k_level_fused64(DevMPS m, LevelArgs g, const Cx<double>* Lin, Cx<double>* Lout) {
+  extern __shared__ __align__(256) unsigned char smem[];
+  const int* rank = m.rank + (size_t)g.slot * (m.n + 1);
+  const int D = rank[g.k], Dp = rank[g.k + 1], W = 2 * Dp;
+  const int P = max(1, 16 / D), u0 = g.u_lo + blockIdx.x * P, u1 = min(u0 + P, g.u_hi);
+  const int c0 = max(g.cb[u0], g.c_lo), c1 = min(g.cb[u1], g.c_hi);
+  if (c0 >= c1) return;
+  Cx<double>* Ts = (Cx<double>*)(smem + gate::gemm_tile_bytes<256>());   // [rows][2 D']
+  const Cx<double>* Bk = (const Cx<double>*)m.B + (size_t)g.slot * m.slot_elems + m.site_off[g.k];
+  const Cx<double>* Lu = Lin + (size_t)(u0 - g.node_base) * D * D;
+  const int rows = (u1 - u0) * D;
+  gate::tile_gemm<double, 256, false>(
+      rows, W, D, [&](int i, int q) { return Lu[i * D + q]; }, [&](int q, int j) { return Bk[q * W + j]; },
+      [&](int i, int j, Cx<double> v) { Ts[i * W + j] = v; }, smem);
+  const int32_t* par = g.parent + c0;
+  const uint8_t* ed = g.edge + c0;
+  gate::tile_gemm<double, 256, false>(
+      Dp, (c1 - c0) * Dp, 2 * D,
+      [&](int i, int q) {
+        const int h = q >= D;
+        return conj(Bk[(q - h * D) * W + h * Dp + i]);
+      },
+      [&](int q, int n) {
+        const int h = q >= D, ch = n / Dp, let = ed[ch];
+        const int jj = (let == 1 || let == 2) ? 1 - h : h;
+        const Cx<double> t = Ts[((par[ch] - u0) * D + q - h * D) * W + jj * Dp + n - ch * Dp];
+        if (let == 2) return h ? cx<double>(-t.y, t.x) : cx<double>(t.y, -t.x);   // i T_0, -i T_1
+        return let == 3 && h ? cx<double>(-t.x, -t.y) : t;
+      },
+      [&](int i, int n, Cx<double> v) {
+        const int ch = n / Dp;
+        Lout[((size_t)(c0 + ch - g.c_lo) * Dp + i) * Dp + n - ch * Dp] = v;
+      },
+      smem);
+}
+
+cudaError_t launch_level_fused(const DevMPS& m, int prec, int slot, int k, int D, int Dp, int u_lo, int u_hi,
+                               int node_base, int c_lo, int c_hi, const int32_t* cb, const int32_t* parent,
+                               const uint8_t* edge, const void* L, void* Lout, cudaStream_t st) {
+  if (c_lo >= c_hi) return cudaSuccess;
+  const LevelArgs g{slot, k, u_lo, u_hi, node_base, c_lo, c_hi, cb, parent, edge};
+  const int nu = u_hi - u_lo;
+  cudaError_t e;
+  if (prec == MPS_PREC_FP64) {
+    const int P = std::max(1, 16 / D), rows = std::min(nu, P) * D;
+    const size_t smem = gate::gemm_tile_bytes<256>() + sizeof(Cx<double>) * (size_t)rows * 2 * Dp;
+    if ((e = gate::raise_smem_limit<k_level_fused64>()) != cudaSuccess) return e;
+    k_level_fused64<<<(nu + P - 1) / P, 256, smem, st>>>(m, g, (const Cx<double>*)L, (Cx<double>*)Lout);
+    return cudaGetLastError();
+  }
+  const int P = std::max(1, 64 / D);
+  const size_t smem = sizeof(Cx<float>) * ((size_t)D * 2 * Dp + 64 * (size_t)(D + 1) + 64 * (size_t)2 * Dp);
+  auto go = [&](auto dp) {
+    constexpr auto kern = k_level_fused<decltype(dp)::value>;
+    cudaError_t r = gate::raise_smem_limit<kern>();
+    if (r != cudaSuccess) return r;
+    kern<<<(nu + P - 1) / P, 256, smem, st>>>(m, g, (const Cx<float>*)L, (Cx<float>*)Lout);
+    return cudaGetLastError();
+  };
+  if (Dp <= 8) return go(std::integral_constant<int, 8>{});
+  if (Dp <= 16) return go(std::integral_constant<int, 16>{});
+  if (Dp <= 32) return go(std::integral_constant<int, 32>{});
+  return go(std::integral_constant<int, 64>{});
 }
 
 // <P> (unnormalised) of a string closing at site k with letter P on node u:
@@ -333,12 +637,12 @@ __global__ void __launch_bounds__(256) k_level_close(DevMPS m, int slot, int k, 
 }
 
 cudaError_t launch_env_T(const DevMPS& m, int prec, int slot, int k, const void* L, void* T, int n_nodes,
-                         cudaStream_t st) {
+                         const int32_t* cb, cudaStream_t st) {
   if (n_nodes <= 0) return cudaSuccess;
   if (prec == MPS_PREC_FP64)
-    k_level_T<double><<<dim3(n_nodes, 2), 256, 0, st>>>(m, slot, k, (const Cx<double>*)L, (Cx<double>*)T);
+    k_level_T<double><<<dim3(n_nodes, 2), 256, 0, st>>>(m, slot, k, (const Cx<double>*)L, (Cx<double>*)T, cb);
   else
-    k_level_T<float><<<dim3(n_nodes, 2), 256, 0, st>>>(m, slot, k, (const Cx<float>*)L, (Cx<float>*)T);
+    k_level_T<float><<<dim3(n_nodes, 2), 256, 0, st>>>(m, slot, k, (const Cx<float>*)L, (Cx<float>*)T, cb);
   return cudaGetLastError();
 }
 
@@ -368,6 +672,11 @@ cudaError_t launch_env_child(const DevMPS& m, int prec, int slot, int k, const v
 }
 
 // ------------------------------------------------------------------ energy sum
+// E = sum_i a_i <P_i> in FP64, compensated throughout: each thread runs a Neumaier sum over
+// its terms, pairs (sum, correction) are then merged by TwoSum in a fixed tree. A block
+// covers 256 threads x kTermsPerThread terms; the block that finishes last merges the
+// blocks' pairs in block order, so the result does not depend on the schedule.
+constexpr int kTermsPerThread = 4;
 __device__ __forceinline__ void neumaier_add(double& s, double& c, double v) {
   const double t = s + v;
   if (fabs(s) >= fabs(v))
@@ -376,54 +685,91 @@ __device__ __forceinline__ void neumaier_add(double& s, double& c, double v) {
     c += (v - t) + s;
   s = t;
 }
+__device__ __forceinline__ void merge_pair(double& s, double& c, double s2, double c2) {
+  const double t = s + s2, b = t - s;
+  c = (c + c2) + ((s - (t - b)) + (s2 - b));
+  s = t;
+}
+// The sum over a block's threads, in thread 0.
+__device__ __forceinline__ void block_merge(double& s, double& c, double (*sh)[2]) {
+  for (int o = 1; o < 32; o <<= 1) {
+    const double s2 = __shfl_down_sync(0xffffffffu, s, o), c2 = __shfl_down_sync(0xffffffffu, c, o);
+    merge_pair(s, c, s2, c2);
+  }
+  const int warp = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    sh[warp][0] = s;
+    sh[warp][1] = c;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int w = 1; w < 8; ++w) merge_pair(s, c, sh[w][0], sh[w][1]);
+}
 
 template <class R>
-__global__ void __launch_bounds__(1024) k_energy_sum(int64_t n_terms, const double* coeff, const double* vals,
-                                                     const Cx<R>* R0, double id_coeff, int64_t id_term,
-                                                     double* out) {
-  __shared__ double ps[1024], pc[1024];
+__global__ void __launch_bounds__(256) k_energy_sum(int64_t n_terms, const double* coeff, const double* vals,
+                                                    const Cx<R>* R0, double id_coeff, int64_t id_term, double* part,
+                                                    unsigned* done, double* out) {
+  __shared__ double sh[8][2];
+  __shared__ bool last;
   const double norm = (double)R0[0].x;
-  const int64_t chunk = (n_terms + 1023) / 1024;
-  const int64_t b = (int64_t)threadIdx.x * chunk, e = min(n_terms, b + chunk);
+  const double2* v2 = reinterpret_cast<const double2*>(vals);
+  double2* o2 = reinterpret_cast<double2*>(out + 4);
   double s = 0.0, c = 0.0;
-  for (int64_t t = b; t < e; ++t) {
-    double re, im;
-    if (t == id_term) {
-      re = 1.0;
-      im = 0.0;
-    } else {
-      re = vals[2 * t] / norm;
-      im = vals[2 * t + 1] / norm;
-      neumaier_add(s, c, coeff[t] * re);
+#pragma unroll
+  for (int i = 0; i < kTermsPerThread; ++i) {
+    const int64_t t = ((int64_t)blockIdx.x * kTermsPerThread + i) * 256 + threadIdx.x;
+    if (t < n_terms) {
+      double2 v = make_double2(1.0, 0.0);
+      if (t != id_term) {
+        v = v2[t];
+        v.x /= norm;
+        v.y /= norm;
+        neumaier_add(s, c, coeff[t] * v.x);
+      }
+      o2[t] = v;
     }
-    out[4 + 2 * t] = re;
-    out[5 + 2 * t] = im;
   }
-  ps[threadIdx.x] = s;
-  pc[threadIdx.x] = c;
-  __syncthreads();
+  block_merge(s, c, sh);
   if (threadIdx.x == 0) {
-    double S = 0.0, Cc = 0.0;
-    for (int i = 0; i < 1024; ++i) {
-      neumaier_add(S, Cc, ps[i]);
-      neumaier_add(S, Cc, pc[i]);
-    }
-    neumaier_add(S, Cc, id_coeff);
-    out[0] = S + Cc;
+    part[2 * blockIdx.x] = s;
+    part[2 * blockIdx.x + 1] = c;
+    __threadfence();
+    last = atomicAdd(done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  s = c = 0.0;
+  const int per = (gridDim.x + 255) / 256;
+  for (int i = 0; i < per; ++i) {
+    const unsigned b = threadIdx.x * per + i;
+    if (b < gridDim.x) merge_pair(s, c, __ldcg(part + 2 * b), __ldcg(part + 2 * b + 1));
+  }
+  __syncthreads();
+  block_merge(s, c, sh);
+  if (threadIdx.x == 0) {
+    neumaier_add(s, c, id_coeff);
+    out[0] = s + c;
     out[1] = norm;
+    *done = 0;   // ready for the next measurement of this handle
   }
 }
 
-cudaError_t launch_energy_sum(const DevMPS& m, int prec, int slot, MeasDev& w, int64_t n_terms,
-                              const double* coeff_dev, double id_coeff, int64_t id_term, cudaStream_t st) {
-  (void)m;
-  (void)slot;
+int64_t energy_sum_blocks(int64_t n_terms) {
+  const int64_t per = 256 * kTermsPerThread;
+  return n_terms > 0 ? (n_terms + per - 1) / per : 1;
+}
+
+cudaError_t launch_energy_sum(int prec, MeasDev& w, int64_t n_terms, const double* coeff_dev, double id_coeff,
+                              int64_t id_term, cudaStream_t st) {
+  const unsigned grid = (unsigned)energy_sum_blocks(n_terms);
   if (prec == MPS_PREC_FP64)
-    k_energy_sum<double><<<1, 1024, 0, st>>>(n_terms, coeff_dev, w.vals, (const Cx<double>*)w.R, id_coeff,
-                                             id_term, w.out);
+    k_energy_sum<double><<<grid, 256, 0, st>>>(n_terms, coeff_dev, w.vals, (const Cx<double>*)w.R, id_coeff, id_term,
+                                               w.part, w.done, w.out);
   else
-    k_energy_sum<float><<<1, 1024, 0, st>>>(n_terms, coeff_dev, w.vals, (const Cx<float>*)w.R, id_coeff,
-                                            id_term, w.out);
+    k_energy_sum<float><<<grid, 256, 0, st>>>(n_terms, coeff_dev, w.vals, (const Cx<float>*)w.R, id_coeff, id_term,
+                                              w.part, w.done, w.out);
   return cudaGetLastError();
 }
 

@@ -64,31 +64,39 @@ struct MeasDev {
   void* Q;          // complex<R> [n][4][chi*chi]: Q_k^P = sum_ij conj(P_ij) Bhat_k^i (B_k^j)^+ per letter P
   double* vals;     // [n_terms][2] re, im of unnormalised <P>
   double* out;      // [4 + n_terms*2]: E, norm, ...
+  double* part;     // [energy_sum_blocks][2]: (sum, correction) per block of the energy sum
+  unsigned* done;   // blocks of the energy sum that have finished (zero between calls)
 };
 
 
 // Thread-local message returned by mps_last_error() (defined with the C ABI).
 void set_error_message(const char* msg);
 
-// ranks: the slot's n+1 bond ranks on the host (ranks[k] = left dimension of site k);
-// site_off: the n site offsets on the host (DevMPS::site_off is the device copy).
-cudaError_t launch_right_envs(const DevMPS& m, int prec, int slot, const int* ranks, const int64_t* site_off,
-                              MeasDev& w, cudaStream_t st, int* launches);
+// ranks: the slot's n+1 bond ranks on the host (ranks[k] = left dimension of site k).
+cudaError_t launch_right_envs(const DevMPS& m, int prec, int slot, const int* ranks, MeasDev& w, cudaStream_t st,
+                              int* launches);
 // Chunked trie levels. Environment buffers: L holds node u's D_k x D_k block (row-major,
 // leading dimension D_k) at u chi^2 complex entries; T holds T_j[u] = L[u] B_k^j
 // (D_k x D_{k+1}, leading dimension D_{k+1}) at (2u + j) chi^2. Node indices in cnode /
 // parent are absolute trie indices; node_base is the trie index of buffer entry 0.
+// cb: first child of each of the n_nodes nodes (nodes without children are left out).
 cudaError_t launch_env_T(const DevMPS& m, int prec, int slot, int k, const void* L, void* T, int n_nodes,
-                         cudaStream_t st);
+                         const int32_t* cb, cudaStream_t st);
+// A level whose bonds are both <= kFusedMax: T in shared memory, children [c_lo, c_hi) of
+// parents [u_lo, u_hi) (trie indices; cb[u] = first child of node u) into Lout.
+constexpr int kFusedMax = 64;
+cudaError_t launch_level_fused(const DevMPS& m, int prec, int slot, int k, int D, int Dp, int u_lo, int u_hi,
+                               int node_base, int c_lo, int c_hi, const int32_t* cb, const int32_t* parent,
+                               const uint8_t* edge, const void* L, void* Lout, cudaStream_t st);
 cudaError_t launch_env_close(const DevMPS& m, int prec, int slot, int k, const void* L, const void* Q,
                              const int32_t* cnode, const uint8_t* cletter, const int32_t* cterm, int n_closes,
                              int node_base, double* vals, cudaStream_t st);
 cudaError_t launch_env_child(const DevMPS& m, int prec, int slot, int k, const void* T, const int32_t* parent,
                              const uint8_t* edge, int n_children, int node_base, void* Lout, cudaStream_t st);
-// E = sum_t coeff_t Re(vals_t) / norm + id_coeff (Neumaier, fixed order); also writes
+// E = sum_t coeff_t Re(vals_t) / norm + id_coeff (compensated, fixed order); also writes
 // normalised <P_t> to out[4 + 2t], out[0] = E, out[1] = norm.
-cudaError_t launch_energy_sum(const DevMPS& m, int prec, int slot, MeasDev& w, int64_t n_terms,
-                              const double* coeff_dev, double id_coeff, int64_t id_term,
-                              cudaStream_t st);
+int64_t energy_sum_blocks(int64_t n_terms);
+cudaError_t launch_energy_sum(int prec, MeasDev& w, int64_t n_terms, const double* coeff_dev, double id_coeff,
+                              int64_t id_term, cudaStream_t st);
 
 }  // namespace mpsvqe

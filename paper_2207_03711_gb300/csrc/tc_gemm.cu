@@ -30,7 +30,9 @@
 //                   registers, bounds-checked stores of C
 //   warps 10..13    split each loaded stage in shared memory: hi over the loaded tile,
 //                   lo beside it (same swizzled offsets), then a proxy fence so the
-//                   tensor core sees the stores
+//                   tensor core sees the stores. An operand that all tiles share comes
+//                   split already, as two planes, which halves this work and takes 32 KB
+//                   of the 224 KB that a K tile moves through shared memory
 // The pipeline counters run on across a CTA's tiles, so the loads and MMAs of the next
 // tile overlap the epilogue of the previous one. Every mbarrier wait is bounded: a wait
 // that runs out records an error code in *err, and the kernel still passes its final
@@ -45,6 +47,7 @@
 #include <algorithm>
 
 #include "kernels.cuh"
+#include "smem_limit.cuh"
 #include "tc_gemm.cuh"
 
 namespace mpsvqe {
@@ -56,7 +59,7 @@ constexpr int TILE_A = BM * BK * 4;                   // 16 KB
 constexpr int TILE_B = BN * BK * 4;                   // 16 KB
 constexpr int STAGE_BYTES = 2 * TILE_A + 2 * TILE_B;  // hi and lo of both operands: 64 KB
 constexpr int NBARS = 3 * STAGES + 4;                 // full, split, empty per stage; ready, free per buffer
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 8 * NBARS + 16;
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 8 * NBARS + 16 + 4 * STAGES;
 constexpr int NTHREADS = 448;
 constexpr int NEPI = 256;                             // epilogue threads (warps 2..9)
 constexpr int EPI_COLS = BN / 2;                      // columns per epilogue thread
@@ -178,9 +181,36 @@ __device__ __forceinline__ float tf32_rna(float v) {
   return __uint_as_float(b);
 }
 
+// What a K tile of the second operand is, and where the product goes.
+//   kPlain     rows n0.. of B; C row-major (optionally with the columns of each group of
+//              cmod spread to a stride of cpad, the gap written as zeros)
+//   kChildren  environments of trie children (env_tc.cu): B is T^T, the rows (j, re/im, c) of
+//              T_j over columns (node, a), leading dimension tdn per node. Column tile
+//              (child, c0) at inner index (i, re/im, a) is the box of T^T at the child's
+//              parent and (j, re/im') with a sign, which its letter gives; rows of the product
+//              are (c', re/im) and go to L[child][c'][c] as complex entries.
+enum Mode { kPlain, kChildren };
+struct Children {
+  const int32_t* parent = nullptr;
+  const uint8_t* edge = nullptr;
+  int node_base = 0, nc = 0, Dp = 0, tdn = 0, seg_tiles = 0;
+  Cx<float>* L = nullptr;
+};
+// Letter l, inner segment seg = 2 i + re/im of W_i = sum_j P_ij T_j (I: (T_0, T_1); X: (T_1,
+// T_0); Y: (-i T_1, i T_0); Z: (T_0, -T_1)) -> row block 2 j + re/im' of T^T and the sign.
+__device__ __forceinline__ int child_block(int l, int seg, float* sign) {
+  const int i = seg >> 1, ri = seg & 1;
+  *sign = (l == 2 && i != ri) || (l == 3 && i == 1) ? -1.f : 1.f;
+  // Y: Re(-i t) = Im t, Im(-i t) = -Re t; Re(i t) = -Im t, Im(i t) = Re t
+  return l == 0 || l == 3 ? seg : l == 1 ? 2 * (1 - i) + ri : 2 * (1 - i) + (1 - ri);
+}
+
+// PRE: A comes already split (planes hi and lo), as the operands do that all tiles share.
+template <bool PRE, Mode MODE>
 __global__ void __launch_bounds__(NTHREADS, 1)
-    k_gemm_tf32x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, float* C,
-                  int64_t ldc, int M, int N, int K, int* err) {
+    k_gemm_tf32x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmAl,
+                  const __grid_constant__ CUtensorMap tmB, float* C, int64_t ldc, int M, int N, int K, int cmod,
+                  int cpad, const __grid_constant__ Children chd, int* err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   // barriers: full[s] (TMA), split[s] (hi/lo written), empty[s] (MMAs done), ready[b], freed[b]
@@ -191,9 +221,23 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   uint64_t* ready = bars + 3 * STAGES;
   uint64_t* freed = bars + 3 * STAGES + 2;
   uint32_t* tmem_slot = (uint32_t*)(bars + NBARS);
+  float* sgn = (float*)(tmem_slot + 4);   // sign of the B tile in each stage
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nk = (K + BK - 1) / BK;
-  const int tiles_n = (N + BN - 1) / BN, tiles = tiles_n * ((M + BM - 1) / BM);
+  const int tiles_m = (M + BM - 1) / BM;
+  const int tiles_n = MODE == kPlain ? (N + BN - 1) / BN : chd.nc * ((chd.Dp + BN - 1) / BN);
+  const int tiles = tiles_n * tiles_m;
+  // plain: A may be the long side, columns vary fastest; children: rows do, so that CTAs
+  // side by side share a child's tile
+  auto tile_at = [&](int tile, int* mt, int* nt) {
+    if (MODE == kPlain) {
+      *mt = tile / tiles_n;
+      *nt = tile % tiles_n;
+    } else {
+      *nt = tile / tiles_m;
+      *mt = tile % tiles_m;
+    }
+  };
   // persistent: this CTA takes tiles blockIdx.x, blockIdx.x + gridDim.x, ...; the
   // pipeline counters (stage and accumulator phases) run on across its tiles
   const int my_tiles = blockIdx.x < tiles ? (tiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
@@ -216,14 +260,23 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0 && lane == 0) {
-    // ---- TMA producer: the FP32 tiles of A and B, into the hi slots of the stage
+    // ---- TMA producer: the FP32 tiles of A and B into the hi slots of the stage (A
+    // already split: both planes)
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
     int g = 0;
     bool ok = true;
     for (int n = 0; n < my_tiles && ok; ++n) {
-      const int tile = blockIdx.x + n * gridDim.x;
-      const int m0 = (tile / tiles_n) * BM, n0 = (tile % tiles_n) * BN;
+      int mt, nt;
+      tile_at(blockIdx.x + n * gridDim.x, &mt, &nt);
+      const int m0 = mt * BM;
+      int letter = 0, x0 = 0, y0 = nt * BN;
+      if (MODE == kChildren) {
+        const int per = (chd.Dp + BN - 1) / BN, ch = nt / per;
+        letter = chd.edge[ch];
+        x0 = (chd.parent[ch] - chd.node_base) * chd.tdn;
+        y0 = (nt - ch * per) * BN;
+      }
       for (int kt = 0; kt < nk; ++kt, ++g) {
         const int s = g % STAGES;
         if (g >= STAGES && !mbar_wait(smem_u32(&empty[s]), ((g / STAGES) & 1) ^ 1, err, 1)) {
@@ -232,9 +285,18 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         }
         unsigned char* st = base + s * STAGE_BYTES;
         const uint32_t fb = smem_u32(&full[s]);
-        mbar_arrive_expect_tx(fb, TILE_A + TILE_B);
+        int x = kt * BK, y = y0;
+        if (MODE == kChildren) {
+          const int seg = kt / chd.seg_tiles;
+          x = x0 + (kt - seg * chd.seg_tiles) * BK;
+          float sg;
+          y = child_block(letter, seg, &sg) * chd.Dp + y0;
+          sgn[s] = sg;   // released by the arrival below
+        }
+        mbar_arrive_expect_tx(fb, (PRE ? 2 : 1) * TILE_A + TILE_B);
         tma_load_2d(smem_u32(st), &tmA, kt * BK, m0, fb);
-        tma_load_2d(smem_u32(st + 2 * TILE_A), &tmB, kt * BK, n0, fb);
+        if (PRE) tma_load_2d(smem_u32(st + TILE_A), &tmAl, kt * BK, m0, fb);
+        tma_load_2d(smem_u32(st + 2 * TILE_A), &tmB, x, y, fb);
       }
     }
     // no copy may still be landing in shared memory when the CTA exits: wait (bounded)
@@ -265,8 +327,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       float4* al = (float4*)(st + TILE_A);
       float4* bh = (float4*)(st + 2 * TILE_A);
       float4* bl = (float4*)(st + 2 * TILE_A + TILE_B);
+      const float sg = MODE == kChildren ? sgn[s] : 1.f;
 #pragma unroll 4
-      for (int v = ct; v < TILE_A / 16; v += NCONV) {
+      for (int v = ct; v < (PRE ? 0 : TILE_A / 16); v += NCONV) {
         const float4 x = ah[v];
         float4 h, l;
         h.x = tf32_rna(x.x); l.x = tf32_rna(x.x - h.x);
@@ -278,7 +341,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       }
 #pragma unroll 4
       for (int v = ct; v < TILE_B / 16; v += NCONV) {
-        const float4 x = bh[v];
+        float4 x = bh[v];
+        if (MODE == kChildren) x = make_float4(sg * x.x, sg * x.y, sg * x.z, sg * x.w);
         float4 h, l;
         h.x = tf32_rna(x.x); l.x = tf32_rna(x.x - h.x);
         h.y = tf32_rna(x.y); l.y = tf32_rna(x.y - h.y);
@@ -302,6 +366,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t st = smem_u32(base + s * STAGE_BYTES);
       const uint32_t acc = tmem + (uint32_t)(b * BN);
+      // the two products with a low part first: the accumulator is 2^-11 times smaller then,
+      // and so is what its truncation takes; four truncations at full size are left per
+      // tile instead of twelve
 #pragma unroll
       for (int ks = 0; ks < BK / 8; ++ks) {
         // K step of 8 TF32 = 32 bytes inside each 128-byte swizzled row
@@ -309,10 +376,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const uint64_t al = sw128_kmajor_desc(st + TILE_A + ks * 32);
         const uint64_t bh = sw128_kmajor_desc(st + 2 * TILE_A + ks * 32);
         const uint64_t bl = sw128_kmajor_desc(st + 2 * TILE_A + TILE_B + ks * 32);
-        mma_tf32(acc, ah, bh, idesc, ks > 0 ? 1u : 0u);
-        mma_tf32(acc, ah, bl, idesc, 1u);
+        mma_tf32(acc, ah, bl, idesc, ks > 0 ? 1u : 0u);
         mma_tf32(acc, al, bh, idesc, 1u);
       }
+#pragma unroll
+      for (int ks = 0; ks < BK / 8; ++ks)
+        mma_tf32(acc, sw128_kmajor_desc(st + ks * 32), sw128_kmajor_desc(st + 2 * TILE_A + ks * 32), idesc, 1u);
       mma_commit(smem_u32(&empty[s]));   // stage s free once these finish
       mma_commit(smem_u32(&ready[b]));   // K tile g complete in accumulator b
     }
@@ -325,8 +394,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     bool ok = true;
     int g = 0;
     for (int n = 0; n < my_tiles && ok; ++n) {
-      const int tile = blockIdx.x + n * gridDim.x;
-      const int m0 = (tile / tiles_n) * BM, n0 = (tile % tiles_n) * BN + c_lo;
+      int mt, nt;
+      tile_at(blockIdx.x + n * gridDim.x, &mt, &nt);
+      const int m0 = mt * BM, n0 = nt * BN + c_lo;
       float sum[EPI_COLS];
 #pragma unroll
       for (int c = 0; c < EPI_COLS; ++c) sum[c] = 0.f;
@@ -348,16 +418,57 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         mbar_arrive(smem_u32(&freed[b]));
       }
       const int row = m0 + q * 32 + lane;
-      if (ok && row < M) {
-        float* out = C + (size_t)row * ldc + n0;
-        if (vec && n0 + EPI_COLS <= N) {
+      if (MODE == kChildren) {
+        // lanes 2x and 2x + 1 hold the real and imaginary rows of one c': each takes half of
+        // the columns of both
+        const int per = (chd.Dp + BN - 1) / BN, ch = nt / per, cc = (nt - ch * per) * BN + c_lo;
+        const bool odd = lane & 1;
+        Cx<float> z[EPI_COLS / 2];
 #pragma unroll
-          for (int c = 0; c < EPI_COLS; c += 4)
-            *reinterpret_cast<float4*>(out + c) = make_float4(sum[c], sum[c + 1], sum[c + 2], sum[c + 3]);
+        for (int c = 0; c < EPI_COLS / 2; ++c) {
+          const float mine = odd ? sum[c + EPI_COLS / 2] : sum[c];
+          const float got = __shfl_xor_sync(0xffffffffu, odd ? sum[c] : sum[c + EPI_COLS / 2], 1);
+          z[c] = odd ? cx<float>(got, mine) : cx<float>(mine, got);
+        }
+        if (ok && row < M) {
+          const int c0 = cc + (odd ? EPI_COLS / 2 : 0);
+          Cx<float>* out = chd.L + ((size_t)ch * chd.Dp + (row >> 1)) * chd.Dp + c0;
+          if ((chd.Dp & 1) == 0 && c0 + EPI_COLS / 2 <= chd.Dp) {
+#pragma unroll
+            for (int c = 0; c < EPI_COLS / 2; c += 2)
+              *reinterpret_cast<float4*>(out + c) = make_float4(z[c].x, z[c].y, z[c + 1].x, z[c + 1].y);
+          } else {
+#pragma unroll
+            for (int c = 0; c < EPI_COLS / 2; ++c)
+              if (c0 + c < chd.Dp) out[c] = z[c];
+          }
+        }
+      } else if (ok && row < M) {
+        if (cmod) {
+          int u = n0 / cmod, x = n0 - u * cmod;
+          float* out = C + (size_t)row * ldc + (size_t)u * cpad;
+#pragma unroll
+          for (int c = 0; c < EPI_COLS; ++c) {
+            if (n0 + c < N) {
+              out[x] = sum[c];
+              if (++x == cmod) {
+                for (; x < cpad; ++x) out[x] = 0.f;
+                x = 0;
+                out += cpad;
+              }
+            }
+          }
         } else {
+          float* out = C + (size_t)row * ldc + n0;
+          if (vec && n0 + EPI_COLS <= N) {
 #pragma unroll
-          for (int c = 0; c < EPI_COLS; ++c)
-            if (n0 + c < N) out[c] = sum[c];
+            for (int c = 0; c < EPI_COLS; c += 4)
+              *reinterpret_cast<float4*>(out + c) = make_float4(sum[c], sum[c + 1], sum[c + 2], sum[c + 3]);
+          } else {
+#pragma unroll
+            for (int c = 0; c < EPI_COLS; ++c)
+              if (n0 + c < N) out[c] = sum[c];
+          }
         }
       }
     }
@@ -423,31 +534,54 @@ cudaError_t launch_pad_rows(const float* x, int64_t ld_in, int M, int K, float* 
   return cudaGetLastError();
 }
 
-cudaError_t launch_gemm_tf32x3(const Plane& A, const Plane& B, int M, int N, int K, float* C, int64_t ldc, int* err,
-                               cudaStream_t st) {
+template <bool PRE, Mode MODE>
+static cudaError_t launch(const Plane& A, const float* a_lo, const Plane& B, int M, int N, int K, int b_rows, int b_cols,
+                          float* C, int64_t ldc, int cmod, int cpad, const Children& chd, int* err, cudaStream_t st) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  if ((A.ld & 3) || (B.ld & 3) || ((uintptr_t)A.p & 15) || ((uintptr_t)B.p & 15)) return cudaErrorInvalidValue;
-  CUtensorMap am, bm;
+  if ((A.ld & 3) || (B.ld & 3) || ((uintptr_t)A.p & 15) || ((uintptr_t)B.p & 15) || ((uintptr_t)a_lo & 15))
+    return cudaErrorInvalidValue;
+  CUtensorMap am, al, bm;
   cudaError_t e;
   if ((e = make_map(&am, A.p, M, K, A.ld, BM)) != cudaSuccess) return e;
-  if ((e = make_map(&bm, B.p, N, K, B.ld, BN)) != cudaSuccess) return e;
-  static std::once_flag once[64];
-  static cudaError_t attr[64];
+  if ((e = make_map(&al, PRE ? a_lo : A.p, M, K, A.ld, BM)) != cudaSuccess) return e;
+  if ((e = make_map(&bm, B.p, b_rows, b_cols, B.ld, BN)) != cudaSuccess) return e;
+  if ((e = gate::raise_smem_limit<k_gemm_tf32x3<PRE, MODE>>()) != cudaSuccess) return e;
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  std::call_once(once[dev], [dev] {
-    attr[dev] = cudaFuncSetAttribute(k_gemm_tf32x3, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-  });
-  if (attr[dev] != cudaSuccess) return attr[dev];
   // persistent grid: one CTA per SM at most (197 KB of shared memory each)
   static int sm_count[64] = {0};
   if (!sm_count[dev] && (e = cudaDeviceGetAttribute(&sm_count[dev], cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
     return e;
-  const int64_t tiles = (int64_t)((N + BN - 1) / BN) * ((M + BM - 1) / BM);
+  const int64_t tiles = (int64_t)(MODE == kPlain ? (N + BN - 1) / BN : chd.nc * ((chd.Dp + BN - 1) / BN)) * ((M + BM - 1) / BM);
   const int grid = (int)std::min<int64_t>(tiles, sm_count[dev]);
-  k_gemm_tf32x3<<<grid, NTHREADS, SMEM_BYTES, st>>>(am, bm, C, ldc, M, N, K, err);
+  k_gemm_tf32x3<PRE, MODE><<<grid, NTHREADS, SMEM_BYTES, st>>>(am, al, bm, C, ldc, M, N, K, cmod, cpad, chd, err);
   return cudaGetLastError();
+}
+
+cudaError_t launch_gemm_tf32x3(const Plane& A, const Plane& B, int M, int N, int K, float* C, int64_t ldc, int* err,
+                               cudaStream_t st) {
+  return launch<false, kPlain>(A, nullptr, B, M, N, K, N, K, C, ldc, 0, 0, Children{}, err, st);
+}
+
+cudaError_t launch_gemm_presplit(const Plane& A, const float* a_lo, const Plane& B, int M, int N, int K, float* C,
+                                 int64_t ldc, int cmod, int cpad, int* err, cudaStream_t st) {
+  return launch<true, kPlain>(A, a_lo, B, M, N, K, N, K, C, ldc, cmod == cpad ? 0 : cmod, cpad, Children{}, err, st);
+}
+
+cudaError_t launch_gemm_children(const Plane& A, const float* a_lo, const Plane& Tt, int U, int D, int Dn, int Dp,
+                                 const int32_t* parent, const uint8_t* edge, int node_base, int nc, Cx<float>* L,
+                                 int* err, cudaStream_t st) {
+  Children chd;
+  chd.parent = parent;
+  chd.edge = edge;
+  chd.node_base = node_base;
+  chd.nc = nc;
+  chd.Dp = Dp;
+  chd.tdn = Dn;
+  chd.seg_tiles = (D + BK - 1) / BK;
+  chd.L = L;
+  return launch<true, kChildren>(A, a_lo, Tt, 2 * Dp, nc * Dp, 4 * chd.seg_tiles * BK, 4 * Dp, U * Dn, nullptr, 0, 0, 0,
+                                 chd, err, st);
 }
 
 }  // namespace tc

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 
+#include "cx.cuh"
+
 namespace mpsvqe {
 namespace tc {
 
@@ -26,6 +28,20 @@ cudaError_t launch_pad_rows(const float* x, int64_t ld_in, int M, int K, float* 
 // misaligned planes.
 cudaError_t launch_gemm_tf32x3(const Plane& A, const Plane& B, int M, int N, int K, float* C, int64_t ldc, int* err,
                                cudaStream_t st);
+
+
+// The same with A given as hi plane A and lo plane a_lo (same leading dimension). C's
+// columns of each group of cmod may be spread to a stride of cpad (gaps become zeros).
+cudaError_t launch_gemm_presplit(const Plane& A, const float* a_lo, const Plane& B, int M, int N, int K, float* C,
+                                 int64_t ldc, int cmod, int cpad, int* err, cudaStream_t st);
+
+// Environments of nc trie children: L[child][c'][c] = sum over (i, a) of conj(B^i[a][c'])
+// W_i[a][c], W_i = sum_j P_ij T_j[parent]. A, a_lo: planes of 2 Dp rows (c', re/im) over
+// inner indices (i, re/im, a), a padded with zeros to a multiple of 32; Tt: T^T, rows
+// (j, re/im, c) over columns (node, a) of U nodes at a stride of Dn >= D (a multiple of 4).
+cudaError_t launch_gemm_children(const Plane& A, const float* a_lo, const Plane& Tt, int U, int D, int Dn, int Dp,
+                                 const int32_t* parent, const uint8_t* edge, int node_base, int nc, Cx<float>* L,
+                                 int* err, cudaStream_t st);
 
 }  // namespace tc
 }  // namespace mpsvqe
