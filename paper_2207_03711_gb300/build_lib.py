@@ -1,8 +1,9 @@
 """Build the in-tree CUDA library libmpsvqe.so for sm_103a (GB300).
 
-Six translation units compiled in parallel (host.cpp with g++; gate.cu, kernels.cu,
-api.cu, tc_gemm.cu and env_tc.cu with nvcc), linked with nvcc into paper_2207_03711_gb300/libmpsvqe.so.
-The CUDA runtime is linked statically, so the library only needs the driver.
+host.cpp with g++ and the .cu files with nvcc, all in parallel (the gate engine's
+instances are spread over several files for that), linked with nvcc into
+paper_2207_03711_gb300/libmpsvqe.so. The CUDA runtime is linked statically, so the library
+only needs the driver.
 """
 import os
 import shutil
@@ -46,7 +47,9 @@ def build(force=False, verbose=False):
          os.path.join(CSRC, "host.cpp"),
          "-o", os.path.join(OBJ, "host.o")],
     ]
-    for name in ("gate", "kernels", "api", "tc_gemm", "env_tc"):
+    units = ("gate_fp64", "gate_mixed1", "gate_mixed2", "gate_mixed8", "gate_raw", "gate", "kernels", "api", "tc_gemm",
+             "env_tc")
+    for name in units:
         jobs.append([nvcc, *ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", *inc,
                      "-c", os.path.join(CSRC, name + ".cu"), "-o", os.path.join(OBJ, name + ".o")])
     with ThreadPoolExecutor(len(jobs)) as ex:
@@ -55,9 +58,8 @@ def build(force=False, verbose=False):
         for o in outs:
             sys.stdout.write(o)
     tmp = LIB + ".tmp"
-    _run([nvcc, *ARCH, "-shared", "-o", tmp, os.path.join(OBJ, "host.o"), os.path.join(OBJ, "gate.o"), os.path.join(OBJ, "kernels.o"),
-          os.path.join(OBJ, "api.o"), os.path.join(OBJ, "tc_gemm.o"),
-          os.path.join(OBJ, "env_tc.o"), "-lpthread"])
+    objs = [os.path.join(OBJ, name + ".o") for name in ("host",) + units]
+    _run([nvcc, *ARCH, "-shared", "-o", tmp, *objs, "-lpthread"])
     os.replace(tmp, LIB)
     return LIB
 

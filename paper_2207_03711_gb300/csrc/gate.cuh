@@ -23,7 +23,7 @@ namespace mpsvqe {
 namespace gate {
 
 // -------------------------------------------------------------------- bidiagonalisation
-// T = Q B P^H (LAPACK reflector conventions) with a single cluster barrier per
+// T = Q B P^H (LAPACK reflector conventions) with one exposed cluster barrier per
 // step: the updates by right reflector k-1 and left reflector k go over the trailing
 // columns together, the next row comes out of that pass, and the product z with the next
 // right reflector is formed from the unscaled row (its norm, hence its scale, is known one
@@ -56,8 +56,7 @@ __device__ __forceinline__ void root_and_inverse(double x, double* root, double*
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-x * y, y, 1.0);
   y = fma(y * e, fma(0.375, e, 0.5), y);
-  const double r = x * y;
-  *root = fma(0.5 * y, fma(-r, r, x), r);
+  *root = x * y;
   *inv = y;
 }
 __device__ __forceinline__ float inverse(float d) {
@@ -82,12 +81,13 @@ __device__ __forceinline__ void reflector(Cx<R> alpha, R xn2, Cx<R>* tau, R* bet
   }
   R nrm, inv;
   root_and_inverse(n2, &nrm, &inv);
+  // |alpha - beta|^2 = |alpha|^2 + nrm^2 + 2 |Re alpha| nrm, without waiting for alpha - beta
+  const R ax = alpha.x >= R(0) ? alpha.x : -alpha.x;
+  const R rd = inverse(fma(R(2) * ax, nrm, R(2) * n2 - xn2));
   const R b = alpha.x >= R(0) ? -nrm : nrm, rb = alpha.x >= R(0) ? -inv : inv;
   *beta = b;
   *tau = cx<R>((b - alpha.x) * rb, -alpha.y * rb);
-  const Cx<R> den = cx<R>(alpha.x - b, alpha.y);
-  const R rd = inverse(norm2(den));
-  *scale = cx<R>(den.x * rd, -den.y * rd);
+  *scale = cx<R>((alpha.x - b) * rd, -alpha.y * rd);
 }
 
 // Per own column: left factor, pending and new row entry (the pending right update uses
@@ -102,13 +102,12 @@ struct Bidiag {
   Cx<R>* T;            // own columns, leading dimension ld (>= r)
   int ld;
   int zrows;
-  Cx<R>* zp;           // [2][C][gmax][zrows] z partials
+  Cx<R>* zp;           // [2][C VG][zrows] z partials, one per virtual rank
   Cx<R>* colp;         // [2][zrows] next column before its right update
-  Cx<R>* sc;           // [0..1] row entry of the next column, [2]: X of the leading row, [3..7]: scalars
-  R* nrmp;             // [2][C] partial |row|^2
+  Cx<R>* sc;           // [0..1] row entry of the next column, [3..7]: scalars
+  R* nrmp;             // [2][C VG] partial |row|^2
   Cx<R>*xs, *us;       // [zrows] X conj(right scale), the column (unscaled left reflector)
   ColState<R>* cs;     // [own]
-  R* part;             // [24] per-warp partial sums
   R *dd, *ee;
   Cx<R>*tau, *scl;     // factor and scale per reflector of the side the back-transformation needs
   Cx<R>* Y;            // global [.][ystride]: the reflector vectors of that side
@@ -118,255 +117,286 @@ struct Bidiag {
 // log2 of the smallest power of two >= rows, at least a warp's.
 __device__ __forceinline__ int row_shift(int rows) { return rows <= 32 ? 5 : 32 - __clz(rows - 1); }
 
-template <class R, int NT, int C>
-__device__ __forceinline__ void bidiagonalize_cluster(const Bidiag<R> b, const int gmax, const int r, const int p,
+// Virtual ranks: pair pi of columns belongs to rank pi mod (C VG), of which block pi mod C
+// holds VG. Sums over columns are formed per virtual rank and added in a fixed tree, so the
+// result has the same bits for every C with the same C VG: how many blocks a slot gets can
+// follow from how many slots run.
+template <class R, int NT, int C, int VG>
+__device__ __forceinline__ void bidiagonalize_cluster(const Bidiag<R> b, const int r, const int p,
                                                       const bool right_side, const unsigned rank) {
   const int tid = threadIdx.x;
-  // On this chip a SM does two FP64 operations a clock: scalar work in FP64 runs in one
-  // warp and is passed on through shared memory. In FP32 every warp does it for itself,
-  // which saves the barrier.
-  constexpr bool kOneWarp = sizeof(R) == 8;
-  constexpr int GL = 8, NG = NT / GL;   // lanes per column, columns at a time
-  constexpr int kLogNT = NT == 512 ? 9 : NT == 256 ? 8 : 7;
-  static_assert(NT == 1 << kLogNT, "threads: a power of two");
+  constexpr int GL = 8;                  // lanes per column in pass 1
+  constexpr int NG = (NT - 64) / GL;     // columns at a time: all warps but two
+  constexpr int NV = C * VG;             // virtual ranks
   const int own = 2 * (((p >> 1) + C - 1 - (int)rank) / C);   // p is even: pairs are never split
-  Cx<R> tauR = cx<R>(0, 0), scR = cx<R>(0, 0);
   for (int i = tid; i < own; i += NT) b.cs[i].rn = cx<R>(0, 0);
-  for (int k = 0; k < p; ++k) {
-    const int par = k & 1, rows = r - k;
-    const bool have_old = k > 0;
-    // ---- the next column and the right-update vector X, one thread per row
-    const int rsh = row_shift(rows);
-    if (tid < (1 << rsh)) {
-      R pn = 0;
-      Cx<R> pd = cx<R>(0, 0);
-      if (tid < rows) {
-        Cx<R> col, X = cx<R>(0, 0);
-        if (!have_old) {
-          col = peer<C>(b.T, 0)[tid];
-        } else {
-          const Cx<R>* zq = b.zp + par * C * gmax * b.zrows + tid;
-          const Cx<R> a = b.colp[par * b.zrows + tid];
-          Cx<R> zc[C];
+  // The right reflector of a row waits for the blocks' partial norms. One block, and FP64,
+  // form it during pass 2 (with a cluster barrier of its own, hidden there); in FP32 that
+  // barrier costs more than the reflector, which goes beside the sums of z after the step's
+  // one barrier (chi = 64: 322 k cycles per gate against 345 k; FP64 1 861 k against 1 807 k).
+  constexpr bool kEarly = C == 1 || sizeof(R) == 8;
+  const bool last_warp = tid >= NT - 32;
+  auto send_norm = [&](int first, int lnext, int npar) {
+    // lane pairs over the pairs of one virtual rank, in the order of its columns
+    const int l = tid & 31;
 #pragma unroll
-          for (int c = 0; c < C; ++c) zc[c] = zq[c * gmax * b.zrows];
-          if (min(gmax, NT >> rsh) == 2) {
+    for (int g = 0; g < VG; ++g) {
+      R nn = 0;
+      // columns of virtual rank g at or after `first`: pairs lp = g mod VG
+      const int lp0 = (first >> 1) + ((g - (first >> 1)) % VG + VG) % VG;
+      for (int lc = 2 * (lp0 + (l >> 1) * VG) + (l & 1); lc < own; lc += 32 * VG)
+        if (lc >= first && lc != lnext) nn += norm2(b.cs[lc].rn);
 #pragma unroll
-            for (int c = 0; c < C; ++c) zc[c] = zc[c] + zq[(c * gmax + 1) * b.zrows];
-          }
+      for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, o);
+      if (l < C) peer<C>(b.nrmp, l)[npar * NV + (int)rank + C * g] = nn;
+    }
+    if (l < C && lnext >= 0) peer<C>(b.sc, l)[npar] = b.cs[lnext].rn;
+    __syncwarp();
+  };
+  auto right_reflector = [&](int k, int npar) {
+    Cx<R> tauR, scR;
+    R betaR, rc[NV];
 #pragma unroll
-          for (int h = C / 2; h > 0; h >>= 1)
+    for (int c = 0; c < NV; ++c) rc[c] = b.nrmp[npar * NV + c];
 #pragma unroll
-            for (int c = 0; c < h; ++c) zc[c] = zc[c] + zc[c + h];
-          const Cx<R> z = zc[0];
-          X = tauR * (a + scR * z);
-          col = a - X;
-          b.xs[tid] = X * conj(scR);
-        }
-        b.us[tid] = col;
-        if (tid > 0) {
-          pn = norm2(col);
-          cmac_conj(pd, col, X);
-        } else {
-          b.sc[2] = X;
-        }
-      }
+    for (int h = NV / 2; h > 0; h >>= 1)
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        pn += __shfl_xor_sync(0xffffffffu, pn, o);
-        pd.x += __shfl_xor_sync(0xffffffffu, pd.x, o);
-        pd.y += __shfl_xor_sync(0xffffffffu, pd.y, o);
-      }
-      if ((tid & 31) == 0) {
-        b.part[tid >> 5] = pn;
-        b.part[8 + (tid >> 5)] = pd.x;
-        b.part[16 + (tid >> 5)] = pd.y;
+      for (int c = 0; c < h; ++c) rc[c] += rc[c + h];
+    reflector(conj(b.sc[npar]), rc[0], &tauR, &betaR, &scR);
+    if (tid == NT - 32) {
+      b.sc[6] = tauR;
+      b.sc[7] = scR;
+      b.ee[k] = betaR;
+      if (right_side) {
+        b.tau[k] = tauR;
+        b.scl[k] = scR;
       }
     }
-    __syncthreads();
-    // ---- left reflector u = (1, col scL) of that column; g = u^H (X conj(scR))
-    Cx<R> scL, ct, g;
-    if (!kOneWarp || tid < 32) {
-      R xn2 = b.part[0], betaL;
-      Cx<R> dot = cx<R>(b.part[8], b.part[16]), tauL;
+  };
+  for (int k = 0; k < p; ++k) {
+    const int par = k & 1, npar = par ^ 1, rows = r - k;
+    const bool have_old = k > 0;
+    // conj(col) X and |col|^2 per row, in place of the first two z partials of that row, which
+    // its own thread has read by then (the peers write that buffer again after the next
+    // cluster barrier)
+    Cx<R>* pd = b.zp + par * NV * b.zrows;
+    Cx<R>* pn = pd + b.zrows;
+    // ---- sums of z, the right-update vector X and the next column, one thread per row
+    Cx<R> a = cx<R>(0, 0), z = a;
+    if (have_old) {
+      if (!kEarly && last_warp) right_reflector(k - 1, par);
+      if (tid < rows) {
+        const Cx<R>* zq = b.zp + par * NV * b.zrows + tid;
+        a = b.colp[par * b.zrows + tid];
+        Cx<R> zc[NV];
 #pragma unroll
-      for (int w = 1; w < 8; ++w)
-        if (w < (1 << rsh) / 32) {
-          xn2 += b.part[w];
-          dot.x += b.part[8 + w];
-          dot.y += b.part[16 + w];
-        }
-      reflector(b.us[0], xn2, &tauL, &betaL, &scL);
-      g = have_old ? (b.sc[2] + conj(scL) * dot) * conj(scR) : cx<R>(0, 0);
-      ct = conj(tauL);
+        for (int c = 0; c < NV; ++c) zc[c] = zq[c * b.zrows];
+#pragma unroll
+        for (int h = NV / 2; h > 0; h >>= 1)
+#pragma unroll
+          for (int c = 0; c < h; ++c) zc[c] = zc[c] + zc[c + h];
+        z = zc[0];
+      }
+      if (!kEarly) __syncthreads();
+    }
+    if (tid < rows) {
+      Cx<R> X = cx<R>(0, 0), col;
+      if (have_old) {
+        const Cx<R> scR = b.sc[7];
+        X = b.sc[6] * (a + scR * z);
+        col = a - X;
+        b.xs[tid] = X * conj(scR);
+      } else {
+        col = peer<C>(b.T, 0)[tid];
+      }
+      b.us[tid] = col;
+      Cx<R> d = cx<R>(0, 0);
+      cmac_conj(d, col, X);
+      pn[tid].x = tid > 0 ? norm2(col) : R(0);
+      pd[tid] = tid > 0 ? d : cx<R>(0, 0);
+    }
+    __syncthreads();
+    // ---- first warp: left reflector u = (1, col scL) of that column; second warp: col^H X;
+    // the others: pass 1, s_j = col^H a_j of the own trailing columns, which needs neither.
+    // (Scalars go through one warp: they would cost every warp the same instructions, and
+    // FP64 runs at two lanes a clock whatever the lanes hold.)
+    const int l0 = 2 * ((((k + 1) >> 1) + C - 1 - (int)rank) / C);   // own pairs from column k (or k + 1) on
+    const int first = 2 * (C * (l0 >> 1) + (int)rank) > k ? l0 : l0 + 1;   // own columns after k
+    if (tid < 32) {
+      R v = 0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (tid + 32 * i < rows) v += pn[tid + 32 * i].x;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      Cx<R> tauL, scL;
+      R betaL;
+      reflector(b.us[0], v, &tauL, &betaL, &scL);
       if (tid == 0) {
         b.dd[k] = betaL;
         if (!right_side) {
           b.tau[k] = tauL;
           b.scl[k] = cx<R>(1, 0);
         }
-        if (kOneWarp) {
-          b.sc[3] = scL;
-          b.sc[4] = ct;
-          b.sc[5] = g;
+        b.sc[3] = scL;
+        b.sc[4] = conj(tauL);
+      }
+    } else if (tid < 64) {
+      if (have_old) {
+        Cx<R> v = cx<R>(0, 0);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (tid - 32 + 32 * i < rows) v = v + pd[tid - 32 + 32 * i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+          v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
         }
+        if (tid == 32) b.sc[5] = v * conj(b.sc[7]);
+      }
+    } else if (k + 1 < p) {
+      const int lane = tid & (GL - 1), grp = (tid - 64) / GL;
+      for (int base = first; base < own; base += NG) {
+        const int lc = base + grp;
+        const bool act = lc < own;
+        Cx<R> s = cx<R>(0, 0);
+        if (act) {
+          // four partial sums: the dependent chain, not the arithmetic, is what this costs
+          const Cx<R>* t = b.T + lc * b.ld + k;
+          Cx<R> sp[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) sp[e] = cx<R>(0, 0);
+          int i = lane == 0 ? GL : lane;
+          for (; i + 3 * GL < rows; i += 4 * GL) {
+            Cx<R> av[4], uv[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              av[e] = t[i + e * GL];
+              uv[e] = b.us[i + e * GL];
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) cmac_conj(sp[e], uv[e], av[e]);
+          }
+#pragma unroll
+          for (int e = 0; e < 3; ++e)
+            if (i + e * GL < rows) cmac_conj(sp[e], b.us[i + e * GL], t[i + e * GL]);
+          s = (sp[0] + sp[1]) + (sp[2] + sp[3]);
+        }
+#pragma unroll
+        for (int o = 1; o < GL; o <<= 1) {
+          s.x += __shfl_xor_sync(0xffffffffu, s.x, o, GL);
+          s.y += __shfl_xor_sync(0xffffffffu, s.y, o, GL);
+        }
+        if (act && lane == 0) b.cs[lc].f = s;
       }
     }
-    if (kOneWarp) {
-      __syncthreads();
-      scL = b.sc[3];
-      ct = b.sc[4];
-      g = b.sc[5];
-    }
+    __syncthreads();
+    const Cx<R> scL = b.sc[3];
     if (!right_side && (k % C) == (int)rank)
       for (int i = tid; i < rows; i += NT) b.Y[(size_t)k * b.ystride + k + i] = i == 0 ? cx<R>(1, 0) : b.us[i] * scL;
     if (k + 1 >= p) break;
-    // ---- pass 1: s_j = u^H a_j of the own trailing columns; then the left factor f_j and
-    // the new row entry r_j, both with the pending right update taken into account
-    const int l0 = 2 * ((((k + 1) >> 1) + C - 1 - (int)rank) / C);   // own pairs from column k (or k + 1) on
-    const int first = 2 * (C * (l0 >> 1) + (int)rank) > k ? l0 : l0 + 1;   // own columns after k
-    const int lane = tid & (GL - 1), grp = tid / GL;
-    auto finish = [&](int lc, Cx<R> s) {
-      const Cx<R> a0 = b.T[lc * b.ld + k], ro = b.cs[lc].rn;
-      s = a0 + conj(scL) * s;
-      Cx<R> rn = a0;
+    // ---- the left factor f_j and the new row entry r_j, with the pending right update taken
+    // into account: u^H (a_j - X conj(scR) r_j') = (a_j - X conj(scR) r_j')_0 + conj(scL)
+    // (col^H a_j - col^H X conj(scR) r_j')
+    for (int lc = first + tid; lc < own; lc += NT) {
+      Cx<R> rn = b.T[lc * b.ld + k], t = b.cs[lc].f;
+      const Cx<R> ro = b.cs[lc].rn;
       if (have_old) {
-        cmsub(s, g, ro);
         cmsub(rn, b.xs[0], ro);
+        cmsub(t, b.sc[5], ro);
       }
-      const Cx<R> f = ct * s;
+      Cx<R> s = rn;
+      cmac_conj(s, scL, t);
+      const Cx<R> f = b.sc[4] * s;
       rn = rn - f;
       b.cs[lc].f = f;
       b.cs[lc].ro = ro;
       b.cs[lc].rn = rn;
       if (right_side) b.Y[(size_t)k * b.ystride + 2 * (C * (lc >> 1) + (int)rank) + (lc & 1)] = conj(rn);
-    };
-    for (int base = first; base < own; base += NG) {
-      const int lc = base + grp;
-      const bool act = lc < own;
-      Cx<R> s = cx<R>(0, 0);
-      if (act) {
-        // four partial sums: the dependent chain, not the arithmetic, is what this costs
-        const Cx<R>* a = b.T + lc * b.ld + k;
-        Cx<R> sp[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) sp[e] = cx<R>(0, 0);
-        int i = lane == 0 ? GL : lane;
-        for (; i + 3 * GL < rows; i += 4 * GL) {
-          Cx<R> av[4], uv[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            av[e] = a[i + e * GL];
-            uv[e] = b.us[i + e * GL];
-          }
-#pragma unroll
-          for (int e = 0; e < 4; ++e) cmac_conj(sp[e], uv[e], av[e]);
-        }
-#pragma unroll
-        for (int e = 0; e < 3; ++e)
-          if (i + e * GL < rows) cmac_conj(sp[e], b.us[i + e * GL], a[i + e * GL]);
-        s = (sp[0] + sp[1]) + (sp[2] + sp[3]);
-      }
-#pragma unroll
-      for (int o = 1; o < GL; o <<= 1) {
-        s.x += __shfl_xor_sync(0xffffffffu, s.x, o, GL);
-        s.y += __shfl_xor_sync(0xffffffffu, s.y, o, GL);
-      }
-      if (act && lane == 0) {
-        if constexpr (kOneWarp)
-          b.cs[lc].f = s;
-        else
-          finish(lc, s);
-      }
     }
     __syncthreads();
-    if constexpr (kOneWarp) {
-      for (int lc = first + tid; lc < own; lc += NT) finish(lc, b.cs[lc].f);
-      __syncthreads();
+    const int lnext = ((k + 1) >> 1) % C == (int)rank ? 2 * (((k + 1) >> 1) / C) + ((k + 1) & 1) : -1;
+    // ---- last warp: partial norm of the new row (columns after k + 1) and its leading entry
+    // to all blocks
+    const int nrow = rows - 1, rsh2 = row_shift(nrow), groups = min(VG, NT >> rsh2);
+    const bool last_busy = (groups << rsh2) > NT - 32;   // it has rows of its own in pass 2
+    if (last_warp && (kEarly || !last_busy)) send_norm(first, lnext, npar);
+    if constexpr (kEarly) {
+      csync_arrive<C>();
+      if (last_warp && !last_busy) {
+        csync_wait<C>();
+        right_reflector(k, npar);
+      }
     }
     // ---- pass 2: both updates, one thread per row and column group; z = sum a_j conj(r_j)
     // over the columns after k + 1; column k + 1 goes out whole
-    const int nrow = rows - 1, rsh2 = row_shift(nrow), groups = min(gmax, NT >> rsh2);
-    const int row = tid & ((1 << rsh2) - 1), cgp = tid >> rsh2, npar = par ^ 1;
-    const int lnext = ((k + 1) >> 1) % C == (int)rank ? 2 * (((k + 1) >> 1) / C) + ((k + 1) & 1) : -1;
+    const int row = tid & ((1 << rsh2) - 1), cgp = tid >> rsh2;
     if (cgp < groups && row < nrow) {
-      Cx<R> z = cx<R>(0, 0), z2 = cx<R>(0, 0);
       const Cx<R> u = b.us[row + 1] * scL;
       const Cx<R> x = have_old ? b.xs[row + 1] : cx<R>(0, 0);
-      int lc = first + cgp;
-      Cx<R>* a = b.T + lc * b.ld + k + 1 + row;
-      if (lc == lnext) {   // first own column: only group 0 can meet it
-        Cx<R> v = *a;
-        cmsub(v, x, b.cs[lc].ro);
-        cmsub(v, b.cs[lc].f, u);
-#pragma unroll
-        for (int c = 0; c < C; ++c) peer<C>(b.colp, c)[npar * b.zrows + row] = v;
-        lc += groups;
-        a += groups * b.ld;
-      }
-      const int step = groups * b.ld;
-      for (; lc + groups < own; lc += 2 * groups, a += 2 * step) {
-        const ColState<R> q = b.cs[lc], q2 = b.cs[lc + groups];
-        Cx<R> v = a[0], v2 = a[step];
-        cmsub(v, x, q.ro);
-        cmsub(v2, x, q2.ro);
-        cmsub(v, q.f, u);
-        cmsub(v2, q2.f, u);
-        a[0] = v;
-        a[step] = v2;
-        cmac_bconj(z, v, q.rn);
-        cmac_bconj(z2, v2, q2.rn);
-      }
-      if (lc < own) {
-        const ColState<R> q = b.cs[lc];
-        Cx<R> v = a[0];
+      Cx<R>* col0 = b.T + k + 1 + row;
+      auto update = [&](int lc, const ColState<R>& q) {
+        Cx<R> v = col0[lc * b.ld];
         cmsub(v, x, q.ro);
         cmsub(v, q.f, u);
-        a[0] = v;
-        cmac_bconj(z, v, q.rn);
-      }
-      z = z + z2;
+        return v;
+      };
+      for (int g = cgp; g < VG; g += groups) {
+        Cx<R> z1 = cx<R>(0, 0), z2 = cx<R>(0, 0);   // even and odd columns of the pairs
+        const int lf = first >> 1;
+        int lp = VG == 1 ? lf : lf + ((g - lf) % VG + VG) % VG;
+        if (lp == lf) {
+          // the first pair: its even column may be gone, or one of them be column k + 1
+          const int lc = 2 * lp;
+          if (lc >= first && lc < own) {
+            const ColState<R> q = b.cs[lc];
+            const Cx<R> v = update(lc, q);
+            if (lc == lnext) {
 #pragma unroll
-      for (int c = 0; c < C; ++c)
-        peer<C>(b.zp, c)[((npar * C + (int)rank) * gmax + cgp) * b.zrows + row] = z;
+              for (int c = 0; c < C; ++c) peer<C>(b.colp, c)[npar * b.zrows + row] = v;
+            } else {
+              col0[lc * b.ld] = v;
+              cmac_bconj(z1, v, q.rn);
+            }
+          }
+          if (lc + 1 < own) {
+            const ColState<R> q = b.cs[lc + 1];
+            const Cx<R> v = update(lc + 1, q);
+            if (lc + 1 == lnext) {
+#pragma unroll
+              for (int c = 0; c < C; ++c) peer<C>(b.colp, c)[npar * b.zrows + row] = v;
+            } else {
+              col0[(lc + 1) * b.ld] = v;
+              cmac_bconj(z2, v, q.rn);
+            }
+          }
+          lp += VG;
+        }
+        for (int lc = 2 * lp; lc < own; lc += 2 * VG) {
+          const ColState<R> q = b.cs[lc], q2 = b.cs[lc + 1];
+          const Cx<R> v = update(lc, q), v2 = update(lc + 1, q2);
+          col0[lc * b.ld] = v;
+          col0[(lc + 1) * b.ld] = v2;
+          cmac_bconj(z1, v, q.rn);
+          cmac_bconj(z2, v2, q2.rn);
+        }
+        z1 = z1 + z2;
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+          peer<C>(b.zp, c)[(npar * NV + (int)rank + C * g) * b.zrows + row] = z1;
+      }
     }
-    // partial norm of the new row (columns after k + 1) and its leading entry
-    if (tid >= NT - 32) {
-      const int l = tid & 31;
-      R nn = 0;
-      for (int lc = first + l; lc < own; lc += 32)
-        if (lc != lnext) nn += norm2(b.cs[lc].rn);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, o);
-      if (l < C) {
-        peer<C>(b.nrmp, l)[npar * C + (int)rank] = nn;
-        if (lnext >= 0) peer<C>(b.sc, l)[npar] = b.cs[lnext].rn;
+    if constexpr (kEarly) {
+      if (!last_warp) {
+        csync_wait<C>();
+      } else if (last_busy) {
+        csync_wait<C>();
+        right_reflector(k, npar);
       }
+    } else if (last_warp && last_busy) {
+      send_norm(first, lnext, npar);
     }
     csync<C>();
-    // ---- right reflector of the new row
-    if (!kOneWarp || tid < 32) {
-      R rn2 = 0, betaR;
-#pragma unroll
-      for (int c = 0; c < C; ++c) rn2 += b.nrmp[npar * C + c];
-      reflector(conj(b.sc[npar]), rn2, &tauR, &betaR, &scR);
-      if (tid == 0) {
-        b.ee[k] = betaR;
-        if (right_side) {
-          b.tau[k] = tauR;
-          b.scl[k] = scR;
-        }
-        if (kOneWarp) {
-          b.sc[6] = tauR;
-          b.sc[7] = scR;
-        }
-      }
-    }
-    if (kOneWarp) {
-      __syncthreads();
-      tauR = b.sc[6];
-      scR = b.sc[7];
-    }
   }
   csync<C>();
 }
@@ -465,43 +495,39 @@ __device__ __forceinline__ int sturm_ge1(const R* b2, int s, int e, R x) {
   return ge;
 }
 
-// Singular values t[0..V) (0-based, descending) of the TGK block [s, e) in FP32 by one
-// warp: 32 shifts per value and pass, each pass narrows a bracket 33-fold. First pass on a
-// log grid over eight decades, then linear to the working precision. lo/hi bracket the
-// values.
-template <int V>
-__device__ __forceinline__ int warp_bisect(const float* b2, int s, int e, const int* t, float top, float* lo,
-                                           float* hi) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int v = 0; v < V; ++v) {
-    lo[v] = 0.f;
-    hi[v] = top;
-  }
-  int passes = 0;
-  for (int it = 0; it < 9; ++it) {
-    float x[V];
-    int ge[V];
-#pragma unroll
-    for (int v = 0; v < V; ++v)
-      x[v] = it == 0 ? top * exp10f(-8.0f * (float)(32 - lane) / 32.0f)
-                     : fmaf(hi[v] - lo[v], (float)(lane + 1) / 33.0f, lo[v]);
-    sturm_ge<float, V>(b2, s, e, x, ge);
-    bool open = false;
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      // counts fall with x: the number of shifts below the value locates it
-      const int m = __popc(__ballot_sync(0xffffffffu, ge[v] >= t[v] + 1));
-      const float nlo = __shfl_sync(0xffffffffu, x[v], max(m - 1, 0));
-      const float nhi = __shfl_sync(0xffffffffu, x[v], min(m, 31));
-      if (m > 0) lo[v] = nlo;
-      if (m < 32) hi[v] = nhi;
-      open = open || hi[v] - lo[v] > 1.2e-7f * hi[v];   // not yet two neighbours of the working precision
+// Singular value t (0-based, descending) of the TGK block [s, e) in FP32 by half a warp: 16
+// shifts a pass, each pass narrows the bracket 17-fold. First pass on a log grid over
+// eight decades, then linear to the working precision or `passes` passes. lo/hi bracket
+// the value; one found to lie below `floor` is left there. Always 16 lanes, so that the
+// shifts, and with them the last bits, do not depend on how many values a block has.
+constexpr int kBisectLanes = 16;
+__device__ __forceinline__ int half_bisect(const float* b2, int s, int e, int t, bool act, float top, float floor,
+                                           int passes, float* lo_out, float* hi_out) {
+  constexpr int LP = kBisectLanes;
+  const int wl = threadIdx.x & 31, lane = wl & (LP - 1), base = wl & ~(LP - 1);
+  float lo = 0.f, hi = top;
+  int it = 0;
+  bool open = act;
+  while (it < passes) {
+    const float x = it == 0 ? top * exp10f(-8.0f * (float)(LP - lane) / (float)(LP + 1))
+                            : fmaf(hi - lo, (float)(lane + 1) / (float)(LP + 1), lo);
+    const bool above = sturm_ge1<float>(b2, s, e, x) >= t + 1;
+    // counts fall with x: the number of shifts below the value locates it
+    const int m = __popc((__ballot_sync(0xffffffffu, above) >> base) & ((1u << LP) - 1u));
+    const float nlo = __shfl_sync(0xffffffffu, x, base + max(m - 1, 0));
+    const float nhi = __shfl_sync(0xffffffffu, x, base + min(m, LP - 1));
+    if (open) {
+      if (m > 0) lo = nlo;
+      if (m < LP) hi = nhi;
     }
-    ++passes;
-    if (!open) break;
+    // not yet two neighbours of the working precision, and not below what is kept
+    open = open && hi - lo > 1.2e-7f * hi && hi > floor;
+    ++it;
+    if (!__any_sync(0xffffffffu, open)) break;
   }
-  return passes;
+  *lo_out = lo;
+  *hi_out = hi;
+  return it;
 }
 
 // Value t of block [s, e) in FP64 from the FP32 bracket, LT = 4 lanes per value (a warp's FP64 operation
@@ -512,8 +538,8 @@ __device__ __forceinline__ int warp_bisect(const float* b2, int s, int e, const 
 // pass), or, when that gained less than a plain section would, evenly. The bracket itself
 // always moves by counts, so a wrong estimate costs a pass and nothing else. Stops at the
 // working precision relative to the value, or at 2^-60 of the largest one.
-__device__ __forceinline__ int lanes_bisect(const double* b2, int s, int e, int t, bool act, double top, float lo_f,
-                                            float hi_f, double* lo_out, double* hi_out) {
+__device__ __forceinline__ int lanes_bisect(const double* b2, int s, int e, int t, bool act, double top, double floor,
+                                            float lo_f, float hi_f, double* lo_out, double* hi_out) {
   constexpr int LT = 4;
   const int wl = threadIdx.x & 31, lane = wl & (LT - 1), base = wl & ~(LT - 1);
   double lo = (double)lo_f * (1.0 - 4e-6), hi = fmin(top, (double)hi_f * (1.0 + 4e-6) + 1e-30);
@@ -577,7 +603,7 @@ __device__ __forceinline__ int lanes_bisect(const double* b2, int s, int e, int 
         even = secant && !(hi - lo < 0.2 * w);
       }
     }
-    done = done || hi - lo <= fmax(2.3e-16 * hi, 8.7e-19);
+    done = done || hi - lo <= fmax(2.3e-16 * hi, 8.7e-19) || hi <= floor;
     if (__all_sync(0xffffffffu, done)) break;
   }
   *lo_out = lo;

@@ -24,6 +24,16 @@ __device__ __forceinline__ void csync() {
   }
 }
 
+// The two halves of a cluster barrier, for work in between; whole warps, every warp both.
+template <int C>
+__device__ __forceinline__ void csync_arrive() {
+  if constexpr (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+template <int C>
+__device__ __forceinline__ void csync_wait() {
+  if constexpr (C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 template <int C>
 __device__ __forceinline__ unsigned crank() {
   if constexpr (C == 1) return 0;
@@ -78,7 +88,6 @@ __device__ __forceinline__ SplitF to_elem(Cx<float> a) {
   const float hx = lead11(a.x), hy = lead11(a.y);
   return SplitF{make_float4(hx, __fadd_rn(a.x, -hx), hy, __fadd_rn(a.y, -hy))};
 }
-__device__ __forceinline__ Cx<double> to_elem(Cx<double> a) { return a; }
 __device__ __forceinline__ void zero(SplitAcc& a) { a.hx = a.hy = a.lx = a.ly = 0.f; }
 __device__ __forceinline__ void zero(Cx<double>& a) { a = cx<double>(0, 0); }
 // acc += a b
@@ -97,17 +106,21 @@ __device__ __forceinline__ Cx<float> value(const SplitAcc& a) {
   return cx<float>(__fadd_rn(a.hx, a.lx), __fadd_rn(a.hy, a.ly));
 }
 __device__ __forceinline__ Cx<double> value(const Cx<double>& a) { return a; }
-template <class R>
-struct Gemm;
-template <>
-struct Gemm<float> {
-  using E = SplitF;
-  using A = SplitAcc;
+__device__ __forceinline__ void zero(Cx<float>& a) { a = cx<float>(0, 0); }
+__device__ __forceinline__ void mac(Cx<float>& c, const Cx<float>& a, const Cx<float>& b) { cmac(c, a, b); }
+__device__ __forceinline__ Cx<float> value(const Cx<float>& a) { return a; }
+// EXACT: split products (FP32)
+template <class R, bool EXACT>
+struct Gemm {
+  using E = Cx<R>;
+  using A = Cx<R>;
+  static __device__ __forceinline__ E elem(Cx<R> a) { return a; }
 };
 template <>
-struct Gemm<double> {
-  using E = Cx<double>;
-  using A = Cx<double>;
+struct Gemm<float, true> {
+  using E = SplitF;
+  using A = SplitAcc;
+  static __device__ __forceinline__ E elem(Cx<float> a) { return to_elem(a); }
 };
 
 // out(m, n) = sum_k a(m, k) b(k, n) for m < M, n < N by one block. The operands come from
@@ -121,9 +134,10 @@ __host__ __device__ constexpr size_t gemm_tile_bytes() {   // of the largest til
   constexpr int TY = NT / 16;
   return 16 * (size_t)((4 * TY) * (kKT + 1) + kKT * (64 + 1));
 }
-template <class R, int NT, int RM, int JN, bool KF, class FA, class FB, class FC>
+template <class R, int NT, int RM, int JN, bool KF, bool EXACT, class FA, class FB, class FC>
 __device__ __forceinline__ void tile_gemm_shape(int M, int N, int K, FA fa, FB fb, FC fc, unsigned char* smem) {
-  using E = typename Gemm<R>::E;
+  using G = Gemm<R, EXACT>;
+  using E = typename G::E;
   constexpr int TY = NT / 16, TM = TY * RM, TN = 16 * JN, KT = kKT;
   constexpr int NA = TM * KT / NT, NB = KT * TN / NT > 0 ? KT * TN / NT : 1;
   E(*As)[KT + 1] = reinterpret_cast<E(*)[KT + 1]>(smem);
@@ -131,7 +145,7 @@ __device__ __forceinline__ void tile_gemm_shape(int M, int N, int K, FA fa, FB f
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   for (int m0 = 0; m0 < M; m0 += TM)
     for (int n0 = 0; n0 < N; n0 += TN) {
-      typename Gemm<R>::A acc[RM][JN];
+      typename G::A acc[RM][JN];
 #pragma unroll
       for (int i = 0; i < RM; ++i)
 #pragma unroll
@@ -155,12 +169,12 @@ __device__ __forceinline__ void tile_gemm_shape(int M, int N, int K, FA fa, FB f
 #pragma unroll
         for (int e = 0; e < NA; ++e) {
           const int x = tid + e * NT;
-          As[x / KT][x % KT] = to_elem(ra[e]);
+          As[x / KT][x % KT] = G::elem(ra[e]);
         }
 #pragma unroll
         for (int e = 0; e < NB; ++e) {
           const int x = tid + e * NT, kk = KF ? x % KT : x / TN, n = KF ? x / KT : x % TN;
-          if (x < KT * TN) Bs[kk][n] = to_elem(rb[e]);
+          if (x < KT * TN) Bs[kk][n] = G::elem(rb[e]);
         }
         __syncthreads();
         if (k0 + KT < K) fetch(k0 + KT);
@@ -205,18 +219,18 @@ __device__ __forceinline__ void tile_gemm_shape(int M, int N, int K, FA fa, FB f
 
 // Shape by the narrow side: what one thread computes is kept at four outputs where the
 // product has them, and small products spread over all threads.
-template <class R, int NT, bool KF, class FA, class FB, class FC>
+template <class R, int NT, bool KF, bool EXACT = true, class FA, class FB, class FC>
 __device__ __forceinline__ void tile_gemm(int M, int N, int K, FA fa, FB fb, FC fc, unsigned char* smem) {
   constexpr int TY = NT / 16;
   if (N <= 16) {
     if (M <= TY)
-      tile_gemm_shape<R, NT, 1, 1, KF>(M, N, K, fa, fb, fc, smem);
+      tile_gemm_shape<R, NT, 1, 1, KF, EXACT>(M, N, K, fa, fb, fc, smem);
     else
-      tile_gemm_shape<R, NT, 4, 1, KF>(M, N, K, fa, fb, fc, smem);
+      tile_gemm_shape<R, NT, 4, 1, KF, EXACT>(M, N, K, fa, fb, fc, smem);
   } else if (N <= 32 && M > TY) {
-    tile_gemm_shape<R, NT, 2, 2, KF>(M, N, K, fa, fb, fc, smem);
+    tile_gemm_shape<R, NT, 2, 2, KF, EXACT>(M, N, K, fa, fb, fc, smem);
   } else {
-    tile_gemm_shape<R, NT, 1, 4, KF>(M, N, K, fa, fb, fc, smem);
+    tile_gemm_shape<R, NT, 1, 4, KF, EXACT>(M, N, K, fa, fb, fc, smem);
   }
 }
 

@@ -16,12 +16,20 @@ __device__ __forceinline__ R rabs(R x) {
 // ldw), in blocks of 8 rows. Each of the two repetitions projects the block out of all
 // earlier rows and then orthonormalises it internally by Cholesky QR (G = W_b W_b^T =
 // L L^T, W_b <- L^{-1} W_b). Row t of the result depends only on rows 0..t, so the
-// leading singular vectors keep their directions. The rows come in with unit norm: a
-// Cholesky pivot below 1e-6 of that (or, in the second repetition, of its diagonal), i.e. a
-// row that is numerically a combination of earlier rows, of its own block or before it,
-// counts as a collapse. coef: >= 8 k shared scratch (used once k > 8); small: >= 128 shared.
+// leading singular vectors keep their directions. The rows come in with unit norm. A row of
+// which only theta is left beside the rows before it keeps theta of its own direction
+// against eps of rounding, so eps / theta of sigma / sigma_0 is what M' loses by it: a
+// squared theta below collapse_limit counts as a collapse. coef: >= 8 k shared scratch (used
+// once k > 8); small: >= 128 shared.
+template <class R>
+__device__ __forceinline__ R collapse_limit(R sigma, R sigma0) {
+  const R t = sigma0 > R(0) ? sigma / sigma0 : R(1);
+  const R lim = sizeof(R) == 4 ? R(0.36) * t * t : R(0.01) * t * t;
+  return fmin(R(1e-6), fmax(sizeof(R) == 4 ? R(1e-11) : R(1e-26), lim));
+}
 template <class R, int NT>
-__device__ void orthonormalize_rows_block(R* W, int ldw, int k, int p, R* coef, R* small, int* collapsed) {
+__device__ void orthonormalize_rows_block(R* W, int ldw, int k, int p, const R* sig, R* coef, R* small,
+                                          int* collapsed) {
   const int tid = threadIdx.x;
   for (int b0 = 0; b0 < k; b0 += 8) {
     const int nb = min(8, k - b0);
@@ -81,7 +89,7 @@ __device__ void orthonormalize_rows_block(R* W, int ldw, int k, int p, R* coef, 
             R d = gjj;
 #pragma unroll
             for (int u = 0; u < j; ++u) d -= Lm[j][u] * Lm[j][u];
-            if (!(d > R(1e-6) * (rep == 0 ? fmax(gjj, R(1)) : gjj))) {
+            if (!(d > (rep == 0 ? collapse_limit(sig[b0 + j], sig[0]) : R(1e-6) * gjj))) {
               ++*collapsed;
               d = gjj > R(0) ? gjj * R(1e-30) : R(1e-30);
             }
@@ -143,7 +151,8 @@ __device__ void jacobi_columns(Cx<R>* X, int ldx, int ncols, int len, double zer
   int G = 1;
   while (G < 32 && G * MAXE < len) G <<= 1;
   const int npairs = (ncols + 1) >> 1;
-  while (G < 32 && G < len && (NT / (2 * G)) >= npairs) G <<= 1;
+  // (as for 256 threads, whatever NT: the lanes of a dot product fix its last bits)
+  while (G < 32 && G < len && (256 / (2 * G)) >= npairs) G <<= 1;
   const int ept = (len + G - 1) / G;
   const int ngroups = NT / G, grp = threadIdx.x / G, lane = threadIdx.x - grp * G;
   const R tol = R(2) * (sizeof(R) == 8 ? R(2.220446049250313e-16) : R(1.1920929e-7)) * sqrt((R)len);
