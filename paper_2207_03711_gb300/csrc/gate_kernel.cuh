@@ -52,6 +52,19 @@ __device__ __forceinline__ int bond_cap(int b, int n, int chi) {
 
 namespace gate {
 
+// s + c += a b without rounding errors beyond c's: TwoProd by FMA and TwoSum (Knuth), the
+// step of the compensated dot product "Dot2" (Ogita, Rump and Oishi, 2005). The _rn
+// intrinsics keep the compiler from contracting the products into the sums.
+__device__ __forceinline__ void dot2_acc(float a, float b, float& s, float& c) {
+  const float p = __fmul_rn(a, b);
+  const float ep = fmaf(a, b, -p);
+  const float t = __fadd_rn(s, p);
+  const float bv = __fsub_rn(t, s);
+  const float et = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bv)), __fsub_rn(p, bv));
+  s = t;
+  c = __fadd_rn(c, __fadd_rn(ep, et));
+}
+
 // Shared-memory plan of one block. Two areas have several tenants in turn:
 //   exchange  GEMM tiles of the contraction | exchange buffers of the bidiagonalisation |
 //             TGK arrays, its blocks, singular values, orderings
@@ -88,9 +101,9 @@ struct Plan {
     for (size_t b : {twist, nsr, nsc, ychunk, tiles})
       if (b > work) work = b;
     total = fixed + exch + work;
-    // small caps: room for the whole Jacobi matrix, and for longer chunks
-    const size_t cap = 227 * 1024 - 1024, want = up(sizeof(Cx<R>) * (size_t)mmax * (mmax + 1));
-    if (want > work && want <= 96 * 1024 && fixed + exch + want <= cap) {
+    // room for the whole Jacobi matrix where a block has it, and for longer chunks
+    const size_t cap = 227 * 1024 - 1024, want = up(sizeof(R) * (size_t)mmax * (mmax + 1));
+    if (want > work && fixed + exch + want <= cap) {
       work = want;
       total = fixed + exch + work;
     }
@@ -581,12 +594,24 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
 #pragma unroll
       for (int ij = 0; ij < 4; ++ij) {
         Cx<R> v = cx<R>(0, 0);
+        if constexpr (kF64) {
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-          if constexpr (!kF64) cmac(v, Ul[ij * 4 + kk], th4[kk]);
+          for (int kk = 0; kk < 4; ++kk) cmac(v, Uh[ij * 4 + kk], th4[kk]);
+        } else {
+          // one rounding per entry, against the matrix in 48 bits
+          float cr = 0.f, ci = 0.f;
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk) {
+            const Cx<float> u = Uh[ij * 4 + kk], l = Ul[ij * 4 + kk], t = th4[kk];
+            dot2_acc(u.x, t.x, v.x, cr);
+            dot2_acc(-u.y, t.y, v.x, cr);
+            dot2_acc(u.x, t.y, v.y, ci);
+            dot2_acc(u.y, t.x, v.y, ci);
+            cr = fmaf(-l.y, t.y, fmaf(l.x, t.x, cr));
+            ci = fmaf(l.y, t.x, fmaf(l.x, t.y, ci));
+          }
+          v = cx<float>(__fadd_rn(v.x, cr), __fadd_rn(v.y, ci));
         }
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) cmac(v, Uh[ij * 4 + kk], th4[kk]);
         W[(size_t)(2 * a + (ij >> 1)) * ncol + (ij & 1) * rr + cc] = v;
         const Cx<R> mv = la * v;
         *e[ij] = tall ? mv : conj(mv);
@@ -823,11 +848,8 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
       }
     }
     __syncthreads();
-    const int k = misc[0];
-    if (tid == 0) {
-      st_max_rank = max(st_max_rank, k);
-      st_max_iters = max(st_max_iters, passes);
-    }
+    int k = misc[0];
+    if (tid == 0) st_max_iters = max(st_max_iters, passes);
     PHASE(2);
 
     // (4) singular vectors of B from twisted factorisations of TGK - sigma. Leading minors
@@ -835,7 +857,7 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
     // only serial chain, one multiply-add a step); the pivots' reciprocals p_{i-1} / p_i,
     // the twist where |gamma| is smallest and the ratios of neighbouring entries by whole
     // warps; then the running products of the ratios outward from the twist.
-    const int kcv = (k + C - 1 - (int)rank_c) / C;   // own vectors t = rank_c + C i
+    int kcv = (k + C - 1 - (int)rank_c) / C;   // own vectors t = rank_c + C i
     {
       constexpr int STEP = SturmGroup<R>::v;
       const R big = kF64 ? R(1e300) : R(1e30);
@@ -1039,10 +1061,66 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
         csync<C>();
       }
       __syncthreads();
+      if (misc[1] != 0) {
+        // degenerate without a split: Jacobi on the bidiagonal by the first block. Columns of
+        // B^T (tall) or B (wide) converge to sigma_t times the wanted vector.
+        if (tid == 0) ++st_bad;
+        Wc = Wn;
+        if (rank_c == 0) {
+          const int ldx = tp + 1;
+          R* X = sizeof(R) * (size_t)tp * ldx <= L.work ? (R*)work : (R*)xout;
+          for (int e = tid; e < tp * tp; e += NT) {
+            const int c = e / tp, q = e - c * tp;   // entry q of column c: B[c][q] or B[q][c]
+            R v = q == c ? dd[c] * down : R(0);
+            if (tall && q == c + 1) v = ee[c] * down;
+            if (!tall && q + 1 == c) v = ee[q] * down;
+            X[(size_t)c * ldx + q] = v;
+          }
+          __syncthreads();
+          const double zero2 = (double)Eps<R>::v * Eps<R>::v * 16.0 * total * (double)down * (double)down;
+          jacobi_columns<R, NT, 8>(X, ldx, tp, zero2, max_sweeps, &misc[2]);
+          for (int p = tid; p < tp; p += NT) {
+            double acc = 0.0;
+            for (int q = 0; q < tp; ++q) acc = fma((double)X[(size_t)p * ldx + q], (double)X[(size_t)p * ldx + q], acc);
+            sig2d[p] = acc;
+          }
+          __syncthreads();
+          for (int p = tid; p < tp; p += NT) {
+            const double v = sig2d[p];
+            int rk = 0;
+            for (int q = 0; q < tp; ++q) {
+              const double w = sig2d[q];
+              rk += (w > v) || (w == v && q < p);
+            }
+            order[rk] = p;
+          }
+          __syncthreads();
+          if (tid == 0) {
+            const double s0 = sig2d[order[0]];
+            int kj = 0;
+            while (kj < kk && sig2d[order[kj]] > cutoff * cutoff * s0) ++kj;
+            if (kj == 0) kj = 1;
+            for (int cb = 0; cb < C; ++cb) peer<C>(misc, cb)[0] = kj;
+          }
+          __syncthreads();
+          const int kj = misc[0];
+          for (int t = tid; t < kj; t += NT) {
+            const R v = (R)sqrt(sig2d[order[t]]);
+            for (int cb = 0; cb < C; ++cb) peer<C>(sig, cb)[t] = v;
+          }
+          for (int e = tid; e < kj * tp; e += NT) {
+            const int t = e / tp, q = e - t * tp, p = order[t];
+            Wn[e] = (R)((double)X[(size_t)p * ldx + q] / sqrt(sig2d[p]));
+          }
+        }
+        csync<C>();
+        k = misc[0];
+        kcv = (k + C - 1 - (int)rank_c) / C;
+      }
+      if (tid == 0) st_max_rank = max(st_max_rank, k);
     }
     PHASE(4);
-    int kf = k;                                  // kept count of the path taken
-    if (misc[1] == 0) {
+    {
       // (5) back-transformation: x_t = P w_t (tall) or Q [w_t; 0] (wide) is the right
       //     singular vector v_t of M' (length ncol)
       const int nref = tall ? tp - 1 : tp;
@@ -1072,66 +1150,7 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
         if (lane == 0 && total > 0.0) dw_acc += fmax(0.0, total - kept) / total;
         for (int t = lane; t < k; t += 32) lam[(size_t)bond * chi + t] = (double)(sig[t] * back);
       }
-    } else {
-      // (5') degenerate spectrum without a split: one-sided Jacobi by the first block on the
-      //      columns X = conj rows of M' (rebuilt from W and lambda_{n-1})
-      if (tid == 0) ++st_bad;
-      if (rank_c == 0) {
-        const int ldx = ncol + 1;
-        Cx<R>* X = sizeof(Cx<R>) * (size_t)mrows * ldx <= L.work ? T : Y;
-        for (int idx = tid; idx < mrows * ncol; idx += NT) {
-          const int row = idx / ncol, q = idx - row * ncol;
-          const R la = laml ? (R)__ldcg(laml + (row >> 1)) : R(1);
-          X[(size_t)row * ldx + q] = conj(la * ldcg(W + (size_t)row * ncol + q));
-        }
-        __syncthreads();
-        const double zero2 = (double)Eps<R>::v * Eps<R>::v * 16.0 * total;
-        jacobi_columns<R, NT, 8>(X, ldx, mrows, ncol, zero2, max_sweeps, &misc[2]);
-        for (int p = tid; p < mrows; p += NT) {
-          double acc = 0.0;
-          for (int q = 0; q < ncol; ++q) acc += (double)norm2(X[(size_t)p * ldx + q]);
-          sig2d[p] = acc;
-        }
-        __syncthreads();
-        for (int p = tid; p < mrows; p += NT) {
-          const double v = sig2d[p];
-          int rk = 0;
-          for (int q = 0; q < mrows; ++q) {
-            const double w = sig2d[q];
-            rk += (w > v) || (w == v && q < p);
-          }
-          order[rk] = p;
-        }
-        __syncthreads();
-        if (tid == 0) {
-          const double s0 = sig2d[order[0]];
-          const int kmax = min(chi, min(mrows, ncol));
-          int kk2 = 0;
-          while (kk2 < kmax && sig2d[order[kk2]] > cutoff * cutoff * s0) ++kk2;
-          if (kk2 == 0) kk2 = 1;
-          double all = 0.0, dropped = 0.0;
-          for (int t = 0; t < mrows; ++t) all += sig2d[order[t]];
-          for (int t = kk2; t < mrows; ++t) dropped += sig2d[order[t]];
-          if (all > 0.0) dw_acc += dropped / all;
-          for (int cb = 0; cb < C; ++cb) peer<C>(misc, cb)[0] = kk2;
-          st_max_rank = max(st_max_rank, kk2);
-        }
-        __syncthreads();
-        const int kj = misc[0];
-        for (int t = tid; t < kj; t += NT) lam[(size_t)bond * chi + t] = (double)(R)sqrt(sig2d[order[t]]);
-        for (int idx = tid; idx < kj * ncol; idx += NT) {
-          const int t = idx / ncol, q = idx - t * ncol;
-          const int p = order[t];
-          const R inv = (R)(1.0 / sqrt(sig2d[p]));
-          const Cx<R> v = inv * X[(size_t)p * ldx + q];   // column p of X = sigma * v_t
-          xout[idx] = v;
-          if (kF64) Bn1[idx] = conj(v);
-        }
-      }
-      csync<C>();
-      kf = misc[0];
     }
-    const int kcf = (kf + C - 1 - (int)rank_c) / C;
     csync<C>();
     Cx<R>* xv = xout;
     if constexpr (!kF64) {
@@ -1141,10 +1160,10 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
       Cx<float>* E = (Cx<float>*)work;
       SplitF* chunk = (SplitF*)(E + ((size_t)L.kc * chi + 1) / 2 * 2);
       if constexpr (RAW) {
-        newton_schulz_cluster<NT, C>(xout, kf, ncol, kcf, rank_c, E, chunk, xout2, xout2);
+        newton_schulz_cluster<NT, C>(xout, k, ncol, kcv, rank_c, E, chunk, xout2, xout2);
         __syncthreads();
         // the caller's tensors take V by component; xout2 then holds conj(V) rows
-        for (int i = 0; i < kcf; ++i) {
+        for (int i = 0; i < kcv; ++i) {
           const int t = rank_c + C * i;
           for (int q = tid; q < ncol; q += NT) {
             const Cx<R> v = xout2[(size_t)t * ncol + q];
@@ -1153,7 +1172,7 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
           }
         }
       } else {
-        newton_schulz_cluster<NT, C>(xout, kf, ncol, kcf, rank_c, E, chunk, xout2, Bn1);
+        newton_schulz_cluster<NT, C>(xout, k, ncol, kcv, rank_c, E, chunk, xout2, Bn1);
       }
       xv = xout2;
       csync<C>();
@@ -1164,17 +1183,17 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
     {
       const int mper = (mrows + C - 1) / C, m0 = min(mrows, mper * (int)rank_c), mn = min(mper, mrows - m0);
       tile_gemm<R, NT, true>(
-          mn, kf, ncol, [&](int mi, int q) { return ldcg(W + (m0 + mi) * ncol + q); },
+          mn, k, ncol, [&](int mi, int q) { return ldcg(W + (m0 + mi) * ncol + q); },
           [&](int q, int t) { return ldcg(xv + t * ncol + q); },
-          [&](int mi, int t, Cx<R> v) { st_site<RAW>(Bn + (m0 + mi) * kf + t, v); }, work);
+          [&](int mi, int t, Cx<R> v) { st_site<RAW>(Bn + (m0 + mi) * k + t, v); }, work);
     }
     if (tid == 0) {
-      ranks[bond + 1] = kf;
-      if (rank_c == 0) rank[bond + 1] = kf;
+      ranks[bond + 1] = k;
+      if (rank_c == 0) rank[bond + 1] = k;
     }
     csync<C>();
     PHASE(6);
-    if (tid == 0) alg_flops += flops_per_gate(rl, rm, rr, kf);
+    if (tid == 0) alg_flops += flops_per_gate(rl, rm, rr, k);
   }
 #undef PHASE
   if (rank_c == 0 && tid == 0) {

@@ -141,23 +141,24 @@ __device__ void orthonormalize_rows_block(R* W, int ldw, int k, int p, const R* 
   }
 }
 
-// One-sided (Hestenes) Jacobi on the `ncols` columns of X (each of length `len`,
-// column stride ldx), used when the bidiagonal route reports a collapsed vector
-// (numerically degenerate singular values without a split). Columns converge to
-// sigma_p times a singular vector; columns below sqrt(zero2) are numerically zero.
+// One-sided (Hestenes) Jacobi on the n columns of the real n x n matrix X (column stride
+// ldx), used when Gram-Schmidt reports a collapsed vector (numerically degenerate singular
+// values without a split). It runs on the bidiagonal factor, not on the complex M': a
+// quarter of the arithmetic, and the back-transformation takes its vectors like any
+// others. Columns converge to sigma_p times a singular vector; columns below sqrt(zero2)
+// are numerically zero. n <= 32 MAXE.
 template <class R, int NT, int MAXE>
-__device__ void jacobi_columns(Cx<R>* X, int ldx, int ncols, int len, double zero2, int max_sweeps,
-                               int* noconv) {
+__device__ void jacobi_columns(R* X, int ldx, int n, double zero2, int max_sweeps, int* noconv) {
   int G = 1;
-  while (G < 32 && G * MAXE < len) G <<= 1;
-  const int npairs = (ncols + 1) >> 1;
+  while (G < 32 && G * MAXE < n) G <<= 1;
+  const int npairs = (n + 1) >> 1;
   // (as for 256 threads, whatever NT: the lanes of a dot product fix its last bits)
-  while (G < 32 && G < len && (256 / (2 * G)) >= npairs) G <<= 1;
-  const int ept = (len + G - 1) / G;
+  while (G < 32 && G < n && (256 / (2 * G)) >= npairs) G <<= 1;
+  const int ept = (n + G - 1) / G;
   const int ngroups = NT / G, grp = threadIdx.x / G, lane = threadIdx.x - grp * G;
-  const R tol = R(2) * (sizeof(R) == 8 ? R(2.220446049250313e-16) : R(1.1920929e-7)) * sqrt((R)len);
-  const int mm = ncols + (ncols & 1);  // even number of players; index ncols is a dummy
-  bool converged = ncols <= 1;
+  const R tol = R(2) * (sizeof(R) == 8 ? R(2.220446049250313e-16) : R(1.1920929e-7)) * sqrt((R)n);
+  const int mm = n + (n & 1);  // even number of players; index n is a dummy
+  bool converged = n <= 1;
   int sweep = 0;
   for (; sweep < max_sweeps && !converged; ++sweep) {
     int rotated = 0;
@@ -169,50 +170,45 @@ __device__ void jacobi_columns(Cx<R>* X, int ldx, int ncols, int len, double zer
           p = r;
           q = mm - 1;
         } else if (pi < mm / 2) {
-          p = (r + pi) % (mm - 1);
-          q = (r - pi + (mm - 1)) % (mm - 1);
+          p = r + pi;
+          if (p >= mm - 1) p -= mm - 1;
+          q = r - pi;
+          if (q < 0) q += mm - 1;
         }
-        const bool active = pi < mm / 2 && p < ncols && q < ncols;
-        Cx<R>* xp = X + (size_t)p * ldx;
-        Cx<R>* xq = X + (size_t)q * ldx;
-        Cx<R> vp[MAXE], vq[MAXE];
-        R al = 0, be = 0;
-        Cx<R> ga = cx<R>(0, 0);
+        const bool active = pi < mm / 2 && p < n && q < n;
+        R* xp = X + (size_t)p * ldx;
+        R* xq = X + (size_t)q * ldx;
+        R vp[MAXE], vq[MAXE];
+        R al = 0, be = 0, ga = 0;
 #pragma unroll
         for (int e = 0; e < MAXE; ++e) {
           const int idx = lane + e * G;
-          if (active && e < ept && idx < len) {
-            vp[e] = xp[idx];
-            vq[e] = xq[idx];
-          } else {
-            vp[e] = cx<R>(0, 0);
-            vq[e] = cx<R>(0, 0);
-          }
-          al += norm2(vp[e]);
-          be += norm2(vq[e]);
-          cmac_conj(ga, vp[e], vq[e]);
+          const bool in = active && e < ept && idx < n;
+          vp[e] = in ? xp[idx] : R(0);
+          vq[e] = in ? xq[idx] : R(0);
+          al = fma(vp[e], vp[e], al);
+          be = fma(vq[e], vq[e], be);
+          ga = fma(vp[e], vq[e], ga);
         }
         for (int o = G >> 1; o > 0; o >>= 1) {
           al += __shfl_xor_sync(0xffffffffu, al, o, G);
           be += __shfl_xor_sync(0xffffffffu, be, o, G);
-          ga.x += __shfl_xor_sync(0xffffffffu, ga.x, o, G);
-          ga.y += __shfl_xor_sync(0xffffffffu, ga.y, o, G);
+          ga += __shfl_xor_sync(0xffffffffu, ga, o, G);
         }
-        const R ag = sqrt(norm2(ga));
+        const R ag = rabs(ga);
         if (active && ag > R(0) && (double)fmin(al, be) > zero2 && ag > tol * sqrt(al) * sqrt(be)) {
-          const R zeta = (be - al) / (R(2) * ag);
+          const R zeta = (be - al) / (R(2) * ga);
           const R az = rabs(zeta);
           const R t = az > R(1e15) ? R(0.5) / zeta : copysign(R(1), zeta) / (az + sqrt(R(1) + zeta * zeta));
           if (t != R(0)) {
             const R cs = R(1) / sqrt(R(1) + t * t), sn = cs * t;
-            const Cx<R> sph = cx<R>(sn * ga.x / ag, sn * ga.y / ag);
 #pragma unroll
             for (int e = 0; e < MAXE; ++e) {
               const int idx = lane + e * G;
-              if (e < ept && idx < len) {
-                const Cx<R> a = vp[e], b = vq[e];
-                xp[idx] = cs * a - conj(sph) * b;
-                xq[idx] = sph * a + cs * b;
+              if (e < ept && idx < n) {
+                const R a = vp[e], b = vq[e];
+                xp[idx] = cs * a - sn * b;
+                xq[idx] = sn * a + cs * b;
               }
             }
             rotated = 1;
