@@ -133,7 +133,6 @@ struct mps_s {
   std::vector<cudaEvent_t> kev;
   std::vector<uint8_t> kev_kind;   // per used pair: 0 tensor-core GEMM, 1 close
   size_t kev_used = 0;
-  size_t tc_floats = 0;
   double* d_theta = nullptr;
   size_t theta_cap = 0;
   uint8_t* d_occ = nullptr;
@@ -277,18 +276,28 @@ static int ensure_theta(mps_s* m, size_t count) {
 
 // Chunked measurement plan. The prefix trie is walked depth first in chunks of
 // consecutive nodes of one level, so only one chunk per level is live: level k keeps
-// environment buffers (L: chi^2, T: 2 chi^2 complex entries per node) for cap[k] nodes.
-// cap[k] = min(nodes of level k, U) with U set by a per-handle budget (4 GiB of level
-// buffers for chi <= 128, 48 GiB above) spread over the levels; in mixed precision the
-// tensor-core scratch holds tc_nodes nodes (about 1 GiB for chi <= 128, 4 GiB above).
-constexpr int kTcMinDim = 128;    // levels with both bonds >= 128 use the tensor cores
+// environment buffers (L: chi^2, T, where a route needs it: 2 chi^2 complex entries per
+// node) for cap[k] nodes. cap[k] = min(nodes of level k, U) with U set by a per-handle
+// budget (4 GiB of level buffers for chi <= 128, 48 GiB above) spread over the levels.
+// Mixed-precision levels with both bonds >= kTcMinDim use the tensor cores. Against the
+// fused FP32 kernel (k_level_fused) on a 24-qubit molecular Hamiltonian: 2.8 ms instead of
+// 3.8 at bonds of 34, 3.1 / 4.5 at 40, 4.1 / 5.9 at 49, 5.1 / 8.8 at 64; against the tiled
+// FP32 kernels (k_level_T, k_level_child) 4.3 / 5.2 at 96 and 6.6 / 9.6 at 127 (16-qubit
+// Hamiltonian). At 32 and less a tile is mostly padding. With fewer nodes than SMs the fused
+// kernel is one wave whatever their number and one launch instead of three: with 100 strings
+// 0.87 ms instead of 1.01 at 34, 1.08 / 1.10 at 49, 1.24 / 1.09 at 64, so bonds up to 48
+// want kTcMinNodes.
+constexpr int kTcMinDim = 33, kTcMinNodes = 152, kTcAnyNodes = 49;
 struct MeasPlan {
   std::vector<int32_t> cap;
   size_t level_bytes = 0, tc_bytes = 0;
 };
-// Bytes of T per node: two D x D' blocks, or T^T with its padded node stride.
-static size_t t_bytes(int chi, size_t es) {
-  return chi <= kFusedMax ? 0 : 2 * (size_t)chi * env_tc_node_stride(chi) * es;
+// Entries of L per node.
+static size_t l_entries(int chi, bool mixed) { return mixed ? env_node<float>(chi) : env_node<double>(chi); }
+// Bytes of T per node: two D x D' blocks, or T^T with its padded node stride. The fused
+// levels keep T in shared memory.
+static size_t t_bytes(int chi, size_t es, bool mixed) {
+  return chi <= (mixed ? std::min(kTcMinDim - 1, kFusedMax) : kFusedMax) ? 0 : 2 * (size_t)chi * env_rows(chi) * es;
 }
 static MeasPlan meas_plan(const Trie& t, int chi, size_t es, bool mixed, size_t budget = 0) {
   MeasPlan p;
@@ -299,15 +308,15 @@ static MeasPlan meas_plan(const Trie& t, int chi, size_t es, bool mixed, size_t 
   p.cap.assign(t.n, 0);
   for (int k = 0; k < t.n_levels; ++k) {
     p.cap[k] = std::min(t.level_nodes[k], U);
-    // bonds up to kFusedMax keep T in shared memory
-    p.level_bytes += (size_t)p.cap[k] * (chi2 * es + t_bytes(chi, es));
+    p.level_bytes += (size_t)p.cap[k] * (l_entries(chi, mixed) * es + t_bytes(chi, es, mixed));
   }
   if (mixed && chi >= kTcMinDim) p.tc_bytes = env_tc_scratch_floats(chi) * sizeof(float);
   return p;
 }
 
 static int ensure_meas(mps_s* m, ham_s* h) {
-  const size_t chi2 = (size_t)m->chi * m->chi;
+  const bool mixed = m->prec == MPS_MIXED;
+  const size_t chi2 = (size_t)m->chi * m->chi, chiL = l_entries(m->chi, mixed);
   const int64_t terms = std::max<int64_t>(1, (int64_t)h->terms.size());
   reset_alloc_count();
   if (!m->w.R) {
@@ -316,10 +325,10 @@ static int ensure_meas(mps_s* m, ham_s* h) {
     m->w.R = p;
     TRY(dev_alloc(&p, (size_t)m->dm.slot_elems * m->es, "B-hat", m->st));
     m->w.Bhat = p;
-    TRY(dev_alloc(&p, (size_t)m->n * 4 * chi2 * m->es, "per-letter right blocks", m->st));
+    TRY(dev_alloc(&p, (size_t)m->n * 4 * chiL * m->es, "per-letter right blocks", m->st));
     m->w.Q = p;
   }
-  const MeasPlan plan = meas_plan(h->trie, m->chi, m->es, m->prec == MPS_MIXED, m->meas_budget);
+  const MeasPlan plan = meas_plan(h->trie, m->chi, m->es, mixed, m->meas_budget);
   m->lvl_L.resize(m->n, nullptr);
   m->lvl_T.resize(m->n, nullptr);
   m->lvl_cap.resize(m->n, 0);
@@ -329,9 +338,9 @@ static int ensure_meas(mps_s* m, ham_s* h) {
     dfree(m->lvl_T[k], m->st);
     m->lvl_L[k] = m->lvl_T[k] = nullptr;
     m->lvl_cap[k] = 0;
-    TRY(dev_alloc(&m->lvl_L[k], (size_t)plan.cap[k] * chi2 * m->es, "environment buffer", m->st));
-    if (m->chi > kFusedMax)
-      TRY(dev_alloc(&m->lvl_T[k], (size_t)plan.cap[k] * t_bytes(m->chi, m->es), "T buffer", m->st));
+    TRY(dev_alloc(&m->lvl_L[k], (size_t)plan.cap[k] * chiL * m->es, "environment buffer", m->st));
+    if (const size_t t = t_bytes(m->chi, m->es, mixed))
+      TRY(dev_alloc(&m->lvl_T[k], (size_t)plan.cap[k] * t, "T buffer", m->st));
     m->lvl_cap[k] = plan.cap[k];
   }
   if (plan.tc_bytes && !m->tc.scratch) {
@@ -451,8 +460,8 @@ static int upload_reset(mps_s* m, int slot0, int count, const uint8_t* occ_rows)
 // level k has its environments L in lvl_L[k]; T_j = L B_k^j goes to lvl_T[k], the
 // strings that close at level k are evaluated from it, and the children are built and
 // walked chunk by chunk. Mixed precision runs the contractions of levels whose bonds
-// are both >= kTcMinDim on the tensor cores (env_tc.cu), the others on the CUDA-core
-// tile kernels; both use the same buffer layouts.
+// are both >= kTcMinDim on the tensor cores (env_tc.cu), the others on the CUDA cores; L
+// has the same layout for all.
 struct MeasWalk {
   mps_s* m;
   ham_s* h;
@@ -484,9 +493,8 @@ static int meas_chunk(MeasWalk& c, int k, int u0, int u1) {
   const int U = u1 - u0, D = c.r[k], Dp = c.r[k + 1];
   void* L = m->lvl_L[k];
   void* T = m->lvl_T[k];
-  // the tensor-core route reads L in place as rows of 2D floats, which TMA needs 16-byte
-  // aligned: levels with an odd left bond stay on the CUDA-core kernels
-  const bool tc = m->prec == MPS_MIXED && m->tc.scratch && D >= kTcMinDim && Dp >= kTcMinDim && (D & 1) == 0;
+  const bool tc = m->prec == MPS_MIXED && m->tc.scratch && D >= kTcMinDim && Dp >= kTcMinDim &&
+                  (U >= kTcMinNodes || std::max(D, Dp) >= kTcAnyNodes);
   const bool fused = !tc && D <= kFusedMax && Dp <= kFusedMax;
   const bool leaf = k + 1 >= t.n_levels || k + 1 >= m->n;
   if (tc && !leaf) {
@@ -520,17 +528,20 @@ static int meas_chunk(MeasWalk& c, int k, int u0, int u1) {
   }
   if (leaf) return MPS_OK;
   const auto& par = t.parent[k + 1];
-  int64_t a = std::lower_bound(par.begin(), par.end(), u0) - par.begin();
+  const int64_t c0 = std::lower_bound(par.begin(), par.end(), u0) - par.begin();
+  int64_t a = c0;
   const int64_t c1 = std::lower_bound(par.begin(), par.end(), u1) - par.begin();
   while (a < c1) {
     int64_t b = a + 1;
     while (b < c1 && b - a < m->lvl_cap[k + 1]) ++b;
     if (tc) {
-      // the shared operands of site k live in the scratch, which the deeper levels of
-      // the previous sub-chunk have used for their own sites: rebuild them
-      const Cx<float>* Bk = (const Cx<float>*)m->dm.B + (size_t)c.slot * m->dm.slot_elems + m->site_off[k];
-      CU(env_tc_site(m->tc, Bk, D, Dp, m->st));
-      ++c.launches;
+      if (a > c0) {
+        // the shared operands of site k live in the scratch, which the deeper levels of
+        // the previous sub-chunk have used for their own sites: rebuild them
+        const Cx<float>* Bk = (const Cx<float>*)m->dm.B + (size_t)c.slot * m->dm.slot_elems + m->site_off[k];
+        CU(env_tc_site(m->tc, Bk, D, Dp, m->st));
+        ++c.launches;
+      }
       cudaEvent_t e0, e1;
       TRY(next_event_pair(m, &e0, &e1));
       const int nch = (int)(b - a);
@@ -568,10 +579,10 @@ static int run_measure(mps_s* m, ham_s* h, int slot, double* out_host, bool term
   CU(launch_right_envs(m->dm, m->prec, slot, c.r.data(), m->w, m->st, &c.launches));
   const Trie& t = h->trie;
   if (t.n_levels > 0) {
-    // root environment L_0 = [1] (one node, D_0 = 1)
+    // root environment L_0 = [1] (one node, D_0 = 1, in FP32 with its row's second entry)
     static const double one_d[2] = {1.0, 0.0};
-    static const float one_f[2] = {1.0f, 0.0f};
-    CU(cudaMemcpyAsync(m->lvl_L[0], m->prec == MPS_FP64 ? (const void*)one_d : (const void*)one_f, m->es,
+    static const float one_f[4] = {1.0f, 0.0f, 0.0f, 0.0f};
+    CU(cudaMemcpyAsync(m->lvl_L[0], m->prec == MPS_FP64 ? (const void*)one_d : (const void*)one_f, 16,
                        cudaMemcpyHostToDevice, m->st));
     TRY(meas_chunk(c, 0, 0, t.level_nodes[0]));
   }
@@ -769,7 +780,7 @@ int mps_estimate_bytes(int n_qubits, int chi, int precision, int n_slots, circ_t
              + S * (8 + 16 + 64 + n + 24) + (size_t)n * 8;
   const size_t chi2 = (size_t)chi * chi;
   b += (size_t)(n + 1) * chi2 * es + slot * es;     // right environments, B-hat
-  b += (size_t)n * 4 * chi2 * es;                   // per-letter right blocks
+  b += (size_t)n * 4 * l_entries(chi, precision == MPS_MIXED) * es;   // per-letter right blocks
   if (circ) b += circ->comp.gates.size() * sizeof(GateRec) + circ->comp.mats.size() * 16 +
                  S * std::max(1, circ->comp.n_params) * 8;
   if (ham) {

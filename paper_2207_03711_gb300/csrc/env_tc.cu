@@ -23,16 +23,18 @@
 //           A2 row (c', re) = [ Re B^0[:, c'],  Im B^0[:, c'],  Re B^1[:, c'],  Im B^1[:, c'] ],
 //           A2 row (c', im) = [-Im B^0[:, c'],  Re B^0[:, c'], -Im B^1[:, c'],  Re B^1[:, c'] ],
 //           each a range padded with zeros to a multiple of 32; the product goes to the
-//           children's L as complex entries.
+//           children's L as complex entries. Bonds up to 64 put two children into one
+//           tile of 128 columns.
 // No layout pass is left around the GEMMs: packing W and placing the children took 12 % of
 // a 64-qubit chi = 256 measurement (11.5 + 7.6 of 148 ms, a 10-orbital Hamiltonian).
-// Both run on tc_gemm.cu (tcgen05, compensated TF32 splits). Level buffers are dense: L[u]
-// at u D^2 (leading dimension D); T^T has a stride of Dn floats per node, D rounded up to a
-// multiple of 4 (TMA rows and boxes start on 16-byte boundaries).
+// Both run on tc_gemm.cu (tcgen05, compensated TF32 splits). L[u] has an even leading
+// dimension (env_ld) and Dn rows, D rounded up to a multiple of 4, zeros in the ones added;
+// so T^T has Dn columns per node (TMA rows and boxes start on 16-byte boundaries).
 #include <cstdint>
 
 #include "cx.cuh"
 #include "env_tc.cuh"
+#include "kernels.cuh"
 #include "tc_gemm.cuh"
 
 namespace mpsvqe {
@@ -54,16 +56,18 @@ __device__ __forceinline__ void split_store(float z, float* hi, float* lo) {
   *lo = __uint_as_float(b);
 }
 
-// BT (4D' x 2D) and A2 (2D' x 4 Dk, Dk = D rounded up to 32) from site k (B[b][j][c] at
+// BT (4D' x 2D, leading dimension 2 env_ld(D)) and A2 (2D' x 4 Dk, Dk = D rounded up to 32) from site k (B[b][j][c] at
 // (b 2 + j) D' + c), hi and lo planes.
 __global__ void k_tc_site_operands(const Cx<float>* Bk, int D, int Dp, int Dk, float* bt, float* bt_lo, float* a2,
                                    float* a2_lo) {
-  const int64_t nbt = (int64_t)4 * Dp * 2 * D, na2 = (int64_t)2 * Dp * 4 * Dk;
+  const int ldb = 2 * env_ld<float>(D);
+  const int64_t nbt = (int64_t)4 * Dp * ldb, na2 = (int64_t)2 * Dp * 4 * Dk;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nbt + na2;
        i += (int64_t)gridDim.x * blockDim.x) {
     if (i < nbt) {
-      const int64_t row = i / (2 * D);
-      const int col = (int)(i - row * 2 * D);
+      const int64_t row = i / ldb;
+      const int col = (int)(i - row * ldb);
+      if (col >= 2 * D) continue;   // never loaded
       const int c = (int)(row % Dp), ro = (int)(row / Dp) & 1, j = (int)(row / Dp) >> 1;
       const int b = col >> 1, ri = col & 1;
       const Cx<float> z = Bk[((size_t)b * 2 + j) * Dp + c];   // B^j[b][c]
@@ -90,7 +94,7 @@ namespace {
 struct Parts {
   float *bt, *bt_lo, *a2, *a2_lo;
 };
-int64_t part_bt(int chi) { return ((int64_t)8 * chi * chi + 63) & ~(int64_t)63; }
+int64_t part_bt(int chi) { return ((int64_t)8 * chi * env_ld<float>(chi) + 63) & ~(int64_t)63; }
 int64_t part_a2(int chi) { return ((int64_t)8 * chi * pad32(chi) + 63) & ~(int64_t)63; }
 Parts carve(float* base, int chi) {
   return {base, base + part_bt(chi), base + 2 * part_bt(chi), base + 2 * part_bt(chi) + part_a2(chi)};
@@ -110,11 +114,12 @@ cudaError_t env_tc_T(const EnvTc& s, const Cx<float>* L, float* Tt, int U, int D
                      cudaEvent_t e0, cudaEvent_t e1) {
   if (U <= 0) return cudaSuccess;
   const Parts p = carve(s.scratch, s.chi);
-  const int Dn = env_tc_node_stride(D);
+  const int Dn = env_rows(D);
+  const int64_t ld = 2 * env_ld<float>(D);
   cudaError_t e;
   if (e0 && (e = cudaEventRecord(e0, st)) != cudaSuccess) return e;
-  e = tc::launch_gemm_presplit(tc::Plane{p.bt, 2 * (int64_t)D}, p.bt_lo, tc::Plane{(const float*)L, 2 * (int64_t)D},
-                               4 * Dp, U * D, 2 * D, Tt, (int64_t)U * Dn, D, Dn, s.err, st);
+  e = tc::launch_gemm_presplit(tc::Plane{p.bt, ld}, p.bt_lo, tc::Plane{(const float*)L, ld},
+                               4 * Dp, U * Dn, 2 * D, Tt, (int64_t)U * Dn, s.err, st);
   if (e != cudaSuccess) return e;
   if (e1 && (e = cudaEventRecord(e1, st)) != cudaSuccess) return e;
   return cudaSuccess;
@@ -125,7 +130,7 @@ cudaError_t env_tc_children(const EnvTc& s, const float* Tt, const int32_t* pare
                             cudaEvent_t e1) {
   if (nc <= 0) return cudaSuccess;
   const Parts p = carve(s.scratch, s.chi);
-  const int Dn = env_tc_node_stride(D);
+  const int Dn = env_rows(D);
   cudaError_t e;
   if (e0 && (e = cudaEventRecord(e0, st)) != cudaSuccess) return e;
   e = tc::launch_gemm_children(tc::Plane{p.a2, 4 * (int64_t)pad32(D)}, p.a2_lo, tc::Plane{Tt, (int64_t)U * Dn}, U, D,

@@ -248,15 +248,17 @@ __global__ void __launch_bounds__(256) k_letter_blocks(DevMPS m, int slot, const
         }
     }
   }
-  Cx<R>* q = Q + (size_t)k * 4 * m.chi * m.chi;
-  const size_t chi2 = (size_t)m.chi * m.chi;
+  const int ld = env_ld<R>(Dl);
+  const size_t chi2 = (size_t)m.chi * env_ld<R>(m.chi);
+  Cx<R>* q = Q + (size_t)k * 4 * chi2;
 #pragma unroll
   for (int i = 0; i < TI; ++i)
 #pragma unroll
     for (int j = 0; j < TI; ++j) {
       const int r = m0 + ty + 16 * i, c = n0 + tx + 16 * j;
       if (r < Dl && c < Dl) {
-        const size_t o = (size_t)r * Dl + c;
+        const size_t o = (size_t)r * ld + c;
+        if (c == Dl - 1 && ld > Dl) q[chi2 + o + 1] = q[2 * chi2 + o + 1] = q[3 * chi2 + o + 1] = cx<R>(0, 0);
         const Cx<R> d = g01[i][j] - g10[i][j];
         q[chi2 + o] = g01[i][j] + g10[i][j];
         q[2 * chi2 + o] = cx<R>(-d.y, d.x);   // i G01 - i G10
@@ -327,8 +329,6 @@ __device__ __forceinline__ void letter_entries(uint8_t l, int* ii, int* jj, Cx<R
   }
 }
 
-// Level buffers are dense: node u of level k holds L at u Dk^2 (leading dimension Dk)
-// and, on the CUDA-core route, T_j at (2u + j) Dk Dk1 (leading dimension Dk1).
 // T_j[u] = L_k[u] B_k^j  (Dk x Dk)(Dk x Dk1), grid (nodes, 2)
 template <class R>
 __global__ void __launch_bounds__(256) k_level_T(DevMPS m, int slot, int k, const Cx<R>* Lin, Cx<R>* T,
@@ -340,7 +340,8 @@ __global__ void __launch_bounds__(256) k_level_T(DevMPS m, int slot, int k, cons
   const int* rank = m.rank + (size_t)slot * (m.n + 1);
   const int Dk = rank[k], Dk1 = rank[k + 1];
   const Cx<R>* Bk = (const Cx<R>*)m.B + (size_t)slot * m.slot_elems + m.site_off[k];
-  GemmTerm<R> t{Lin + (size_t)u * Dk * Dk, Dk, false, Bk + j * Dk1, 2 * Dk1, cx<R>(1, 0), false};
+  const int ld = env_ld<R>(Dk);
+  GemmTerm<R> t{Lin + u * env_node<R>(Dk), ld, false, Bk + j * Dk1, 2 * Dk1, cx<R>(1, 0), false};
   block_gemm<R, 256>(Dk, Dk1, Dk, &t, 1, T + ((size_t)u * 2 + j) * Dk * Dk1, Dk1, As, Bs);
 }
 
@@ -362,7 +363,12 @@ __global__ void __launch_bounds__(256) k_level_child(DevMPS m, int slot, int k, 
   GemmTerm<R> t[2];
   for (int e = 0; e < 2; ++e)
     t[e] = GemmTerm<R>{Bk + ii[e] * Dk1, 2 * Dk1, true, T + ((size_t)u * 2 + jj[e]) * Dk * Dk1, Dk1, sg[e], false};
-  block_gemm<R, 256>(Dk1, Dk1, Dk, t, 2, Lout + (size_t)c * Dk1 * Dk1, Dk1, As, Bs);
+  const int ld = env_ld<R>(Dk1);
+  Cx<R>* out = Lout + c * env_node<R>(Dk1);
+  block_gemm<R, 256>(Dk1, Dk1, Dk, t, 2, out, ld, As, Bs);
+  for (int64_t e = threadIdx.x + (int64_t)Dk1 * ld; e < env_node<R>(Dk1); e += 256) out[e] = cx<R>(0, 0);
+  if (ld > Dk1)
+    for (int r = threadIdx.x; r < Dk1; r += 256) out[(size_t)r * ld + Dk1] = cx<R>(0, 0);
 }
 
 // Fused level for bonds up to 64: both T_j of a group of parents stay in shared memory and
@@ -397,12 +403,13 @@ __global__ void __launch_bounds__(256) k_level_fused(DevMPS m, LevelArgs g, cons
   Cx<float>* Ts = Ls + 64 * (D + 1);            // [rows][2 D']
   const Cx<float>* Bk = (const Cx<float>*)m.B + (size_t)g.slot * m.slot_elems + m.site_off[g.k];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int rows = (u1 - u0) * D;
-  const Cx<float>* Lu = Lin + (size_t)(u0 - g.node_base) * D * D;
+  const int rows = (u1 - u0) * D, ld = env_ld<float>(D), ldp = env_ld<float>(Dp);
+  const int64_t node = env_node<float>(D);
+  const Cx<float>* Lu = Lin + (u0 - g.node_base) * node;
   for (int e = tid; e < D * W; e += 256) Bs[e] = Bk[e];
   for (int e = tid; e < rows * D; e += 256) {
     const int r = e / D, c = e - r * D;
-    Ls[r * (D + 1) + c] = Lu[e];
+    Ls[r * (D + 1) + c] = Lu[r / D * node + r % D * ld + c];
   }
   __syncthreads();
   {
@@ -482,15 +489,17 @@ __global__ void __launch_bounds__(256) k_level_fused(DevMPS m, LevelArgs g, cons
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       if (n0 + tx + 16 * j >= ncol) continue;
-      Cx<float>* o = Lout + (size_t)(c0 + ch[j] - g.c_lo) * Dp * Dp + cc[j];
+      Cx<float>* o = Lout + (c0 + ch[j] - g.c_lo) * env_node<float>(Dp) + cc[j];
 #pragma unroll
       for (int i = 0; i < RM; ++i) {
         const int r = ty + 16 * i;
-        if (r >= Dp) continue;
+        if (r >= env_rows(Dp)) continue;
         Cx<float> v = acc[i][j];
         if (let[j] == 2) v = cx<float>(-v.y, v.x);       // s1 = i
         if (let[j] == 3) v = cx<float>(-v.x, -v.y);      // s1 = -1
-        o[(size_t)r * Dp] = v;
+        if (r >= Dp) v = cx<float>(0.f, 0.f);
+        o[(size_t)r * ldp] = v;
+        if (ldp > Dp && cc[j] == Dp - 1) o[(size_t)r * ldp + 1] = cx<float>(0.f, 0.f);
       }
     }
   }
@@ -567,7 +576,7 @@ cudaError_t launch_level_fused(const DevMPS& m, int prec, int slot, int k, int D
 // sum_ab L[u][a][b] conj(Q_k^P[a][b]), Q_k^P = sum_ij conj(P_ij) Bhat_k^i (B_k^j)^+ from the
 // right-environment pass. This equals sum_ij P_ij <Bhat_k^i, L[u] B_k^j>_F (Eq. 11 with
 // the right part contracted first) and reads one D x D block of the node instead of the
-// two D x D' blocks of T. Both blocks are contiguous with leading dimension D.
+// two D x D' blocks of T. Both blocks are contiguous with leading dimension env_ld(D).
 template <class R>
 __global__ void __launch_bounds__(256) k_level_close(DevMPS m, int slot, int k, const int32_t* cnode,
                                                      const uint8_t* cletter, const int32_t* cterm,
@@ -575,12 +584,12 @@ __global__ void __launch_bounds__(256) k_level_close(DevMPS m, int slot, int k, 
                                                      int node_base) {
   __shared__ double red[2][8];
   const int c = blockIdx.x;
-  const int chi2 = m.chi * m.chi;
+  const int chi2 = m.chi * env_ld<R>(m.chi);
   const int* rank = m.rank + (size_t)slot * (m.n + 1);
-  const int Dk = rank[k];
-  const Cx<R>* Lu = L + (size_t)(cnode[c] - node_base) * Dk * Dk;
+  const int Dk = rank[k], ld = env_ld<R>(Dk);
+  const Cx<R>* Lu = L + (cnode[c] - node_base) * env_node<R>(Dk);
   const Cx<R>* Qp = Q + ((size_t)k * 4 + (cletter[c] & 3)) * chi2;
-  const int n = Dk * Dk;
+  const int n = Dk * ld;
   double re = 0.0, im = 0.0;
   // R = float: FP32 products summed in FP32 over runs of 8 entries, the runs summed in
   // FP64. GB300's FP64 (and FP32 -> FP64 conversion) throughput is a small fraction of

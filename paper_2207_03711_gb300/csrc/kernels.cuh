@@ -61,7 +61,7 @@ cudaError_t launch_circuit(const DevMPS& m, int prec, const CircDev& c, int64_t 
 struct MeasDev {
   void* R;          // complex<R> [n+1][chi*chi] right identity environments R_k
   void* Bhat;       // complex<R> like one slot of B: B_k^i R_{k+1}
-  void* Q;          // complex<R> [n][4][chi*chi]: Q_k^P = sum_ij conj(P_ij) Bhat_k^i (B_k^j)^+ per letter P
+  void* Q;          // complex<R> [n][4][chi env_ld(chi)]: Q_k^P = sum_ij conj(P_ij) Bhat_k^i (B_k^j)^+ per letter P
   double* vals;     // [n_terms][2] re, im of unnormalised <P>
   double* out;      // [4 + n_terms*2]: E, norm, ...
   double* part;     // [energy_sum_blocks][2]: (sum, correction) per block of the energy sum
@@ -75,9 +75,23 @@ void set_error_message(const char* msg);
 // ranks: the slot's n+1 bond ranks on the host (ranks[k] = left dimension of site k).
 cudaError_t launch_right_envs(const DevMPS& m, int prec, int slot, const int* ranks, MeasDev& w, cudaStream_t st,
                               int* launches);
+// Leading dimension of a D x D environment L: an FP32 row starts on a 16-byte boundary, so
+// that the tensor-core route can read it in place; the entry an odd D leaves over is zero.
+// The per-letter right blocks have the same layout.
+template <class R>
+__host__ __device__ constexpr int env_ld(int D) {
+  return sizeof(R) == 4 ? D + (D & 1) : D;
+}
+// Entries from one node's L to the next. FP32 rounds the rows up to a multiple of 4, zeros
+// below the D-th, so that the columns (node, row) of T^T start on 16-byte boundaries too.
+__host__ __device__ constexpr int env_rows(int D) { return (D + 3) & ~3; }
+template <class R>
+__host__ __device__ constexpr int64_t env_node(int D) {
+  return sizeof(R) == 4 ? (int64_t)env_rows(D) * env_ld<R>(D) : (int64_t)D * D;
+}
 // Chunked trie levels. Environment buffers: L holds node u's D_k x D_k block (row-major,
-// leading dimension D_k) at u chi^2 complex entries; T holds T_j[u] = L[u] B_k^j
-// (D_k x D_{k+1}, leading dimension D_{k+1}) at (2u + j) chi^2. Node indices in cnode /
+// leading dimension env_ld(D_k)) at u env_node(D_k) complex entries; T holds T_j[u] =
+// L[u] B_k^j (D_k x D_{k+1}, dense) at (2u + j) D_k D_{k+1}. Node indices in cnode /
 // parent are absolute trie indices; node_base is the trie index of buffer entry 0.
 // cb: first child of each of the n_nodes nodes (nodes without children are left out).
 cudaError_t launch_env_T(const DevMPS& m, int prec, int slot, int k, const void* L, void* T, int n_nodes,

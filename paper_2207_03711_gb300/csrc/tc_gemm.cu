@@ -59,7 +59,7 @@ constexpr int TILE_A = BM * BK * 4;                   // 16 KB
 constexpr int TILE_B = BN * BK * 4;                   // 16 KB
 constexpr int STAGE_BYTES = 2 * TILE_A + 2 * TILE_B;  // hi and lo of both operands: 64 KB
 constexpr int NBARS = 3 * STAGES + 4;                 // full, split, empty per stage; ready, free per buffer
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 8 * NBARS + 16 + 4 * STAGES;
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 8 * NBARS + 16 + 8 * STAGES;
 constexpr int NTHREADS = 448;
 constexpr int NEPI = 256;                             // epilogue threads (warps 2..9)
 constexpr int EPI_COLS = BN / 2;                      // columns per epilogue thread
@@ -182,8 +182,7 @@ __device__ __forceinline__ float tf32_rna(float v) {
 }
 
 // What a K tile of the second operand is, and where the product goes.
-//   kPlain     rows n0.. of B; C row-major (optionally with the columns of each group of
-//              cmod spread to a stride of cpad, the gap written as zeros)
+//   kPlain     rows n0.. of B; C row-major
 //   kChildren  environments of trie children (env_tc.cu): B is T^T, the rows (j, re/im, c) of
 //              T_j over columns (node, a), leading dimension tdn per node. Column tile
 //              (child, c0) at inner index (i, re/im, a) is the box of T^T at the child's
@@ -193,8 +192,11 @@ enum Mode { kPlain, kChildren };
 struct Children {
   const int32_t* parent = nullptr;
   const uint8_t* edge = nullptr;
-  int node_base = 0, nc = 0, Dp = 0, tdn = 0, seg_tiles = 0;
+  int node_base = 0, nc = 0, Dp = 0, ldp = 0, tdn = 0, seg_tiles = 0;
+  int pack = 1;   // children per column tile: bonds up to 64 share it, 64 columns each
   Cx<float>* L = nullptr;
+  __host__ __device__ int per() const { return (Dp + BN - 1) / BN; }               // column tiles per child
+  __host__ __device__ int tiles_n() const { return (nc + pack - 1) / pack * per(); }
 };
 // Letter l, inner segment seg = 2 i + re/im of W_i = sum_j P_ij T_j (I: (T_0, T_1); X: (T_1,
 // T_0); Y: (-i T_1, i T_0); Z: (T_0, -T_1)) -> row block 2 j + re/im' of T^T and the sign.
@@ -209,8 +211,8 @@ __device__ __forceinline__ int child_block(int l, int seg, float* sign) {
 template <bool PRE, Mode MODE>
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_gemm_tf32x3(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmAl,
-                  const __grid_constant__ CUtensorMap tmB, float* C, int64_t ldc, int M, int N, int K, int cmod,
-                  int cpad, const __grid_constant__ Children chd, int* err) {
+                  const __grid_constant__ CUtensorMap tmB, float* C, int64_t ldc, int M, int N, int K,
+                  const __grid_constant__ Children chd, int* err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   // barriers: full[s] (TMA), split[s] (hi/lo written), empty[s] (MMAs done), ready[b], freed[b]
@@ -221,11 +223,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   uint64_t* ready = bars + 3 * STAGES;
   uint64_t* freed = bars + 3 * STAGES + 2;
   uint32_t* tmem_slot = (uint32_t*)(bars + NBARS);
-  float* sgn = (float*)(tmem_slot + 4);   // sign of the B tile in each stage
+  float* sgn = (float*)(tmem_slot + 4);   // signs of the B tile's two halves in each stage
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nk = (K + BK - 1) / BK;
   const int tiles_m = (M + BM - 1) / BM;
-  const int tiles_n = MODE == kPlain ? (N + BN - 1) / BN : chd.nc * ((chd.Dp + BN - 1) / BN);
+  const int tiles_n = MODE == kPlain ? (N + BN - 1) / BN : chd.tiles_n();
   const int tiles = tiles_n * tiles_m;
   // plain: A may be the long side, columns vary fastest; children: rows do, so that CTAs
   // side by side share a child's tile
@@ -270,12 +272,17 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       int mt, nt;
       tile_at(blockIdx.x + n * gridDim.x, &mt, &nt);
       const int m0 = mt * BM;
-      int letter = 0, x0 = 0, y0 = nt * BN;
+      int letter[2] = {0, 0}, x0[2] = {0, 0}, y0 = nt * BN;
       if (MODE == kChildren) {
-        const int per = (chd.Dp + BN - 1) / BN, ch = nt / per;
-        letter = chd.edge[ch];
-        x0 = (chd.parent[ch] - chd.node_base) * chd.tdn;
-        y0 = (nt - ch * per) * BN;
+        const int per = chd.per(), grp = nt / per;
+        y0 = (nt - grp * per) * BN;
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+          // a last tile without its second child loads the first one twice
+          const int ch = min(grp * chd.pack + (p < chd.pack ? p : 0), chd.nc - 1);
+          letter[p] = chd.edge[ch];
+          x0[p] = (chd.parent[ch] - chd.node_base) * chd.tdn;
+        }
       }
       for (int kt = 0; kt < nk; ++kt, ++g) {
         const int s = g % STAGES;
@@ -285,18 +292,23 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         }
         unsigned char* st = base + s * STAGE_BYTES;
         const uint32_t fb = smem_u32(&full[s]);
-        int x = kt * BK, y = y0;
+        int x[2] = {kt * BK, 0}, y[2] = {y0, 0};
         if (MODE == kChildren) {
           const int seg = kt / chd.seg_tiles;
-          x = x0 + (kt - seg * chd.seg_tiles) * BK;
-          float sg;
-          y = child_block(letter, seg, &sg) * chd.Dp + y0;
-          sgn[s] = sg;   // released by the arrival below
+#pragma unroll
+          for (int p = 0; p < 2; ++p) {
+            x[p] = x0[p] + (kt - seg * chd.seg_tiles) * BK;
+            float sg;
+            y[p] = child_block(letter[p], seg, &sg) * chd.Dp + y0;
+            sgn[2 * s + p] = sg;   // released by the arrival below
+          }
         }
         mbar_arrive_expect_tx(fb, (PRE ? 2 : 1) * TILE_A + TILE_B);
         tma_load_2d(smem_u32(st), &tmA, kt * BK, m0, fb);
         if (PRE) tma_load_2d(smem_u32(st + TILE_A), &tmAl, kt * BK, m0, fb);
-        tma_load_2d(smem_u32(st + 2 * TILE_A), &tmB, x, y, fb);
+        tma_load_2d(smem_u32(st + 2 * TILE_A), &tmB, x[0], y[0], fb);
+        if (MODE == kChildren && chd.pack == 2)   // boxes of half a tile
+          tma_load_2d(smem_u32(st + 2 * TILE_A + TILE_B / 2), &tmB, x[1], y[1], fb);
       }
     }
     // no copy may still be landing in shared memory when the CTA exits: wait (bounded)
@@ -327,7 +339,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       float4* al = (float4*)(st + TILE_A);
       float4* bh = (float4*)(st + 2 * TILE_A);
       float4* bl = (float4*)(st + 2 * TILE_A + TILE_B);
-      const float sg = MODE == kChildren ? sgn[s] : 1.f;
+      const float sg0 = MODE == kChildren ? sgn[2 * s] : 1.f, sg1 = MODE == kChildren ? sgn[2 * s + 1] : 1.f;
 #pragma unroll 4
       for (int v = ct; v < (PRE ? 0 : TILE_A / 16); v += NCONV) {
         const float4 x = ah[v];
@@ -342,7 +354,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 #pragma unroll 4
       for (int v = ct; v < TILE_B / 16; v += NCONV) {
         float4 x = bh[v];
-        if (MODE == kChildren) x = make_float4(sg * x.x, sg * x.y, sg * x.z, sg * x.w);
+        if (MODE == kChildren) {
+          const float sg = v < TILE_B / 32 ? sg0 : sg1;   // one child: the two are the same
+          x = make_float4(sg * x.x, sg * x.y, sg * x.z, sg * x.w);
+        }
         float4 h, l;
         h.x = tf32_rna(x.x); l.x = tf32_rna(x.x - h.x);
         h.y = tf32_rna(x.y); l.y = tf32_rna(x.y - h.y);
@@ -421,7 +436,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       if (MODE == kChildren) {
         // lanes 2x and 2x + 1 hold the real and imaginary rows of one c': each takes half of
         // the columns of both
-        const int per = (chd.Dp + BN - 1) / BN, ch = nt / per, cc = (nt - ch * per) * BN + c_lo;
+        const int per = chd.per(), grp = nt / per;
+        const int ch = chd.pack == 2 ? 2 * grp + c_lo / EPI_COLS : grp;
+        const int cc = chd.pack == 2 ? 0 : (nt - grp * per) * BN + c_lo;
         const bool odd = lane & 1;
         Cx<float> z[EPI_COLS / 2];
 #pragma unroll
@@ -430,45 +447,32 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           const float got = __shfl_xor_sync(0xffffffffu, odd ? sum[c] : sum[c + EPI_COLS / 2], 1);
           z[c] = odd ? cx<float>(got, mine) : cx<float>(mine, got);
         }
-        if (ok && row < M) {
+        // rows of A past M are zeros, and so are the rows of L that they give
+        if (ok && row < 2 * env_rows(chd.Dp) && ch < chd.nc) {
           const int c0 = cc + (odd ? EPI_COLS / 2 : 0);
-          Cx<float>* out = chd.L + ((size_t)ch * chd.Dp + (row >> 1)) * chd.Dp + c0;
-          if ((chd.Dp & 1) == 0 && c0 + EPI_COLS / 2 <= chd.Dp) {
+          Cx<float>* out = chd.L + ch * env_node<float>(chd.Dp) + (int64_t)(row >> 1) * chd.ldp + c0;
+          if (c0 + EPI_COLS / 2 <= chd.Dp) {
 #pragma unroll
             for (int c = 0; c < EPI_COLS / 2; c += 2)
               *reinterpret_cast<float4*>(out + c) = make_float4(z[c].x, z[c].y, z[c + 1].x, z[c + 1].y);
           } else {
 #pragma unroll
-            for (int c = 0; c < EPI_COLS / 2; ++c)
+            for (int c = 0; c < EPI_COLS / 2; ++c) {
               if (c0 + c < chd.Dp) out[c] = z[c];
+              else if (c0 + c < chd.ldp) out[c] = cx<float>(0.f, 0.f);
+            }
           }
         }
       } else if (ok && row < M) {
-        if (cmod) {
-          int u = n0 / cmod, x = n0 - u * cmod;
-          float* out = C + (size_t)row * ldc + (size_t)u * cpad;
+        float* out = C + (size_t)row * ldc + n0;
+        if (vec && n0 + EPI_COLS <= N) {
 #pragma unroll
-          for (int c = 0; c < EPI_COLS; ++c) {
-            if (n0 + c < N) {
-              out[x] = sum[c];
-              if (++x == cmod) {
-                for (; x < cpad; ++x) out[x] = 0.f;
-                x = 0;
-                out += cpad;
-              }
-            }
-          }
+          for (int c = 0; c < EPI_COLS; c += 4)
+            *reinterpret_cast<float4*>(out + c) = make_float4(sum[c], sum[c + 1], sum[c + 2], sum[c + 3]);
         } else {
-          float* out = C + (size_t)row * ldc + n0;
-          if (vec && n0 + EPI_COLS <= N) {
 #pragma unroll
-            for (int c = 0; c < EPI_COLS; c += 4)
-              *reinterpret_cast<float4*>(out + c) = make_float4(sum[c], sum[c + 1], sum[c + 2], sum[c + 3]);
-          } else {
-#pragma unroll
-            for (int c = 0; c < EPI_COLS; ++c)
-              if (n0 + c < N) out[c] = sum[c];
-          }
+          for (int c = 0; c < EPI_COLS; ++c)
+            if (n0 + c < N) out[c] = sum[c];
         }
       }
     }
@@ -536,7 +540,7 @@ cudaError_t launch_pad_rows(const float* x, int64_t ld_in, int M, int K, float* 
 
 template <bool PRE, Mode MODE>
 static cudaError_t launch(const Plane& A, const float* a_lo, const Plane& B, int M, int N, int K, int b_rows, int b_cols,
-                          float* C, int64_t ldc, int cmod, int cpad, const Children& chd, int* err, cudaStream_t st) {
+                          float* C, int64_t ldc, const Children& chd, int* err, cudaStream_t st) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   if ((A.ld & 3) || (B.ld & 3) || ((uintptr_t)A.p & 15) || ((uintptr_t)B.p & 15) || ((uintptr_t)a_lo & 15))
     return cudaErrorInvalidValue;
@@ -544,7 +548,7 @@ static cudaError_t launch(const Plane& A, const float* a_lo, const Plane& B, int
   cudaError_t e;
   if ((e = make_map(&am, A.p, M, K, A.ld, BM)) != cudaSuccess) return e;
   if ((e = make_map(&al, PRE ? a_lo : A.p, M, K, A.ld, BM)) != cudaSuccess) return e;
-  if ((e = make_map(&bm, B.p, b_rows, b_cols, B.ld, BN)) != cudaSuccess) return e;
+  if ((e = make_map(&bm, B.p, b_rows, b_cols, B.ld, BN / chd.pack)) != cudaSuccess) return e;
   if ((e = gate::raise_smem_limit<k_gemm_tf32x3<PRE, MODE>>()) != cudaSuccess) return e;
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -552,20 +556,20 @@ static cudaError_t launch(const Plane& A, const float* a_lo, const Plane& B, int
   static int sm_count[64] = {0};
   if (!sm_count[dev] && (e = cudaDeviceGetAttribute(&sm_count[dev], cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
     return e;
-  const int64_t tiles = (int64_t)(MODE == kPlain ? (N + BN - 1) / BN : chd.nc * ((chd.Dp + BN - 1) / BN)) * ((M + BM - 1) / BM);
+  const int64_t tiles = (int64_t)(MODE == kPlain ? (N + BN - 1) / BN : chd.tiles_n()) * ((M + BM - 1) / BM);
   const int grid = (int)std::min<int64_t>(tiles, sm_count[dev]);
-  k_gemm_tf32x3<PRE, MODE><<<grid, NTHREADS, SMEM_BYTES, st>>>(am, al, bm, C, ldc, M, N, K, cmod, cpad, chd, err);
+  k_gemm_tf32x3<PRE, MODE><<<grid, NTHREADS, SMEM_BYTES, st>>>(am, al, bm, C, ldc, M, N, K, chd, err);
   return cudaGetLastError();
 }
 
 cudaError_t launch_gemm_tf32x3(const Plane& A, const Plane& B, int M, int N, int K, float* C, int64_t ldc, int* err,
                                cudaStream_t st) {
-  return launch<false, kPlain>(A, nullptr, B, M, N, K, N, K, C, ldc, 0, 0, Children{}, err, st);
+  return launch<false, kPlain>(A, nullptr, B, M, N, K, N, K, C, ldc, Children{}, err, st);
 }
 
 cudaError_t launch_gemm_presplit(const Plane& A, const float* a_lo, const Plane& B, int M, int N, int K, float* C,
-                                 int64_t ldc, int cmod, int cpad, int* err, cudaStream_t st) {
-  return launch<true, kPlain>(A, a_lo, B, M, N, K, N, K, C, ldc, cmod == cpad ? 0 : cmod, cpad, Children{}, err, st);
+                                 int64_t ldc, int* err, cudaStream_t st) {
+  return launch<true, kPlain>(A, a_lo, B, M, N, K, N, K, C, ldc, Children{}, err, st);
 }
 
 cudaError_t launch_gemm_children(const Plane& A, const float* a_lo, const Plane& Tt, int U, int D, int Dn, int Dp,
@@ -577,10 +581,12 @@ cudaError_t launch_gemm_children(const Plane& A, const float* a_lo, const Plane&
   chd.node_base = node_base;
   chd.nc = nc;
   chd.Dp = Dp;
+  chd.ldp = env_ld<float>(Dp);
+  chd.pack = Dp <= BN / 2 ? 2 : 1;
   chd.tdn = Dn;
   chd.seg_tiles = (D + BK - 1) / BK;
   chd.L = L;
-  return launch<true, kChildren>(A, a_lo, Tt, 2 * Dp, nc * Dp, 4 * chd.seg_tiles * BK, 4 * Dp, U * Dn, nullptr, 0, 0, 0,
+  return launch<true, kChildren>(A, a_lo, Tt, 2 * Dp, nc * Dp, 4 * chd.seg_tiles * BK, 4 * Dp, U * Dn, nullptr, 0,
                                  chd, err, st);
 }
 

@@ -29,11 +29,9 @@ cudaError_t launch_pad_rows(const float* x, int64_t ld_in, int M, int K, float* 
 cudaError_t launch_gemm_tf32x3(const Plane& A, const Plane& B, int M, int N, int K, float* C, int64_t ldc, int* err,
                                cudaStream_t st);
 
-
-// The same with A given as hi plane A and lo plane a_lo (same leading dimension). C's
-// columns of each group of cmod may be spread to a stride of cpad (gaps become zeros).
+// The same with A given as hi plane A and lo plane a_lo (same leading dimension).
 cudaError_t launch_gemm_presplit(const Plane& A, const float* a_lo, const Plane& B, int M, int N, int K, float* C,
-                                 int64_t ldc, int cmod, int cpad, int* err, cudaStream_t st);
+                                 int64_t ldc, int* err, cudaStream_t st);
 
 // Environments of nc trie children: L[child][c'][c] = sum over (i, a) of conj(B^i[a][c'])
 // W_i[a][c], W_i = sum_j P_ij T_j[parent]. A, a_lo: planes of 2 Dp rows (c', re/im) over
