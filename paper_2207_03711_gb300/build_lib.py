@@ -48,7 +48,7 @@ def build(force=False, verbose=False):
          "-o", os.path.join(OBJ, "host.o")],
     ]
     units = ("gate_fp64", "gate_mixed1", "gate_mixed2", "gate_mixed8", "gate_raw", "gate", "kernels", "api", "tc_gemm",
-             "env_tc")
+             "env_tc", "env_fp64_tc")
     for name in units:
         jobs.append([nvcc, *ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", *inc,
                      "-c", os.path.join(CSRC, name + ".cu"), "-o", os.path.join(OBJ, name + ".o")])

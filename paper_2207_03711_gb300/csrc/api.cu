@@ -12,6 +12,7 @@
 
 #include "../../include/mpsvqe.h"
 #include "host.hpp"
+#include "env_fp64_tc.cuh"
 #include "env_tc.cuh"
 #include "kernels.cuh"
 
@@ -128,6 +129,7 @@ struct mps_s {
   std::vector<int32_t> lvl_cap;
   size_t meas_budget = 0;          // 0: the default of meas_plan
   EnvTc tc{};
+  EnvFp64 tc64{};
   // optional per-launch timing of the tensor-core GEMMs (mps_set_kernel_timing)
   bool ktime = false;
   std::vector<cudaEvent_t> kev;
@@ -161,6 +163,7 @@ struct mps_s {
     for (void* p : lvl_L) dfree(p, st);
     for (void* p : lvl_T) dfree(p, st);
     dfree(tc.scratch, st);
+    dfree(tc64.scratch, st);
     dfree(tc.err, st);
     dfree(w.vals, st);
     dfree(w.out, st);
@@ -288,9 +291,16 @@ static int ensure_theta(mps_s* m, size_t count) {
 // 0.87 ms instead of 1.01 at 34, 1.08 / 1.10 at 49, 1.24 / 1.09 at 64, so bonds up to 48
 // want kTcMinNodes.
 constexpr int kTcMinDim = 33, kTcMinNodes = 152, kTcAnyNodes = 49;
+// FP64 levels with both bonds in this range multiply by digits on the tensor cores
+// (env_fp64_tc.cu). Against the fused FP64 kernel (k_level_fused64), an 18-qubit molecular
+// Hamiltonian and 30 random strings: 3.5 ms instead of 3.0 and 1.3 instead of 0.9 at bonds of
+// 16, 4.2 / 6.8 and 1.8 / 2.0 at 20, 4.4 / 8.8 and 1.9 / 2.3 at 24, 8.6 / 62 and 3.1 / 16 at
+// 64. Up to 512 the 64-bit sums cannot overflow.
+constexpr int kFp64TcMinDim = 17, kFp64TcMaxDim = 512;
 struct MeasPlan {
   std::vector<int32_t> cap;
   size_t level_bytes = 0, tc_bytes = 0;
+  int batch = 0;   // FP64: nodes of a batch on the tensor cores
 };
 // Entries of L per node.
 static size_t l_entries(int chi, bool mixed) { return mixed ? env_node<float>(chi) : env_node<double>(chi); }
@@ -311,6 +321,10 @@ static MeasPlan meas_plan(const Trie& t, int chi, size_t es, bool mixed, size_t 
     p.level_bytes += (size_t)p.cap[k] * (l_entries(chi, mixed) * es + t_bytes(chi, es, mixed));
   }
   if (mixed && chi >= kTcMinDim) p.tc_bytes = env_tc_scratch_floats(chi) * sizeof(float);
+  if (!mixed && chi >= kFp64TcMinDim) {
+    p.batch = std::min(env_fp64_batch(chi), *std::max_element(p.cap.begin(), p.cap.end()));
+    p.tc_bytes = p.batch ? env_fp64_scratch(chi, p.batch) : 0;
+  }
   return p;
 }
 
@@ -343,7 +357,19 @@ static int ensure_meas(mps_s* m, ham_s* h) {
       TRY(dev_alloc(&m->lvl_T[k], (size_t)plan.cap[k] * t, "T buffer", m->st));
     m->lvl_cap[k] = plan.cap[k];
   }
-  if (plan.tc_bytes && !m->tc.scratch) {
+  if (!mixed && plan.batch > m->tc64.batch) {
+    dfree(m->tc64.scratch, m->st);
+    m->tc64.scratch = nullptr;
+    m->tc64.batch = 0;
+    void* p;
+    TRY(dev_alloc(&p, plan.tc_bytes, "tensor-core scratch", m->st));
+    m->tc64.scratch = (char*)p;
+    m->tc64.batch = plan.batch;
+    m->tc64.chi = m->chi;
+    if (!m->tc.err) TRY(dalloc(&m->tc.err, 1, m->st));
+    m->tc64.err = m->tc.err;
+  }
+  if (mixed && plan.tc_bytes && !m->tc.scratch) {
     void* p;
     TRY(dev_alloc(&p, plan.tc_bytes, "tensor-core scratch", m->st));
     m->tc.scratch = (float*)p;
@@ -495,7 +521,9 @@ static int meas_chunk(MeasWalk& c, int k, int u0, int u1) {
   void* T = m->lvl_T[k];
   const bool tc = m->prec == MPS_MIXED && m->tc.scratch && D >= kTcMinDim && Dp >= kTcMinDim &&
                   (U >= kTcMinNodes || std::max(D, Dp) >= kTcAnyNodes);
-  const bool fused = !tc && D <= kFusedMax && Dp <= kFusedMax;
+  const bool tc64 = m->prec == MPS_FP64 && m->tc64.scratch && std::min(D, Dp) >= kFp64TcMinDim &&
+                    std::max(D, Dp) <= kFp64TcMaxDim;
+  const bool fused = !tc && !tc64 && D <= kFusedMax && Dp <= kFusedMax;
   const bool leaf = k + 1 >= t.n_levels || k + 1 >= m->n;
   if (tc && !leaf) {
     const Cx<float>* Bk = (const Cx<float>*)m->dm.B + (size_t)c.slot * m->dm.slot_elems + m->site_off[k];
@@ -508,7 +536,7 @@ static int meas_chunk(MeasWalk& c, int k, int u0, int u1) {
     m->stats.tc_gemm_launches += 1;
     m->stats.tc_gemm_flops += 2.0 * ((double)U * D) * (4.0 * Dp) * (2.0 * D);
   } else if (!tc) {
-    if (!fused && !leaf) {
+    if (!fused && !tc64 && !leaf) {
       CU(launch_env_T(m->dm, m->prec, c.slot, k, L, T, U, c.h->d_cbegin[k] + u0, m->st));
       ++c.launches;
     }
@@ -550,6 +578,19 @@ static int meas_chunk(MeasWalk& c, int k, int u0, int u1) {
       c.launches += 1;
       m->stats.tc_gemm_launches += 1;
       m->stats.tc_gemm_flops += 2.0 * (2.0 * Dp) * ((double)nch * Dp) * (4.0 * D);
+    } else if (tc64) {
+      // batches of parents; the scratch is the deeper levels' too
+      CU(env_fp64_site(m->tc64, (const Cx<double>*)m->dm.B + (size_t)c.slot * m->dm.slot_elems + m->site_off[k], D, Dp, m->st));
+      ++c.launches;
+      for (int64_t x = a; x < b;) {
+        const int ub = par[x], ue = std::min(ub + m->tc64.batch, par[b - 1] + 1);
+        const int64_t y = std::lower_bound(par.begin() + x, par.begin() + b, ue) - par.begin();
+        CU(env_fp64_T(m->tc64, (const Cx<double>*)L + (size_t)(ub - u0) * D * D, ue - ub, D, Dp, m->st));
+        CU(env_fp64_children(m->tc64, c.h->d_parent[k + 1] + x, c.h->d_edge[k + 1] + x, (int)(y - x), ub, ue - ub, D, Dp,
+                             (Cx<double>*)m->lvl_L[k + 1] + (size_t)(x - a) * Dp * Dp, m->st));
+        c.launches += 4;
+        x = y;
+      }
     } else if (fused) {
       CU(launch_level_fused(m->dm, m->prec, c.slot, k, D, Dp, par[a], par[b - 1] + 1, u0, (int)a, (int)b,
                             c.h->d_cbegin[k], c.h->d_parent[k + 1], c.h->d_edge[k + 1], L, m->lvl_L[k + 1], m->st));

@@ -171,7 +171,12 @@ __global__ void __launch_bounds__(256) k_renv_chain(DevMPS m, int slot, Cx<R>* R
     gate::csync<C>();
   }
 }
-// One product of one site over a grid (large bonds).
+// One product of one site over a grid (large bonds): tiles of 16 rows and kRenvCols columns, the
+// shortest time for a product of a serial chain. FP64 is bound by the FP64 lanes of the few
+// SMs that have a tile, so its tiles are as small as the threads of a block allow (18 sites,
+// chi = 64: 1.79 ms with 64 columns).
+template <class R>
+constexpr int kRenvCols = sizeof(R) == 4 ? 64 : 16;
 template <class R>
 __global__ void __launch_bounds__(256) k_renv_step(DevMPS m, int slot, int k, int stage, Cx<R>* Renv, Cx<R>* Bhat) {
   extern __shared__ __align__(256) unsigned char smem[];
@@ -180,8 +185,7 @@ __global__ void __launch_bounds__(256) k_renv_step(DevMPS m, int slot, int k, in
   const int Dl = rank[k], Dr = rank[k + 1];
   const Cx<R>* Bk = (const Cx<R>*)m.B + (size_t)slot * m.slot_elems + m.site_off[k];
   Cx<R>* Bh = Bhat + m.site_off[k];
-  // blockIdx.y: column slabs of 64 (the tile shape's width)
-  const int N = stage == 0 ? Dr : Dl, n0 = blockIdx.y * 64, nn = min(64, N - n0);
+  const int N = stage == 0 ? Dr : Dl, n0 = blockIdx.y * kRenvCols<R>, nn = min(kRenvCols<R>, N - n0);
   if (nn <= 0) return;
   const int M = stage == 0 ? 2 * Dl : Dl, per = (M + gridDim.x - 1) / gridDim.x, m0 = min(M, per * (int)blockIdx.x),
             mn = min(per, M - m0);
@@ -297,9 +301,9 @@ static cudaError_t right_envs_t(const DevMPS& m, int slot, const int* ranks, Cx<
   } else {
     for (int k = m.n - 1; k >= 0; --k) {
       const int Dl = ranks[k], Dr = ranks[k + 1];
-      // slabs of 16 rows: the shortest time for one product of a serial chain
-      k_renv_step<R><<<dim3((2 * Dl + 15) / 16, (Dr + 63) / 64), 256, smem, st>>>(m, slot, k, 0, Renv, Bhat);
-      k_renv_step<R><<<dim3((Dl + 15) / 16, (Dl + 63) / 64), 256, smem, st>>>(m, slot, k, 1, Renv, Bhat);
+      constexpr int cw = kRenvCols<R>;
+      k_renv_step<R><<<dim3((2 * Dl + 15) / 16, (Dr + cw - 1) / cw), 256, smem, st>>>(m, slot, k, 0, Renv, Bhat);
+      k_renv_step<R><<<dim3((Dl + 15) / 16, (Dl + cw - 1) / cw), 256, smem, st>>>(m, slot, k, 1, Renv, Bhat);
     }
     *launches += 2 * m.n;
   }

@@ -118,6 +118,7 @@ def test_tensor_core_levels_with_unaligned_nodes(ranks):
 
 
 @pytest.mark.parametrize("n,chi,prec", [(2, 2, G.MPS_FP64), (9, 16, G.MPS_FP64), (13, 64, G.MPS_FP64),
+                                        (11, 16, G.MPS_FP64), (11, 17, G.MPS_FP64), (13, 50, G.MPS_FP64), (14, 65, G.MPS_FP64),
                                         (9, 5, G.MPS_MIXED), (13, 32, G.MPS_MIXED), (13, 33, G.MPS_MIXED),
                                         (13, 50, G.MPS_MIXED), (13, 63, G.MPS_MIXED), (14, 64, G.MPS_MIXED),
                                         (14, 65, G.MPS_MIXED)])
