@@ -2,6 +2,7 @@
 // orchestration of the kernels in kernels.cu. See include/mpsvqe.h for the contract.
 #include <algorithm>
 #include <array>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -11,9 +12,9 @@
 #include <vector>
 
 #include "../../include/mpsvqe.h"
-#include "host.hpp"
 #include "env_fp64_tc.cuh"
 #include "env_tc.cuh"
+#include "host.hpp"
 #include "kernels.cuh"
 
 using namespace mpsvqe;
@@ -409,6 +410,29 @@ static int sum_slot_flops(mps_s* m, int slot0, int count, double* total) {
   return MPS_OK;
 }
 
+// Slots whose gate chains the calls in progress run on a device, this call's included:
+// launch_circuit spreads a slot over several SMs only while there are SMs to spare. The
+// results have the same bits either way.
+class SlotsInFlight {
+ public:
+  explicit SlotsInFlight(int n) : n_(n) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) c_ = &count_[dev];
+    if (c_) *c_ += n_;
+  }
+  ~SlotsInFlight() {
+    if (c_) *c_ -= n_;
+  }
+  SlotsInFlight(const SlotsInFlight&) = delete;
+  int now() const { return c_ ? c_->load() : n_; }
+
+ private:
+  static std::atomic<int> count_[64];
+  std::atomic<int>* c_ = nullptr;
+  int n_;
+};
+std::atomic<int> SlotsInFlight::count_[64];
+
 // Apply the circuit to slots [slot0, slot0 + count) with per-slot parameters thetas
 // ([count][n_params], host; null keeps the device copy). Optional per-slot host arrays:
 // start (first gate), shift_gate / shift_phi (angle shift of one parametric gate).
@@ -444,8 +468,9 @@ static int run_circuit(mps_s* m, circ_s* c, int slot0, int count, const double* 
   TRY(sum_slot_flops(m, slot0, count, &flops0));
   CU(cudaEventRecord(m->ev[0], m->st));
   int launches = 0;
+  const SlotsInFlight load(m->st ? count : 0);   // calls on the default stream run one after the other
   for (int64_t g0 = g_begin; g0 < G; g0 += chunk) {
-    CU(launch_circuit(m->dm, m->prec, cd, g0, std::min(G, g0 + chunk), slot0, count, m->d_theta, m->cutoff,
+    CU(launch_circuit(m->dm, m->prec, cd, g0, std::min(G, g0 + chunk), slot0, count, m->st ? load.now() : count, m->d_theta, m->cutoff,
                       m->max_sweeps, m->st));
     ++launches;
   }

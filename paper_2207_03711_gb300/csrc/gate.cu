@@ -17,19 +17,22 @@ template <class R, int NT, int C, int VG, bool RAW>
 int max_clusters(int chi);
 
 // Blocks per slot in mixed precision. chi <= 16: one (a step of these sizes is shorter than
-// a cluster barrier is worth). chi 17..64: the most of 8, 4, 2, 1 with which all slots still
-// run at once, with the same bits for each (8 virtual ranks). chi > 64: 8, M' needs their
-// shared memory.
+// a cluster barrier is worth). chi 17..64: the most of 8, 4, 2, 1 with which all running slots
+// (of all calls in progress) still run at once, with the same bits for each (8 virtual ranks).
+// A chi = 64 gate takes 263 us with 8 blocks (up to 14 slots), 294 with 4, 342 with 2 and 477
+// with 1 (152 slots); one block alone took 746 us before clusters, and 415 and 442 us a gate at
+// 73 and 152 slots. Serving 152 single slots with 8 blocks each would run 14 at a time: 2 860 us
+// a round of gates instead of 477. chi > 64: 8, M' needs their shared memory.
 template <bool RAW>
 static cudaError_t launch_mixed(const DevMPS& m, const CircDev& c, int64_t g0, int64_t g1, int slot0, int count,
-                                const double* theta, double cutoff, int max_sweeps, cudaStream_t st) {
+                                int running, const double* theta, double cutoff, int max_sweeps, cudaStream_t st) {
   if (m.chi <= 16)
     return launch_cluster<float, 256, 1, 2, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
   if constexpr (!RAW) {
-    if (m.chi <= 64 && count > max_clusters<float, 256, 8, 1, RAW>(m.chi)) {
-      if (count <= max_clusters<float, 256, 4, 2, RAW>(m.chi))
+    if (m.chi <= 64 && running > max_clusters<float, 256, 8, 1, RAW>(m.chi)) {
+      if (running <= max_clusters<float, 256, 4, 2, RAW>(m.chi))
         return launch_cluster<float, 256, 4, 2, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
-      if (count <= max_clusters<float, 256, 2, 4, RAW>(m.chi))
+      if (running <= max_clusters<float, 256, 2, 4, RAW>(m.chi))
         return launch_cluster<float, 256, 2, 4, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
       return launch_cluster<float, 512, 1, 8, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
     }
@@ -38,10 +41,10 @@ static cudaError_t launch_mixed(const DevMPS& m, const CircDev& c, int64_t g0, i
 }
 
 cudaError_t launch_circuit(const DevMPS& m, int prec, const CircDev& c, int64_t g0, int64_t g1, int slot0, int count,
-                           const double* theta, double cutoff, int max_sweeps, cudaStream_t st) {
+                           int running, const double* theta, double cutoff, int max_sweeps, cudaStream_t st) {
   if (prec == MPS_PREC_FP64)
     return launch_cluster<double, 256, 8, 1, false>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
-  return launch_mixed<false>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
+  return launch_mixed<false>(m, c, g0, g1, slot0, count, running, theta, cutoff, max_sweeps, st);
 }
 
 }  // namespace mpsvqe
@@ -134,7 +137,7 @@ extern "C" int mps_apply_gates_noalloc(int n_qubits, int chi, void* site_tensors
   const double* theta = (const double*)(base + off_dw + 128);   // never read: every gate is fixed
   for (int64_t g0 = 0; g0 < n_gates; g0 += 16384) {
     const int64_t g1 = g0 + 16384 < n_gates ? g0 + 16384 : n_gates;
-    if (launch_mixed<true>(d, c, g0, g1, 0, 1, theta, std::ldexp(1.0, -20), 60, st) != cudaSuccess) return MPS_ECUDA;
+    if (launch_mixed<true>(d, c, g0, g1, 0, 1, 1, theta, std::ldexp(1.0, -20), 60, st) != cudaSuccess) return MPS_ECUDA;
   }
   if (discarded_weight) {
     // the discarded weight and the status words sit next to each other in the array:

@@ -32,6 +32,8 @@ namespace gate {
 // z partials, the next column before its right update, the partial norms of the row.
 // The trailing matrix is read twice and written once per step, where two separate half
 // steps read and write it twice.
+// chi = 64 in mixed precision (128 steps): 667 k cycles in one block with two barriers a step, 322 k
+// so on eight.
 // LAPACK-style reflector H = I - tau v v^H, v_0 = 1, for x = (alpha, tail) with ||tail||^2 =
 // xn2: H^H x = beta e_1 with beta real, v = scale tail. A vector whose squared norm is
 // within 16x of the smallest normal number counts as zero: the squares that make up that

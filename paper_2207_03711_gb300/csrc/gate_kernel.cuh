@@ -5,9 +5,15 @@
 // truncated SVD (bidiagonal route; one-sided Jacobi for spectra that stay degenerate),
 // Eq. (10) updates. One evaluation's gate chain is serial, so what a gate costs is its own
 // latency; a cluster of C blocks spreads every stage of it over C SMs, and keeps M' in
-// distributed shared memory where one block's is too small. C depends on the precision and
-// the bond cap only, never on how many slots run together, so a slot's result does not
-// depend on its company.
+// distributed shared memory where one block's is too small. Where C depends on how many slots
+// run together, C VG (virtual ranks: how the columns and the sums are dealt out) does not, so a
+// slot's result does not depend on its company.
+//
+// A gate is bound by the latency of its serial stages, not by bandwidth or arithmetic. Time of a
+// gate of a saturated circuit, with one block per slot before and now: FP64 chi = 16 1 000 and
+// 115 us, chi = 64 16.8 and 1.6 ms; mixed chi = 16 60 and 38 us (one block still), chi = 33 280
+// and 135, chi = 64 746 and 263 us, chi = 128 (M' in L2 before, in shared memory now) 6.5 and
+// 0.74 ms.
 #pragma once
 #include <atomic>
 #include <type_traits>

@@ -52,9 +52,10 @@ struct CircDev {
 cudaError_t launch_reset(const DevMPS& m, int prec, int slot0, int count, const uint8_t* occ_dev,
                          cudaStream_t st);
 
-// Apply gates [g0, g1) to slots [slot0, slot0+count); theta_dev: [count][n_params].
+// Apply gates [g0, g1) to slots [slot0, slot0+count); theta_dev: [count][n_params]. running:
+// slots that share the device, these included (it decides the speed only).
 cudaError_t launch_circuit(const DevMPS& m, int prec, const CircDev& c, int64_t g0, int64_t g1,
-                           int slot0, int count, const double* theta_dev, double cutoff,
+                           int slot0, int count, int running, const double* theta_dev, double cutoff,
                            int max_sweeps, cudaStream_t st);
 
 // Measurement workspace (device) for one slot at a time.

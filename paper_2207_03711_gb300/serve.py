@@ -2,8 +2,8 @@
 
 Requests of different sizes (qubits, bond dimension, precision) are admitted while
 device memory allows. Each admitted request owns an MPS handle on its own CUDA stream,
-so the gate chains of all requests in flight run side by side on the device (one thread
-block, i.e. one SM, per evaluation slot); a request that finishes releases its memory and
+so the gate chains of all requests in flight run side by side on the device (one
+thread-block cluster per evaluation slot, smaller the more slots run); a request that finishes releases its memory and
 the loop admits the next ones that fit (first fit in arrival order). Every result is
 computed by the same deterministic kernels as a lone call, so it does not depend on what
 else is in flight. A request can be cancelled (Future.cancel) until it starts running.

@@ -144,3 +144,36 @@ def test_fused_levels_and_energy_sum(n, chi, prec):
     assert np.abs(G.mps_expect_paulis(M, codes) - ref).max() <= tol
     H = G.ham_create(codes, coeff)
     assert abs(G.mps_energy(M, H) - float(coeff @ ref.real)) <= tol * np.abs(coeff).sum()
+
+
+@pytest.mark.parametrize("n_threads", [3, 20])
+def test_results_do_not_depend_on_calls_in_progress(n_threads):
+    """Handles on streams of their own, driven from threads: the blocks per slot follow the
+    number of running slots, the bits do not."""
+    import threading
+
+    import torch
+    n, chi = 10, 20
+    ranks = syn.full_ranks(n, chi)
+    st = mps.random_canonical(n, ranks, syn.random_mps_gaussians(n, ranks, 7))
+    bonds = np.tile(np.arange(n - 1, dtype=np.int32), 6)
+    U = np.array([np.linalg.qr(z)[0] for z in syn.random_gate_matrices(len(bonds), 5)])
+    streams = [torch.cuda.Stream() for _ in range(n_threads)]
+    handles = [G.mps_create(n, chi, G.MPS_MIXED, cuda_stream=s.cuda_stream) for s in streams]
+    alone = G.mps_create(n, chi, G.MPS_MIXED)
+
+    def run(M):
+        G.mps_set_state(M, st.B, st.lam)
+        G.mps_apply_gates(M, bonds, U)
+
+    run(alone)
+    ref = G.mps_get_state(alone)
+    threads = [threading.Thread(target=run, args=(M,)) for M in handles]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for M in handles:
+        got = G.mps_get_state(M)
+        for a, b in zip(ref[1] + ref[2], got[1] + got[2]):
+            assert np.array_equal(a, b)
