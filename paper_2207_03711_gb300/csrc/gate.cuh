@@ -1,5 +1,5 @@
 // Device code of the gate engine: one two-site gate (Eqs. 7-10) by a thread-block cluster
-// of C blocks (C = 1: one block). See gate.cu for the kernel that strings these together.
+// of C blocks (C = 1: one block). See gate_kernel.cuh for the kernel that strings these together.
 //
 // M' (tall orientation: T = M' or M'^H, tr x tp, tr >= tp) is spread over the cluster by
 // columns: column q belongs to block (q / 2) mod C and stays in that block's shared memory

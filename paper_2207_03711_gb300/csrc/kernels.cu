@@ -1,8 +1,11 @@
 // CUDA kernels of the MPS-VQE hot path for sm_103a (GB300).
 //
 //  k_reset        product-state reference (Sec. III-D: X gates on the occupied qubits).
-//  k_right_envs   right identity environments R_k and B^_k = B_k R_{k+1}.
-//  k_level_T/child/close   one level of the Pauli-string prefix trie (Eq. 11 generalised).
+//  k_renv_chain, k_renv_step   right identity environments R_k and B^_k = B_k R_{k+1}.
+//  k_letter_blocks   per-letter right blocks, from which closing strings are evaluated.
+//  k_level_fused, k_level_T/child   one level of the Pauli-string prefix trie (Eq. 11
+//                 generalised) on the CUDA cores; env_tc.cu and env_fp64_tc.cu: larger bonds.
+//  k_level_close  the strings that end at a level.
 //  k_energy_sum   E = sum_i a_i <P_i> (Eq. 2) with Neumaier compensation in FP64.
 #include <cfloat>
 #include <cmath>
