@@ -165,6 +165,7 @@ struct mps_s {
     for (void* p : lvl_T) dfree(p, st);
     dfree(tc.scratch, st);
     dfree(tc64.scratch, st);
+    dfree(tc64.bal, st);
     dfree(tc.err, st);
     dfree(w.vals, st);
     dfree(w.out, st);
@@ -362,12 +363,13 @@ static int ensure_meas(mps_s* m, ham_s* h) {
     dfree(m->tc64.scratch, m->st);
     m->tc64.scratch = nullptr;
     m->tc64.batch = 0;
+    if (!m->tc.err) TRY(dalloc(&m->tc.err, 1, m->st));
+    if (!m->tc64.bal) TRY(dalloc(&m->tc64.bal, (size_t)m->n * m->chi, m->st));
     void* p;
     TRY(dev_alloc(&p, plan.tc_bytes, "tensor-core scratch", m->st));
     m->tc64.scratch = (char*)p;
     m->tc64.batch = plan.batch;
     m->tc64.chi = m->chi;
-    if (!m->tc.err) TRY(dalloc(&m->tc.err, 1, m->st));
     m->tc64.err = m->tc.err;
   }
   if (mixed && plan.tc_bytes && !m->tc.scratch) {
@@ -605,12 +607,12 @@ static int meas_chunk(MeasWalk& c, int k, int u0, int u1) {
       m->stats.tc_gemm_flops += 2.0 * (2.0 * Dp) * ((double)nch * Dp) * (4.0 * D);
     } else if (tc64) {
       // batches of parents; the scratch is the deeper levels' too
-      CU(env_fp64_site(m->tc64, (const Cx<double>*)m->dm.B + (size_t)c.slot * m->dm.slot_elems + m->site_off[k], D, Dp, m->st));
+      CU(env_fp64_site(m->tc64, (const Cx<double>*)m->dm.B + (size_t)c.slot * m->dm.slot_elems + m->site_off[k], k, D, Dp, m->st));
       ++c.launches;
       for (int64_t x = a; x < b;) {
         const int ub = par[x], ue = std::min(ub + m->tc64.batch, par[b - 1] + 1);
         const int64_t y = std::lower_bound(par.begin() + x, par.begin() + b, ue) - par.begin();
-        CU(env_fp64_T(m->tc64, (const Cx<double>*)L + (size_t)(ub - u0) * D * D, ue - ub, D, Dp, m->st));
+        CU(env_fp64_T(m->tc64, (const Cx<double>*)L + (size_t)(ub - u0) * D * D, k, ue - ub, D, Dp, m->st));
         CU(env_fp64_children(m->tc64, c.h->d_parent[k + 1] + x, c.h->d_edge[k + 1] + x, (int)(y - x), ub, ue - ub, D, Dp,
                              (Cx<double>*)m->lvl_L[k + 1] + (size_t)(x - a) * Dp * Dp, m->st));
         c.launches += 4;
@@ -643,6 +645,10 @@ static int run_measure(mps_s* m, ham_s* h, int slot, double* out_host, bool term
   m->kev_used = 0;
   CU(cudaEventRecord(m->ev[2], m->st));
   CU(launch_right_envs(m->dm, m->prec, slot, c.r.data(), m->w, m->st, &c.launches));
+  if (const int top = *std::max_element(c.r.begin(), c.r.end()); m->tc64.scratch && top >= kFp64TcMinDim) {
+    CU(env_fp64_balance(m->tc64, m->dm, slot, top, (const Cx<double>*)m->w.R, m->st));
+    ++c.launches;
+  }
   const Trie& t = h->trie;
   if (t.n_levels > 0) {
     // root environment L_0 = [1] (one node, D_0 = 1, in FP32 with its row's second entry)
@@ -853,6 +859,7 @@ int mps_estimate_bytes(int n_qubits, int chi, int precision, int n_slots, circ_t
     const size_t T = ham->terms.size();
     const MeasPlan plan = meas_plan(ham->trie, chi, es, precision == MPS_MIXED);
     b += plan.level_bytes + plan.tc_bytes + (4 + 4 * T) * 8;   // chunk buffers, tensor-core scratch, values
+    if (plan.batch) b += (size_t)n * chi * 4;                  // balance of the bonds
     b += T * (8 + 4 + 1 + 4) + (size_t)ham->trie.total_nodes * 9;   // coefficients and the trie arrays
   }
   *bytes = b;

@@ -15,6 +15,15 @@
 // so, 3.9 in the levels that use it; against 128-bit arithmetic the rms error of 16 strings is
 // 0.4 - 1.4e-16 at bonds of 24 .. 64, of the FP64 kernels 0.7 - 1.9e-16.
 //
+// One scale for a row wants entries of like weight, which a gauge B_k -> B_k X, B_{k+1} ->
+// X^-1 B_{k+1} on a bond takes away from both operands at once: the products do not notice a
+// diagonal X, 55 bits below the largest entry do (a spread of 2^20 cost 1e-12 of <P>, 2^30
+// 5e-10). So the inner index of every product is balanced first: entry b of L's rows (of T's
+// columns) is taken times 2^x, entry b of the site operand times 2^-x, where 2^x is the weight of
+// b in the state (k_balance). That is exact, costs an addition per exponent, and makes a state
+// with a gauge of powers of two give the bits it gives without; x = 0 where the site tensors are
+// right-canonical.
+//
 // A level is, for a batch of nodes (see env_tc.cu for the real form of the products):
 //   k_split_L       digits of L's rows (node, a), inner (b, re/im)
 //   k_gemm_digits   T^T: rows (j, re/im, c) over columns (node, a), FP64
@@ -36,6 +45,7 @@ namespace mpsvqe {
 namespace {
 constexpr int kDigits = 8;
 constexpr int kNoScale = 1 << 20;   // exponent of a row with an infinity or NaN
+constexpr int kNone = -8000;        // exponent of zero
 constexpr int BM = 128, BN = 64, BK = 64;   // 64 BF16 = one 128-byte swizzle row
 constexpr int kDrain = 256 / BK;            // K tiles that the accumulators take exactly
 constexpr int PLANE_A = BM * BK * 2, PLANE_B = BN * BK * 2;
@@ -46,11 +56,12 @@ constexpr int TMEM_COLS = kDigits * BN;
 __host__ __device__ constexpr int pad8(int d) { return (d + 7) & ~7; }
 __host__ __device__ constexpr int pad64(int d) { return (d + 63) & ~63; }
 
-// Exponent e with |x| < 2^e (of the largest entry of a row; 0 rows: far below all).
-__device__ __forceinline__ int exponent_of(double x) {
+// Exponent e with |x| 2^s < 2^e.
+__device__ __forceinline__ int exponent_of(double x, int s) {
   const int b = (__double2hiint(x) >> 20) & 0x7ff;
-  return b == 0x7ff ? kNoScale : x == 0.0 ? -1100 : max(b, 1) - 1022;
+  return b == 0x7ff ? kNoScale : x == 0.0 ? kNone : max(b, 1) - 1022 + s;
 }
+__device__ __forceinline__ int exponent_of(Cx<double> z, int s) { return max(exponent_of(z.x, s), exponent_of(z.y, s)); }
 // x 2^(55 - e) rounded to a whole number, digits' offset added: digit p (p = 0 the highest) is
 // (y >> 7 (7 - p)) - 64, of 7 bits but the highest, which takes all that is left.
 __device__ __forceinline__ long long to_fixed(double x, int e) {
@@ -72,85 +83,115 @@ __device__ __forceinline__ int digit(long long y, int p) {
 }
 __device__ __forceinline__ int warp_max(int v) { return __reduce_max_sync(0xffffffffu, v); }
 // Two neighbouring entries into the planes at o (even), plane stride ps.
-__device__ __forceinline__ void store_digits(uint16_t* o, int64_t ps, double x0, double x1, int e) {
-  const long long y0 = to_fixed(x0, e), y1 = to_fixed(x1, e);
+__device__ __forceinline__ void store_digits(uint16_t* o, int64_t ps, double x0, int e0, double x1, int e1) {
+  const long long y0 = to_fixed(x0, e0), y1 = to_fixed(x1, e1);
 #pragma unroll
   for (int p = 0; p < kDigits; ++p)
     *reinterpret_cast<uint32_t*>(o + p * ps) = bf16_of(digit(y0, p)) | bf16_of(digit(y1, p)) << 16;
 }
 
+// Balance of the left bond's indices of every site: x with 2^x about the norm of the state that
+// index b stands for to the right (the root of R_k[b][b], to the nearest power of two), raised
+// where that norm comes from cancellation to what the entries of row b weigh against the norms
+// right of the site. So the balanced site operand stays below 1 and the balanced L is a part of
+// <psi|psi>. One warp an index; grid (indices / 8, sites).
+__device__ __forceinline__ int norm_exponent(double r2) {
+  if (!(r2 > 0.0)) return kNone;
+  const int b = __double2hiint(r2) >> 20;
+  return b == 0x7ff ? kNoScale : (max(b, 1) - 1022) >> 1;
+}
+__global__ void __launch_bounds__(256) k_balance(DevMPS m, int slot, const Cx<double>* Renv, int* bal) {
+  const int* rank = m.rank + (size_t)slot * (m.n + 1);
+  const int k = blockIdx.y, D = rank[k], Dp = rank[k + 1];
+  const int b = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (b >= D) return;
+  const size_t chi2 = (size_t)m.chi * m.chi;
+  const Cx<double>* R = Renv + (size_t)k * chi2;
+  const Cx<double>* Rn = R + chi2;
+  const Cx<double>* row = (const Cx<double>*)m.B + (size_t)slot * m.slot_elems + m.site_off[k] + (size_t)b * 2 * Dp;
+  int x = norm_exponent(R[(size_t)b * (D + 1)].x);
+  for (int q = lane; q < 2 * Dp; q += 32) {
+    const int c = q < Dp ? q : q - Dp;
+    x = max(x, exponent_of(row[q], k == m.n - 1 ? 0 : norm_exponent(Rn[(size_t)c * (Dp + 1)].x)) - 1);
+  }
+  x = warp_max(x);
+  if (lane == 0) bal[(size_t)k * m.chi + b] = x > 4000 || x < -4000 ? 0 : x;
+}
+
 // Row r = (u, a) of L: 2D reals (b, re/im), one warp a row.
-__global__ void __launch_bounds__(256) k_split_L(const Cx<double>* L, int64_t rows, int D, uint16_t* out, int* ex) {
+__global__ void __launch_bounds__(256) k_split_L(const Cx<double>* L, int64_t rows, int D, const int* bal, uint16_t* out,
+                                                 int* ex) {
   const int64_t r = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31, ld = pad8(2 * D);
   if (r >= rows) return;
   const Cx<double>* x = L + r * D;
-  int e = -1100;
-  for (int b = lane; b < D; b += 32) e = max(e, max(exponent_of(x[b].x), exponent_of(x[b].y)));
+  int e = kNone;
+  for (int b = lane; b < D; b += 32) e = max(e, exponent_of(x[b], bal[b]));
   e = warp_max(e);
   if (lane == 0) ex[r] = e;
   for (int b = lane; 2 * b < ld; b += 32) {
     const Cx<double> z = b < D ? x[b] : cx<double>(0, 0);
-    store_digits(out + r * ld + 2 * b, rows * ld, z.x, z.y, e);
+    const int eb = b < D ? e - bal[b] : e;
+    store_digits(out + r * ld + 2 * b, rows * ld, z.x, eb, z.y, eb);
   }
 }
 
 // Column (u, c) of T: ranges (j, re/im) of D entries a, each padded to pad8(D); one warp a column.
-__global__ void __launch_bounds__(256) k_split_T(const double* Tt, int U, int D, int Dp, uint16_t* out, int* ex) {
+__global__ void __launch_bounds__(256) k_split_T(const double* Tt, int U, int D, int Dp, const int* bal, uint16_t* out,
+                                                 int* ex) {
   const int64_t rows = (int64_t)U * Dp, r = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31, ds = pad8(D);
   if (r >= rows) return;
   const int64_t u = r / Dp, c = r - u * Dp, ldt = (int64_t)U * D;
   const double* t = Tt + c * ldt + u * D;
-  int e = -1100;
+  int e = kNone;
   for (int s = 0; s < 4; ++s)
-    for (int a = lane; a < D; a += 32) e = max(e, exponent_of(t[(int64_t)s * Dp * ldt + a]));
+    for (int a = lane; a < D; a += 32) e = max(e, exponent_of(t[(int64_t)s * Dp * ldt + a], bal[a]));
   e = warp_max(e);
   if (lane == 0) ex[r] = e;
   for (int s = 0; s < 4; ++s)
     for (int a = 2 * lane; a < ds; a += 64) {
       const double* x = t + (int64_t)s * Dp * ldt + a;
-      store_digits(out + (r * 4 + s) * ds + a, rows * 4 * ds, a < D ? x[0] : 0.0, a + 1 < D ? x[1] : 0.0, e);
+      const bool i0 = a < D, i1 = a + 1 < D;
+      store_digits(out + (r * 4 + s) * ds + a, rows * 4 * ds, i0 ? x[0] : 0.0, i0 ? e - bal[a] : e, i1 ? x[1] : 0.0,
+                   i1 ? e - bal[a + 1] : e);
     }
 }
 
 // Shared operands of a site (layouts as in env_tc.cu): BT, 4D' rows of 2D; A2, 2D' rows of
 // eight ranges of pad64(D): the four ranges (i, re/im) and the same with the other sign.
-__global__ void __launch_bounds__(256) k_split_site(const Cx<double>* Bk, int D, int Dp, uint16_t* bt, int* bt_ex, uint16_t* a2,
-                                                    int* a2_ex) {
+__global__ void __launch_bounds__(256) k_split_site(const Cx<double>* Bk, int D, int Dp, const int* bal, uint16_t* bt,
+                                                    int* bt_ex, uint16_t* a2, int* a2_ex) {
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r < 4 * Dp) {
     const int c = r % Dp, ro = r / Dp & 1, j = r / Dp >> 1, ld = pad8(2 * D);
-    int e = -1100;
-    for (int b = lane; b < D; b += 32) {
-      const Cx<double> z = Bk[((size_t)b * 2 + j) * Dp + c];
-      e = max(e, max(exponent_of(z.x), exponent_of(z.y)));
-    }
+    int e = kNone;
+    for (int b = lane; b < D; b += 32) e = max(e, exponent_of(Bk[((size_t)b * 2 + j) * Dp + c], -bal[b]));
     e = warp_max(e);
     if (lane == 0) bt_ex[r] = e;
     for (int b = lane; 2 * b < ld; b += 32) {
       const Cx<double> z = b < D ? Bk[((size_t)b * 2 + j) * Dp + c] : cx<double>(0, 0);
-      store_digits(bt + (int64_t)r * ld + 2 * b, (int64_t)4 * Dp * ld, ro ? z.y : z.x, ro ? z.x : -z.y, e);
+      const int eb = b < D ? e + bal[b] : e;
+      store_digits(bt + (int64_t)r * ld + 2 * b, (int64_t)4 * Dp * ld, ro ? z.y : z.x, eb, ro ? z.x : -z.y, eb);
     }
   } else if (r < 6 * Dp) {
     const int q = r - 4 * Dp, ro = q & 1, cp = q >> 1, ds = pad64(D), ld = 8 * ds;
-    int e = -1100;
-    for (int a = lane; a < 2 * D; a += 32) {
-      const Cx<double> z = Bk[(size_t)a * Dp + cp];   // (a, i) in one index
-      e = max(e, max(exponent_of(z.x), exponent_of(z.y)));
-    }
+    int e = kNone;
+    for (int a = lane; a < 2 * D; a += 32) e = max(e, exponent_of(Bk[(size_t)a * Dp + cp], -bal[a >> 1]));   // (a, i) in one index
     e = warp_max(e);
     if (lane == 0) a2_ex[q] = e;
     for (int x = 2 * lane; x < ld; x += 64) {
       const int seg = x / ds, a = x - seg * ds, i = seg >> 1 & 1, ri = seg & 1;
       double v[2];
+      int ek[2];
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
+        ek[k] = a + k < D ? e + bal[a + k] : e;
         const Cx<double> z = a + k < D ? Bk[((size_t)(a + k) * 2 + i) * Dp + cp] : cx<double>(0, 0);
         v[k] = ro == ri ? z.x : ro ? -z.y : z.y;   // re row [Br, Bi] per i, im row [-Bi, Br]
         if (seg >= 4) v[k] = -v[k];
       }
-      store_digits(a2 + (int64_t)q * ld + x, (int64_t)2 * Dp * ld, v[0], v[1], e);
+      store_digits(a2 + (int64_t)q * ld + x, (int64_t)2 * Dp * ld, v[0], ek[0], v[1], ek[1]);
     }
   }
 }
@@ -403,17 +444,23 @@ Parts carve(char* base, int chi, int nb) {
 int env_fp64_batch(int chi) { return std::max(16, (int)((size_t(512) << 20) / (128 * (size_t)chi * chi))); }
 size_t env_fp64_scratch(int chi, int batch) { return carve(nullptr, chi, batch).bytes; }
 
-cudaError_t env_fp64_site(const EnvFp64& s, const Cx<double>* Bk, int D, int Dp, cudaStream_t st) {
-  const Parts p = carve(s.scratch, s.chi, s.batch);
-  k_split_site<<<(6 * Dp + 7) / 8, 256, 0, st>>>(Bk, D, Dp, p.bt, p.bt_ex, p.a2, p.a2_ex);
+cudaError_t env_fp64_balance(const EnvFp64& s, const DevMPS& m, int slot, int top, const Cx<double>* Renv, cudaStream_t st) {
+  k_balance<<<dim3((top + 7) / 8, m.n), 256, 0, st>>>(m, slot, Renv, s.bal);
   return cudaGetLastError();
 }
 
-cudaError_t env_fp64_T(const EnvFp64& s, const Cx<double>* L, int U, int D, int Dp, cudaStream_t st) {
+cudaError_t env_fp64_site(const EnvFp64& s, const Cx<double>* Bk, int k, int D, int Dp, cudaStream_t st) {
+  const Parts p = carve(s.scratch, s.chi, s.batch);
+  k_split_site<<<(6 * Dp + 7) / 8, 256, 0, st>>>(Bk, D, Dp, s.bal + (size_t)k * s.chi, p.bt, p.bt_ex, p.a2, p.a2_ex);
+  return cudaGetLastError();
+}
+
+cudaError_t env_fp64_T(const EnvFp64& s, const Cx<double>* L, int k, int U, int D, int Dp, cudaStream_t st) {
   if (U <= 0) return cudaSuccess;
+  const int* bal = s.bal + (size_t)k * s.chi;
   const Parts p = carve(s.scratch, s.chi, s.batch);
   const int64_t rows = (int64_t)U * D, cols = (int64_t)U * Dp;
-  k_split_L<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(L, rows, D, p.l, p.l_ex);
+  k_split_L<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(L, rows, D, bal, p.l, p.l_ex);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   DigitGemm g;
@@ -426,7 +473,7 @@ cudaError_t env_fp64_T(const EnvFp64& s, const Cx<double>* L, int U, int D, int 
   g.b_ex = p.l_ex;
   g.T = p.T;
   if ((e = launch<false>(g, p.bt, pad8(2 * D), p.l, pad8(2 * D), s.err, st)) != cudaSuccess) return e;
-  k_split_T<<<(unsigned)((cols + 7) / 8), 256, 0, st>>>(p.T, U, D, Dp, p.t, p.t_ex);
+  k_split_T<<<(unsigned)((cols + 7) / 8), 256, 0, st>>>(p.T, U, D, Dp, bal, p.t, p.t_ex);
   return cudaGetLastError();
 }
 
