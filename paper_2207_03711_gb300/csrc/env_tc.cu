@@ -30,6 +30,7 @@
 // Both run on tc_gemm.cu (tcgen05, compensated TF32 splits). L[u] has an even leading
 // dimension (env_ld) and Dn rows, D rounded up to a multiple of 4, zeros in the ones added;
 // so T^T has Dn columns per node (TMA rows and boxes start on 16-byte boundaries).
+#include <algorithm>
 #include <cstdint>
 
 #include "cx.cuh"
@@ -41,54 +42,66 @@ namespace mpsvqe {
 
 static inline int pad32(int d) { return (d + 31) / 32 * 32; }
 
-// The tensor core truncates its accumulator after each product. A truncation takes half a
-// unit in the last place on average, 2^-23 / 2 / m of a value with mantissa m, so a K tile
-// with its four products at full size loses (1 + 2 + 3 + 4) / 4 of that: a fixed fraction
-// kLoss of the sum whatever its terms, which two products a level over dozens of levels
-// add up. The operand that all tiles share carries the inverse factor.
-constexpr float kLoss = 9.0e-8f;
-__device__ __forceinline__ void split_store(float z, float* hi, float* lo) {
+// The tensor core truncates its accumulator after each product of 8 inner indices: half a unit
+// in the last place on average, 2^-24 / m of a sum with mantissa m, which two products a level
+// over dozens of levels add up. With mantissas spread evenly over their logarithm that is the
+// fraction 2/3 2^-24 = 4.0e-8 of the sum (least squares: E[m] / E[m^2]). In a 32-wide K tile a
+// term loses it once for its own group of 8, measured 3.7e-8, and again for each later group
+// of the tile, less where that group has few entries n in the shared operand's row (few terms
+// leave few bits to cut): 1.2e-8 for n = 1, 1.9 for 2, 2.9 for 4, 3.3 for 8, which kLater (1 -
+// 0.62^n) follows. A tile whose only entry is a power of two (sites that pass an index through)
+// has exact products and loses nothing. The operand that all tiles share carries the
+// inverse factor entry by entry. One factor of 9.0e-8 for every entry, right for dense rows, moved <P> by 1.5e-5 over 100
+// sites that pass the bond through.
+constexpr float kOwn = 3.7e-8f, kLater = 3.3e-8f;
+// One row of a K tile by a warp, an entry a lane: hi and lo planes of z (1 + loss).
+__device__ __forceinline__ void split_store(float z, float* hi, float* lo, bool store) {
+  const unsigned nz = __ballot_sync(0xffffffffu, z != 0.f);
+  float loss = kOwn;
+#pragma unroll
+  for (int g = 1; g < 4; ++g)
+    if (g > (int)(threadIdx.x & 31) / 8) loss += kLater * (1.0f - exp2f(-0.69f * (float)__popc(nz >> (8 * g) & 255u)));
+  const bool exact = __popc(nz) == 1 && (__float_as_uint(z) & 0x7fffffu) == 0;
   uint32_t b;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(b) : "f"(z));
   const float h = __uint_as_float(b);
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(b) : "f"(fmaf(z, kLoss, z - h)));
-  *hi = h;
-  *lo = __uint_as_float(b);
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(b) : "f"(fmaf(z, exact ? 0.f : loss, z - h)));
+  if (store) {
+    *hi = h;
+    *lo = __uint_as_float(b);
+  }
 }
 
 // BT (4D' x 2D, leading dimension 2 env_ld(D)) and A2 (2D' x 4 Dk, Dk = D rounded up to 32) from site k (B[b][j][c] at
-// (b 2 + j) D' + c), hi and lo planes.
-__global__ void k_tc_site_operands(const Cx<float>* Bk, int D, int Dp, int Dk, float* bt, float* bt_lo, float* a2,
-                                   float* a2_lo) {
-  const int ldb = 2 * env_ld<float>(D);
-  const int64_t nbt = (int64_t)4 * Dp * ldb, na2 = (int64_t)2 * Dp * 4 * Dk;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nbt + na2;
-       i += (int64_t)gridDim.x * blockDim.x) {
+// (b 2 + j) D' + c), hi and lo planes. One warp a row of a K tile, rows fastest: neighbouring
+// warps share the sectors that they read.
+__global__ void __launch_bounds__(256) k_tc_site_operands(const Cx<float>* Bk, int D, int Dp, int Dk, float* bt, float* bt_lo,
+                                                          float* a2, float* a2_lo) {
+  const int ldb = 2 * env_ld<float>(D), lane = threadIdx.x & 31;
+  const int64_t nbt = (int64_t)4 * Dp * ((2 * D + 31) / 32), na2 = (int64_t)2 * Dp * (4 * Dk / 32);
+  for (int64_t i = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5); i < nbt + na2; i += (int64_t)gridDim.x * 8) {
     if (i < nbt) {
-      const int64_t row = i / ldb;
-      const int col = (int)(i - row * ldb);
-      if (col >= 2 * D) continue;   // never loaded
+      const int64_t row = i % (4 * Dp);
+      const int col = (int)(i / (4 * Dp)) * 32 + lane;
       const int c = (int)(row % Dp), ro = (int)(row / Dp) & 1, j = (int)(row / Dp) >> 1;
       const int b = col >> 1, ri = col & 1;
-      const Cx<float> z = Bk[((size_t)b * 2 + j) * Dp + c];   // B^j[b][c]
+      const Cx<float> z = b < D ? Bk[((size_t)b * 2 + j) * Dp + c] : cx<float>(0.f, 0.f);   // B^j[b][c]
       // re row: (Br, -Bi) per b; im row: (Bi, Br) per b
-      split_store(ro == 0 ? (ri == 0 ? z.x : -z.y) : (ri == 0 ? z.y : z.x), bt + i, bt_lo + i);
+      const int64_t o = row * ldb + col;
+      split_store(ro == 0 ? (ri == 0 ? z.x : -z.y) : (ri == 0 ? z.y : z.x), bt + o, bt_lo + o, b < D);
     } else {
-      const int64_t e = i - nbt, row = e / (4 * Dk);
-      const int col = (int)(e - row * 4 * Dk);
+      const int64_t e = i - nbt, row = e % (2 * Dp);
+      const int col = (int)(e / (2 * Dp)) * 32 + lane;
       const int ro = (int)(row & 1), cp = (int)(row >> 1);
       const int ii = col / (2 * Dk), ri = (col / Dk) & 1, a = col % Dk;
       const Cx<float> z = a < D ? Bk[((size_t)a * 2 + ii) * Dp + cp] : cx<float>(0.f, 0.f);   // B^i[a][c']
       // re row [Br, Bi] per i, im row [-Bi, Br] per i
-      split_store(ro == 0 ? (ri == 0 ? z.x : z.y) : (ri == 0 ? -z.y : z.x), a2 + e, a2_lo + e);
+      const int64_t o = row * 4 * Dk + col;
+      split_store(ro == 0 ? (ri == 0 ? z.x : z.y) : (ri == 0 ? -z.y : z.x), a2 + o, a2_lo + o, true);
     }
   }
 }
 
-static inline int grid_for(int64_t total) {
-  const int64_t b = (total + 255) / 256;
-  return (int)(b < 152 * 32 ? (b > 0 ? b : 1) : 152 * 32);
-}
 
 namespace {
 struct Parts {
@@ -106,7 +119,9 @@ size_t env_tc_scratch_floats(int chi) { return (size_t)(2 * part_bt(chi) + 2 * p
 cudaError_t env_tc_site(const EnvTc& s, const Cx<float>* Bk, int D, int Dp, cudaStream_t st) {
   const Parts p = carve(s.scratch, s.chi);
   const int Dk = pad32(D);
-  k_tc_site_operands<<<grid_for(8 * (int64_t)Dp * (D + Dk)), 256, 0, st>>>(Bk, D, Dp, Dk, p.bt, p.bt_lo, p.a2, p.a2_lo);
+  const int64_t warps = (int64_t)4 * Dp * ((2 * D + 31) / 32) + (int64_t)2 * Dp * (4 * Dk / 32);
+  const int grid = (int)std::min<int64_t>((warps + 7) / 8, 152 * 32);
+  k_tc_site_operands<<<grid, 256, 0, st>>>(Bk, D, Dp, Dk, p.bt, p.bt_lo, p.a2, p.a2_lo);
   return cudaGetLastError();
 }
 

@@ -3,6 +3,7 @@
 * FP64: a diagonal gauge on the bonds (column c of B_k times g_c, row c of B_{k+1} over g_c)
   leaves the state as it is. Every product of the contraction sums terms in which g cancels,
   so with powers of two the result has the same bits, and it is the oracle's to FP64.
+* Mixed: sites that pass a bond through are exact on the tensor cores, however many.
 """
 import numpy as np
 import pytest
@@ -20,12 +21,12 @@ def lib():
     return G.load_library()
 
 
-def _polarised(n, ranks, seed):
-    """Random right-canonical state with O(1) expectations of strings of Z."""
+def _polarised(n, ranks, seed, bias=2.0):
+    """Random right-canonical state that prefers |0> where its bonds leave it the choice."""
     g = syn.random_mps_gaussians(n, ranks, seed)
     r = [1] + list(ranks) + [1]
     for k in range(n):
-        g[k][:r[k + 1]] *= 2.0
+        g[k][:r[k + 1]] *= bias
     return mps.random_canonical(n, ranks, g)
 
 
@@ -64,3 +65,33 @@ def test_fp64_does_not_depend_on_a_bond_gauge(n, chi, spread):
     # two products a level, each off by a few units of the last place of <psi|psi> = 1
     ref = np.array([mps.expect_string(st, c) for c in codes]) / mps.norm2(st)
     assert np.abs(gauged - ref).max() <= n * 16 * 2.0 ** -53
+
+
+def _with_idle_sites(st, at, count):
+    """st with `count` sites in |0> that pass bond `at` - 1 through."""
+    D = st.B[at].shape[0]
+    idle = np.zeros((D, 2, D), dtype=complex)
+    idle[:, 0, :] = np.eye(D)
+    return st.B[:at] + [idle.copy() for _ in range(count)] + st.B[at:], \
+        st.lam[:at] + [st.lam[at - 1]] * count + st.lam[at:]
+
+
+# a bond of one packed tile, of one tile and of two column tiles
+@pytest.mark.parametrize("n,chi", [(18, 64), (20, 100), (22, 160)])
+def test_mixed_sites_that_pass_a_bond_through_are_exact(n, chi):
+    """100 idle sites in the middle of a state: their products are single terms with factor 1,
+    exact but for the first, which may drop the last bit of an entry of L (its two 11-bit parts
+    hold 23 bits and a sign of 24). <P> is sum L conj(Q) with ||L||_F <= ||rho||_F <= 1 and
+    ||Q||_F <= sqrt(chi), so that is at most sqrt(chi) 2^-23, doubled for the two products."""
+    ranks = syn.full_ranks(n, chi)
+    st = _polarised(n, ranks, chi + 3, bias=8.0)
+    at, idle = n // 2, 100
+    codes = np.zeros((6, n), dtype=np.uint8)      # pairs of Z and some X around the idle sites
+    for c, (p, q, l) in zip(codes, [(at - 1, at, 3), (at - 2, at, 3), (at - 2, at + 1, 3), (0, at, 3), (at - 1, at, 1), (1, at, 2)]):
+        c[p], c[q] = l, 3
+    long = np.concatenate([codes[:, :at], np.zeros((len(codes), idle), dtype=np.uint8), codes[:, at:]], axis=1)
+    short = _measure(st.B, st.lam, chi, G.MPS_MIXED, codes)
+    B, lam = _with_idle_sites(st, at, idle)
+    v = _measure(B, lam, chi, G.MPS_MIXED, long)
+    assert np.abs(short).max() > 0.6              # a systematic factor would be seen
+    assert np.abs(v - short).max() <= 2 * np.sqrt(chi) * 2.0 ** -23
