@@ -288,11 +288,12 @@ static int ensure_theta(mps_s* m, size_t count) {
 // fused FP32 kernel (k_level_fused) on a 24-qubit molecular Hamiltonian: 2.8 ms instead of
 // 3.8 at bonds of 34, 3.1 / 4.5 at 40, 4.1 / 5.9 at 49, 5.1 / 8.8 at 64; against the tiled
 // FP32 kernels (k_level_T, k_level_child) 4.3 / 5.2 at 96 and 6.6 / 9.6 at 127 (16-qubit
-// Hamiltonian). At 32 and less a tile is mostly padding. With fewer nodes than SMs the fused
-// kernel is one wave whatever their number and one launch instead of three: with 100 strings
-// 0.87 ms instead of 1.01 at 34, 1.08 / 1.10 at 49, 1.24 / 1.09 at 64, so bonds up to 48
-// want kTcMinNodes.
-constexpr int kTcMinDim = 33, kTcMinNodes = 152, kTcAnyNodes = 49;
+// Hamiltonian). At 32 and less a tile is mostly padding. The rule reads bonds only: the two
+// routes round differently, and a string's value must not follow from how many other strings
+// are asked or how the trie is cut. With fewer nodes than SMs the fused kernel, one launch
+// instead of three, would be ahead at the small end: with 100 strings 0.87 ms instead of 1.01 at 34,
+// 1.08 / 1.10 at 49, 1.24 / 1.09 at 64.
+constexpr int kTcMinDim = 33;
 // FP64 levels with both bonds in this range multiply by digits on the tensor cores
 // (env_fp64_tc.cu). Against the fused FP64 kernel (k_level_fused64), an 18-qubit molecular
 // Hamiltonian and 30 random strings: 3.5 ms instead of 3.0 and 1.3 instead of 0.9 at bonds of
@@ -546,8 +547,7 @@ static int meas_chunk(MeasWalk& c, int k, int u0, int u1) {
   const int U = u1 - u0, D = c.r[k], Dp = c.r[k + 1];
   void* L = m->lvl_L[k];
   void* T = m->lvl_T[k];
-  const bool tc = m->prec == MPS_MIXED && m->tc.scratch && D >= kTcMinDim && Dp >= kTcMinDim &&
-                  (U >= kTcMinNodes || std::max(D, Dp) >= kTcAnyNodes);
+  const bool tc = m->prec == MPS_MIXED && m->tc.scratch && D >= kTcMinDim && Dp >= kTcMinDim;
   const bool tc64 = m->prec == MPS_FP64 && m->tc64.scratch && std::min(D, Dp) >= kFp64TcMinDim &&
                     std::max(D, Dp) <= kFp64TcMaxDim;
   const bool fused = !tc && !tc64 && D <= kFusedMax && Dp <= kFusedMax;

@@ -95,3 +95,19 @@ def test_mixed_sites_that_pass_a_bond_through_are_exact(n, chi):
     v = _measure(B, lam, chi, G.MPS_MIXED, long)
     assert np.abs(short).max() > 0.6              # a systematic factor would be seen
     assert np.abs(v - short).max() <= 2 * np.sqrt(chi) * 2.0 ** -23
+
+
+# bonds of 33..48, where few nodes and many would favour different kernels; 64: two children a tile
+@pytest.mark.parametrize("n,chi", [(14, 34), (14, 48), (15, 64)])
+def test_mixed_values_do_not_depend_on_the_company(n, chi):
+    """A string's value is the same alone, among hundreds and with chunks of 16 nodes: every
+    number of a level comes out of the same sums in the same order."""
+    st = _polarised(n, syn.full_ranks(n, chi), chi + 5)
+    codes = _random_strings(n, 400, chi)
+    M = G.mps_create(n, chi, G.MPS_MIXED)
+    G.mps_set_state(M, st.B, st.lam)
+    v = G.mps_expect_paulis(M, codes)
+    for i in (0, 7, 200, 399):
+        assert np.array_equal(G.mps_expect_paulis(M, codes[i:i + 1]), v[i:i + 1])
+    G.mps_set_meas_budget(M, 1)
+    assert np.array_equal(G.mps_expect_paulis(M, codes), v)
