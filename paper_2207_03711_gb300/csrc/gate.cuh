@@ -41,11 +41,12 @@ namespace gate {
 // so the norm could come out as 0 while alpha is not, and 1 / (alpha - beta) would be a
 // division by zero. The identity is taken there and the entries (absolutely that small)
 // are dropped from the bidiagonal. The root and the reciprocals are the hardware estimates
-// with Newton-Raphson steps, whose dependent chain is a quarter of a library square root's
+// with a Newton-Raphson step, whose dependent chain is a quarter of a library square root's
 // and four divisions': it runs twice per step of a serial recurrence.
-// FP64 takes one third-order step from the 22-bit estimates (e the residual: 1 + e/2 +
-// 3 e^2 / 8 for the inverse root, 1 + e + e^2 for the inverse), which is shorter in
-// dependent operations than two second-order steps; FP64 latency is what it costs.
+// FP64 takes one step of third order (Chebyshev's iteration: the binomial series of
+// (1 - e)^(-1/2) and (1 - e)^-1 in the residual e, up to e^2) from estimates of 20 bits, which is
+// shorter in dependent operations than two Newton-Raphson steps; FP64 latency is what it costs.
+// Both are within one and a half units of the last place over the range used.
 __device__ __forceinline__ void root_and_inverse(float x, float* root, float* inv) {
   const float y = rsqrtf(x);
   float r = x * y;

@@ -645,6 +645,18 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
       csync<C>();
       continue;
     }
+    // a norm whose square is near the largest number: the reduction works on 2^-8 M' (its
+    // reflectors take up to 4 times a squared norm, and the reciprocal estimate is 0 for the two
+    // highest exponents)
+    const bool huge = total >= (kF64 ? 0x1p1008 : 0x1p112);
+    if (huge) {
+      const int rows = tall ? mrows : ncol;
+      for (int it = tid; it < 2 * nq * rows; it += NT) {
+        Cx<R>* e = T + (size_t)(it / rows) * ld + it % rows;
+        *e = R(0x1p-8) * *e;
+      }
+      csync<C>();
+    }
     PHASE(0);
     // (3) Eq. (9): bidiagonalise T = Q B P^H (B real)
     {
@@ -1154,7 +1166,7 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
         for (int t = lane; t < k; t += 32) kept += ((double)sig[t] * bk) * ((double)sig[t] * bk);
         for (int o = 16; o > 0; o >>= 1) kept += __shfl_xor_sync(0xffffffffu, kept, o);
         if (lane == 0 && total > 0.0) dw_acc += fmax(0.0, total - kept) / total;
-        for (int t = lane; t < k; t += 32) lam[(size_t)bond * chi + t] = (double)(sig[t] * back);
+        for (int t = lane; t < k; t += 32) lam[(size_t)bond * chi + t] = (double)(sig[t] * back) * (huge ? 256.0 : 1.0);
       }
     }
     csync<C>();

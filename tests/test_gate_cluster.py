@@ -177,3 +177,34 @@ def test_results_do_not_depend_on_calls_in_progress(n_threads):
         got = G.mps_get_state(M)
         for a, b in zip(ref[1] + ref[2], got[1] + got[2]):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec,scales", [(G.MPS_MIXED, (0, 58, 61, 62, 63)), (G.MPS_FP64, (0, 500, 509, 510, 511))])
+@pytest.mark.parametrize("n,chi", [(2, 2), (8, 16), (12, 40)])
+def test_gate_on_a_state_of_large_norm(prec, scales, n, chi):
+    """The reduction works up to the largest norm whose square is a number: the squared norm of
+    M' is 2^(2 scale) here, so twice scale stays below 128 (1024)."""
+    bond = n // 2 - 1
+    U = np.linalg.qr(syn.random_gate_matrices(1, n)[0])[0]
+    eps = 2.0 ** -53 if prec == G.MPS_FP64 else 2.0 ** -24
+    for seed in range(4):
+        r = syn.full_ranks(n, chi)
+        st = mps.random_canonical(n, r, syn.random_mps_gaussians(n, r, seed))
+        ll = mps.left_lambda(st, bond)
+        out = []
+        for s in scales:
+            M = G.mps_create(n, chi, prec)
+            B = list(st.B)
+            B[bond] = B[bond] * 2.0 ** s
+            G.mps_set_state(M, B, st.lam)
+            G.mps_apply_gates(M, np.array([bond], dtype=np.int32), U[None])
+            rg, sites, lams = G.mps_get_state(M)
+            M.close()
+            V = sites[bond + 1].reshape(rg[bond], -1)
+            block = ll[:, None, None, None] * np.einsum("aib,bjc->aijc", sites[bond] * 2.0 ** -s, sites[bond + 1])
+            assert np.abs(V @ V.conj().T - np.eye(len(V))).max() <= 128 * eps
+            out.append((lams[bond] * 2.0 ** -s, block))
+        for lam, block in out[1:]:
+            # the steps round differently only where sums are split at absolute places
+            assert np.abs(lam - out[0][0]).max() <= 128 * eps
+            assert np.linalg.norm(block - out[0][1]) <= 128 * eps
