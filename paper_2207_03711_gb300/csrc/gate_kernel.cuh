@@ -1128,7 +1128,8 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
           }
           for (int e = tid; e < kj * tp; e += NT) {
             const int t = e / tp, q = e - t * tp, p = order[t];
-            Wn[e] = (R)((double)X[(size_t)p * ldx + q] / sqrt(sig2d[p]));
+            // M' = 0 (a gate that annihilates the state): any unit vector is its singular vector
+            Wn[e] = sig2d[p] > 0.0 ? (R)((double)X[(size_t)p * ldx + q] / sqrt(sig2d[p])) : R(q == t ? 1 : 0);
           }
         }
         csync<C>();

@@ -208,3 +208,21 @@ def test_gate_on_a_state_of_large_norm(prec, scales, n, chi):
             # the steps round differently only where sums are split at absolute places
             assert np.abs(lam - out[0][0]).max() <= 128 * eps
             assert np.linalg.norm(block - out[0][1]) <= 128 * eps
+
+
+@pytest.mark.parametrize("prec", [G.MPS_FP64, G.MPS_MIXED])
+@pytest.mark.parametrize("chi", [2, 16, 40])
+@pytest.mark.parametrize("ranks", [[1, 1, 2, 2, 2], [2, 2, 1, 1, 1], [2, 2, 2, 2, 2]])
+def test_gate_that_annihilates_the_state(prec, chi, ranks):
+    """M' = 0, tall, wide and square: one Schmidt number 0, a unit vector in B_{n+1}, zeros in B_n."""
+    n, bond = 6, 1
+    rng = np.random.default_rng(chi)
+    r = [1] + ranks + [1]
+    B = [rng.normal(size=(r[k], 2, r[k + 1])) + 0j for k in range(n)]
+    M = G.mps_create(n, chi, prec)
+    G.mps_set_state(M, B, [np.ones(x) for x in ranks])
+    G.mps_apply_gates(M, np.array([bond], dtype=np.int32), np.zeros((1, 4, 4), dtype=complex))
+    rg, sites, lams = G.mps_get_state(M)
+    assert rg[bond] == 1 and lams[bond][0] == 0.0
+    assert not sites[bond].any()
+    assert np.linalg.norm(sites[bond + 1]) == 1.0
