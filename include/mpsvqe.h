@@ -157,11 +157,14 @@ int mps_set_svd_params(mps_t mps, double cutoff, int max_sweeps);
 
 /* Memory of the trie measurement (Sec. III-C; no counterpart in the paper's text). The
  * prefix trie of the strings is walked depth first in chunks of consecutive nodes of one
- * level, each level keeping environment buffers (3 chi^2 complex entries per node) for
- * one chunk: bytes bounds the sum of those buffers (at least 16 nodes per level); the
- * tensor-core scratch of mixed precision then takes a quarter of bytes (at least 64 MiB).
- * 0 restores the default, 4 GiB for chi <= 128 and 48 GiB above, which mps_estimate_bytes
- * assumes. Results do not depend on the chunking. */
+ * level, each level keeping environment buffers (up to 3 chi^2 complex entries per node,
+ * odd bonds of mixed precision padded to an even leading dimension and a multiple of 4
+ * rows) for one chunk: bytes bounds the sum of those buffers, padding aside (at least 16
+ * nodes per level). The tensor cores' scratch comes on top: 128 chi^2 bytes in mixed
+ * precision; in FP64 384 chi^2 for a site and 128 chi^2 per node of a batch, which is no
+ * larger than a chunk nor than 512 MiB (at least 16 nodes). 0 restores the default, 4 GiB
+ * for chi <= 128 and 48 GiB above, which mps_estimate_bytes assumes. What an earlier
+ * budget held is given back. Results do not depend on the chunking. */
 int mps_set_meas_budget(mps_t mps, size_t bytes);
 
 /* Sec. III-A, Eqs. (7)-(10), for every gate of circ on slot 0 in order: contract

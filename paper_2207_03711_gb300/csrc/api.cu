@@ -977,6 +977,9 @@ int mps_set_meas_budget(mps_t m, size_t bytes) {
     p = nullptr;
   }
   std::fill(m->lvl_cap.begin(), m->lvl_cap.end(), 0);
+  dfree(m->tc64.scratch, m->st);
+  m->tc64.scratch = nullptr;
+  m->tc64.batch = 0;
   m->meas_budget = bytes;
   return MPS_OK;
 }

@@ -5,8 +5,11 @@
   so with powers of two the result has the same bits, and it is the oracle's to FP64.
 * Mixed: sites that pass a bond through are exact on the tensor cores, however many.
 """
+import ctypes
+
 import numpy as np
 import pytest
+import torch
 
 import paper_2207_03711_gb300 as G
 from oracle import mps
@@ -111,3 +114,37 @@ def test_mixed_values_do_not_depend_on_the_company(n, chi):
         assert np.array_equal(G.mps_expect_paulis(M, codes[i:i + 1]), v[i:i + 1])
     G.mps_set_meas_budget(M, 1)
     assert np.array_equal(G.mps_expect_paulis(M, codes), v)
+
+
+def _pool_used():
+    """Bytes in use of the device's memory pool, which the library allocates from."""
+    torch.cuda.synchronize()
+    cu = ctypes.CDLL("libcuda.so.1")
+    dev, pool, used = ctypes.c_int(), ctypes.c_void_p(), ctypes.c_uint64()
+    assert cu.cuCtxGetDevice(ctypes.byref(dev)) == 0
+    assert cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), dev) == 0
+    assert cu.cuMemPoolGetAttribute(pool, 7, ctypes.byref(used)) == 0   # CU_MEMPOOL_ATTR_USED_MEM_CURRENT
+    return used.value
+
+
+@pytest.mark.parametrize("prec", [G.MPS_FP64, G.MPS_MIXED])
+def test_a_smaller_budget_gives_the_memory_back(prec):
+    n, chi = 16, 64
+    st = _polarised(n, syn.full_ranks(n, chi), 3)
+    codes = _random_strings(n, 2000, 4)
+    torch.zeros(1, device="cuda")
+
+    def held(budgets):
+        before = _pool_used()
+        M = G.mps_create(n, chi, prec)
+        G.mps_set_state(M, st.B, st.lam)
+        for b in budgets:
+            G.mps_set_meas_budget(M, b)
+            G.mps_expect_paulis(M, codes)
+        used = _pool_used() - before
+        M.close()
+        return used
+
+    small = held([1])
+    assert held([0]) > 2 * small
+    assert held([0, 1]) == small
