@@ -47,8 +47,10 @@ def build(force=False, verbose=False):
          os.path.join(CSRC, "host.cpp"),
          "-o", os.path.join(OBJ, "host.o")],
     ]
-    units = ("gate_fp64", "gate_mixed1", "gate_mixed2", "gate_mixed8", "gate_raw", "gate", "kernels", "api", "tc_gemm",
-             "env_tc", "env_fp64_tc")
+    # the longest to compile first
+    units = ("gate_fp64_8", "gate_mixed_8", "gate_raw", "gate_mixed_1", "gate_mixed_2", "gate_mixed_2g",
+             "gate_fp64_2", "gate_fp64_2g", "gate_mixed_16", "env_fp64_tc", "tc_gemm",
+             "kernels", "api", "env_tc", "gate")
     for name in units:
         jobs.append([nvcc, *ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", *inc,
                      "-c", os.path.join(CSRC, name + ".cu"), "-o", os.path.join(OBJ, name + ".o")])

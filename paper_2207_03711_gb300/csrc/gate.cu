@@ -9,42 +9,65 @@
 
 namespace mpsvqe {
 
-template <class R, int NT, int C, int VG, bool RAW>
+template <class R, int NT, int C, int VG, bool RAW, bool TG>
 cudaError_t launch_cluster(const DevMPS& m, const CircDev& c, int64_t g0, int64_t g1, int slot0, int count,
                            const double* theta, double cutoff, int max_sweeps, cudaStream_t st);
-// Slots that run at once on the current device (one thread block per SM).
-template <class R, int NT, int C, int VG, bool RAW>
+// Slots that run at once on the current device (one thread block per SM); 0 where chi does not fit.
+template <class R, int NT, int C, int VG, bool RAW, bool TG>
 int max_clusters(int chi);
 
-// Blocks per slot in mixed precision. chi <= 16: one (a step of these sizes is shorter than
-// a cluster barrier is worth). chi 17..64: the most of 8, 4, 2, 1 with which all running slots
-// (of all calls in progress) still run at once, with the same bits for each (8 virtual ranks).
-// A chi = 64 gate takes 263 us with 8 blocks (up to 14 slots), 294 with 4, 342 with 2 and 477
-// with 1 (152 slots); one block alone took 746 us before clusters, and 415 and 442 us a gate at
-// 73 and 152 slots. Serving 152 single slots with 8 blocks each would run 14 at a time: 2 860 us
-// a round of gates instead of 477. chi > 64: 8, M' needs their shared memory.
-template <bool RAW>
-static cudaError_t launch_mixed(const DevMPS& m, const CircDev& c, int64_t g0, int64_t g1, int slot0, int count,
-                                int running, const double* theta, double cutoff, int max_sweeps, cudaStream_t st) {
-  if (m.chi <= 16)
-    return launch_cluster<float, 256, 1, 2, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
-  if constexpr (!RAW) {
-    if (m.chi <= 64 && running > max_clusters<float, 256, 8, 1, RAW>(m.chi)) {
-      if (running <= max_clusters<float, 256, 4, 2, RAW>(m.chi))
-        return launch_cluster<float, 256, 4, 2, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
-      if (running <= max_clusters<float, 256, 2, 4, RAW>(m.chi))
-        return launch_cluster<float, 256, 2, 4, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
-      return launch_cluster<float, 512, 1, 8, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
-    }
-  }
-  return launch_cluster<float, 256, 8, 1, RAW>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
+namespace {
+struct Engine {
+  decltype(&launch_cluster<float, 256, 8, 1, false, false>) launch;
+  int (*slots)(int chi);
+};
+template <class R, int NT, int C, int VG, bool TG>
+constexpr Engine engine() {
+  return {launch_cluster<R, NT, C, VG, false, TG>, max_clusters<R, NT, C, VG, false, TG>};
 }
+// Blocks per slot: the most with which all running slots (of all calls in progress) still run at
+// once, else the instance that runs most of them; each has the same bits (8 virtual ranks). One
+// slot finishes soonest on eight blocks, but a gate costs the fewest SM cycles in one. Time of a
+// gate of a UCCSD circuit in us, at 14 / 76 / 152 / 304 slots, and with one block a slot before
+// clusters (any number up to 152 / 304):
+//   mixed  chi = 33  114 / 158 / 218 / 433       209 - 212 / 423
+//          chi = 64  197 / 315 / 423 / 820       415 - 442 / 849
+//          chi = 72  161 / 276 / 542 / 1 060     569 - 601 / 1 157
+//          chi = 128 252 / 590 / 1 078 / 1 953   1 186 - 1 275 / 2 351
+//   FP64   chi = 16  185 / 206 / 402 / 792       1 545 - 1 599 / 3 116 (random rotations)
+//          chi = 64  694 / 924 / 1 820           3 963 - 4 062
+// (From 77 slots on caps of 33 are 2 %, of 65 to 67 8 % behind the one-block engine of old.)
+// Eight blocks for all in FP64 and above chi = 64 took 1 876 and 6 158 us (FP64), 2 900 - 7 200 us
+// (mixed, chi = 65 - 128) at 152 slots. One block holds M' up to chi = 70, two up to 96 (FP64 72);
+// above, two blocks keep part of it in L2. Mixed chi <= 16 takes one block always: a step of
+// these sizes is shorter than a cluster barrier is worth.
+constexpr Engine kMixed[] = {engine<float, 256, 8, 1, false>(), engine<float, 256, 4, 2, false>(),
+                             engine<float, 256, 2, 4, false>(), engine<float, 256, 2, 4, true>(),
+                             engine<float, 512, 1, 8, false>()};
+constexpr Engine kFp64[] = {engine<double, 256, 8, 1, false>(), engine<double, 256, 4, 2, false>(),
+                            engine<double, 256, 2, 4, false>(), engine<double, 256, 2, 4, true>()};
+template <int N>
+const Engine& choose(const Engine (&of)[N], int chi, int running) {
+  const Engine* best = &of[0];
+  int most = 0;
+  for (const Engine& e : of) {
+    const int n = e.slots(chi);
+    if (n > most) {
+      best = &e;
+      most = n;
+    }
+    if (n >= running) break;
+  }
+  return *best;
+}
+}  // namespace
 
 cudaError_t launch_circuit(const DevMPS& m, int prec, const CircDev& c, int64_t g0, int64_t g1, int slot0, int count,
                            int running, const double* theta, double cutoff, int max_sweeps, cudaStream_t st) {
-  if (prec == MPS_PREC_FP64)
-    return launch_cluster<double, 256, 8, 1, false>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
-  return launch_mixed<false>(m, c, g0, g1, slot0, count, running, theta, cutoff, max_sweeps, st);
+  if (prec != MPS_PREC_FP64 && m.chi <= 16)
+    return launch_cluster<float, 256, 1, 2, false, false>(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
+  const Engine& e = prec == MPS_PREC_FP64 ? choose(kFp64, m.chi, running) : choose(kMixed, m.chi, running);
+  return e.launch(m, c, g0, g1, slot0, count, theta, cutoff, max_sweeps, st);
 }
 
 }  // namespace mpsvqe
@@ -137,7 +160,8 @@ extern "C" int mps_apply_gates_noalloc(int n_qubits, int chi, void* site_tensors
   const double* theta = (const double*)(base + off_dw + 128);   // never read: every gate is fixed
   for (int64_t g0 = 0; g0 < n_gates; g0 += 16384) {
     const int64_t g1 = g0 + 16384 < n_gates ? g0 + 16384 : n_gates;
-    if (launch_mixed<true>(d, c, g0, g1, 0, 1, 1, theta, std::ldexp(1.0, -20), 60, st) != cudaSuccess) return MPS_ECUDA;
+    const auto launch = chi <= 16 ? launch_cluster<float, 256, 1, 2, true, false> : launch_cluster<float, 256, 8, 1, true, false>;
+    if (launch(d, c, g0, g1, 0, 1, theta, std::ldexp(1.0, -20), 60, st) != cudaSuccess) return MPS_ECUDA;
   }
   if (discarded_weight) {
     // the discarded weight and the status words sit next to each other in the array:

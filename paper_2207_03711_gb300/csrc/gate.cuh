@@ -100,10 +100,25 @@ struct alignas(16) ColState {
   Cx<R> f, ro, rn, pad;
 };
 
+// Own columns of T by local index, leading dimension ld (>= r): in shared memory, the first gc
+// (even) of them in global memory where a block's shared memory does not hold them all. The
+// columns leave the reduction in order, so the ones in global memory are read the least.
+template <class R>
+struct Columns {
+  Cx<R>*s, *g;   // g: null where all fit (known at compile time: the engine's TG)
+  int ld, gc;
+  template <bool TG>
+  __device__ __forceinline__ Cx<R>* at(int lc) const {
+    if constexpr (!TG) return s + lc * ld;
+    return lc < gc ? g + lc * ld : s + (lc - gc) * ld;
+  }
+};
+
 template <class R>
 struct Bidiag {
-  Cx<R>* T;            // own columns, leading dimension ld (>= r)
-  int ld;
+  Columns<R> T;        // own columns
+  int gc0;             // columns of block 0 in global memory,
+  size_t gstride;      // and from one block's to the next
   int zrows;
   Cx<R>* zp;           // [2][C VG][zrows] z partials, one per virtual rank
   Cx<R>* colp;         // [2][zrows] next column before its right update
@@ -124,7 +139,7 @@ __device__ __forceinline__ int row_shift(int rows) { return rows <= 32 ? 5 : 32 
 // holds VG. Sums over columns are formed per virtual rank and added in a fixed tree, so the
 // result has the same bits for every C with the same C VG: how many blocks a slot gets can
 // follow from how many slots run.
-template <class R, int NT, int C, int VG>
+template <class R, int NT, int C, int VG, bool TG>
 __device__ __forceinline__ void bidiagonalize_cluster(const Bidiag<R> b, const int r, const int p,
                                                       const bool right_side, const unsigned rank) {
   const int tid = threadIdx.x;
@@ -142,17 +157,24 @@ __device__ __forceinline__ void bidiagonalize_cluster(const Bidiag<R> b, const i
   auto send_norm = [&](int first, int lnext, int npar) {
     // lane pairs over the pairs of one virtual rank, in the order of its columns
     const int l = tid & 31;
+    R nn[VG];
 #pragma unroll
     for (int g = 0; g < VG; ++g) {
-      R nn = 0;
+      nn[g] = 0;
       // columns of virtual rank g at or after `first`: pairs lp = g mod VG
       const int lp0 = (first >> 1) + ((g - (first >> 1)) % VG + VG) % VG;
       for (int lc = 2 * (lp0 + (l >> 1) * VG) + (l & 1); lc < own; lc += 32 * VG)
-        if (lc >= first && lc != lnext) nn += norm2(b.cs[lc].rn);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, o);
-      if (l < C) peer<C>(b.nrmp, l)[npar * NV + (int)rank + C * g] = nn;
+        if (lc >= first && lc != lnext) nn[g] += norm2(b.cs[lc].rn);
     }
+    // side by side: one after the other, VG chains of five shuffles were the longest of a step
+    // in one block
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int g = 0; g < VG; ++g) nn[g] += __shfl_xor_sync(0xffffffffu, nn[g], o);
+#pragma unroll
+    for (int g = 0; g < VG; ++g)
+      if (l < C) peer<C>(b.nrmp, l)[npar * NV + (int)rank + C * g] = nn[g];
     if (l < C && lnext >= 0) peer<C>(b.sc, l)[npar] = b.cs[lnext].rn;
     __syncwarp();
   };
@@ -210,7 +232,8 @@ __device__ __forceinline__ void bidiagonalize_cluster(const Bidiag<R> b, const i
         col = a - X;
         b.xs[tid] = X * conj(scR);
       } else {
-        col = peer<C>(b.T, 0)[tid];
+        // column 0 is block 0's
+        col = TG && b.gc0 ? ldcg(b.T.g - (size_t)rank * b.gstride + tid) : peer<C>(b.T.s, 0)[tid];
       }
       b.us[tid] = col;
       Cx<R> d = cx<R>(0, 0);
@@ -265,25 +288,30 @@ __device__ __forceinline__ void bidiagonalize_cluster(const Bidiag<R> b, const i
         Cx<R> s = cx<R>(0, 0);
         if (act) {
           // four partial sums: the dependent chain, not the arithmetic, is what this costs
-          const Cx<R>* t = b.T + lc * b.ld + k;
-          Cx<R> sp[4];
+          auto dot = [&](const Cx<R>* t) {
+            Cx<R> sp[4];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) sp[e] = cx<R>(0, 0);
-          int i = lane == 0 ? GL : lane;
-          for (; i + 3 * GL < rows; i += 4 * GL) {
-            Cx<R> av[4], uv[4];
+            for (int e = 0; e < 4; ++e) sp[e] = cx<R>(0, 0);
+            int i = lane == 0 ? GL : lane;
+            for (; i + 3 * GL < rows; i += 4 * GL) {
+              Cx<R> av[4], uv[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              av[e] = t[i + e * GL];
-              uv[e] = b.us[i + e * GL];
+              for (int e = 0; e < 4; ++e) {
+                av[e] = t[i + e * GL];
+                uv[e] = b.us[i + e * GL];
+              }
+#pragma unroll
+              for (int e = 0; e < 4; ++e) cmac_conj(sp[e], uv[e], av[e]);
             }
 #pragma unroll
-            for (int e = 0; e < 4; ++e) cmac_conj(sp[e], uv[e], av[e]);
-          }
-#pragma unroll
-          for (int e = 0; e < 3; ++e)
-            if (i + e * GL < rows) cmac_conj(sp[e], b.us[i + e * GL], t[i + e * GL]);
-          s = (sp[0] + sp[1]) + (sp[2] + sp[3]);
+            for (int e = 0; e < 3; ++e)
+              if (i + e * GL < rows) cmac_conj(sp[e], b.us[i + e * GL], t[i + e * GL]);
+            return (sp[0] + sp[1]) + (sp[2] + sp[3]);
+          };
+          if (TG && lc < b.T.gc)
+            s = dot(b.T.g + lc * b.T.ld + k);
+          else
+            s = dot(b.T.s + (TG ? lc - b.T.gc : lc) * b.T.ld + k);
         }
 #pragma unroll
         for (int o = 1; o < GL; o <<= 1) {
@@ -302,7 +330,7 @@ __device__ __forceinline__ void bidiagonalize_cluster(const Bidiag<R> b, const i
     // into account: u^H (a_j - X conj(scR) r_j') = (a_j - X conj(scR) r_j')_0 + conj(scL)
     // (col^H a_j - col^H X conj(scR) r_j')
     for (int lc = first + tid; lc < own; lc += NT) {
-      Cx<R> rn = b.T[lc * b.ld + k], t = b.cs[lc].f;
+      Cx<R> rn = b.T.template at<TG>(lc)[k], t = b.cs[lc].f;
       const Cx<R> ro = b.cs[lc].rn;
       if (have_old) {
         cmsub(rn, b.xs[0], ro);
@@ -337,13 +365,13 @@ __device__ __forceinline__ void bidiagonalize_cluster(const Bidiag<R> b, const i
     if (cgp < groups && row < nrow) {
       const Cx<R> u = b.us[row + 1] * scL;
       const Cx<R> x = have_old ? b.xs[row + 1] : cx<R>(0, 0);
-      Cx<R>* col0 = b.T + k + 1 + row;
-      auto update = [&](int lc, const ColState<R>& q) {
-        Cx<R> v = col0[lc * b.ld];
+      Cx<R>* col0 = b.T.s + k + 1 + row - (TG ? b.T.gc * b.T.ld : 0);   // of the columns in shared memory
+      auto update = [&](Cx<R> v, const ColState<R>& q) {
         cmsub(v, x, q.ro);
         cmsub(v, q.f, u);
         return v;
       };
+      auto entry = [&](int lc) { return TG ? b.T.template at<TG>(lc) + k + 1 + row : col0 + lc * b.T.ld; };
       for (int g = cgp; g < VG; g += groups) {
         Cx<R> z1 = cx<R>(0, 0), z2 = cx<R>(0, 0);   // even and odd columns of the pairs
         const int lf = first >> 1;
@@ -353,33 +381,59 @@ __device__ __forceinline__ void bidiagonalize_cluster(const Bidiag<R> b, const i
           const int lc = 2 * lp;
           if (lc >= first && lc < own) {
             const ColState<R> q = b.cs[lc];
-            const Cx<R> v = update(lc, q);
+            Cx<R>* at = entry(lc);
+            const Cx<R> v = update(*at, q);
             if (lc == lnext) {
 #pragma unroll
               for (int c = 0; c < C; ++c) peer<C>(b.colp, c)[npar * b.zrows + row] = v;
             } else {
-              col0[lc * b.ld] = v;
+              *at = v;
               cmac_bconj(z1, v, q.rn);
             }
           }
           if (lc + 1 < own) {
             const ColState<R> q = b.cs[lc + 1];
-            const Cx<R> v = update(lc + 1, q);
+            Cx<R>* at = entry(lc + 1);
+            const Cx<R> v = update(*at, q);
             if (lc + 1 == lnext) {
 #pragma unroll
               for (int c = 0; c < C; ++c) peer<C>(b.colp, c)[npar * b.zrows + row] = v;
             } else {
-              col0[(lc + 1) * b.ld] = v;
+              *at = v;
               cmac_bconj(z2, v, q.rn);
             }
           }
           lp += VG;
         }
+        if constexpr (TG) {
+          // columns in global memory: those of two pairs on their way at a time
+          Cx<R>* cg = b.T.g + k + 1 + row;
+          const int ge = min(b.T.gc, own);
+          while (2 * lp < ge) {
+            const bool two = 2 * (lp + VG) < ge;
+            Cx<R> in[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              if (e < 2 || two) in[e] = cg[(2 * (lp + e / 2 * VG) + (e & 1)) * b.T.ld];
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+              if (e == 0 || two) {
+                const int lc = 2 * (lp + e * VG);
+                const ColState<R> q = b.cs[lc], q2 = b.cs[lc + 1];
+                const Cx<R> v = update(in[2 * e], q), v2 = update(in[2 * e + 1], q2);
+                cg[lc * b.T.ld] = v;
+                cg[(lc + 1) * b.T.ld] = v2;
+                cmac_bconj(z1, v, q.rn);
+                cmac_bconj(z2, v2, q2.rn);
+              }
+            lp += two ? 2 * VG : VG;
+          }
+        }
         for (int lc = 2 * lp; lc < own; lc += 2 * VG) {
           const ColState<R> q = b.cs[lc], q2 = b.cs[lc + 1];
-          const Cx<R> v = update(lc, q), v2 = update(lc + 1, q2);
-          col0[lc * b.ld] = v;
-          col0[(lc + 1) * b.ld] = v2;
+          const Cx<R> v = update(col0[lc * b.T.ld], q), v2 = update(col0[(lc + 1) * b.T.ld], q2);
+          col0[lc * b.T.ld] = v;
+          col0[(lc + 1) * b.T.ld] = v2;
           cmac_bconj(z1, v, q.rn);
           cmac_bconj(z2, v2, q2.rn);
         }

@@ -76,11 +76,14 @@ __device__ __forceinline__ void dot2_acc(float a, float b, float& s, float& c) {
 //             TGK arrays, its blocks, singular values, orderings
 //   work      own columns of T | pivots of the twisted factorisations | chunks of W, V or
 //             reflectors and the rows of E | GEMM tiles of the site update
-template <class R, int NT, int C, int VG>
+// TG: T does not fit; as many columns as the rest of an SM's shared memory holds stay there.
+template <class R, int NT, int C, int VG, bool TG>
 struct Plan {
   static constexpr size_t kFixed = 3072;   // gate, record, reductions, ranks, site offsets
+  static constexpr size_t kCap = 227 * 1024 - 1024;
   size_t fixed, exch, work, total;
   int mmax, cl, kc;
+  int vb;   // vectors whose twisted factorisations are in shared memory together
   __host__ __device__ static size_t up(size_t b) { return (b + 255) & ~(size_t)255; }
   // leading dimension of T: 8 (mod 16) complex<float> entries, so that the two 8-lane
   // column walks of a half warp fall into different banks
@@ -89,17 +92,22 @@ struct Plan {
     mmax = 2 * chi;
     cl = 2 * ((chi + C - 1) / C);
     kc = (chi + C - 1) / C;
+    vb = kc;
+    if (TG) {
+      const int fit = (int)(96 * 1024 / (sizeof(R) * 2 * 2 * mmax));
+      if (fit < vb) vb = fit;
+    }
     fixed = up(kFixed + sizeof(R) * 2 * mmax + sizeof(Cx<R>) * 2 * mmax);
     const size_t bidiag = up(sizeof(Cx<R>) * ((size_t)2 * C * VG * mmax + 4 * (size_t)mmax + 4 * cl + 8) +
                              sizeof(R) * 2 * C * VG);
     const size_t post = up(sizeof(R) * (2 * 2 * (size_t)mmax + 2 * mmax) + sizeof(float) * 2 * mmax +
                            (8 + 2 * 4) * (size_t)mmax + 256 * sizeof(R) + 48 + sizeof(int) * (8 * (size_t)mmax + 4) +
-                           sizeof(R) * 2 * kc * (2 * (size_t)mmax / SturmGroup<R>::v + 1));
+                           sizeof(R) * 2 * vb * (2 * (size_t)mmax / SturmGroup<R>::v + 1));
     const size_t tiles = up(gemm_tile_bytes<NT>());
     exch = bidiag > post ? bidiag : post;
     if (tiles > exch) exch = tiles;
-    const size_t t = up(sizeof(Cx<R>) * (size_t)cl * lead(mmax));
-    const size_t twist = up(sizeof(R) * (size_t)kc * 2 * 2 * mmax);
+    const size_t t = TG ? 0 : up(sizeof(Cx<R>) * (size_t)cl * lead(mmax));
+    const size_t twist = up(sizeof(R) * (size_t)vb * 2 * 2 * mmax);
     const size_t nsr = up(sizeof(R) * ((size_t)kc * chi + (size_t)chi * 33));
     const size_t nsc = sizeof(R) == 4 ? up(8 * (size_t)kc * chi + 16 * (size_t)chi * 33 + 16) : 0;
     const size_t ychunk = up(sizeof(Cx<R>) * 16 * (size_t)mmax);   // at least 16 reflectors
@@ -108,8 +116,11 @@ struct Plan {
       if (b > work) work = b;
     total = fixed + exch + work;
     // room for the whole Jacobi matrix where a block has it, and for longer chunks
-    const size_t cap = 227 * 1024 - 1024, want = up(sizeof(R) * (size_t)mmax * (mmax + 1));
-    if (want > work && fixed + exch + want <= cap) {
+    const size_t want = up(sizeof(R) * (size_t)mmax * (mmax + 1));
+    if (TG && total < kCap) {
+      work = (kCap - fixed - exch) & ~(size_t)255;
+      total = fixed + exch + work;
+    } else if (want > work && fixed + exch + want <= kCap) {
       work = want;
       total = fixed + exch + work;
     }
@@ -147,33 +158,36 @@ template <class R, int NT, int C>
 __device__ __forceinline__ R real_defect(const R* W, int k, int p, int kcv, unsigned rank, R* E, R* chunk, R* red) {
   const int tid = threadIdx.x;
   constexpr int QC = 32, LDC = 33, SP = C == 1 ? 16 : 8;
-  R acc[SP];
-#pragma unroll
-  for (int s = 0; s < SP; ++s) acc[s] = R(0);
   const int npair = kcv * k;
-  for (int q0 = 0; q0 < p; q0 += QC) {
-    load_chunk<NT>(W, k, p, q0, [&](int at, R v) { chunk[at] = v; });
+  // once, but for many vectors in two or four blocks
+  for (int e0 = tid; e0 - tid < (C == 2 || C == 4 ? npair : 1); e0 += SP * NT) {
+    R acc[SP];
 #pragma unroll
-    for (int s = 0; s < SP; ++s) {
-      const int e = tid + s * NT;
-      if (e < npair) {
-        const int i = e / k, j = e - i * k;
-        const R* wi = chunk + (rank + C * i) * LDC;
-        const R* wj = chunk + j * LDC;
-        R a = acc[s];
+    for (int s = 0; s < SP; ++s) acc[s] = R(0);
+    for (int q0 = 0; q0 < p; q0 += QC) {
+      load_chunk<NT>(W, k, p, q0, [&](int at, R v) { chunk[at] = v; });
+#pragma unroll
+      for (int s = 0; s < SP; ++s) {
+        const int e = e0 + s * NT;
+        if (e < npair) {
+          const int i = e / k, j = e - i * k;
+          const R* wi = chunk + (rank + C * i) * LDC;
+          const R* wj = chunk + j * LDC;
+          R a = acc[s];
 #pragma unroll 8
-        for (int q = 0; q < QC; ++q) a = fma(wi[q], wj[q], a);
-        acc[s] = a;
+          for (int q = 0; q < QC; ++q) a = fma(wi[q], wj[q], a);
+          acc[s] = a;
+        }
       }
     }
-  }
-  __syncthreads();
+    __syncthreads();
 #pragma unroll
-  for (int s = 0; s < SP; ++s) {
-    const int e = tid + s * NT;
-    if (e < npair) {
-      const int i = e / k, j = e - i * k;
-      E[e] = acc[s] - (j == (int)rank + C * i ? R(1) : R(0));
+    for (int s = 0; s < SP; ++s) {
+      const int e = e0 + s * NT;
+      if (e < npair) {
+        const int i = e / k, j = e - i * k;
+        E[e] = acc[s] - (j == (int)rank + C * i ? R(1) : R(0));
+      }
     }
   }
   __syncthreads();
@@ -228,14 +242,15 @@ __device__ __forceinline__ void newton_schulz_cluster(const Cx<float>* X, int k,
   auto load = [&](int q0) {
     return load_chunk<NT>(X, k, len, q0, [&](int at, Cx<float> v) { chunk[at] = to_elem(v); });
   };
-  auto gram = [&](auto sp) {
+  auto gram = [&](auto sp, int r0) {   // rows r0 .. of each thread
     constexpr int NS = decltype(sp)::value;
+    const int i1 = i0 + r0 * istep;
     SplitAcc acc[NS];
     const SplitF* row[NS];
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
       zero(acc[s]);
-      row[s] = chunk + ((int)rank + C * max(min(i0 + s * istep, kcv - 1), 0)) * LDC;
+      row[s] = chunk + ((int)rank + C * max(min(i1 + s * istep, kcv - 1), 0)) * LDC;
     }
     for (int q0 = 0; q0 < len; q0 += QC) {
       load(q0);
@@ -254,7 +269,7 @@ __device__ __forceinline__ void newton_schulz_cluster(const Cx<float>* X, int k,
     if (j < k) {
 #pragma unroll
       for (int s = 0; s < NS; ++s) {
-        const int i = i0 + s * istep;
+        const int i = i1 + s * istep;
         if (i < kcv) {
           const bool diag = j == (int)rank + C * i;
           E[i * k + j] = diag ? cx<float>(__fadd_rn(__fadd_rn(acc[s].hx, -1.0f), acc[s].lx), 0.f) : value(acc[s]);
@@ -263,15 +278,15 @@ __device__ __forceinline__ void newton_schulz_cluster(const Cx<float>* X, int k,
     }
   };
   if (ns <= 1)
-    gram(std::integral_constant<int, 1>{});
+    gram(std::integral_constant<int, 1>{}, 0);
   else if (ns <= 2)
-    gram(std::integral_constant<int, 2>{});
+    gram(std::integral_constant<int, 2>{}, 0);
   else if (ns <= 4)
-    gram(std::integral_constant<int, 4>{});
-  else if (C > 1 || ns <= 8)
-    gram(std::integral_constant<int, 8>{});
+    gram(std::integral_constant<int, 4>{}, 0);
+  else if (C == 8 || ns <= 8)
+    gram(std::integral_constant<int, 8>{}, 0);
   else
-    gram(std::integral_constant<int, C == 1 ? 16 : 8>{});
+    for (int r0 = 0; r0 < ns; r0 += 16) gram(std::integral_constant<int, C == 8 ? 8 : 16>{}, r0);
   for (int q0 = 0; q0 < len; q0 += QC) {
     const int qn = load(q0);
     for (int e = tid; e < kcv * QC; e += NT) {
@@ -435,13 +450,14 @@ __device__ __forceinline__ void st_site(Cx<R>* p, Cx<R> v) {
   }
 }
 
-template <class R, int NT, int C, int VG, bool RAW>
+template <class R, int NT, int C, int VG, bool RAW, bool TG>
 __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t g0, int64_t g1, int slot0,
                                                 const double* theta, double cutoff, int max_sweeps) {
   extern __shared__ __align__(256) unsigned char smem[];
   constexpr bool kF64 = sizeof(R) == 8;
   constexpr int NW = NT / 32;
-  const Plan<R, NT, C, VG> L(m.chi);
+  using P = Plan<R, NT, C, VG, TG>;
+  const P L(m.chi);
   const unsigned rank_c = crank<C>();
   const int blk = blockIdx.x / C, s = slot0 + blk;
   const int n = m.n, chi = m.chi, mmax = 2 * chi;
@@ -466,7 +482,7 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
   int* misc = (int*)(redc + 16);              // [0] k, [1] collapsed, [2] Jacobi caps, [3] splits
   int64_t* soff = (int64_t*)(smem + 1024);    // site offsets (128)
   int* ranks = (int*)(smem + 2048);           // bond ranks (129): every block keeps its own copy
-  R* dd = (R*)(smem + Plan<R, NT, C, VG>::kFixed);
+  R* dd = (R*)(smem + P::kFixed);
   R* ee = dd + mmax;
   Cx<R>* tau = (Cx<R>*)(ee + mmax);
   Cx<R>* scl = tau + mmax;
@@ -486,7 +502,12 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
   int* bstart = be + mmax;                    // unreduced blocks of the TGK: starts (2 mmax + 1),
   int* bpre = bstart + 2 * mmax + 1;          // values asked of the blocks before (2 mmax + 1)
   R* gscale = (R*)(((uintptr_t)(bpre + 2 * mmax + 1) + 15) & ~(uintptr_t)15);
-  Cx<R>* T = (Cx<R>*)work;
+  // columns of T: see Columns. Those in global memory lie where V comes later (12 chi^2 doubles
+  // from there on; all columns of C blocks take less)
+  const size_t gstride = (size_t)L.cl * P::lead(mmax);
+  Columns<R> T;
+  T.s = (Cx<R>*)work;
+  T.g = TG ? xout + rank_c * gstride : nullptr;
 
   const double* th = theta + (size_t)blk * c.n_params;
   int st_max_iters = 0, st_max_rank = 1, st_bad = 0, st_nonfinite = 0, st_badarg = 0;
@@ -563,7 +584,15 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
     const int rl = ranks[bond], rm = ranks[bond + 1], rr = ranks[bond + 2];
     const int mrows = 2 * rl, ncol = 2 * rr;
     const bool tall = mrows >= ncol;
-    const int tr = tall ? mrows : ncol, tp = tall ? ncol : mrows, ld = Plan<R, NT, C, VG>::lead(tr);
+    const int tr = tall ? mrows : ncol, tp = tall ? ncol : mrows;
+    T.ld = P::lead(tr);
+    T.gc = 0;
+    int gc0 = 0;
+    if constexpr (TG) {
+      const int fit = (int)(L.work / (sizeof(Cx<R>) * T.ld)) & ~1, np = tp >> 1;
+      gc0 = max(0, 2 * ((np + C - 1) / C) - fit);
+      T.gc = max(0, 2 * ((np + C - 1 - (int)rank_c) / C) - fit);
+    }
     Cx<R>* Bn = Bslot + soff[bond];
     Cx<R>* Bn1 = Bslot + soff[bond + 1];
     const double* laml = bond > 0 ? lam + (size_t)(bond - 1) * chi : nullptr;
@@ -575,13 +604,13 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
       tile_gemm<R, NT, false>(
           mrows, 2 * nq, rm, [&](int mi, int k) { return ld_site<RAW>(Bn + mi * rm + k); },
           [&](int k, int ni) { return ld_site<RAW>(Bn1 + k * ncol + (ni & 1) * rr + rank_c + C * (ni >> 1)); },
-          [&](int mi, int ni, Cx<R> v) { T[ni * ld + mi] = v; }, exch);
+          [&](int mi, int ni, Cx<R> v) { T.template at<TG>(ni)[mi] = v; }, exch);
     else
       tile_gemm<R, NT, false>(
           2 * nq, ncol, rm,
           [&](int mi, int k) { return ld_site<RAW>(Bn + (2 * (rank_c + C * (mi >> 1)) + (mi & 1)) * rm + k); },
           [&](int k, int ni) { return ld_site<RAW>(Bn1 + k * ncol + ni); },
-          [&](int mi, int ni, Cx<R> v) { T[mi * ld + ni] = v; }, exch);
+          [&](int mi, int ni, Cx<R> v) { T.template at<TG>(mi)[ni] = v; }, exch);
     double fro = 0.0;
     const int qfast = tall ? rl : rr;
     for (int it = tid; it < nq * qfast; it += NT) {
@@ -592,7 +621,7 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
 #pragma unroll
       for (int ij = 0; ij < 4; ++ij) {
         const int i = ij >> 1, j = ij & 1;
-        e[ij] = tall ? T + (size_t)(2 * o + j) * ld + 2 * f + i : T + (size_t)(2 * o + i) * ld + j * rr + f;
+        e[ij] = tall ? T.template at<TG>(2 * o + j) + 2 * f + i : T.template at<TG>(2 * o + i) + j * rr + f;
       }
       const Cx<R> th4[4] = {*e[0], *e[1], *e[2], *e[3]};
       const R la = laml ? (R)__ldcg(laml + a) : R(1);
@@ -652,7 +681,7 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
     if (huge) {
       const int rows = tall ? mrows : ncol;
       for (int it = tid; it < 2 * nq * rows; it += NT) {
-        Cx<R>* e = T + (size_t)(it / rows) * ld + it % rows;
+        Cx<R>* e = T.template at<TG>(it / rows) + it % rows;
         *e = R(0x1p-8) * *e;
       }
       csync<C>();
@@ -662,7 +691,8 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
     {
       Bidiag<R> b;
       b.T = T;
-      b.ld = ld;
+      b.gc0 = gc0;
+      b.gstride = gstride;
       b.zrows = mmax;
       b.zp = (Cx<R>*)exch;
       b.colp = b.zp + (size_t)2 * C * VG * mmax;
@@ -677,7 +707,7 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
       b.scl = scl;
       b.Y = Y;
       b.ystride = mmax;
-      bidiagonalize_cluster<R, NT, C, VG>(b, tr, tp, tall, rank_c);
+      bidiagonalize_cluster<R, NT, C, VG, TG>(b, tr, tp, tall, rank_c);
     }
     PHASE(1);
     // Golub-Kahan tridiagonal off-diagonal (d0, e0, d1, e1, ..., d_{p-1}), scaled by a power
@@ -880,16 +910,19 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
       constexpr int STEP = SturmGroup<R>::v;
       const R big = kF64 ? R(1e300) : R(1e30);
       const int odd = tall ? 0 : 1;
-      R* F = (R*)work;                       // [kcv][2][N]: minors, then reciprocal pivots, ratios, entries
+      R* F = (R*)work;                       // [nv][2][N]: minors, then reciprocal pivots, ratios, entries
       const int ns = N / STEP + 1;
       R* S = gscale;                         // [kcv][2][ns]: scale of each group of steps
       int* rng = order;                      // [kcv][3]: block start, end, twist
       if (warp == NW - 1 && lane < 16 && g + 1 < g1) fetch_gate(g + 1, lane);
       const int v = tid >> 1, dir = tid & 1;
-      const bool act = v < kcv;
+      // vectors v0 .. v0 + nv of the block at a time (all at once, but for large bonds in few blocks)
+      for (int v0 = 0; v0 < (TG ? kcv : 1); v0 += TG ? L.vb : 1) {
+      const int nv = TG ? min(kcv - v0, L.vb) : kcv;
+      const bool act = v < nv;
       int s0 = 0, e0 = N;
       if (act) {
-        const int t = rank_c + C * v;
+        const int t = rank_c + C * (v0 + v);
         const R x = sig[t];
         s0 = bs[t];
         e0 = be[t];
@@ -931,7 +964,7 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
         }
       }
       __syncthreads();
-      for (int w = warp; w < kcv; w += NW) {
+      for (int w = warp; w < nv; w += NW) {
         const int ws = rng[3 * w], we = rng[3 * w + 1];
         R* fu = F + (size_t)2 * w * N;
         R* fd = fu + N;
@@ -963,7 +996,7 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
           }
           __syncwarp();
         }
-        const R lw = sig[rank_c + C * w];
+        const R lw = sig[rank_c + C * (v0 + w)];
         R best = big;
         int at = we - 1;
         for (int i = ws + lane; i < we; i += 32) {
@@ -1017,7 +1050,7 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
         }
       }
       __syncthreads();
-      for (int w = warp; w < kcv; w += NW) {
+      for (int w = warp; w < nv; w += NW) {
         const R* z = F + (size_t)2 * w * N;
         R nrm = 0;
         for (int q = lane; q < tp; q += 32) {
@@ -1026,8 +1059,10 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
         }
         for (int o = 16; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
         const R inv = nrm > R(0) ? R(1) / sqrt(nrm) : R(0);
-        const int t = rank_c + C * w;
+        const int t = rank_c + C * (v0 + w);
         for (int q = lane; q < tp; q += 32) Wa[(size_t)t * tp + q] = z[2 * q + odd] * inv;
+      }
+      if constexpr (TG) __syncthreads();
       }
     }
     csync<C>();
@@ -1159,6 +1194,8 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
         go(std::integral_constant<int, 4>{});
       else if (ncol <= 128)
         go(std::integral_constant<int, 8>{});
+      else if (C < 8 && ncol <= 160)   // (one more copy of the loop costs eight blocks 1 % at other sizes)
+        go(std::integral_constant<int, C < 8 ? 10 : 16>{});
       else
         go(std::integral_constant<int, 16>{});
       if (rank_c == 0 && warp == 0) {
@@ -1233,10 +1270,10 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
 }  // namespace gate
 
 // One translation unit instantiates each (they compile side by side): see gate_*.cu.
-template <class R, int NT, int C, int VG, bool RAW>
+template <class R, int NT, int C, int VG, bool RAW, bool TG>
 static cudaError_t cluster_config(int chi, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at) {
-  const gate::Plan<R, NT, C, VG> L(chi);
-  if (L.total > 227 * 1024 - 1024) return cudaErrorInvalidValue;
+  const gate::Plan<R, NT, C, VG, TG> L(chi);
+  if (L.total > L.kCap) return cudaErrorInvalidValue;
   *cfg = cudaLaunchConfig_t{};
   cfg->blockDim = dim3(NT);
   cfg->dynamicSmemBytes = L.total;
@@ -1246,35 +1283,41 @@ static cudaError_t cluster_config(int chi, cudaLaunchConfig_t* cfg, cudaLaunchAt
   at->val.clusterDim.z = 1;
   cfg->attrs = at;
   cfg->numAttrs = C > 1 ? 1 : 0;
-  return gate::raise_smem_limit<gate::k_circuit<R, NT, C, VG, RAW>>();
+  return gate::raise_smem_limit<gate::k_circuit<R, NT, C, VG, RAW, TG>>();
 }
 
-template <class R, int NT, int C, int VG, bool RAW>
+template <class R, int NT, int C, int VG, bool RAW, bool TG>
 cudaError_t launch_cluster(const DevMPS& m, const CircDev& c, int64_t g0, int64_t g1, int slot0, int count,
                            const double* theta, double cutoff, int max_sweeps, cudaStream_t st) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at[1];
-  cudaError_t e = cluster_config<R, NT, C, VG, RAW>(m.chi, &cfg, at);
+  cudaError_t e = cluster_config<R, NT, C, VG, RAW, TG>(m.chi, &cfg, at);
   if (e != cudaSuccess) return e;
   cfg.gridDim = dim3((unsigned)(count * C));
   cfg.stream = st;
-  return cudaLaunchKernelEx(&cfg, gate::k_circuit<R, NT, C, VG, RAW>, m, c, g0, g1, slot0, theta, cutoff, max_sweeps);
+  return cudaLaunchKernelEx(&cfg, gate::k_circuit<R, NT, C, VG, RAW, TG>, m, c, g0, g1, slot0, theta, cutoff, max_sweeps);
 }
 
-// The registers of one block fill an SM, so the answer does not depend on chi and is asked
-// for once per device; 0 (then fewer blocks per slot are taken) where it cannot be had.
-template <class R, int NT, int C, int VG, bool RAW>
+// 0 where the bond cap does not fit. The registers of one block fill an SM, so else the answer
+// does not depend on chi and is asked for once per device; 0 too (then other instances are
+// taken) where it cannot be had.
+template <class R, int NT, int C, int VG, bool RAW, bool TG>
 int max_clusters(int chi) {
   static std::atomic<int> known[64];
   int dev = 0;
+  if (gate::Plan<R, NT, C, VG, TG>(chi).total > gate::Plan<R, NT, C, VG, TG>::kCap) return 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
   int n = known[dev].load();
+  if (C == 1 && n == 0) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    known[dev].store(n);
+  }
   if (n == 0) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[1];
-    if (cluster_config<R, NT, C, VG, RAW>(chi, &cfg, at) != cudaSuccess) return 0;
+    if (cluster_config<R, NT, C, VG, RAW, TG>(chi, &cfg, at) != cudaSuccess) return 0;
     cfg.gridDim = dim3(C);
-    if (cudaOccupancyMaxActiveClusters(&n, gate::k_circuit<R, NT, C, VG, RAW>, &cfg) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveClusters(&n, gate::k_circuit<R, NT, C, VG, RAW, TG>, &cfg) != cudaSuccess) return 0;
     known[dev].store(n);
   }
   return n;

@@ -226,3 +226,20 @@ def test_gate_that_annihilates_the_state(prec, chi, ranks):
     assert rg[bond] == 1 and lams[bond][0] == 0.0
     assert not sites[bond].any()
     assert np.linalg.norm(sites[bond + 1]) == 1.0
+
+
+# (cap, precision): every number of blocks a slot can get, T wholly in shared memory or partly in L2
+@pytest.mark.parametrize("n,chi,prec", [(8, 9, G.MPS_FP64), (10, 24, G.MPS_FP64), (14, 64, G.MPS_FP64), (14, 80, G.MPS_FP64),
+                                        (14, 65, G.MPS_MIXED), (14, 72, G.MPS_MIXED), (16, 97, G.MPS_MIXED),
+                                        (16, 128, G.MPS_MIXED)])
+def test_blocks_per_slot_do_not_change_results(n, chi, prec):
+    rng = np.random.default_rng(chi)
+    nrot = 9                                   # each doubles the rank of every bond until it is full
+    C = G.circ_create(rng.integers(1, 4, (nrot, n)).astype(np.uint8), np.arange(nrot, dtype=np.int32), np.ones(nrot))
+    H = G.ham_create(rng.integers(0, 4, (40, n)).astype(np.uint8), rng.normal(size=40))
+    M = G.mps_create(n, chi, prec, n_slots=80)
+    theta = rng.uniform(0.3, 2.5, (80, nrot))
+    alone = np.array([G.vqe_energy(M, C, H, t) for t in theta[:2]])
+    assert G.mps_get_stats(M)["max_rank"] > 0.75 * min(chi, 2 ** (n // 2))
+    for count in (8, 16, 39, 80):
+        assert np.array_equal(G.vqe_energy_batch(M, C, H, theta[:count])[:2], alone)
