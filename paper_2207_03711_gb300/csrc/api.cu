@@ -612,9 +612,15 @@ static int meas_chunk(MeasWalk& c, int k, int u0, int u1) {
       for (int64_t x = a; x < b;) {
         const int ub = par[x], ue = std::min(ub + m->tc64.batch, par[b - 1] + 1);
         const int64_t y = std::lower_bound(par.begin() + x, par.begin() + b, ue) - par.begin();
-        CU(env_fp64_T(m->tc64, (const Cx<double>*)L + (size_t)(ub - u0) * D * D, k, ue - ub, D, Dp, m->st));
-        CU(env_fp64_children(m->tc64, c.h->d_parent[k + 1] + x, c.h->d_edge[k + 1] + x, (int)(y - x), ub, ue - ub, D, Dp,
-                             (Cx<double>*)m->lvl_L[k + 1] + (size_t)(x - a) * Dp * Dp, m->st));
+        const int nu = ue - ub, nch = (int)(y - x);
+        cudaEvent_t e0, e1;
+        TRY(next_event_pair(m, &e0, &e1));
+        CU(env_fp64_T(m->tc64, (const Cx<double>*)L + (size_t)(ub - u0) * D * D, k, nu, D, Dp, m->st, e0, e1));
+        TRY(next_event_pair(m, &e0, &e1));
+        CU(env_fp64_children(m->tc64, c.h->d_parent[k + 1] + x, c.h->d_edge[k + 1] + x, nch, ub, nu, D, Dp,
+                             (Cx<double>*)m->lvl_L[k + 1] + (size_t)(x - a) * Dp * Dp, m->st, e0, e1));
+        m->stats.tc_gemm_launches += 2;
+        m->stats.tc_gemm_flops += 2.0 * ((double)nu * D) * (4.0 * Dp) * (2.0 * D) + 2.0 * (2.0 * Dp) * ((double)nch * Dp) * (4.0 * D);
         c.launches += 4;
         x = y;
       }

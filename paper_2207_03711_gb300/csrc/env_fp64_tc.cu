@@ -455,7 +455,8 @@ cudaError_t env_fp64_site(const EnvFp64& s, const Cx<double>* Bk, int k, int D, 
   return cudaGetLastError();
 }
 
-cudaError_t env_fp64_T(const EnvFp64& s, const Cx<double>* L, int k, int U, int D, int Dp, cudaStream_t st) {
+cudaError_t env_fp64_T(const EnvFp64& s, const Cx<double>* L, int k, int U, int D, int Dp, cudaStream_t st, cudaEvent_t e0,
+                       cudaEvent_t e1) {
   if (U <= 0) return cudaSuccess;
   const int* bal = s.bal + (size_t)k * s.chi;
   const Parts p = carve(s.scratch, s.chi, s.batch);
@@ -472,13 +473,15 @@ cudaError_t env_fp64_T(const EnvFp64& s, const Cx<double>* L, int k, int U, int 
   g.a_ex = p.bt_ex;
   g.b_ex = p.l_ex;
   g.T = p.T;
+  if (e0 && (e = cudaEventRecord(e0, st)) != cudaSuccess) return e;
   if ((e = launch<false>(g, p.bt, pad8(2 * D), p.l, pad8(2 * D), s.err, st)) != cudaSuccess) return e;
+  if (e1 && (e = cudaEventRecord(e1, st)) != cudaSuccess) return e;
   k_split_T<<<(unsigned)((cols + 7) / 8), 256, 0, st>>>(p.T, U, D, Dp, bal, p.t, p.t_ex);
   return cudaGetLastError();
 }
 
 cudaError_t env_fp64_children(const EnvFp64& s, const int32_t* parent, const uint8_t* edge, int nc, int node_base, int U, int D,
-                              int Dp, Cx<double>* Lout, cudaStream_t st) {
+                              int Dp, Cx<double>* Lout, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1) {
   if (nc <= 0) return cudaSuccess;
   const Parts p = carve(s.scratch, s.chi, s.batch);
   DigitGemm g;
@@ -497,7 +500,10 @@ cudaError_t env_fp64_children(const EnvFp64& s, const int32_t* parent, const uin
   g.ds = pad8(D);
   g.per = (Dp + BN - 1) / BN;
   g.L = Lout;
-  return launch<true>(g, p.a2, 8 * pad64(D), p.t, 4 * pad8(D), s.err, st);
+  cudaError_t e;
+  if (e0 && (e = cudaEventRecord(e0, st)) != cudaSuccess) return e;
+  if ((e = launch<true>(g, p.a2, 8 * pad64(D), p.t, 4 * pad8(D), s.err, st)) != cudaSuccess) return e;
+  return e1 ? cudaEventRecord(e1, st) : cudaSuccess;
 }
 
 }  // namespace mpsvqe

@@ -148,3 +148,43 @@ def test_a_smaller_budget_gives_the_memory_back(prec):
     small = held([1])
     assert held([0]) > 2 * small
     assert held([0, 1]) == small
+
+
+def test_fp64_levels_of_many_batches():
+    """chi = 256: a batch of the digit products holds 64 nodes, the levels here have hundreds,
+    some without children. Against the oracle, and bit for bit against chunks of 16 nodes."""
+    n, chi = 18, 256
+    st = _polarised(n, syn.full_ranks(n, chi), 6)
+    codes = _random_strings(n, 300, 7)
+    M = G.mps_create(n, chi, G.MPS_FP64)
+    G.mps_set_state(M, st.B, st.lam)
+    v = G.mps_expect_paulis(M, codes)
+    assert G.mps_get_stats(M)["tc_gemm_launches"] > 0
+    G.mps_set_meas_budget(M, 1)
+    assert np.array_equal(G.mps_expect_paulis(M, codes), v)
+    some = np.arange(0, 300, 25)
+    ref = np.array([mps.expect_string(st, codes[i]) for i in some]) / mps.norm2(st)
+    assert np.abs(v[some] - ref).max() <= n * 16 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("prec,tol", [(G.MPS_FP64, 16 * 160 * 2.0 ** -53), (G.MPS_MIXED, 2e-5)])
+def test_ranks_that_fall_fast(prec, tol):
+    """A bond above 64 beside one below the tensor cores' smallest (neither route, nor the fused
+    kernels): loaded tensors may have any ranks within the caps. They are not canonical either:
+    sums of |L| |B| are up to the root of a bond above <psi|psi>."""
+    n, chi = 16, 128
+    ranks = [2, 4, 8, 16, 32, 64, 100, 12, 90, 64, 32, 16, 8, 4, 2]
+    r = [1] + ranks + [1]
+    rng = np.random.default_rng(2)
+    B = [(rng.normal(size=(r[k], 2, r[k + 1])) + 1j * rng.normal(size=(r[k], 2, r[k + 1]))) / np.sqrt(4 * r[k + 1])
+         for k in range(n)]
+    st = mps.MPS(B, [np.ones(x) for x in ranks])
+    codes = _random_strings(n, 60, 8)
+    codes[:20, :6] = 0
+    M = G.mps_create(n, chi, prec)
+    G.mps_set_state(M, B, st.lam)
+    v = G.mps_expect_paulis(M, codes)
+    ref = np.array([mps.expect_string(st, c) for c in codes]) / mps.norm2(st)
+    assert np.abs(v - ref).max() <= tol
+    G.mps_set_meas_budget(M, 1)
+    assert np.array_equal(G.mps_expect_paulis(M, codes), v)
