@@ -294,12 +294,13 @@ static int ensure_theta(mps_s* m, size_t count) {
 // instead of three, would be ahead at the small end: with 100 strings 0.87 ms instead of 1.01 at 34,
 // 1.08 / 1.10 at 49, 1.24 / 1.09 at 64.
 constexpr int kTcMinDim = 33;
-// FP64 levels with both bonds in this range multiply by digits on the tensor cores
+// FP64 levels with both bonds from here on multiply by digits on the tensor cores
 // (env_fp64_tc.cu). Against the fused FP64 kernel (k_level_fused64), an 18-qubit molecular
 // Hamiltonian and 30 random strings: 3.5 ms instead of 3.0 and 1.3 instead of 0.9 at bonds of
 // 16, 4.2 / 6.8 and 1.8 / 2.0 at 20, 4.4 / 8.8 and 1.9 / 2.3 at 24, 8.6 / 62 and 3.1 / 16 at
-// 64. Up to 512 the 64-bit sums cannot overflow.
-constexpr int kFp64TcMinDim = 17, kFp64TcMaxDim = 512;
+// 64.
+constexpr int kFp64TcMinDim = 17;
+static_assert(kMaxChi <= 512, "the 64-bit sums of the digit products");
 struct MeasPlan {
   std::vector<int32_t> cap;
   size_t level_bytes = 0, tc_bytes = 0;
@@ -548,8 +549,7 @@ static int meas_chunk(MeasWalk& c, int k, int u0, int u1) {
   void* L = m->lvl_L[k];
   void* T = m->lvl_T[k];
   const bool tc = m->prec == MPS_MIXED && m->tc.scratch && D >= kTcMinDim && Dp >= kTcMinDim;
-  const bool tc64 = m->prec == MPS_FP64 && m->tc64.scratch && std::min(D, Dp) >= kFp64TcMinDim &&
-                    std::max(D, Dp) <= kFp64TcMaxDim;
+  const bool tc64 = m->prec == MPS_FP64 && m->tc64.scratch && std::min(D, Dp) >= kFp64TcMinDim;
   const bool fused = !tc && !tc64 && D <= kFusedMax && Dp <= kFusedMax;
   const bool leaf = k + 1 >= t.n_levels || k + 1 >= m->n;
   if (tc && !leaf) {

@@ -106,18 +106,14 @@ __device__ __forceinline__ Cx<float> value(const SplitAcc& a) {
   return cx<float>(__fadd_rn(a.hx, a.lx), __fadd_rn(a.hy, a.ly));
 }
 __device__ __forceinline__ Cx<double> value(const Cx<double>& a) { return a; }
-__device__ __forceinline__ void zero(Cx<float>& a) { a = cx<float>(0, 0); }
-__device__ __forceinline__ void mac(Cx<float>& c, const Cx<float>& a, const Cx<float>& b) { cmac(c, a, b); }
-__device__ __forceinline__ Cx<float> value(const Cx<float>& a) { return a; }
-// EXACT: split products (FP32)
-template <class R, bool EXACT>
+template <class R>
 struct Gemm {
   using E = Cx<R>;
   using A = Cx<R>;
   static __device__ __forceinline__ E elem(Cx<R> a) { return a; }
 };
 template <>
-struct Gemm<float, true> {
+struct Gemm<float> {
   using E = SplitF;
   using A = SplitAcc;
   static __device__ __forceinline__ E elem(Cx<float> a) { return to_elem(a); }
@@ -134,9 +130,9 @@ __host__ __device__ constexpr size_t gemm_tile_bytes() {   // of the largest til
   constexpr int TY = NT / 16;
   return 16 * (size_t)((4 * TY) * (kKT + 1) + kKT * (64 + 1));
 }
-template <class R, int NT, int RM, int JN, bool KF, bool EXACT, class FA, class FB, class FC>
+template <class R, int NT, int RM, int JN, bool KF, class FA, class FB, class FC>
 __device__ __forceinline__ void tile_gemm_shape(int M, int N, int K, FA fa, FB fb, FC fc, unsigned char* smem) {
-  using G = Gemm<R, EXACT>;
+  using G = Gemm<R>;
   using E = typename G::E;
   constexpr int TY = NT / 16, TM = TY * RM, TN = 16 * JN, KT = kKT;
   constexpr int NA = TM * KT / NT, NB = KT * TN / NT > 0 ? KT * TN / NT : 1;
@@ -219,18 +215,18 @@ __device__ __forceinline__ void tile_gemm_shape(int M, int N, int K, FA fa, FB f
 
 // Shape by the narrow side: what one thread computes is kept at four outputs where the
 // product has them, and small products spread over all threads.
-template <class R, int NT, bool KF, bool EXACT = true, class FA, class FB, class FC>
+template <class R, int NT, bool KF, class FA, class FB, class FC>
 __device__ __forceinline__ void tile_gemm(int M, int N, int K, FA fa, FB fb, FC fc, unsigned char* smem) {
   constexpr int TY = NT / 16;
   if (N <= 16) {
     if (M <= TY)
-      tile_gemm_shape<R, NT, 1, 1, KF, EXACT>(M, N, K, fa, fb, fc, smem);
+      tile_gemm_shape<R, NT, 1, 1, KF>(M, N, K, fa, fb, fc, smem);
     else
-      tile_gemm_shape<R, NT, 4, 1, KF, EXACT>(M, N, K, fa, fb, fc, smem);
+      tile_gemm_shape<R, NT, 4, 1, KF>(M, N, K, fa, fb, fc, smem);
   } else if (N <= 32 && M > TY) {
-    tile_gemm_shape<R, NT, 2, 2, KF, EXACT>(M, N, K, fa, fb, fc, smem);
+    tile_gemm_shape<R, NT, 2, 2, KF>(M, N, K, fa, fb, fc, smem);
   } else {
-    tile_gemm_shape<R, NT, 1, 4, KF, EXACT>(M, N, K, fa, fb, fc, smem);
+    tile_gemm_shape<R, NT, 1, 4, KF>(M, N, K, fa, fb, fc, smem);
   }
 }
 

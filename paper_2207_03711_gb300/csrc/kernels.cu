@@ -50,10 +50,8 @@ cudaError_t launch_reset(const DevMPS& m, int prec, int slot0, int count, const 
 }
 
 // ------------------------------------------------------------ small tiled GEMM
-// C (Mdim x Ndim, ldc) = sum_t s_t opA_t(A_t) opB_t(B_t) with NTH threads (256 or 512)
-// and 64x64 tiles. opA: A stored Mdim x K (lda), or K x Mdim used as A^H (conjT).
-// opB: B stored K x Ndim (ldb), or Ndim x K used as B^T (transB); conjB conjugates the
-// entries of B as they are loaded.
+// C (Mdim x Ndim, ldc) = sum_t s_t opA_t(A_t) B_t with 256 threads and 64x64 tiles. opA: A
+// stored Mdim x K (lda), or K x Mdim used as A^H (conjT). B stored K x Ndim (ldb).
 template <class R>
 struct GemmTerm {
   const Cx<R>* A;
@@ -62,15 +60,13 @@ struct GemmTerm {
   const Cx<R>* B;
   int ldb;
   Cx<R> s;
-  bool transB;
-  bool conjB = false;
 };
 
 // One 64 x 64 output tile at (m0, n0).
-template <class R, int NTH>
+template <class R>
 __device__ void gemm_tile(int m0, int n0, int Mdim, int Ndim, int K, const GemmTerm<R>* terms, int nterm, Cx<R>* C,
                           int ldc, Cx<R> (*As)[17], Cx<R> (*Bs)[65]) {
-  constexpr int TY = NTH / 16, RPT = 64 / TY;
+  constexpr int NTH = 256, TY = NTH / 16, RPT = 64 / TY;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   Cx<R> acc[RPT][4];
 #pragma unroll
@@ -88,11 +84,9 @@ __device__ void gemm_tile(int m0, int n0, int Mdim, int Ndim, int K, const GemmT
         As[r][cc] = T.s * v;
       }
       for (int e = threadIdx.x; e < 16 * 64; e += NTH) {
-        const int r = T.transB ? (e & 15) : (e >> 6), cc = T.transB ? (e >> 4) : (e & 63);
+        const int r = e >> 6, cc = e & 63;
         const int gk = k0 + r, gn = n0 + cc;
-        Cx<R> v = cx<R>(0, 0);
-        if (gk < K && gn < Ndim) v = T.transB ? T.B[(size_t)gn * T.ldb + gk] : T.B[(size_t)gk * T.ldb + gn];
-        Bs[r][cc] = T.conjB ? conj(v) : v;
+        Bs[r][cc] = gk < K && gn < Ndim ? T.B[(size_t)gk * T.ldb + gn] : cx<R>(0, 0);
       }
       __syncthreads();
 #pragma unroll 4
@@ -119,11 +113,11 @@ __device__ void gemm_tile(int m0, int n0, int Mdim, int Ndim, int K, const GemmT
     }
 }
 
-template <class R, int NTH>
+template <class R>
 __device__ void block_gemm(int Mdim, int Ndim, int K, const GemmTerm<R>* terms, int nterm, Cx<R>* C, int ldc,
                            Cx<R> (*As)[17], Cx<R> (*Bs)[65]) {
   for (int m0 = 0; m0 < Mdim; m0 += 64)
-    for (int n0 = 0; n0 < Ndim; n0 += 64) gemm_tile<R, NTH>(m0, n0, Mdim, Ndim, K, terms, nterm, C, ldc, As, Bs);
+    for (int n0 = 0; n0 < Ndim; n0 += 64) gemm_tile<R>(m0, n0, Mdim, Ndim, K, terms, nterm, C, ldc, As, Bs);
 }
 
 // --------------------------------------------------------- right environments
@@ -348,8 +342,8 @@ __global__ void __launch_bounds__(256) k_level_T(DevMPS m, int slot, int k, cons
   const int Dk = rank[k], Dk1 = rank[k + 1];
   const Cx<R>* Bk = (const Cx<R>*)m.B + (size_t)slot * m.slot_elems + m.site_off[k];
   const int ld = env_ld<R>(Dk);
-  GemmTerm<R> t{Lin + u * env_node<R>(Dk), ld, false, Bk + j * Dk1, 2 * Dk1, cx<R>(1, 0), false};
-  block_gemm<R, 256>(Dk, Dk1, Dk, &t, 1, T + ((size_t)u * 2 + j) * Dk * Dk1, Dk1, As, Bs);
+  GemmTerm<R> t{Lin + u * env_node<R>(Dk), ld, false, Bk + j * Dk1, 2 * Dk1, cx<R>(1, 0)};
+  block_gemm<R>(Dk, Dk1, Dk, &t, 1, T + ((size_t)u * 2 + j) * Dk * Dk1, Dk1, As, Bs);
 }
 
 // L_{k+1}[c] = sum_ij sigma_ij (B_k^i)^+ T_j[parent(c)]
@@ -369,10 +363,10 @@ __global__ void __launch_bounds__(256) k_level_child(DevMPS m, int slot, int k, 
   letter_entries<R>(edge[c], ii, jj, sg);
   GemmTerm<R> t[2];
   for (int e = 0; e < 2; ++e)
-    t[e] = GemmTerm<R>{Bk + ii[e] * Dk1, 2 * Dk1, true, T + ((size_t)u * 2 + jj[e]) * Dk * Dk1, Dk1, sg[e], false};
+    t[e] = GemmTerm<R>{Bk + ii[e] * Dk1, 2 * Dk1, true, T + ((size_t)u * 2 + jj[e]) * Dk * Dk1, Dk1, sg[e]};
   const int ld = env_ld<R>(Dk1);
   Cx<R>* out = Lout + c * env_node<R>(Dk1);
-  block_gemm<R, 256>(Dk1, Dk1, Dk, t, 2, out, ld, As, Bs);
+  block_gemm<R>(Dk1, Dk1, Dk, t, 2, out, ld, As, Bs);
   for (int64_t e = threadIdx.x + (int64_t)Dk1 * ld; e < env_node<R>(Dk1); e += 256) out[e] = cx<R>(0, 0);
   if (ld > Dk1)
     for (int r = threadIdx.x; r < Dk1; r += 256) out[(size_t)r * ld + Dk1] = cx<R>(0, 0);
