@@ -347,7 +347,7 @@ def run_ours(args):
     K, W = args.steps, max(3, args.warmup)
     n_sm = torch.cuda.get_device_properties(local).multi_processor_count
     if K > n_sm:
-        raise SystemExit(f"--steps {K} exceeds the {n_sm} SMs: the timed steps run side by side, one SM each")
+        raise SystemExit(f"--steps {K} exceeds the {n_sm} SMs: the timed steps run side by side, one SM each at least")
     M = G.mps_create(N_QUBITS, CHI, G.MPS_MIXED, n_slots=max(K, W), cuda_stream=stream)
     # thetas of the timed steps in pinned host memory (uploaded inside the timed call)
     th_pinned = torch.empty((K, C.n_params), dtype=torch.float64, pin_memory=True)
@@ -660,7 +660,7 @@ def run_config3(args):
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peaks["fp32_tflops"], "unit": "TFLOP/s",
                          "frac": achieved / peaks["fp32_tflops"], "traffic": None,
                          "peak_source": "measured: cuBLAS SGEMM in this process (FP32 CUDA cores)",
-                         "kernel": "k_circuit<float> (one cluster of 8 blocks per circuit)"},
+                         "kernel": "k_circuit<float> (one cluster of 2 to 8 blocks per circuit)"},
             "breakdown_ms_per_step": {"circuit": float(np.mean(circ_ms)), "measure": float(np.mean(meas_ms))},
             "gradient_norm": float(np.linalg.norm(grad)), "clocks": clocks}
     print(json.dumps(line))

@@ -133,7 +133,9 @@ int circ_destroy(circ_t circ);
 
 /* Allocate n_slots MPS states of n_qubits sites with bond cap chi (Eq. 6) on the
  * current device, each initialised to the all-zero product state. precision:
- * MPS_FP64 (complex128 tensors, FP64 SVD and contractions) or MPS_MIXED (complex64
+ * MPS_FP64 (complex128 tensors, FP64 SVD and contractions; environment contractions of
+ * bonds >= 17 on the tensor cores by exact digit products, 55 bits of each entry below the
+ * largest of its row after a power-of-two balance of the bonds) or MPS_MIXED (complex64
  * tensors, FP32 SVD with a compensated re-orthonormalisation of the kept singular
  * vectors, FP32 gate contractions, environment contractions of bonds >= 33 on the
  * tensor cores with compensated TF32 splits, FP64 Schmidt numbers and energy sums).
@@ -184,7 +186,7 @@ int mps_apply_gates(mps_t mps, int64_t n_gates, const int32_t* bond, const doubl
  * <psi|P_i|psi> / <psi|psi> on slot 0, by exact transfer-matrix contraction over
  * a prefix trie (shared left environments, walked depth first in chunks) and right
  * identity environments. Returns MPS_ETIMEOUT if a bounded wait inside a tensor-core
- * GEMM ran out (mixed precision). */
+ * GEMM ran out. */
 int mps_expect_paulis(mps_t mps, int64_t n_terms, const uint8_t* paulis, double* re, double* im);
 
 /* Checkpoint / inspection of one slot. ranks: n_qubits-1 bond ranks.

@@ -13,7 +13,7 @@
 // gate of a saturated circuit, with one block per slot before and now: FP64 chi = 16 1 000 and
 // 115 us, chi = 64 16.8 and 1.6 ms; mixed chi = 16 60 and 38 us (one block still), chi = 33 280
 // and 135, chi = 64 746 and 263 us, chi = 128 (M' in L2 before, in shared memory now) 6.5 and
-// 0.74 ms.
+// 0.74 ms, all with one slot; with many, see gate.cu.
 #pragma once
 #include <atomic>
 #include <type_traits>
@@ -918,151 +918,151 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
       const int v = tid >> 1, dir = tid & 1;
       // vectors v0 .. v0 + nv of the block at a time (all at once, but for large bonds in few blocks)
       for (int v0 = 0; v0 < (TG ? kcv : 1); v0 += TG ? L.vb : 1) {
-      const int nv = TG ? min(kcv - v0, L.vb) : kcv;
-      const bool act = v < nv;
-      int s0 = 0, e0 = N;
-      if (act) {
-        const int t = rank_c + C * (v0 + v);
-        const R x = sig[t];
-        s0 = bs[t];
-        e0 = be[t];
-        if (dir == 0) {
-          rng[3 * v] = s0;
-          rng[3 * v + 1] = e0;
-        }
-        // entry q of the walk is index i0 + st q; its off-diagonal is b2[i0 + st q + bo]
-        const int st = dir ? -1 : 1, i0 = dir ? e0 - 1 : s0, bo = dir ? 0 : -1, len = e0 - s0;
-        R* f = F + (size_t)(2 * v + dir) * N;
-        R* sg = S + (size_t)(2 * v + dir) * ns;
-        R prev = R(1), cur = -x;
-        f[i0] = cur;
-        int q = 1, gi = 0;
-        for (; q + STEP <= len; q += STEP) {
-          R bb[STEP], o[STEP];
+        const int nv = TG ? min(kcv - v0, L.vb) : kcv;
+        const bool act = v < nv;
+        int s0 = 0, e0 = N;
+        if (act) {
+          const int t = rank_c + C * (v0 + v);
+          const R x = sig[t];
+          s0 = bs[t];
+          e0 = be[t];
+          if (dir == 0) {
+            rng[3 * v] = s0;
+            rng[3 * v + 1] = e0;
+          }
+          // entry q of the walk is index i0 + st q; its off-diagonal is b2[i0 + st q + bo]
+          const int st = dir ? -1 : 1, i0 = dir ? e0 - 1 : s0, bo = dir ? 0 : -1, len = e0 - s0;
+          R* f = F + (size_t)(2 * v + dir) * N;
+          R* sg = S + (size_t)(2 * v + dir) * ns;
+          R prev = R(1), cur = -x;
+          f[i0] = cur;
+          int q = 1, gi = 0;
+          for (; q + STEP <= len; q += STEP) {
+            R bb[STEP], o[STEP];
 #pragma unroll
-          for (int u = 0; u < STEP; ++u) bb[u] = b2[i0 + st * (q + u) + bo];
+            for (int u = 0; u < STEP; ++u) bb[u] = b2[i0 + st * (q + u) + bo];
 #pragma unroll
-          for (int u = 0; u < STEP; ++u) {
-            const R nxt = fma(-x, cur, -(bb[u] * prev));
+            for (int u = 0; u < STEP; ++u) {
+              const R nxt = fma(-x, cur, -(bb[u] * prev));
+              prev = cur;
+              cur = nxt;
+              o[u] = cur;
+            }
+            const R sc = rescale_factor(prev, cur);
+            prev *= sc;
+            cur *= sc;
+            o[STEP - 1] = cur;   // the last of a group is kept scaled; the group's scale beside it
+#pragma unroll
+            for (int u = 0; u < STEP; ++u) f[i0 + st * (q + u)] = o[u];
+            sg[gi++] = sc;
+          }
+          for (; q < len; ++q) {
+            const R nxt = fma(-x, cur, -(b2[i0 + st * q + bo] * prev));
             prev = cur;
             cur = nxt;
-            o[u] = cur;
+            f[i0 + st * q] = cur;
           }
-          const R sc = rescale_factor(prev, cur);
-          prev *= sc;
-          cur *= sc;
-          o[STEP - 1] = cur;   // the last of a group is kept scaled; the group's scale beside it
-#pragma unroll
-          for (int u = 0; u < STEP; ++u) f[i0 + st * (q + u)] = o[u];
-          sg[gi++] = sc;
         }
-        for (; q < len; ++q) {
-          const R nxt = fma(-x, cur, -(b2[i0 + st * q + bo] * prev));
-          prev = cur;
-          cur = nxt;
-          f[i0 + st * q] = cur;
-        }
-      }
-      __syncthreads();
-      for (int w = warp; w < nv; w += NW) {
-        const int ws = rng[3 * w], we = rng[3 * w + 1];
-        R* fu = F + (size_t)2 * w * N;
-        R* fd = fu + N;
-        // reciprocal pivots in place, walking against the recurrence so that the minor
-        // before is still there: entry q needs entries q and q - 1 of its walk
-        const int len = we - ws;
-        for (int hi_q = len; hi_q > 0; hi_q -= 32) {
-          const int q = hi_q - 1 - lane;
-          R r0 = 0, r1 = 0;
-          if (q >= 0) {
+        __syncthreads();
+        for (int w = warp; w < nv; w += NW) {
+          const int ws = rng[3 * w], we = rng[3 * w + 1];
+          R* fu = F + (size_t)2 * w * N;
+          R* fd = fu + N;
+          // reciprocal pivots in place, walking against the recurrence so that the minor
+          // before is still there: entry q needs entries q and q - 1 of its walk
+          const int len = we - ws;
+          for (int hi_q = len; hi_q > 0; hi_q -= 32) {
+            const int q = hi_q - 1 - lane;
+            R r0 = 0, r1 = 0;
+            if (q >= 0) {
 #pragma unroll
-            for (int d = 0; d < 2; ++d) {
-              const R* f = d ? fd : fu;
-              const R* sg = S + (size_t)(2 * w + d) * ns;
-              const int at = d ? we - 1 - q : ws + q, pv = d ? at + 1 : at - 1;
-              R num = q > 0 ? f[pv] : R(1);
-              // q closes group (q - 1) / STEP when q = STEP, 2 STEP, ..., if that group was whole
-              if (q > 0 && q % STEP == 0) num *= sg[q / STEP - 1];
-              const R den = f[at];
-              R r = num * inverse(den);
-              if (!(rabs(r) <= big)) r = -big;   // a zero pivot counts as a tiny negative one
-              (d ? r1 : r0) = r;
+              for (int d = 0; d < 2; ++d) {
+                const R* f = d ? fd : fu;
+                const R* sg = S + (size_t)(2 * w + d) * ns;
+                const int at = d ? we - 1 - q : ws + q, pv = d ? at + 1 : at - 1;
+                R num = q > 0 ? f[pv] : R(1);
+                // q closes group (q - 1) / STEP when q = STEP, 2 STEP, ..., if that group was whole
+                if (q > 0 && q % STEP == 0) num *= sg[q / STEP - 1];
+                const R den = f[at];
+                R r = num * inverse(den);
+                if (!(rabs(r) <= big)) r = -big;   // a zero pivot counts as a tiny negative one
+                (d ? r1 : r0) = r;
+              }
+            }
+            __syncwarp();
+            if (q >= 0) {
+              fu[ws + q] = r0;
+              fd[we - 1 - q] = r1;
+            }
+            __syncwarp();
+          }
+          const R lw = sig[rank_c + C * (v0 + w)];
+          R best = big;
+          int at = we - 1;
+          for (int i = ws + lane; i < we; i += 32) {
+            // gamma_i = -lam - b_{i-1}^2 / dp_{i-1} - b_i^2 / dm_{i+1}
+            R gm = -lw;
+            if (i > ws) gm = fma(-b2[i - 1], fu[i - 1], gm);
+            if (i < we - 1) gm = fma(-b2[i], fd[i + 1], gm);
+            gm = rabs(gm);
+            if (gm < best) {
+              best = gm;
+              at = i;
             }
           }
-          __syncwarp();
-          if (q >= 0) {
-            fu[ws + q] = r0;
-            fd[we - 1 - q] = r1;
+          for (int o = 16; o > 0; o >>= 1) {
+            const R ob = __shfl_xor_sync(0xffffffffu, best, o);
+            const int oa = __shfl_xor_sync(0xffffffffu, at, o);
+            if (ob < best || (ob == best && oa < at)) {
+              best = ob;
+              at = oa;
+            }
           }
-          __syncwarp();
-        }
-        const R lw = sig[rank_c + C * (v0 + w)];
-        R best = big;
-        int at = we - 1;
-        for (int i = ws + lane; i < we; i += 32) {
-          // gamma_i = -lam - b_{i-1}^2 / dp_{i-1} - b_i^2 / dm_{i+1}
-          R gm = -lw;
-          if (i > ws) gm = fma(-b2[i - 1], fu[i - 1], gm);
-          if (i < we - 1) gm = fma(-b2[i], fd[i + 1], gm);
-          gm = rabs(gm);
-          if (gm < best) {
-            best = gm;
-            at = i;
+          if (lane == 0) rng[3 * w + 2] = at;
+          // ratios z_i / z_{i+1} = -b_i / dp_i above the twist, z_i / z_{i-1} = -b_{i-1} / dm_i below
+          for (int i = lane; i < N; i += 32) {
+            R r = 0;
+            if (i >= ws && i < at) r = -bn[i] * fu[i];
+            if (i > at && i < we) r = -bn[i - 1] * fd[i];
+            if (i == at) r = R(1);
+            fu[i] = r;
           }
         }
-        for (int o = 16; o > 0; o >>= 1) {
-          const R ob = __shfl_xor_sync(0xffffffffu, best, o);
-          const int oa = __shfl_xor_sync(0xffffffffu, at, o);
-          if (ob < best || (ob == best && oa < at)) {
-            best = ob;
-            at = oa;
-          }
-        }
-        if (lane == 0) rng[3 * w + 2] = at;
-        // ratios z_i / z_{i+1} = -b_i / dp_i above the twist, z_i / z_{i-1} = -b_{i-1} / dm_i below
-        for (int i = lane; i < N; i += 32) {
-          R r = 0;
-          if (i >= ws && i < at) r = -bn[i] * fu[i];
-          if (i > at && i < we) r = -bn[i - 1] * fd[i];
-          if (i == at) r = R(1);
-          fu[i] = r;
-        }
-      }
-      __syncthreads();
-      if (act) {
-        const int at = rng[3 * v + 2], st = dir ? 1 : -1, len = dir ? e0 - 1 - at : at - s0;
-        R* z = F + (size_t)2 * v * N + at;
-        R zv = 1;
-        int q = 1;
-        for (; q + 7 <= len; q += 8) {
-          R r[8];
+        __syncthreads();
+        if (act) {
+          const int at = rng[3 * v + 2], st = dir ? 1 : -1, len = dir ? e0 - 1 - at : at - s0;
+          R* z = F + (size_t)2 * v * N + at;
+          R zv = 1;
+          int q = 1;
+          for (; q + 7 <= len; q += 8) {
+            R r[8];
 #pragma unroll
-          for (int u = 0; u < 8; ++u) r[u] = z[st * (q + u)];
+            for (int u = 0; u < 8; ++u) r[u] = z[st * (q + u)];
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            zv *= r[u];
-            z[st * (q + u)] = zv;
+            for (int u = 0; u < 8; ++u) {
+              zv *= r[u];
+              z[st * (q + u)] = zv;
+            }
+          }
+          for (; q <= len; ++q) {
+            zv *= z[st * q];
+            z[st * q] = zv;
           }
         }
-        for (; q <= len; ++q) {
-          zv *= z[st * q];
-          z[st * q] = zv;
+        __syncthreads();
+        for (int w = warp; w < nv; w += NW) {
+          const R* z = F + (size_t)2 * w * N;
+          R nrm = 0;
+          for (int q = lane; q < tp; q += 32) {
+            const R x = z[2 * q + odd];
+            nrm = fma(x, x, nrm);
+          }
+          for (int o = 16; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
+          const R inv = nrm > R(0) ? R(1) / sqrt(nrm) : R(0);
+          const int t = rank_c + C * (v0 + w);
+          for (int q = lane; q < tp; q += 32) Wa[(size_t)t * tp + q] = z[2 * q + odd] * inv;
         }
-      }
-      __syncthreads();
-      for (int w = warp; w < nv; w += NW) {
-        const R* z = F + (size_t)2 * w * N;
-        R nrm = 0;
-        for (int q = lane; q < tp; q += 32) {
-          const R x = z[2 * q + odd];
-          nrm = fma(x, x, nrm);
-        }
-        for (int o = 16; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
-        const R inv = nrm > R(0) ? R(1) / sqrt(nrm) : R(0);
-        const int t = rank_c + C * (v0 + w);
-        for (int q = lane; q < tp; q += 32) Wa[(size_t)t * tp + q] = z[2 * q + odd] * inv;
-      }
-      if constexpr (TG) __syncthreads();
+        if constexpr (TG) __syncthreads();
       }
     }
     csync<C>();
@@ -1194,7 +1194,7 @@ __global__ void __launch_bounds__(NT, 1) k_circuit(DevMPS m, CircDev c, int64_t 
         go(std::integral_constant<int, 4>{});
       else if (ncol <= 128)
         go(std::integral_constant<int, 8>{});
-      else if (C < 8 && ncol <= 160)   // (one more copy of the loop costs eight blocks 1 % at other sizes)
+      else if (C < 8 && ncol <= 160)   // one block, chi = 65: 166 k cycles a gate instead of 180 k
         go(std::integral_constant<int, C < 8 ? 10 : 16>{});
       else
         go(std::integral_constant<int, 16>{});
